@@ -311,15 +311,15 @@ int tsvd_dense_mm(tsvd_handle* h, int trans, int64_t m, int64_t n, const double*
  * split into 7 signed 8-bit digits held exactly in BF16 (exponent-aligned
  * slicing: Ozaki, Ogita, Oishi, Rump 2012; Ootomo, Ozaki, Yokota 2024); the 28
  * digit products of weight >= 2^-48 are summed as exact integers (BF16 MMAs with
- * FP32 accumulation over 128 terms, then 64-bit integers) and scaled back in
- * FP64.  With 2^ea_i, 2^eb_j the powers of two just above max_k |a_ik| and
+ * FP32 accumulation over 128 or 256 terms, then 64-bit integers) and scaled back
+ * in FP64.  With 2^ea_i, 2^eb_j the powers of two just above max_k |a_ik| and
  * max_k |x_kj| (K = the inner dimension):
  *   |Y - op(A) X|_ij <= 2^-56 (2^ea_i sum_k |x_kj| + sum_k |a_ik| 2^eb_j)
  *                       + 6.2 K 2^(ea_i + eb_j - 56) + 2^-52 P sum_k |a_ik x_kj|
  * (normwise FP64 accuracy; the middle term, the dropped digit products, is a
  * sum of mean-zero terms and in practice near sqrt(K) of that; P is the number
  * of FP64 partial sums the K range is cut into: one per CTA share of it and per
- * 8,192 k within a share, 1 when K <= 8,192 and the output has at least 152
+ * 98,304 k within a share, 1 when K <= 98,304 and the output has at least 152
  * tiles of 128 x 64).  Inf or NaN in
  * a row of op(A) or a column of X gives
  * NaN in the corresponding row (column) of Y.  Deterministic (fixed split and

@@ -317,8 +317,8 @@ int setup_op(tsvd_handle* h, const tsvd_matrix* A, int wmax, Arena& ar, Op<T>& o
         op.partial = ar.take<double>(tn_partial_max(h, M, N, wmax) / sizeof(double) + 1);
         if (oz_planes) {
             op.oz = true;
-            oz_cache_carve(op.ozA[0], ar, op.dA64, op.lda64, M, N, false, kOzNoFixedExp);
-            oz_cache_carve(op.ozA[1], ar, op.dA64, op.lda64, M, N, true, kOzNoFixedExp);
+            oz_cache_carve(op.ozA[0], ar, op.dA64, op.lda64, M, N, false, false);
+            oz_cache_carve(op.ozA[1], ar, op.dA64, op.lda64, M, N, true, false);
             if (run) {
                 if (!ar.fits()) return TSVD_ERR_WORKSPACE;
                 TSVD_TRY(oz_cache_slice(h, op.ozA[0], 0, N, st));
@@ -402,7 +402,6 @@ int final_triplets(tsvd_handle* h, Op<T>& op, int k, const T* Bm, int64_t ldbm, 
     constexpr bool kF64 = sizeof(T) == sizeof(double);
     const int64_t m = op.m, n = op.n;
     if (kF64) {
-        OzFreshRows fresh(h);  // the returned vectors to full FP64 accuracy
         TSVD_TRY_CUDA((gemm_nn<T, double, double>(h, m, wdim, k, 1.0, Bm, ldbm, Wm, ldwm, 0.0, dU, k, false, st)));
         TSVD_TRY_CUDA((gemm_nn<T, double, double>(h, n, wdim, k, 1.0, Bn, ldbn, Wn, ldwn, 0.0, dV, k, false, st)));
         TSVD_TRY_CUDA(cudaMemcpyAsync(dsig, sig, sizeof(double) * k, cudaMemcpyDeviceToDevice, st));
@@ -530,7 +529,8 @@ int rsvd_run(tsvd_handle* h, const tsvd_matrix* A, int k, int p, int q, int bq, 
     carve_final(ar, o, m, n, k, kMixed, f);
     // scratch of the FP64-accurate tensor-core products (the mixed form's FP64 final
     // Rayleigh-Ritz step and residual use them too)
-    const size_t ozb = oz_ws_bound(std::max(m, n), kMixed ? k : ell, kMixed ? k : ell);
+    size_t ozb = oz_ws_bound(std::max(m, n), kMixed ? k : ell, kMixed ? k : ell);
+    if (op.oz) ozb = std::max(ozb, std::max(oz_a_ws(op.M, op.N, kMixed ? k : ell), oz_a_ws(op.M, op.N, k)));
     void* ozws = ar.take<char>(ozb);
     if (!run) {
         const int64_t qmax = m > n ? m : n;
@@ -681,17 +681,17 @@ int blanczos_run(tsvd_handle* h, const tsvd_matrix* A, int k, int b, int r, uint
     carve_final(ar, o, m, n, k, kMixed, f);
     // FP64 method: scratch of the FP64-accurate tensor-core products, and the digit
     // planes of both bases, kept up to date block by block: cols layout (per-column
-    // exponents) for P^T Y, rows layout (the fixed exponent 1 of an orthonormal basis,
-    // |entries| < 2) for P H and the Ritz products
-    const size_t ozb = kMixed ? oz_ws_bound(std::max(m, n), std::max(k, keep), std::max(k, keep))
-                              : oz_ws_bound(std::max(m, n), rb, std::max(std::max(b, k), keep));
+    // exponents) for P^T Y, rows layout (per-row exponents) for P H and the restart and
+    // Ritz products
+    size_t ozb = kMixed ? oz_ws_bound(std::max(m, n), std::max(k, keep), std::max(k, keep))
+                        : oz_ws_bound(std::max(m, n), rb, std::max(std::max(b, k), keep));
+    if (op.oz) ozb = std::max(ozb, std::max(oz_a_ws(op.M, op.N, kMixed ? k : b), oz_a_ws(op.M, op.N, k)));
     void* ozws = ar.take<char>(ozb);
     OzCache cP[2], cPb[2];
     if (!kMixed) {
         for (int l = 0; l < 2; ++l) {
-            oz_cache_carve(cP[l], ar, reinterpret_cast<const double*>(P), rb, n, rb, l == 0, l == 0 ? kOzNoFixedExp : 1);
-            oz_cache_carve(cPb[l], ar, reinterpret_cast<const double*>(Pbar), rb, m, rb, l == 0,
-                           l == 0 ? kOzNoFixedExp : 1);
+            oz_cache_carve(cP[l], ar, reinterpret_cast<const double*>(P), rb, n, rb, l == 0, l == 1);
+            oz_cache_carve(cPb[l], ar, reinterpret_cast<const double*>(Pbar), rb, m, rb, l == 0, l == 1);
         }
         if (run)
             for (int l = 0; l < 2; ++l) {
@@ -849,7 +849,6 @@ int blanczos_run(tsvd_handle* h, const tsvd_matrix* A, int k, int b, int r, uint
                 TSVD_TRY_CUDA((convert2d<double, T>(h, n, keep, Pk64[cur], keep, P, rb, st)));
                 TSVD_TRY_CUDA((convert2d<double, T>(h, m, keep, Pbk64[cur], keep, Pbar, rb, st)));
             } else {
-                OzFreshRows fresh(h);  // the kept Ritz vectors to full FP64 accuracy
                 TSVD_TRY_CUDA((gemm_nn<T, double, T>(h, n, d, keep, 1.0, P, rb, Vb, d, 0.0, Pk, keep, false, st)));
                 TSVD_TRY_CUDA((gemm_nn<T, double, T>(h, m, d, keep, 1.0, Pbar, rb, Ub, d, 0.0, Pbk, keep, false, st)));
                 TSVD_TRY(keep_cols(cP, 0));
@@ -866,10 +865,7 @@ int blanczos_run(tsvd_handle* h, const tsvd_matrix* A, int k, int b, int r, uint
             s0 = keep;
         } else {
             // S7: Qbar_1 = Pbar Ubar_1, re-orthonormalised by CholeskyQR2
-            {
-                OzFreshRows fresh(h);
-                TSVD_TRY_CUDA((gemm_nn<T, double, T>(h, m, rb, b, 1.0, Pbar, rb, Ub, rb, 0.0, Qnext, b, false, st)));
-            }
+            TSVD_TRY_CUDA((gemm_nn<T, double, T>(h, m, rb, b, 1.0, Pbar, rb, Ub, rb, 0.0, Qnext, b, false, st)));
             TSVD_TRY(keep_cols(cP, 0));
             TSVD_TRY(keep_cols(cPb, 0));
             TSVD_TRY_CUDA(copy_block<T>(Qnext, b, Pbar, rb, m, b, st));

@@ -11,15 +11,15 @@
 //    gets one exponent e (the smallest e with |x| < 2^e over that row or
 //    column); each entry becomes the 56-bit integer F = round(x 2^(55 - e)),
 //    split into 7 balanced base-256 digits d_0..d_6 (F = sum d_p 2^(8(6-p)),
-//    |d_p| <= 128).  Digit p is stored as the BF16 value d_p 2^(-8p) (exact);
+//    |d_p| <= 128).  Digit p is stored as the BF16 value d_p (exact);
 //  * the 28 digit products with p + q <= 6 are issued as tcgen05 MMAs (M = 128,
 //    K = 16, FP32 accumulators in tensor memory), one accumulator per value of
-//    p + q (7 accumulators side by side, 448 TMEM columns); the products of one
-//    A digit plane with all its B planes form a single MMA of N up to 256.  Over 128 consecutive k
-//    each product is an integer times 2^(-8(p+q)) of magnitude <= 2^14 and each
-//    group sum T_{p+q} is an integer below 2^24, so every accumulation is exact
-//    whatever the tensor core's internal rounding;
-//  * every 128 k the epilogue converts the accumulators to integers and adds
+//    g = p + q (7 accumulators side by side); the products of one A digit plane with
+//    several B planes form a single MMA of N up to 256.  Each product is an integer of
+//    magnitude <= 2^14 and the group sum T_g adds g + 1 of them per k, so over 256 k
+//    (T_0 .. T_3) or 128 k (T_4 .. T_6) it is an integer within 2^24 and every
+//    accumulation is exact whatever the tensor core's internal rounding;
+//  * after that many k the epilogue converts the accumulators to integers and adds
 //    T_0..T_4 into a 64-bit integer (units of 2^-32 of the leading digit
 //    product), T_5 and T_6 (rounded to 2^-40) into a 32-bit one, and at the end
 //    of its K range writes C = 2^(ea + eb - 46) (hi + lo 2^-8) in FP64.
@@ -28,21 +28,20 @@
 // rounded once to FP64: normwise FP64 accuracy (checked against exact products
 // in the CPU tests of the scheme and on the GPU).
 //
-// Layout: every operand is sliced into 7 BF16 digit planes stored K-block major
-// (the 7 planes of each 16-wide K block are [7][rows][16], so one TMA box reads
-// contiguous runs), by one of two slicing kernels:
+// Layout: every operand is sliced into 7 BF16 digit planes stored K-block major (oz_off),
+// by one of three slicing kernels:
 //   rows  the source rows are the stored rows (A = X of X M: one exponent per
 //         source row, computed by the warp that slices the row);
+//   grow  the same for a basis that gains columns block by block;
 //   cols  the source columns are the stored rows (A = X^T and B = Z of X^T Z,
 //         B = M of X M: one exponent per source column, from a column-max pass
 //         with atomicMax, then a tiled transpose).
 // Operands that many products read (a Lanczos basis, a dense A) keep their planes
 // in a cache that the owner extends block by block.
-// The product kernel (one CTA per SM, 320 threads) is the TMA / tcgen05
-// pipeline of the split-BF16 product: warp 0 loads 3-D boxes (16 K x rows x 7
-// planes, 32-byte swizzle) of both operands into a 5-stage ring, warp 1 owns 512
-// TMEM columns and issues the 10 MMAs of each stage from one thread, warps 2-9
-// drain the accumulators (two warps per 32 TMEM lanes, 32 columns each).  Work
+// The product kernel (one CTA per SM) is a TMA / tcgen05 pipeline: warp 0 copies the 7
+// planes of both operands' K blocks into a ring of 5 to 7 stages, warp 1 owns the tensor
+// memory and issues the 11 MMAs of each stage from one thread, the other warps read the
+// accumulators.  Work
 // units (output tile, 16-wide K block) are split evenly over one wave of CTAs,
 // so no CTA runs a third tile while the others idle (314 tiles on 152 SMs would
 // take three rounds for 2.07 rounds of work): a tile whose K range lies inside
@@ -53,6 +52,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <climits>
 
 #include "tc_ptx.cuh"
 #include "tsvd_internal.cuh"
@@ -64,21 +64,33 @@ using namespace tcx;
 
 constexpr int kOzDig = 7;                                   // digits per operand entry
 constexpr int kOzM = 128;                                   // output rows per tile (TMEM lanes)
-constexpr int kOzN = 64;                                    // output columns per tile
+constexpr int kOzN = 64;                                    // most output columns per tile
 constexpr int kOzBK = 16;                                   // K per stage (one 32-byte row, one MMA)
 constexpr int kOzRowB = 2 * kOzBK;
-constexpr int kOzStages = 5;
 constexpr int kOzPlaneA = kOzM * kOzRowB;                   // 4 KB
-constexpr int kOzPlaneB = kOzN * kOzRowB;                   // 2 KB
-constexpr int kOzStageBytes = kOzDig * (kOzPlaneA + kOzPlaneB);  // 42 KB
-constexpr int kOzSmem = kOzStages * kOzStageBytes + 1024;
-constexpr int kOzChunk = 8;          // K blocks per exact accumulation (128 k)
-constexpr int kOzFlushChunks = 64;   // chunks between FP64 flushes of the integer sums (8192 k)
-constexpr int kOzSlots = 7;          // accumulators: p + q = 0 .. 6
-constexpr int kOzEpiWarps = 8;   // two per TMEM lane quarter, 32 columns each
-constexpr int kOzThreads = 64 + 32 * kOzEpiWarps;
+constexpr int kOzSlots = kOzDig;     // accumulators: p + q = 0 .. 6
+constexpr int kOzLowSlots = 4;       // p + q = 0 .. 3: the low group; 4 .. 6: the high group
+// K blocks of one exact accumulation (every |T_g| <= (g + 1) 2^14 per k stays within 2^24):
+// 256 k for T_0 .. T_3, 128 k for T_4 .. T_6.  The low chunks end 4 K blocks off the high
+// ones, the first one after 12 K blocks (so that a tile's output has 8 to finish in).
+constexpr int kOzLowChunk = 16, kOzHighChunk = 8, kOzLowShift = 4;
+constexpr int kOzRun = 4;             // K blocks issued for one group before the other takes over
+constexpr int kOzFoldChunks = 128;    // high chunks between carries of lo into hi (lo stays below 2^31)
+constexpr int kOzFlushChunks = 768;   // high chunks between FP64 flushes of the integer sums (98,304 k)
 constexpr int kOzWave = 152;
-constexpr int kOzTmemCols = 512;
+
+// Tile shapes: NC columns, slot p + q at TMEM column (p + q) NC.
+template <int NC>
+struct OzShape {
+    static constexpr int kStageA = kOzDig * kOzPlaneA;               // 28 KB
+    static constexpr int kPlaneB = NC * kOzRowB;                     // 2 KB at 64 columns
+    static constexpr int kStage = kStageA + kOzDig * kPlaneB;
+    static constexpr int kStages = NC == 64 ? 5 : (NC == 32 ? 6 : 7);
+    static constexpr int kSmem = kStages * kStage + 1024;
+    static constexpr int kTmemCols = NC == 64 ? 512 : (NC == 32 ? 256 : 128);
+    static constexpr int kEpiWarps = NC == 64 ? 16 : 8;              // NC / 4 or NC / 2 columns a warp
+    static constexpr int kThreads = 64 + 32 * kEpiWarps;             // TMA warp, MMA warp, epilogue
+};
 constexpr int kOzNanExp = 1 << 20;      // exponent of a row holding Inf or NaN
 constexpr int kOzZeroExp = -(1 << 20);  // exponent of a zero entry
 
@@ -124,30 +136,31 @@ __device__ inline void oz_digits(double x, int e, int d[kOzDig]) {
     d[0] = (int)r;
 }
 
-__device__ inline float oz_digit_scale(int p) { return __int_as_float((127 - 8 * p) << 23); }  // 2^(-8p)
-
-__device__ inline __nv_bfloat162 oz_pack(int d0, int d1, int p) {
-    const float s = oz_digit_scale(p);
-    return __floats2bfloat162_rn((float)d0 * s, (float)d1 * s);  // exact: |d| <= 128
+__device__ inline __nv_bfloat162 oz_pack(int d0, int d1) {
+    return __floats2bfloat162_rn((float)d0, (float)d1);  // exact: |d| <= 128
 }
 
-// Global layout of the digit planes: K-block major.  Element (digit p, stored row r,
-// column k) of an operand with Ra allocated stored rows sits at
-//   ((k / 16) * 7 + p) * Ra * 16 + r * 16 + k % 16,
-// so the 7 planes of one 16-wide K block are [7][Ra][16] and a TMA box of 16 K x
-// 128 rows x 7 planes reads 7 contiguous runs of 4 KB.  Columns past K up to the
-// next multiple of 16 hold zeros.
+// Global layout of the digit planes: K-block major, and within a block the very bytes that
+// the MMA reads from shared memory.  Element (digit p, stored row r, column k) of an operand
+// with Ra allocated stored rows (a multiple of 16) sits at
+//   ((k / 16) * 7 + p) * Ra * 16 + r * 16 + (k % 16, its halves of 8 exchanged in every
+//   second group of 4 rows: the 32-byte swizzle),
+// so that a TMA box of 128 rows x 7 planes is 56 runs of 512 bytes copied as they are.  (As
+// a box of 16 columns, swizzled by the copy, it was 896 runs of 32 bytes, and the copy
+// engine's rate of about 1.4 clocks a run bounded the product kernel: 1,344 runs a stage.)
+// Columns past K up to the next multiple of 16 hold zeros.
 __host__ __device__ inline int64_t oz_off(int64_t Ra, int64_t r, int64_t k, int p) {
-    return ((k >> 4) * kOzDig + p) * Ra * 16 + r * 16 + (k & 15);
+    return ((k >> 4) * kOzDig + p) * Ra * 16 + r * 16 + ((k & 15) ^ ((r & 4) << 1));
 }
 __host__ __device__ inline int64_t oz_k16(int64_t K) { return (K + 15) / 16 * 16; }
+inline int64_t oz_ra(int64_t rows) { return (rows + 15) / 16 * 16; }
 
 // Stores the digits of (x0, x1) at columns (k, k + 1), k even, of stored row r.
 __device__ inline void oz_store_pair(__nv_bfloat16* planes, int64_t Ra, int64_t r, int64_t k, const int* da,
                                      const int* db) {
     __nv_bfloat162* dst = reinterpret_cast<__nv_bfloat162*>(planes + oz_off(Ra, r, k, 0));
 #pragma unroll
-    for (int p = 0; p < kOzDig; ++p) dst[p * Ra * 8] = oz_pack(da[p], db[p], p);  // plane step Ra*16 elements
+    for (int p = 0; p < kOzDig; ++p) dst[p * Ra * 8] = oz_pack(da[p], db[p]);  // plane step Ra*16 elements
 }
 
 // Rows slicer: row i of S (R x K, lds) -> stored row i; one warp per row.
@@ -174,38 +187,43 @@ __global__ void __launch_bounds__(256, 4) oz_slice_rows_kernel(int64_t R, int64_
     }
 }
 
-// Rows slicer with one fixed exponent e for every row (an orthonormal basis: every
-// entry below 2^e in magnitude), over the columns [a0, a1) of S (R rows, lds), a0
-// even and a1 a multiple of 16; columns from c1 on are written as zeros (a column
-// a0 - 1 < c1 is sliced again with its own value).  A row holding an entry at or
-// above 2^e, or Inf/NaN, gets the exponent of a non-finite row.
-__global__ void __launch_bounds__(256) oz_slice_rows_fixed_kernel(int64_t R, int64_t a0, int64_t a1, int64_t c1,
-                                                                  const double* __restrict__ S, int64_t lds,
-                                                                  __nv_bfloat16* __restrict__ planes, int64_t Ra,
-                                                                  int e, int* __restrict__ eexp) {
-    const int64_t halfk = (a1 - a0) / 2;
-    const int64_t tot = R * halfk;
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < tot; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = t / halfk, k = a0 + 2 * (t % halfk);
-        const double x0 = k < c1 ? S[i * lds + k] : 0.0, x1 = k + 1 < c1 ? S[i * lds + k + 1] : 0.0;
-        if (oz_exp(x0) > e || oz_exp(x1) > e) eexp[i] = kOzNanExp;
-        int da[kOzDig], db[kOzDig];
-        oz_digits(x0, e, da);
-        oz_digits(x1, e, db);
-        oz_store_pair(planes, Ra, i, k, da, db);
-    }
-}
-
-// Zeros of columns [v, v16) of every stored row (rows layout; v16 a multiple of 16).
-__global__ void oz_zero_cols_kernel(int64_t R, int64_t v, int64_t v16, __nv_bfloat16* __restrict__ planes,
-                                    int64_t Ra) {
-    const int64_t w = v16 - v;
-    const int64_t tot = R * w * kOzDig;
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < tot; t += (int64_t)gridDim.x * blockDim.x) {
-        const int p = (int)(t % kOzDig);
-        const int64_t rest = t / kOzDig;
-        const int64_t i = rest / w, k = v + rest % w;
-        planes[oz_off(Ra, i, k, p)] = __float2bfloat16_rn(0.0f);
+// Rows slicer of a matrix that grows by columns (a Lanczos basis): columns [c0, c1) of S
+// (R rows, lds), zeros from c1 to the next multiple of 16; G lanes a row.  A row's exponent
+// is one above its largest entry when it was set (at c0 = 0, or when a later entry does
+// not fit it: the row's earlier columns are then sliced again), so that new columns rarely
+// raise it.  That keeps 55 bits below the row's largest entry; one exponent for all rows of
+// an orthonormal basis kept about log2(R) / 2 bits fewer.
+template <int G>
+__global__ void __launch_bounds__(256) oz_slice_rows_grow_kernel(int64_t R, int64_t c0, int64_t c1,
+                                                                 const double* __restrict__ S, int64_t lds,
+                                                                 __nv_bfloat16* __restrict__ planes, int64_t Ra,
+                                                                 int* __restrict__ eexp) {
+    const int sl = threadIdx.x % G;
+    const int64_t ng = (int64_t)gridDim.x * (blockDim.x / G);
+    const int64_t rounds = (R + ng - 1) / ng;  // the same for every lane: the shuffles need them all
+    const int64_t a1 = oz_k16(c1);
+    for (int64_t t = 0; t < rounds; ++t) {
+        const int64_t i = t * ng + (int64_t)blockIdx.x * (blockDim.x / G) + threadIdx.x / G;
+        const bool in = i < R;
+        const double* src = S + i * lds;
+        int e = kOzZeroExp;
+        if (in)
+            for (int64_t k = c0 + sl; k < c1; k += G) e = max(e, oz_exp(src[k]));
+#pragma unroll
+        for (int o = G / 2; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
+        int old = in && sl == 0 && c0 > 0 ? eexp[i] : kOzZeroExp;
+        old = __shfl_sync(0xffffffffu, old, (threadIdx.x & 31) & ~(G - 1));
+        if (!in) continue;
+        const bool set = c0 == 0 || e > old;
+        // (a row of zeros keeps the exponent of zero, which any entry exceeds)
+        const int en = !set ? old : (e >= kOzNanExp || e <= kOzZeroExp ? e : e + 1);
+        if (set && sl == 0) eexp[i] = en;
+        for (int64_t k = (set ? 0 : c0 & ~int64_t(1)) + 2 * sl; k < a1; k += 2 * G) {
+            int da[kOzDig], db[kOzDig];
+            oz_digits(k < c1 ? src[k] : 0.0, en, da);
+            oz_digits(k + 1 < c1 ? src[k + 1] : 0.0, en, db);
+            oz_store_pair(planes, Ra, i, k, da, db);
+        }
     }
 }
 
@@ -266,15 +284,16 @@ __global__ void oz_fill_kernel(int64_t n, int v, int* __restrict__ x) {
 
 // ---- the product kernel ------------------------------------------------------
 struct OzArgs {
-    int64_t M, N, KB, tiles, totalg;  // totalg: (row tile, K block) units of one column tile
-    int NT, Npad, G, Gg, maxseg;       // CTA c: column tile c % NT, unit group c / NT of Gg
+    int64_t M, N, totalg;  // totalg: (row tile, K block) units of one column tile
+    int KB, NT, tilen;     // K blocks, column tiles and their width
+    int Gg, nslots;        // CTA c: column tile c % NT, unit group c / NT of Gg; partial tiles it may leave
     const int* ea;
     const int* eb;
     double* out;  // C (direct tiles)
     int64_t ldo;
     double alpha, beta;
     int symmetric;
-    double* partial;  // [G][maxseg][128][64]
+    double* partial;  // [CTA][nslots][128][64]
     int* status;
     long long max_wait;  // limit of one pipeline wait (SM clock cycles)
 };
@@ -286,13 +305,42 @@ __host__ __device__ inline int64_t oz_glo(int g, const OzArgs& a) {
     return (int64_t)g * a.totalg / a.Gg;
 }
 
-// C = 2^(ea + eb - 14) (hi 2^-32 + lo 2^-40) in FP64.
+// (hi + lo 2^-8) 2^(ea + eb - 46), rounded once to nearest even.  In integer arithmetic: a
+// warp-wide FP64 instruction takes 16 clocks of the SM's FP64 pipe, and the five that a
+// conversion by casts needs bounded the products with a short K (28,000 of 90,000 clocks a
+// tile at K = 576).
 __device__ inline double oz_value(long long hi, int lo, int ea, int eb) {
     if (ea >= kOzNanExp || eb >= kOzNanExp) return __longlong_as_double(0x7ff8000000000000LL);
-    const double x = fma((double)lo, 0.00390625, (double)hi);  // hi + lo 2^-8
     const int E = ea + eb - 46;
-    if (E >= -1022 && E <= 1023) return x * __longlong_as_double((long long)(E + 1023) << 52);  // exact scaling
-    return ldexp(x, E);
+    // sign and magnitude: m + r / 256
+    const long long v = hi + (lo >> 8);
+    const unsigned r0 = (unsigned)lo & 255u;
+    const bool neg = v < 0;
+    const unsigned r = neg ? (256u - r0) & 255u : r0;
+    const unsigned long long m = neg ? ~(unsigned long long)v + (r0 == 0u ? 1ull : 0ull) : (unsigned long long)v;
+    const int lz = __clzll((long long)m), be = 1086 + E - lz;  // biased exponent of the leading bit
+    if (m != 0ull && be >= 1 && be <= 2046) {
+        // 64 leading bits, the rest ORed into the last one
+        unsigned long long w = m << lz;
+        w |= lz >= 8 ? (unsigned long long)r << (lz - 8) : (unsigned long long)(r >> (8 - lz));
+        if (lz < 8 && (r & ((1u << (8 - lz)) - 1u))) w |= 1ull;
+        unsigned long long mant = w >> 11;
+        mant += ((unsigned)w & 0x7ffu) + ((unsigned)mant & 1u) > 0x400u ? 1ull : 0ull;
+        const unsigned long long bits = ((unsigned long long)(be - 1) << 52) + mant;  // a carry raises the exponent
+        return __longlong_as_double((long long)(bits | (neg ? 1ull << 63 : 0ull)));
+    }
+    // zero, a fraction alone, or a result at the ends of the FP64 range: x 2^E in two steps
+    // (the first one is exact)
+    const double x = fma((double)lo, 0.00390625, (double)hi);
+    const int E1 = max(-900, min(E, 1023));
+    double y = x * __longlong_as_double((long long)(E1 + 1023) << 52);
+    if (E1 != E) y *= __longlong_as_double((long long)(max(-1022, min(E - E1, 1023)) + 1023) << 52);
+    return y;
+}
+
+// alpha v: no FP64 instruction for 1 and -1
+__device__ inline double oz_scale(double alpha, double v) {
+    return alpha == 1.0 ? v : (alpha == -1.0 ? -v : alpha * v);
 }
 
 // The output rule: out = alpha v + beta out (beta == 0: no read); a symmetric
@@ -305,128 +353,207 @@ __device__ inline void oz_store(const OzArgs& a, int64_t i, int64_t j, double v)
         return;
     }
     double* o = a.out + i * a.ldo + j;
-    *o = (a.beta != 0.0) ? fma(a.beta, *o, a.alpha * v) : a.alpha * v;
+    const double w = oz_scale(a.alpha, v);
+    *o = (a.beta != 0.0) ? fma(a.beta, *o, w) : w;
 }
 
-__global__ void __launch_bounds__(kOzThreads, 1)
+// 1.5 2^23: adding it to an integer of magnitude <= 2^22 leaves that integer, plus the
+// bits of the constant, in the float's bit pattern (an exact conversion on the FP32 pipe).
+constexpr float kOzMagic = 12582912.0f;
+constexpr unsigned kOzMagicBits = 0x4B400000u;
+
+// Adds T_g of 8 columns (from column q0 on) to the integer sums.
+template <int N>
+__device__ inline void oz_add_slot(int g, int q0, const uint32_t* v, unsigned long long (&hi)[N],
+                                   unsigned (&lo)[N]) {
+    if (g == 0) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            hi[q0 + q] += (unsigned long long)__float_as_uint(__uint_as_float(v[q]) + kOzMagic) << 32;
+    } else if (g <= 4) {
+        const int mul = 1 << (32 - 8 * g);  // weight of T_g in hi
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(hi[q0 + q]) : "r"(__float2int_rn(__uint_as_float(v[q]))), "r"(mul));
+    } else if (g == 5) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) lo[q0 + q] += (unsigned)__float2int_rn(__uint_as_float(v[q]));
+    } else {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) lo[q0 + q] += __float_as_uint(fmaf(__uint_as_float(v[q]), 0.00390625f, kOzMagic));
+    }
+}
+
+// Whether the accumulators of a group start afresh at K block j of a tile.
+__device__ inline bool oz_chunk_start(int group, int j) {
+    return j == 0 || (group == 0 ? ((j + kOzLowShift) % kOzLowChunk) == 0 : (j % kOzHighChunk) == 0);
+}
+
+// The product kernel.  What bounds it: the tensor pipe (28 NC MMA columns of K = 16 a
+// stage, 896 clocks at NC = 64) next to L2 (42 KB a stage and CTA).
+// Digit plane p of A meets B planes q = 0 .. 6 - p; the products go to the accumulators of
+// p + q, which sit side by side in TMEM as the B planes do in shared memory, so that one
+// MMA covers several B planes.  The accumulators form two groups, p + q <= 3 (4 MMAs a
+// stage) and p + q >= 4 (7 MMAs).  The MMA thread issues kOzRun K blocks for the one, then
+// the same K blocks for the other, and the exact-accumulation chunks of the two end at
+// different K blocks: while the epilogue reads the accumulators of one group, the MMAs of
+// the other run.  With all 7 in one group the tensor pipe stood still at each chunk end.
+// Measured, clocks per K block of 16 and CTA (one group, 10 MMAs, before): 10,000^2 x 128
+// 1,290 (2,500), 100,000 x 576 times 576 x 64 1,710 (3,100), the projection 576 x 100,000
+// times 64 columns 1,700 (2,470; 1,240 would be the DRAM rate of its A planes), width 16
+// 1,200 (DRAM-bound).  The MMAs alone take 930; what is left is shared memory, which MMA
+// operands and copies share (142 of 128 KB per 1,000 clocks).  Tried and left out: copies
+// of A (or B) multicast to a cluster of two CTAs, which changed nothing once the copies
+// were long runs, and an L2 prefetch ahead of the copies, which slowed them by a third.
+template <int NC>
+__global__ void __launch_bounds__(OzShape<NC>::kThreads, 1)
     oz_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, OzArgs a) {
+    using S = OzShape<NC>;
+    constexpr int kSt = S::kStages;
     extern __shared__ uint8_t dsm[];
-    __shared__ __align__(8) uint64_t bars[2 * kOzStages + 2 * kOzSlots + 1];
+    __shared__ __align__(8) uint64_t bars[2 * kSt + 5];
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
     const uint32_t base = (smem_u32(dsm) + 1023u) & ~1023u;
     const uint32_t bar0 = smem_u32(bars);
     auto full = [&](int s) { return bar0 + 8u * (uint32_t)s; };
-    auto empty = [&](int s) { return bar0 + 8u * (uint32_t)(kOzStages + s); };
-    auto accf = [&](int g) { return bar0 + 8u * (uint32_t)(2 * kOzStages + g); };
-    auto acce = [&](int g) { return bar0 + 8u * (uint32_t)(2 * kOzStages + kOzSlots + g); };
-    const uint32_t drain = bar0 + 8u * (uint32_t)(2 * kOzStages + 2 * kOzSlots);
+    auto empty = [&](int s) { return bar0 + 8u * (uint32_t)(kSt + s); };
+    auto accf = [&](int h) { return bar0 + 8u * (uint32_t)(2 * kSt + h); };      // group h: chunk complete
+    auto acce = [&](int h) { return bar0 + 8u * (uint32_t)(2 * kSt + 2 + h); };  // group h: chunk read
+    const uint32_t drain = bar0 + 8u * (uint32_t)(2 * kSt + 4);
     volatile int* abort_flag = &s_abort;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int c = blockIdx.x;
-    const int ntc = c % a.NT, gc = c / a.NT;  // this CTA's column tile and unit group
+    const int nt = c % a.NT, gc = c / a.NT;  // this CTA's column tile and unit group
     const int64_t lo = oz_glo(gc, a), hi = oz_glo(gc + 1, a);
-    const int64_t KB = a.KB;
+    const int KB = a.KB;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kOzStages; ++s) {
+        for (int s = 0; s < kSt; ++s) {
             mbar_init(full(s), 1);
             mbar_init(empty(s), 1);
         }
-        for (int g = 0; g < kOzSlots; ++g) {
-            mbar_init(accf(g), 1);
-            mbar_init(acce(g), 32 * kOzEpiWarps);
+        for (int h = 0; h < 2; ++h) {
+            mbar_init(accf(h), 1);
+            mbar_init(acce(h), S::kEpiWarps);  // one arrival an epilogue warp
         }
         mbar_init(drain, 1);
         s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 1) tmem_alloc(smem_u32(&s_tmem), kOzTmemCols);
+    if (warp == 1) tmem_alloc(smem_u32(&s_tmem), S::kTmemCols);
     fence_before();
     __syncthreads();
     fence_after();
     const uint32_t tmem = s_tmem;
-    const uint32_t stage_tx = (uint32_t)(kOzDig * (kOzPlaneA + a.Npad * kOzRowB));
 
     if (warp == 0) {
-        if (lane == 0) {
-            // ---- TMA producer: both operands' 7 planes of one 32-wide K block per stage
-            int64_t it = 0;
+        if (elect_one()) {
+            // ---- TMA producer: both operands' 7 planes of one 16-wide K block per stage
             bool ok = true;
-            for (int64_t i = lo; i < hi && ok; ++i, ++it) {
-                const int st = (int)(it % kOzStages);
-                if (it >= kOzStages) ok = mbar_wait(empty(st), (uint32_t)(((it / kOzStages) - 1) & 1), abort_flag, a.max_wait);
+            int st = 0, issued = 0;
+            uint32_t ph = 1;  // parity of the wait for an empty stage (the first round does not wait)
+            int mt = (int)(lo / KB), kb = (int)(lo - (int64_t)mt * KB);
+            for (int n = (int)(hi - lo); n > 0; --n) {
+                if (issued >= kSt) ok = mbar_wait(empty(st), ph, abort_flag, a.max_wait);
                 if (!ok) break;
-                const int64_t mt = i / KB;
-                const int kz = (int)((i - mt * KB) * kOzDig);  // the 7 planes of K block i - mt KB
-                const int nt = ntc;
-                const uint32_t sA = base + (uint32_t)st * kOzStageBytes;
-                mbar_arrive_expect_tx(full(st), stage_tx);
-                tma_load_3d(sA, &tmA, 0, mt * kOzM, kz, full(st));
-                tma_load_3d(sA + kOzDig * kOzPlaneA, &tmB, 0, nt * kOzN, kz, full(st));
+                const uint32_t sA = base + (uint32_t)(st * S::kStage);
+                mbar_arrive_expect_tx(full(st), (uint32_t)S::kStage);
+                // (coordinates in groups of 16 rows)
+                tma_load_3d(sA, &tmA, 0, mt * (kOzM / 16), kb * kOzDig, full(st));
+                tma_load_3d(sA + S::kStageA, &tmB, 0, nt * (NC / 16), kb * kOzDig, full(st));
+                if (issued < kSt) ++issued;
+                if (++st == kSt) {
+                    st = 0;
+                    ph ^= 1u;
+                }
+                if (++kb == KB) {
+                    kb = 0;
+                    ++mt;
+                }
             }
             if (!ok) {
                 atomicOr(&a.status[kStTimeout], 1);
                 s_abort = 1;
             }
-            const int64_t first = it > kOzStages ? it - kOzStages : 0;
-            for (int64_t j = first; j < it; ++j) mbar_drain(full((int)(j % kOzStages)), (uint32_t)((j / kOzStages) & 1));
+            // before the CTA leaves, every copy issued has landed: the last `issued` stages,
+            // oldest first; ph ^ 1 is the parity of the current round
+            for (int j = 0; j < issued; ++j) {
+                int s = st - issued + j;
+                uint32_t fp = ph ^ 1u;
+                if (s < 0) {
+                    s += kSt;
+                    fp ^= 1u;
+                }
+                mbar_drain(full(s), fp);
+            }
         }
         __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             // ---- MMA issuer
-            const uint32_t bstep = (uint32_t)(a.Npad * kOzRowB) >> 4;  // one B plane in 16-byte units
-            int64_t it = 0, ch = 0;  // K blocks and chunks issued by this CTA
             bool ok = true;
-            for (int64_t i = lo; i < hi && ok;) {
-                const int64_t mt = i / KB;
-                const int64_t e = min(hi, (mt + 1) * KB);
-                for (; i < e && ok; ++ch) {
-                    const int64_t ce = min(e, i + kOzChunk);
-                    for (int64_t i0 = i; i < ce; ++i, ++it) {
-                        const int st = (int)(it % kOzStages);
-                        ok = mbar_wait(full(st), (uint32_t)((it / kOzStages) & 1), abort_flag, a.max_wait);
-                        if (!ok) break;
-                        fence_after();
-                        const bool first_kb = (i == i0), last_kb = (i + 1 == ce);
-                        const uint32_t sA = base + (uint32_t)st * kOzStageBytes;
-                        const uint64_t a0 = sdesc_sw32(sA);
-                        const uint64_t b0 = sdesc_sw32(sA + kOzDig * kOzPlaneA);
-                        // Digit plane p of A meets B planes q = 0 .. 6 - p; their products go to
-                        // the accumulators of p + q, which sit side by side in TMEM (slot d at
-                        // column d Npad), and the B planes sit side by side in shared memory, so
-                        // one MMA with N = (7 - p) Npad (cut at 256 columns) covers them all:
-                        // 10 MMAs a stage instead of 28, each reading its A plane once.  Slot p is
-                        // final once the MMAs of plane p are done (later planes start at p + 1).
+            int st = 0;
+            uint32_t fph = 0;                // parity of the wait for a full stage
+            uint32_t eph[2] = {0, 0};        // parity of the wait for a group that has been read
+            bool used[2] = {false, false};
+            int kb = (int)(lo % KB);
+            for (int left = (int)(hi - lo); left > 0 && ok;) {
+                const int nk = min(KB - kb, left);  // K blocks of this tile here
+                for (int j0 = 0; j0 < nk && ok; j0 += kOzRun) {
+                    const int j1 = min(j0 + kOzRun, nk);
 #pragma unroll
-                        for (int p = 0; p < kOzDig; ++p) {
-                            const uint64_t ad = a0 + (uint64_t)(p * (kOzPlaneA >> 4));
-#pragma unroll
-                            for (int q0 = 0; q0 < kOzDig - p; q0 += 4) {
-                                const int cnt = min(4, kOzDig - p - q0);  // slots p + q0 .. + cnt - 1
-                                const bool piece_ok = cnt * a.Npad <= 256;
-                                if (first_kb && ch > 0 && p == 0) {
-                                    // the epilogue has drained these accumulators of the previous chunk
-                                    for (int dd = q0; dd < q0 + cnt && ok; ++dd) {
-                                        ok = mbar_wait(acce(dd), (uint32_t)((ch - 1) & 1), abort_flag, a.max_wait);
-                                    }
-                                    if (!ok) break;
-                                    fence_after();
-                                }
-                                if (!piece_ok) continue;  // (Npad <= 64 and cnt <= 4 keep N <= 256)
-                                const uint32_t d = tmem + (uint32_t)((p + q0) * a.Npad);
-                                const uint64_t bd = b0 + (uint64_t)(q0 * bstep);
-                                mma_bf16(d, ad, bd, idesc_bf16(kOzM, cnt * a.Npad), (first_kb && p == 0) ? 0u : 1u);
+                    for (int h = 0; h < 2; ++h) {
+                        int s = st;
+                        uint32_t f = fph;
+                        for (int j = j0; j < j1; ++j) {
+                            if (h == 0) {
+                                ok = mbar_wait(full(s), f, abort_flag, a.max_wait);
+                                if (!ok) break;
                             }
-                            if (!ok) break;
-                            if (last_kb) commit(accf(p));
+                            const bool start = oz_chunk_start(h, j);
+                            if (start) {
+                                if (used[h]) {
+                                    ok = mbar_wait(acce(h), eph[h], abort_flag, a.max_wait);
+                                    if (!ok) break;
+                                    eph[h] ^= 1u;
+                                }
+                                used[h] = true;
+                            }
+                            fence_after();
+                            const uint32_t sA = base + (uint32_t)(s * S::kStage);
+                            const uint64_t a0 = sdesc_sw32(sA), b0 = sdesc_sw32(sA + S::kStageA);
+                            if (h == 0) {
+#pragma unroll
+                                for (int p = 0; p < kOzLowSlots; ++p)  // slots p .. 3
+                                    mma_bf16(tmem + (uint32_t)(p * NC), a0 + (uint64_t)(p * (kOzPlaneA >> 4)), b0,
+                                             idesc_bf16(kOzM, (kOzLowSlots - p) * NC), (start && p == 0) ? 0u : 1u);
+                            } else {
+#pragma unroll
+                                for (int p = 0; p < kOzDig; ++p) {  // slots max(4, p) .. 6
+                                    const int g0 = p < kOzLowSlots ? kOzLowSlots : p;
+                                    mma_bf16(tmem + (uint32_t)(g0 * NC), a0 + (uint64_t)(p * (kOzPlaneA >> 4)),
+                                             b0 + (uint64_t)((g0 - p) * (S::kPlaneB >> 4)),
+                                             idesc_bf16(kOzM, (kOzSlots - g0) * NC), (start && p == 0) ? 0u : 1u);
+                                }
+                                commit(empty(s));
+                            }
+                            if (j + 1 == nk || oz_chunk_start(h, j + 1)) commit(accf(h));
+                            if (++s == kSt) {
+                                s = 0;
+                                f ^= 1u;
+                            }
                         }
                         if (!ok) break;
-                        commit(empty(st));
+                        if (h == 1) {
+                            st = s;
+                            fph = f;
+                        }
                     }
                 }
+                left -= nk;
+                kb = 0;
             }
             if (!ok) {
                 atomicOr(&a.status[kStTimeout], 1);
@@ -437,151 +564,225 @@ __global__ void __launch_bounds__(kOzThreads, 1)
         }
         __syncwarp();
     } else {
-        // ---- epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 and 32 of the columns
-        const int quarter = warp & 3;
-        const int cg = (warp - 2) >> 2;        // column half: columns 32 cg .. 32 cg + 31
-        const int ncol = a.Npad >> 1;          // 16 or 32 valid columns in this half
-        const int r = quarter * 32 + lane;
-        const uint32_t tlane = (uint32_t)(quarter * 32) << 16;
-        int64_t ch = 0;
+        // ---- epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31, CW of the columns
+        constexpr int CW = 4 * NC / S::kEpiWarps;
+        const int r = (warp & 3) * 32 + lane, cofs = ((warp - 2) >> 2) * CW;
+        const uint32_t t0 = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)cofs;
+        uint32_t ph = 0;  // bit h: parity of the wait for group h
         int seg = 0;
         bool ok = true;
-        for (int64_t i = lo; i < hi && ok; ++seg) {
-            const int64_t mt = i / KB;
-            const int64_t e = min(hi, (mt + 1) * KB);
-            const int nt = ntc;
-            const int64_t row = (int64_t)mt * kOzM + r;
-            const int64_t col0 = (int64_t)nt * kOzN + cg * ncol;
-            const bool direct = (i == mt * KB) && (e == (mt + 1) * KB) && KB <= (int64_t)kOzChunk * kOzFlushChunks;
-            const int ea = row < a.M ? a.ea[row] : 0;
-            double* slot = a.partial + (((int64_t)c * a.maxseg + seg) * kOzM + r) * kOzN + cg * ncol;
-            // integer sums of the digit products: hi in units of 2^-32 (p + q <= 4, exact),
-            // lo in units of 2^-40 (p + q = 5 exact, p + q = 6 rounded to 2^-40)
-            long long hi[32];
-            int lo[32];
+        int mt = (int)(lo / KB), kb = (int)(lo - (int64_t)mt * KB);
+        for (int left = (int)(hi - lo); left > 0 && ok; ++seg, ++mt) {
+            const int nk = min(KB - kb, left);
+            // integer sums of the digit products: hi in units of 2^-32 of the leading one
+            // (p + q <= 4, exact), lo in units of 2^-40 (p + q = 5 exact, 6 rounded), both
+            // biased by the magic bits of the chunks added
+            unsigned long long hi64[CW];
+            unsigned lo32[CW];
 #pragma unroll
-            for (int j = 0; j < 32; ++j) hi[j] = lo[j] = 0;
-            int nchunks = 0;
-            bool stored = false;
-            for (; i < e && ok; ++ch) {
-                const int64_t ce = min(e, i + kOzChunk);
-#pragma unroll
-                for (int g = 0; g < kOzSlots; ++g) {
-                    int w_ok = 1;
-                    if (lane == 0) w_ok = mbar_wait_sleep(accf(g), (uint32_t)(ch & 1), abort_flag, a.max_wait) ? 1 : 0;
-                    w_ok = __shfl_sync(0xffffffffu, w_ok, 0);
-                    if (!w_ok) {
-                        if (lane == 0) {
-                            atomicOr(&a.status[kStTimeout], 1);
-                            s_abort = 1;
-                        }
-                        ok = false;
-                        break;
-                    }
-                    fence_after();
-                    // slot g holds T_g 2^(-8g), T_g an integer below 2^24: read it in one
-                    // load and hand the accumulator back before converting, so the next
-                    // chunk's products into it need not wait for the conversion
-                    const uint32_t taddr = tmem + tlane + (uint32_t)(g * a.Npad + cg * ncol);
-                    float v[32];
-                    if (ncol == 32)
-                        tmem_ld32(taddr, v);
-                    else
-                        tmem_ld16(taddr, v);
-                    fence_before();
-                    mbar_arrive(acce(g));
-                    const float mul = oz_digit_scale(-g);
-#pragma unroll
-                    for (int q = 0; q < 32; ++q) {
-                        if (q < ncol) {
-                            if (g <= 4)
-                                hi[q] += (long long)__float2int_rn(v[q] * mul) << (8 * (4 - g));
-                            else if (g == 5)
-                                lo[q] += __float2int_rn(v[q] * mul);
-                            else
-                                lo[q] += (__float2int_rn(v[q] * mul) + 128) >> 8;
-                        }
-                    }
-                }
-                if (!ok) break;
-                i = ce;
-                ++nchunks;
-                const bool seg_end = (i == e);
-                if (!(seg_end || nchunks % kOzFlushChunks == 0)) continue;
-                if (direct) {
-                    // the whole tile's K range in this CTA: the final output
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) {
-                        const int64_t col = col0 + j;
-                        if (j < ncol && row < a.M && col < a.N)
-                            oz_store(a, row, col, oz_value(hi[j], lo[j], ea, a.eb[col]));
-                    }
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) {
-                        const int64_t col = col0 + j;
-                        if (j < ncol) {
-                            const double v = (row < a.M && col < a.N) ? oz_value(hi[j], lo[j], ea, a.eb[col]) : 0.0;
-                            slot[j] = stored ? slot[j] + v : v;
-                        }
-                        hi[j] = lo[j] = 0;
-                    }
-                    stored = true;
-                }
+            for (int q = 0; q < CW; ++q) {
+                hi64[q] = 0ull;
+                lo32[q] = 0u;
             }
+            int nlow = 0, nhigh = 0, nfold = 0;  // chunks added (nfold: since the last carry)
+            bool stored = false;
+            int jl = min(nk, kOzLowChunk - kOzLowShift), jh = min(nk, kOzHighChunk);  // next chunk ends
+            for (bool more = true; more && ok;) {
+                const int h = jl <= jh ? 0 : 1;  // the group whose chunk ends next (both at nk: low first)
+                int w_ok = 1;
+                if (lane == 0) w_ok = mbar_wait(accf(h), (ph >> h) & 1u, abort_flag, a.max_wait) ? 1 : 0;
+                w_ok = __shfl_sync(0xffffffffu, w_ok, 0);
+                if (!w_ok) {
+                    if (lane == 0) {
+                        atomicOr(&a.status[kStTimeout], 1);
+                        s_abort = 1;
+                    }
+                    ok = false;
+                    break;
+                }
+                ph ^= 1u << h;
+                fence_after();
+                // Slot g holds T_g, an integer within 2^24.  8 columns are converted while the
+                // next 8 are read; the group goes back to the MMA thread as soon as its last
+                // columns are in registers.  T_0 (at most 2^22) and T_6, rounded to 2^-40,
+                // convert on the FP32 pipe, the others by F2I.  The loop over slots stays
+                // rolled: unrolled, the scheduler gathers so many conversions that the sums
+                // no longer fit the 168 registers of a thread.
+                const int g1 = h == 0 ? kOzLowSlots : kOzSlots;
+                uint32_t buf[2][8];
+                const int g0 = h == 0 ? 0 : kOzLowSlots;
+                tmem_ld8_async(t0 + g0 * NC, buf[0]);
+                tmem_wait8(buf[0]);
+#pragma unroll 1
+                for (int g = g0; g < g1; ++g) {
+                    const bool lastg = g + 1 == g1;
+#pragma unroll
+                    for (int q = 0; q < CW; q += 8) {
+                        const int b = (q >> 3) & 1;
+                        const bool lastq = q + 8 == CW;
+                        // (one buffer where 8 columns are all: NC = 16)
+                        if (CW > 8 && !(lastq && lastg))
+                            tmem_ld8_async(lastq ? t0 + (g + 1) * NC : t0 + g * NC + q + 8, buf[b ^ 1]);
+                        if (CW == 8 && lastg) {
+                            fence_before();
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(acce(h));
+                        }
+                        oz_add_slot<CW>(g, q, buf[b], hi64, lo32);
+                        if (CW == 8 && !lastg) {
+                            tmem_ld8_async(t0 + (g + 1) * NC, buf[0]);
+                            tmem_wait8(buf[0]);
+                        }
+                        if (CW > 8 && !(lastq && lastg)) tmem_wait8(buf[b ^ 1]);
+                        if (CW > 8 && q + 16 == CW && lastg) {
+                            fence_before();
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(acce(h));
+                        }
+                    }
+                }
+                if (h == 0) {
+                    ++nlow;
+                    jl = jl == nk ? INT_MAX : min(nk, jl + kOzLowChunk);
+                } else {
+                    ++nhigh;
+                    jh = jh == nk ? INT_MAX : min(nk, jh + kOzHighChunk);
+                    if (++nfold == kOzFoldChunks) {
+                        nfold = 0;
+#pragma unroll
+                        for (int q = 0; q < CW; ++q) {  // hi + lo 2^-8 unchanged
+                            const int t = (int)(lo32[q] - (unsigned)kOzFoldChunks * kOzMagicBits);
+                            hi64[q] += (unsigned long long)(long long)(t >> 8);
+                            lo32[q] = (unsigned)(t & 255);
+                        }
+                    }
+                }
+                more = jl != INT_MAX || jh != INT_MAX;
+                if (more && nhigh < kOzFlushChunks) continue;
+                // output: two columns an iteration of a rolled loop that shifts the sums down
+                // (their conversion, unrolled over all columns, would not fit the registers)
+                const int64_t row = (int64_t)mt * kOzM + r, col0 = (int64_t)nt * NC + cofs;
+                const int ea = row < a.M ? a.ea[row] : 0;
+                const int eb_lane = lane < CW && col0 + lane < a.N ? a.eb[col0 + lane] : 0;  // column col0 + lane
+                const unsigned long long bias = (unsigned long long)((unsigned)nlow * kOzMagicBits) << 32;
+                const unsigned lobias = (unsigned)nfold * kOzMagicBits;
+                const bool direct = nk == KB && KB <= kOzHighChunk * kOzFlushChunks;
+                const bool pair = !direct || (!a.symmetric && (a.ldo & 1) == 0 &&
+                                              (reinterpret_cast<uintptr_t>(a.out) & 15) == 0);
+                // segments whose tile is cut between CTAs (at most the first and the last one
+                // unless the tile is longer than one flush) leave a partial tile
+                const int islot = KB <= kOzHighChunk * kOzFlushChunks ? (seg ? 1 : 0) : seg;
+                double* o = direct ? a.out + row * a.ldo + col0
+                                   : a.partial + (((int64_t)c * a.nslots + islot) * kOzM + r) * kOzN + cofs;
+#pragma unroll 1
+                for (int cc = 0; cc < CW; cc += 2) {
+                    const int eb0 = __shfl_sync(0xffffffffu, eb_lane, cc);
+                    const int eb1 = __shfl_sync(0xffffffffu, eb_lane, cc + 1);
+                    const int64_t col = col0 + cc;  // columns col, col + 1
+                    if (row < a.M && col < a.N) {
+                        const bool two = col + 1 < a.N;
+                        double2 w = make_double2(0.0, 0.0);
+                        w.x = oz_value((long long)(hi64[0] - bias), (int)(lo32[0] - lobias), ea, eb0);
+                        if (two) w.y = oz_value((long long)(hi64[1] - bias), (int)(lo32[1] - lobias), ea, eb1);
+                        double* oq = o + cc;
+                        if (pair && two) {
+                            if (direct) {
+                                w.x = oz_scale(a.alpha, w.x);
+                                w.y = oz_scale(a.alpha, w.y);
+                            }
+                            if (direct ? a.beta != 0.0 : stored) {
+                                const double2 z = *reinterpret_cast<const double2*>(oq);
+                                const double beta = direct ? a.beta : 1.0;
+                                w.x = fma(beta, z.x, w.x);
+                                w.y = fma(beta, z.y, w.y);
+                            }
+                            *reinterpret_cast<double2*>(oq) = w;
+                        } else if (direct) {
+                            oz_store(a, row, col, w.x);
+                            if (two) oz_store(a, row, col + 1, w.y);
+                        } else {
+                            *oq = stored ? *oq + w.x : w.x;
+                        }
+                    }
+#pragma unroll
+                    for (int q = 0; q < CW; ++q) {
+                        hi64[q] = q + 2 < CW ? hi64[q + 2 < CW ? q + 2 : 0] : 0ull;
+                        lo32[q] = q + 2 < CW ? lo32[q + 2 < CW ? q + 2 : 0] : 0u;
+                    }
+                }
+                stored = true;
+                nlow = nhigh = nfold = 0;
+            }
+            left -= nk;
+            kb = 0;
         }
     }
     fence_before();
     __syncthreads();
     if (warp == 1) {
         fence_after();
-        tmem_dealloc(tmem, kOzTmemCols);
+        tmem_dealloc(tmem, S::kTmemCols);
     }
 }
 
-// Tiles whose K range is split over CTAs (or longer than one 64-bit
-// accumulation): the parts are added in CTA order and the output rule applied.
-__global__ void oz_fixup_kernel(OzArgs a) {
-    __shared__ int s_g0, s_g1;
-    const int64_t t = blockIdx.y;
-    const int64_t KB = a.KB;
-    const int mt = (int)(t / a.NT), nt = (int)(t % a.NT);
+// Tiles whose K range is split over CTAs (or longer than one 64-bit accumulation): the
+// parts are added in CTA order and the output rule applied.  Block (x, y): 1/32 of the
+// tile that unit group y + 1 starts in (cut tiles; a group that starts in a tile which
+// an earlier group also starts inside leaves it to that one), of column tile z; with
+// every tile split (long K), y is the row tile.
+__global__ void __launch_bounds__(256) oz_fixup_kernel(OzArgs a) {
+    __shared__ int s_g0, s_nc, s_mt;
+    __shared__ int64_t s_slot[kOzWave];
+    const int KB = a.KB, nt = blockIdx.z;
+    const bool all = KB > kOzHighChunk * kOzFlushChunks;
     if (threadIdx.x == 0) {
-        auto group_of = [&](int64_t u) {
-            int g = (int)(u * a.Gg / a.totalg);
-            while (g + 1 < a.Gg && oz_glo(g + 1, a) <= u) ++g;
-            while (g > 0 && oz_glo(g, a) > u) --g;
-            return g;
-        };
-        s_g0 = group_of((int64_t)mt * KB);
-        s_g1 = group_of((int64_t)(mt + 1) * KB - 1);
+        int mt, nc = 0, g0 = 0;
+        if (all) {
+            mt = blockIdx.y;
+            const int64_t u = (int64_t)mt * KB;
+            g0 = (int)(u * a.Gg / a.totalg);
+            while (g0 + 1 < a.Gg && oz_glo(g0 + 1, a) <= u) ++g0;
+            while (g0 > 0 && oz_glo(g0, a) > u) --g0;
+            nc = 1;
+        } else {
+            const int g = (int)blockIdx.y + 1;
+            const int64_t u = oz_glo(g, a);
+            mt = (int)(u / KB);
+            g0 = g - 1;
+            // cut here, and the group before starts at or before the tile
+            if (u > (int64_t)mt * KB && oz_glo(g0, a) <= (int64_t)mt * KB) nc = 1;
+        }
+        if (nc)
+            while (g0 + nc < a.Gg && oz_glo(g0 + nc, a) < (int64_t)(mt + 1) * KB) ++nc;
+        s_g0 = g0;
+        s_nc = nc;
+        s_mt = mt;
     }
     __syncthreads();
-    if (s_g0 == s_g1 && KB <= (int64_t)kOzChunk * kOzFlushChunks) return;  // written by its CTA
-    // the partial tile of each contributing CTA (column tile nt of groups g0..g1, in order)
-    __shared__ int64_t s_slot[kOzWave];
-    const int nc = s_g1 - s_g0 + 1;
+    const int nc = s_nc, mt = s_mt;
+    if (nc == 0) return;
+    // the partial tile of each contributing CTA, in order
     for (int j = threadIdx.x; j < nc; j += blockDim.x) {
         const int g = s_g0 + j;
-        const int cc = g * a.NT + nt;
-        const int seg = (int)(mt - oz_glo(g, a) / KB);
-        s_slot[j] = ((int64_t)cc * a.maxseg + seg) * kOzM * kOzN;
+        const int64_t cc = (int64_t)g * a.NT + nt;
+        int seg = (int)(mt - oz_glo(g, a) / KB);
+        if (!all && seg > 1) seg = 1;
+        s_slot[j] = (cc * a.nslots + seg) * kOzM * kOzN;
     }
     __syncthreads();
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= kOzM * kOzN) return;
     const int r = idx / kOzN, cl = idx % kOzN;
-    const int64_t row = (int64_t)mt * kOzM + r, col = (int64_t)nt * kOzN + cl;
-    if (row >= a.M || col >= a.N) return;
-    // eight loads in flight, added in CTA order (the same sum as a sequential loop)
+    const int64_t row = (int64_t)mt * kOzM + r, col = (int64_t)nt * a.tilen + cl;
+    if (cl >= a.tilen || row >= a.M || col >= a.N) return;
+    // sixteen loads in flight, added in CTA order (the same sum as a sequential loop)
     double acc = 0.0;
     int j = 0;
-    for (; j + 8 <= nc; j += 8) {
-        double v[8];
+    for (; j + 16 <= nc; j += 16) {
+        double v[16];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = a.partial[s_slot[j + u] + idx];
+        for (int u = 0; u < 16; ++u) v[u] = a.partial[s_slot[j + u] + idx];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) acc += v[u];
+        for (int u = 0; u < 16; ++u) acc += v[u];
     }
     for (; j < nc; ++j) acc += a.partial[s_slot[j] + idx];
     oz_store(a, row, col, acc);
@@ -589,56 +790,60 @@ __global__ void oz_fixup_kernel(OzArgs a) {
 
 // ---- host side -------------------------------------------------------------------
 struct OzPlan {
-    int64_t M, N, K, KB, tiles, totalg;
-    int MT, NT, Npad, G, Gg, maxseg;
+    int64_t M, N, K, tiles, totalg;
+    int KB, MT, NT, tilen, G, Gg, nslots;
 };
 
+// Column tiles of 16, 32 or 64 columns (7 accumulators of 64 fill the tensor memory).
 OzPlan oz_plan(int64_t M, int64_t N, int64_t K) {
     OzPlan p{};
     p.M = M;
     p.N = N;
     p.K = K;
+    p.tilen = N <= 16 ? 16 : (N <= 32 ? 32 : kOzN);
     p.MT = (int)((M + kOzM - 1) / kOzM);
-    p.NT = (int)((N + kOzN - 1) / kOzN);
-    p.Npad = N <= 32 ? 32 : kOzN;
-    p.KB = std::max<int64_t>(1, (K + kOzBK - 1) / kOzBK);
+    p.NT = (int)((N + p.tilen - 1) / p.tilen);
+    p.KB = (int)std::max<int64_t>(1, (K + kOzBK - 1) / kOzBK);
     p.tiles = (int64_t)p.MT * p.NT;
     p.totalg = (int64_t)p.MT * p.KB;
     p.Gg = (int)std::max<int64_t>(1, std::min<int64_t>(kOzWave / p.NT, p.totalg));
     p.G = p.Gg * p.NT;
-    p.maxseg = 1;
+    int maxseg = 1;
     OzArgs a{};
     a.KB = p.KB;
-    a.tiles = p.tiles;
     a.totalg = p.totalg;
-    a.G = p.G;
     a.Gg = p.Gg;
     for (int g = 0; g < p.Gg; ++g) {
         const int64_t lo = oz_glo(g, a), hi = oz_glo(g + 1, a);
-        if (hi > lo) p.maxseg = std::max<int>(p.maxseg, (int)((hi - 1) / p.KB - lo / p.KB + 1));
+        if (hi > lo) maxseg = std::max<int>(maxseg, (int)((hi - 1) / p.KB - lo / p.KB + 1));
     }
+    // partial tiles of a CTA: its first and its last, or all where a tile is longer than
+    // one 64-bit accumulation
+    p.nslots = p.KB <= kOzHighChunk * kOzFlushChunks ? std::min(maxseg, 2) : maxseg;
     return p;
 }
 
 inline size_t oz_planes_bytes(int64_t rows, int64_t K) {
-    return align256((size_t)kOzDig * (size_t)rows * (size_t)oz_k16(K) * 2);
+    return align256((size_t)kOzDig * (size_t)oz_ra(rows) * (size_t)oz_k16(K) * 2);
 }
 
-// 3-D tensor map of one operand: dims {16, rows, 7 x K blocks}, strides {32 B,
-// Ra x 32 B}, box 16 x box_rows x 7, 32-byte swizzle (rows past `rows` read zeros).
+// 3-D tensor map of one operand: dims {16 rows = 256 elements, groups of 16 rows, 7 x K
+// blocks}, box 512 bytes x box_rows / 16 x 7, copied byte for byte.  Groups past
+// `rows` read zeros; the rows past it in the last group hold anything, and only reach output
+// rows (columns) that do not exist.
 bool make_oz_map(CUtensorMap* map, const void* planes, int64_t rows, int64_t Ra, int64_t K, int box_rows) {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
-    const cuuint64_t dims[3] = {16, (cuuint64_t)rows, (cuuint64_t)(kOzDig * (oz_k16(K) / 16))};
-    const cuuint64_t strides[2] = {32, (cuuint64_t)Ra * 32};
-    const cuuint32_t box[3] = {16u, (cuuint32_t)box_rows, (cuuint32_t)kOzDig};
+    const cuuint64_t dims[3] = {256, (cuuint64_t)(oz_ra(rows) / 16), (cuuint64_t)(kOzDig * (oz_k16(K) / 16))};
+    const cuuint64_t strides[2] = {512, (cuuint64_t)Ra * 32};
+    const cuuint32_t box[3] = {256u, (cuuint32_t)(box_rows / 16), (cuuint32_t)kOzDig};
     const cuuint32_t estr[3] = {1, 1, 1};
     return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(planes), dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 inline size_t oz_partial_bytes(const OzPlan& p) {
-    return align256(sizeof(double) * (size_t)p.G * p.maxseg * kOzM * kOzN);
+    return align256(sizeof(double) * (size_t)p.G * p.nslots * kOzM * kOzN);
 }
 
 // One operand of the product kernel: `rows` stored rows of K digits each in the
@@ -654,7 +859,7 @@ int oz_slice_rows(tsvd_handle* h, int64_t R, int64_t K, const double* S, int64_t
     if (R == 0) return TSVD_OK;
     const int64_t blocks = std::min<int64_t>((R + 7) / 8, (int64_t)h->sm_count * 16);
     h->launches++;
-    oz_slice_rows_kernel<<<(unsigned)blocks, 256, 0, st>>>(R, K, S, lds, planes, R, eexp);
+    oz_slice_rows_kernel<<<(unsigned)blocks, 256, 0, st>>>(R, K, S, lds, planes, oz_ra(R), eexp);
     TSVD_TRY_CUDA(cudaGetLastError());
     return TSVD_OK;
 }
@@ -663,7 +868,7 @@ int oz_slice_rows(tsvd_handle* h, int64_t R, int64_t K, const double* S, int64_t
 int oz_slice_cols(tsvd_handle* h, int64_t K, int64_t R, const double* S, int64_t lds, bool upper,
                   __nv_bfloat16* planes, int* eexp, cudaStream_t st, int64_t Ra = -1, int64_t r0 = 0) {
     if (R == 0) return TSVD_OK;
-    if (Ra < 0) Ra = R;
+    if (Ra < 0) Ra = oz_ra(R);
     const unsigned gx = (unsigned)((R + 31) / 32);
     int64_t gy = std::min<int64_t>((K + 255) / 256, std::max<int64_t>(1, (int64_t)h->sm_count * 8 / gx));
     const int64_t rows_per = (K + gy - 1) / gy;
@@ -679,28 +884,36 @@ int oz_slice_cols(tsvd_handle* h, int64_t K, int64_t R, const double* S, int64_t
     return TSVD_OK;
 }
 
-int oz_run(tsvd_handle* h, const OzPlan& p, const OzView& va, const OzView& vb, double* partial, double* out,
-           int64_t ldo, double alpha, double beta, bool symmetric, int* status, cudaStream_t st) {
-    if (p.tiles > 65535) return TSVD_ERR_UNSUPPORTED;  // one fix-up grid row per tile
+template <int NC>
+int oz_launch(tsvd_handle* h, int grid, const CUtensorMap& mA, const CUtensorMap& mB, const OzArgs& a,
+              cudaStream_t st) {
+    using S = OzShape<NC>;
     static thread_local int configured = -1;
     if (configured != h->device) {
-        TSVD_TRY_CUDA(cudaFuncSetAttribute(oz_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kOzSmem));
+        TSVD_TRY_CUDA(cudaFuncSetAttribute(oz_gemm_kernel<NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kSmem));
         configured = h->device;
     }
+    h->launches++;
+    oz_gemm_kernel<NC><<<grid, S::kThreads, S::kSmem, st>>>(mA, mB, a);
+    TSVD_TRY_CUDA(cudaGetLastError());
+    return TSVD_OK;
+}
+
+int oz_run(tsvd_handle* h, const OzPlan& p, const OzView& va, const OzView& vb, double* partial, double* out,
+           int64_t ldo, double alpha, double beta, bool symmetric, int* status, cudaStream_t st) {
+    if (p.tiles > 65535) return TSVD_ERR_UNSUPPORTED;
     CUtensorMap mA, mB;
     if (!make_oz_map(&mA, va.planes, p.M, va.Ra, p.K, kOzM)) return TSVD_ERR_CUDA;
-    if (!make_oz_map(&mB, vb.planes, p.N, vb.Ra, p.K, p.Npad)) return TSVD_ERR_CUDA;
+    if (!make_oz_map(&mB, vb.planes, p.N, vb.Ra, p.K, p.tilen)) return TSVD_ERR_CUDA;
     OzArgs a{};
     a.M = p.M;
     a.N = p.N;
     a.KB = p.KB;
-    a.tiles = p.tiles;
     a.totalg = p.totalg;
     a.NT = p.NT;
-    a.Npad = p.Npad;
-    a.G = p.G;
+    a.tilen = p.tilen;
     a.Gg = p.Gg;
-    a.maxseg = p.maxseg;
+    a.nslots = p.nslots;
     a.ea = va.exps;
     a.eb = vb.exps;
     a.out = out;
@@ -711,12 +924,16 @@ int oz_run(tsvd_handle* h, const OzPlan& p, const OzView& va, const OzView& vb, 
     a.partial = partial;
     a.status = status;
     a.max_wait = h->max_wait;
-    h->launches++;
-    oz_gemm_kernel<<<p.G, kOzThreads, kOzSmem, st>>>(mA, mB, a);
-    TSVD_TRY_CUDA(cudaGetLastError());
-    if (partial) {
+    if (p.tilen == 16)
+        TSVD_TRY(oz_launch<16>(h, p.G, mA, mB, a, st));
+    else if (p.tilen == 32)
+        TSVD_TRY(oz_launch<32>(h, p.G, mA, mB, a, st));
+    else
+        TSVD_TRY(oz_launch<64>(h, p.G, mA, mB, a, st));
+    const unsigned parts = p.KB > kOzHighChunk * kOzFlushChunks ? (unsigned)p.MT : (unsigned)(p.Gg - 1);
+    if (parts > 0) {
         h->launches++;
-        oz_fixup_kernel<<<dim3((kOzM * kOzN + 255) / 256, (unsigned)p.tiles), 256, 0, st>>>(a);
+        oz_fixup_kernel<<<dim3(kOzM * kOzN / 256, parts, (unsigned)p.NT), 256, 0, st>>>(a);
         TSVD_TRY_CUDA(cudaGetLastError());
     }
     return TSVD_OK;
@@ -745,13 +962,14 @@ size_t oz_ws_bound(int64_t qmax, int64_t smax, int64_t bmax) {
 namespace {
 
 OzView view_of(const __nv_bfloat16* planes, int64_t rows, int64_t K, const int* exps) {
-    return OzView{planes, rows, K, rows, exps};
+    return OzView{planes, rows, K, oz_ra(rows), exps};
 }
 
 // The cached planes of columns [0, s) (cols layout: stored rows) or of the first s
 // columns of every row (rows layout: K = s).
 OzView view_of_cache(const OzCache& c, int64_t s) {
-    return c.cols_layout ? OzView{c.planes, s, c.rows, c.cols, c.exps} : OzView{c.planes, c.rows, s, c.rows, c.exps};
+    return c.cols_layout ? OzView{c.planes, s, c.rows, oz_ra(c.cols), c.exps}
+                         : OzView{c.planes, c.rows, s, oz_ra(c.rows), c.exps};
 }
 
 }  // namespace
@@ -782,6 +1000,10 @@ size_t oz_nn_ws(int64_t q, int64_t s, int64_t b, bool cached_x) {
     ar.take<int>((size_t)p.N);
     ar.take<char>(oz_partial_bytes(p));
     return ar.off;
+}
+
+size_t oz_a_ws(int64_t M, int64_t N, int64_t w) {
+    return std::max(oz_nn_ws(M, N, w, true), oz_tn_ws(M, N, w, false, true));
 }
 
 int oz_gemm_tn(tsvd_handle* h, int64_t q, int64_t s, int64_t b, const double* X, int64_t ldx, const double* Z,
@@ -842,19 +1064,19 @@ int oz_gemm_nn(tsvd_handle* h, int64_t q, int64_t s, int64_t b, double alpha, co
 size_t oz_cache_bytes(int64_t rows, int64_t cols, bool cols_layout) {
     Arena ar;
     OzCache c;
-    oz_cache_carve(c, ar, nullptr, 0, rows, cols, cols_layout, kOzNoFixedExp);
+    oz_cache_carve(c, ar, nullptr, 0, rows, cols, cols_layout, false);
     return ar.off;
 }
 
 void oz_cache_carve(OzCache& c, Arena& ar, const double* src, int64_t ld, int64_t rows, int64_t cols,
-                    bool cols_layout, int fixed_exp) {
+                    bool cols_layout, bool grows) {
     c = OzCache{};
     c.src = src;
     c.ld = ld;
     c.rows = rows;
     c.cols = cols;
     c.cols_layout = cols_layout;
-    c.fixed_exp = fixed_exp;
+    c.grows = grows;
     const int64_t srows = cols_layout ? cols : rows, K = cols_layout ? rows : cols;
     c.planes = reinterpret_cast<__nv_bfloat16*>(ar.take<char>(oz_planes_bytes(srows, K)));
     c.exps = ar.take<int>((size_t)srows);
@@ -866,20 +1088,17 @@ int oz_cache_slice(tsvd_handle* h, OzCache& c, int64_t c0, int64_t c1, cudaStrea
     if (c1 > c0) {
         if (c.cols_layout) {
             // stored rows [c0, c1): the columns' own exponents
-            TSVD_TRY(oz_slice_cols(h, c.rows, c1 - c0, c.src + c0, c.ld, false, c.planes, c.exps + c0, st, c.cols,
+            TSVD_TRY(oz_slice_cols(h, c.rows, c1 - c0, c.src + c0, c.ld, false, c.planes, c.exps + c0, st,
+                                   oz_ra(c.cols),
                                    c0));
-        } else if (c.fixed_exp != kOzNoFixedExp) {
-            if (c0 == 0) {
-                h->launches++;
-                oz_fill_kernel<<<(unsigned)((c.rows + 255) / 256), 256, 0, st>>>(c.rows, c.fixed_exp, c.exps);
-            }
-            // the window with the rest of its last 16-wide K block (written as zeros)
-            const int64_t a0 = c0 & ~int64_t(1), a1 = oz_k16(c1);
-            const int64_t tot = c.rows * ((a1 - a0) / 2);
-            const int64_t blocks = std::min<int64_t>((tot + 255) / 256, (int64_t)h->sm_count * 32);
+        } else if (c.grows) {
+            const int64_t w = (c1 - c0 + 1) / 2;  // column pairs of a row
+            const int g = w >= 32 ? 32 : (w >= 16 ? 16 : 8);
+            const unsigned blocks = (unsigned)std::min<int64_t>((c.rows * g + 255) / 256, (int64_t)h->sm_count * 32);
             h->launches++;
-            oz_slice_rows_fixed_kernel<<<(unsigned)std::max<int64_t>(1, blocks), 256, 0, st>>>(
-                c.rows, a0, a1, c1, c.src, c.ld, c.planes, c.rows, c.fixed_exp, c.exps);
+            const auto kern = g == 32 ? oz_slice_rows_grow_kernel<32>
+                                      : (g == 16 ? oz_slice_rows_grow_kernel<16> : oz_slice_rows_grow_kernel<8>);
+            kern<<<std::max(1u, blocks), 256, 0, st>>>(c.rows, c0, c1, c.src, c.ld, c.planes, oz_ra(c.rows), c.exps);
             TSVD_TRY_CUDA(cudaGetLastError());
         } else {
             // per-row exponents need the whole rows at once
@@ -893,23 +1112,12 @@ int oz_cache_slice(tsvd_handle* h, OzCache& c, int64_t c0, int64_t c1, cudaStrea
 
 int oz_cache_truncate(tsvd_handle* h, OzCache& c, int64_t v, cudaStream_t st) {
     if (v >= c.valid) return TSVD_OK;
+    c.valid = 0;
+    // Rows layout: a row's exponent may stem from the columns dropped here (a block that
+    // was not orthonormal, or not finite), and a product of the first v columns reads the
+    // whole last K block: the rest is sliced again.
+    if (!c.cols_layout && v > 0) return oz_cache_slice(h, c, 0, v, st);
     c.valid = v < 0 ? 0 : v;
-    if (!c.cols_layout && c.valid % 16 != 0) {
-        // a product of the first `valid` columns reads the whole last K block: zero its rest
-        const int64_t tot = c.rows * (oz_k16(c.valid) - c.valid) * kOzDig;
-        h->launches++;
-        oz_zero_cols_kernel<<<(unsigned)std::min<int64_t>((tot + 255) / 256, (int64_t)h->sm_count * 32), 256, 0,
-                              st>>>(c.rows, c.valid, oz_k16(c.valid), c.planes, c.rows);
-        TSVD_TRY_CUDA(cudaGetLastError());
-    }
-    if (!c.cols_layout && c.fixed_exp != kOzNoFixedExp) {
-        // a row's exponent may carry the mark of an entry out of range in the columns
-        // dropped here (a block that was not orthonormal yet): start again from the
-        // fixed exponent; the dropped columns are sliced again when rewritten
-        h->launches++;
-        oz_fill_kernel<<<(unsigned)((c.rows + 255) / 256), 256, 0, st>>>(c.rows, c.fixed_exp, c.exps);
-        TSVD_TRY_CUDA(cudaGetLastError());
-    }
     return TSVD_OK;
 }
 

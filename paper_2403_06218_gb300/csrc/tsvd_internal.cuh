@@ -22,12 +22,11 @@ struct OzCache {
     const double* src = nullptr;
     int64_t ld = 0, rows = 0, cols = 0;
     bool cols_layout = false;
-    int fixed_exp = 0;  // rows layout of an orthonormal basis: every row's exponent
+    bool grows = false;  // rows layout: columns are added block by block (a Lanczos basis)
     __nv_bfloat16* planes = nullptr;
     int* exps = nullptr;
     int64_t valid = 0;
 };
-constexpr int kOzNoFixedExp = -(1 << 30);
 }  // namespace tsvd
 
 // CUDA-event timing per kernel class (TSVD_FLAG_PROFILE).
@@ -54,9 +53,6 @@ struct tsvd_handle {
     int* oz_status = nullptr;
     // operands whose digit planes are kept for the current call (owned by the caller)
     std::vector<const tsvd::OzCache*> oz_caches;
-    // set by OzFreshRows: products slice their left operand afresh instead of
-    // reading a rows-layout basis cache
-    bool oz_fresh_rows = false;
     // limit, in SM clock cycles, of one bounded wait of the pipelined product kernels
     // and of the Jacobi grid barrier (2e9, about 1 s; tsvd_set_wait_limit lowers it)
     long long max_wait = 2000000000LL;
@@ -296,6 +292,9 @@ size_t oz_tn_ws(int64_t q, int64_t s, int64_t b, bool symmetric, bool cached_x =
 size_t oz_nn_ws(int64_t q, int64_t s, int64_t b, bool cached_x = false);
 // Scratch that covers every product with q <= qmax, s <= smax, b <= bmax (and s, b swapped).
 size_t oz_ws_bound(int64_t qmax, int64_t smax, int64_t bmax);
+// Scratch of the products of a dense A (M x N) and A^T, both in digit-plane caches, with a
+// block of width w.
+size_t oz_a_ws(int64_t M, int64_t N, int64_t w);
 // C (s x b, ldc) = X^T Z, X (q x s, ldx), Z (q x b, ldz); symmetric: Z == X, C mirrored.
 // xc: cached planes of X (cols layout, s <= xc->valid) instead of slicing X.
 int oz_gemm_tn(tsvd_handle* h, int64_t q, int64_t s, int64_t b, const double* X, int64_t ldx, const double* Z,
@@ -311,7 +310,7 @@ int oz_gemm_nn(tsvd_handle* h, int64_t q, int64_t s, int64_t b, double alpha, co
 // then valid = c1), and the lookup the products use.
 size_t oz_cache_bytes(int64_t rows, int64_t cols, bool cols_layout);
 void oz_cache_carve(OzCache& c, Arena& ar, const double* src, int64_t ld, int64_t rows, int64_t cols,
-                    bool cols_layout, int fixed_exp);
+                    bool cols_layout, bool grows);
 int oz_cache_slice(tsvd_handle* h, OzCache& c, int64_t c0, int64_t c1, cudaStream_t st);
 // Columns from v on are about to be rewritten: valid = min(valid, v).
 int oz_cache_truncate(tsvd_handle* h, OzCache& c, int64_t v, cudaStream_t st);
@@ -324,20 +323,6 @@ struct OzCacheScope {
     explicit OzCacheScope(tsvd_handle* hh) : h(hh), n0(hh->oz_caches.size()) {}
     void add(const OzCache* c) { h->oz_caches.push_back(c); }
     ~OzCacheScope() { h->oz_caches.resize(n0); }
-};
-
-// Within its lifetime the FP64 products slice their left operand afresh, with one
-// exponent per row, instead of reading the rows-layout planes of a basis cache.
-// Those planes give every row the fixed exponent of an orthonormal basis (entries
-// below 2), so a basis of n rows, with entries near n^-1/2, keeps about log2(n)/2
-// bits fewer than FP64 there.  The cache serves the CGS-CQR2 updates, whose
-// coefficients are computed from the same planes; the restart and Ritz products,
-// whose results the next cycle takes as exact Ritz vectors, slice afresh.
-struct OzFreshRows {
-    tsvd_handle* h;
-    bool prev;
-    explicit OzFreshRows(tsvd_handle* hh) : h(hh), prev(hh->oz_fresh_rows) { h->oz_fresh_rows = true; }
-    ~OzFreshRows() { h->oz_fresh_rows = prev; }
 };
 
 // Makes the FP64 products of one call run on the tensor cores with `bytes` of
