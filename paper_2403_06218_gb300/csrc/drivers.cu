@@ -905,12 +905,18 @@ namespace {
 // application is projected back onto the complement.
 struct CgBufs {
     double *R, *P, *AP, *T, *H, *rr, *rr_new, *pap, *bb, *alpha, *beta, *part, *cpart;
+    void* ozws;  // tensor-core scratch of either side's projections
+    size_t ozbytes;
+    int* status;
 };
 
 template <typename F1, typename F2>
 int cg_side(tsvd_handle* h, int64_t rows, int k, const double* Q, const double* rhs, const double* s, F1 op1, F2 op2,
             double* X, const tsvd_backward_opts* o, CgBufs& b, cudaStream_t st, int* iters, double* resid) {
     const size_t bytes = sizeof(double) * (size_t)rows * k;
+    const size_t ozneed = oz_standalone_ws(rows, k, k);
+    OzStandalone oz(h, rows, k, Q, k, b.ozws, ozneed <= b.ozbytes ? ozneed : 0, b.status);
+    TSVD_TRY(oz.slice(st));
     auto project = [&](double* Z) -> int {
         TSVD_TRY_CUDA((gemm_tn<double, double>(h, rows, k, k, Q, k, Z, k, b.H, k, false, b.part, st)));
         TSVD_TRY_CUDA((gemm_nn<double, double, double>(h, rows, k, k, -1.0, Q, k, b.H, k, 1.0, Z, k, false, st)));
@@ -1001,6 +1007,10 @@ int svd_backward_run(tsvd_handle* h, const tsvd_matrix* A, int k, const double* 
     for (double** v : {&b.rr, &b.rr_new, &b.pap, &b.bb, &b.alpha, &b.beta}) *v = ar.take<double>(k);
     b.part = ar.take<double>(tn_partial_max(h, mx, k, k) / sizeof(double) + 1);
     b.cpart = ar.take<double>(coldot_ws(mx, k) / sizeof(double) + 1);
+    // the complement projections run on the tensor cores, from planes of U (then V) sliced once
+    b.ozbytes = std::max(oz_standalone_ws(m, k, k), oz_standalone_ws(n, k, k));
+    b.ozws = ar.take<char>(b.ozbytes);
+    b.status = status;
     if (!run) {
         *sizing = ar.off + 256;
         return TSVD_OK;

@@ -719,7 +719,7 @@ cudaError_t gemm_tn(tsvd_handle* h, int64_t q, int64_t s, int64_t b, const TI* X
                    (double)sizeof(TI) * (double)q * (symmetric ? b : s + b) + (double)sizeof(TC) * s * b, st);
     if constexpr (std::is_same<TI, double>::value && std::is_same<TC, double>::value) {
         const OzCache* xc = h->oz_ws ? oz_find_cache(h, X, ldx, q, s, true) : nullptr;
-        if (h->oz_ws && oz_worth(s, b, q) && oz_tn_ws(q, s, b, symmetric, xc != nullptr) <= h->oz_bytes) {
+        if (h->oz_ws && oz_worth(s, b, q) && oz_tn_ws(q, s, b, symmetric, xc != nullptr, h->oz_dig) <= h->oz_bytes) {
             const int rc = oz_gemm_tn(h, q, s, b, X, ldx, Z, ldz, C, ldc, symmetric, h->oz_ws, h->oz_bytes,
                                       h->oz_status, st, xc);
             return rc == TSVD_OK ? cudaSuccess : cudaErrorUnknown;
@@ -817,7 +817,7 @@ cudaError_t gemm_nn(tsvd_handle* h, int64_t q, int64_t s, int64_t b, double alph
     if constexpr (std::is_same<TX, double>::value && std::is_same<TM, double>::value &&
                   std::is_same<TY, double>::value) {
         const OzCache* xc = h->oz_ws ? oz_find_cache(h, X, ldx, q, s, false) : nullptr;
-        if (h->oz_ws && s > 0 && oz_worth(q, b, s) && oz_nn_ws(q, s, b, xc != nullptr) <= h->oz_bytes) {
+        if (h->oz_ws && s > 0 && oz_worth(q, b, s) && oz_nn_ws(q, s, b, xc != nullptr, h->oz_dig) <= h->oz_bytes) {
             const int rc = oz_gemm_nn(h, q, s, b, alpha, X, ldx, M, ldm, beta, Y, ldy, upper, h->oz_ws, h->oz_bytes,
                                       h->oz_status, st, xc);
             return rc == TSVD_OK ? cudaSuccess : cudaErrorUnknown;

@@ -63,15 +63,15 @@ namespace {
 using namespace tcx;
 
 constexpr int kOzDig = 7;                                   // digits per operand entry
+constexpr int kOzWideDig = 8;                               // of the wide form
 constexpr int kOzM = 128;                                   // output rows per tile (TMEM lanes)
 constexpr int kOzN = 64;                                    // most output columns per tile
 constexpr int kOzBK = 16;                                   // K per stage (one 32-byte row, one MMA)
 constexpr int kOzRowB = 2 * kOzBK;
 constexpr int kOzPlaneA = kOzM * kOzRowB;                   // 4 KB
-constexpr int kOzSlots = kOzDig;     // accumulators: p + q = 0 .. 6
-constexpr int kOzLowSlots = 4;       // p + q = 0 .. 3: the low group; 4 .. 6: the high group
+constexpr int kOzLowSlots = 4;       // p + q = 0 .. 3: the low group; 4 .. 6 (or 7): the high group
 // K blocks of one exact accumulation (every |T_g| <= (g + 1) 2^14 per k stays within 2^24):
-// 256 k for T_0 .. T_3, 128 k for T_4 .. T_6.  The low chunks end 4 K blocks off the high
+// 256 k for T_0 .. T_3, 128 k for the others.  The low chunks end 4 K blocks off the high
 // ones, the first one after 12 K blocks (so that a tile's output has 8 to finish in).
 constexpr int kOzLowChunk = 16, kOzHighChunk = 8, kOzLowShift = 4;
 constexpr int kOzRun = 4;             // K blocks issued for one group before the other takes over
@@ -79,13 +79,13 @@ constexpr int kOzFoldChunks = 128;    // high chunks between carries of lo into 
 constexpr int kOzFlushChunks = 768;   // high chunks between FP64 flushes of the integer sums (98,304 k)
 constexpr int kOzWave = 152;
 
-// Tile shapes: NC columns, slot p + q at TMEM column (p + q) NC.
-template <int NC>
+// Tile shapes: NC columns, D digits, slot p + q at TMEM column (p + q) NC.
+template <int NC, int D>
 struct OzShape {
-    static constexpr int kStageA = kOzDig * kOzPlaneA;               // 28 KB
+    static constexpr int kStageA = D * kOzPlaneA;                    // 28 (32) KB
     static constexpr int kPlaneB = NC * kOzRowB;                     // 2 KB at 64 columns
-    static constexpr int kStage = kStageA + kOzDig * kPlaneB;
-    static constexpr int kStages = NC == 64 ? 5 : (NC == 32 ? 6 : 7);
+    static constexpr int kStage = kStageA + D * kPlaneB;
+    static constexpr int kStages = D == 7 ? (NC == 64 ? 5 : (NC == 32 ? 6 : 7)) : (NC == 64 ? 4 : (NC == 32 ? 5 : 6));
     static constexpr int kSmem = kStages * kStage + 1024;
     static constexpr int kTmemCols = NC == 64 ? 512 : (NC == 32 ? 256 : 128);
     static constexpr int kEpiWarps = NC == 64 ? 16 : 8;              // NC / 4 or NC / 2 columns a warp
@@ -106,8 +106,9 @@ __device__ inline int oz_exp(double x) {
 
 __device__ inline int oz_norm_exp(int e) { return e <= kOzZeroExp ? 0 : e; }
 
-// round(x 2^(55 - e)) (ties away from zero) as balanced base-256 digits.
-__device__ inline void oz_digits(double x, int e, int d[kOzDig]) {
+// round(x 2^(8 D - 1 - e)) (ties away from zero) as D balanced base-256 digits.
+template <int D>
+__device__ inline void oz_digits(double x, int e, int (&d)[D]) {
     const uint64_t u = (uint64_t)__double_as_longlong(x);
     const int be = (int)((u >> 52) & 0x7FF);
     uint64_t m = u & ((1ull << 52) - 1);
@@ -118,7 +119,7 @@ __device__ inline void oz_digits(double x, int e, int d[kOzDig]) {
     }
     int64_t F = 0;
     if (be != 0x7FF && e < kOzNanExp && m != 0) {
-        const int sh = q + 55 - e;  // <= 2 when |x| < 2^e
+        const int sh = q + 8 * D - 1 - e;  // <= 8 D - 54 when |x| < 2^e
         if (sh >= 0) {
             F = (int64_t)(m << sh);
         } else if (sh > -54) {
@@ -128,8 +129,8 @@ __device__ inline void oz_digits(double x, int e, int d[kOzDig]) {
     }
     int64_t r = F;
 #pragma unroll
-    for (int p = kOzDig - 1; p >= 1; --p) {
-        const int lo = (int)((r + 128) & 255) - 128;
+    for (int p = D - 1; p >= 1; --p) {
+        const int lo = (int)(((unsigned)r + 128u) & 255u) - 128;
         d[p] = lo;
         r = (r - lo) >> 8;
     }
@@ -143,27 +144,30 @@ __device__ inline __nv_bfloat162 oz_pack(int d0, int d1) {
 // Global layout of the digit planes: K-block major, and within a block the very bytes that
 // the MMA reads from shared memory.  Element (digit p, stored row r, column k) of an operand
 // with Ra allocated stored rows (a multiple of 16) sits at
-//   ((k / 16) * 7 + p) * Ra * 16 + r * 16 + (k % 16, its halves of 8 exchanged in every
+//   ((k / 16) * D + p) * Ra * 16 + r * 16 + (k % 16, its halves of 8 exchanged in every
 //   second group of 4 rows: the 32-byte swizzle),
 // so that a TMA box of 128 rows x 7 planes is 56 runs of 512 bytes copied as they are.  (As
 // a box of 16 columns, swizzled by the copy, it was 896 runs of 32 bytes, and the copy
 // engine's rate of about 1.4 clocks a run bounded the product kernel: 1,344 runs a stage.)
 // Columns past K up to the next multiple of 16 hold zeros.
+template <int D>
 __host__ __device__ inline int64_t oz_off(int64_t Ra, int64_t r, int64_t k, int p) {
-    return ((k >> 4) * kOzDig + p) * Ra * 16 + r * 16 + ((k & 15) ^ ((r & 4) << 1));
+    return ((k >> 4) * D + p) * Ra * 16 + r * 16 + ((k & 15) ^ ((r & 4) << 1));
 }
 __host__ __device__ inline int64_t oz_k16(int64_t K) { return (K + 15) / 16 * 16; }
 inline int64_t oz_ra(int64_t rows) { return (rows + 15) / 16 * 16; }
 
 // Stores the digits of (x0, x1) at columns (k, k + 1), k even, of stored row r.
-__device__ inline void oz_store_pair(__nv_bfloat16* planes, int64_t Ra, int64_t r, int64_t k, const int* da,
-                                     const int* db) {
-    __nv_bfloat162* dst = reinterpret_cast<__nv_bfloat162*>(planes + oz_off(Ra, r, k, 0));
+template <int D>
+__device__ inline void oz_store_pair(__nv_bfloat16* planes, int64_t Ra, int64_t r, int64_t k, const int (&da)[D],
+                                     const int (&db)[D]) {
+    __nv_bfloat162* dst = reinterpret_cast<__nv_bfloat162*>(planes + oz_off<D>(Ra, r, k, 0));
 #pragma unroll
-    for (int p = 0; p < kOzDig; ++p) dst[p * Ra * 8] = oz_pack(da[p], db[p]);  // plane step Ra*16 elements
+    for (int p = 0; p < D; ++p) dst[p * Ra * 8] = oz_pack(da[p], db[p]);  // plane step Ra*16 elements
 }
 
 // Rows slicer: row i of S (R x K, lds) -> stored row i; one warp per row.
+template <int D>
 __global__ void __launch_bounds__(256, 4) oz_slice_rows_kernel(int64_t R, int64_t K, const double* __restrict__ S,
                                                             int64_t lds, __nv_bfloat16* __restrict__ planes,
                                                             int64_t Ra, int* __restrict__ eexp) {
@@ -179,7 +183,7 @@ __global__ void __launch_bounds__(256, 4) oz_slice_rows_kernel(int64_t R, int64_
         e = oz_norm_exp(e);
         if (lane == 0) eexp[i] = e;
         for (int64_t k = 2 * lane; k < K16; k += 64) {
-            int da[kOzDig], db[kOzDig];
+            int da[D], db[D];
             oz_digits(k < K ? src[k] : 0.0, e, da);
             oz_digits(k + 1 < K ? src[k + 1] : 0.0, e, db);
             oz_store_pair(planes, Ra, i, k, da, db);
@@ -249,6 +253,7 @@ __global__ void __launch_bounds__(256) oz_colmax_kernel(int64_t K, int64_t R, co
 
 // Cols slicer: column j of S (K x R, lds) -> stored row r0 + j, tiles of 64 k x 32 j,
 // zeros past K up to the next multiple of 16.
+template <int D>
 __global__ void __launch_bounds__(256) oz_slice_cols_kernel(int64_t K, int64_t R, const double* __restrict__ S,
                                                             int64_t lds, int upper, const int* __restrict__ eexp,
                                                             __nv_bfloat16* __restrict__ planes, int64_t Ra,
@@ -270,7 +275,7 @@ __global__ void __launch_bounds__(256) oz_slice_cols_kernel(int64_t K, int64_t R
         const int64_t j = j0 + jj;
         if (j >= R) break;
         const int e = oz_norm_exp(eexp[j]);
-        int da[kOzDig], db[kOzDig];
+        int da[D], db[D];
         oz_digits(tile[2 * kp][jj], e, da);
         oz_digits(tile[2 * kp + 1][jj], e, db);
         oz_store_pair(planes, Ra, r0 + j, k, da, db);
@@ -305,25 +310,26 @@ __host__ __device__ inline int64_t oz_glo(int g, const OzArgs& a) {
     return (int64_t)g * a.totalg / a.Gg;
 }
 
-// (hi + lo 2^-8) 2^(ea + eb - 46), rounded once to nearest even.  In integer arithmetic: a
+// (hi + lo 2^-F) 2^(ea + eb - 46), rounded once to nearest even.  In integer arithmetic: a
 // warp-wide FP64 instruction takes 16 clocks of the SM's FP64 pipe, and the five that a
 // conversion by casts needs bounded the products with a short K (28,000 of 90,000 clocks a
 // tile at K = 576).
+template <int F>
 __device__ inline double oz_value(long long hi, int lo, int ea, int eb) {
     if (ea >= kOzNanExp || eb >= kOzNanExp) return __longlong_as_double(0x7ff8000000000000LL);
     const int E = ea + eb - 46;
-    // sign and magnitude: m + r / 256
-    const long long v = hi + (lo >> 8);
-    const unsigned r0 = (unsigned)lo & 255u;
+    // sign and magnitude: m + r 2^-F
+    const long long v = hi + (lo >> F);
+    const unsigned r0 = (unsigned)lo & ((1u << F) - 1u);
     const bool neg = v < 0;
-    const unsigned r = neg ? (256u - r0) & 255u : r0;
+    const unsigned r = neg ? ((1u << F) - r0) & ((1u << F) - 1u) : r0;
     const unsigned long long m = neg ? ~(unsigned long long)v + (r0 == 0u ? 1ull : 0ull) : (unsigned long long)v;
     const int lz = __clzll((long long)m), be = 1086 + E - lz;  // biased exponent of the leading bit
     if (m != 0ull && be >= 1 && be <= 2046) {
         // 64 leading bits, the rest ORed into the last one
         unsigned long long w = m << lz;
-        w |= lz >= 8 ? (unsigned long long)r << (lz - 8) : (unsigned long long)(r >> (8 - lz));
-        if (lz < 8 && (r & ((1u << (8 - lz)) - 1u))) w |= 1ull;
+        w |= lz >= F ? (unsigned long long)r << (lz - F) : (unsigned long long)(r >> (F - lz));
+        if (lz < F && (r & ((1u << (F - lz)) - 1u))) w |= 1ull;
         unsigned long long mant = w >> 11;
         mant += ((unsigned)w & 0x7ffu) + ((unsigned)mant & 1u) > 0x400u ? 1ull : 0ull;
         const unsigned long long bits = ((unsigned long long)(be - 1) << 52) + mant;  // a carry raises the exponent
@@ -331,7 +337,7 @@ __device__ inline double oz_value(long long hi, int lo, int ea, int eb) {
     }
     // zero, a fraction alone, or a result at the ends of the FP64 range: x 2^E in two steps
     // (the first one is exact)
-    const double x = fma((double)lo, 0.00390625, (double)hi);
+    const double x = fma((double)lo, F == 8 ? 0x1p-8 : 0x1p-16, (double)hi);
     const int E1 = max(-900, min(E, 1023));
     double y = x * __longlong_as_double((long long)(E1 + 1023) << 52);
     if (E1 != E) y *= __longlong_as_double((long long)(max(-1022, min(E - E1, 1023)) + 1023) << 52);
@@ -362,8 +368,9 @@ __device__ inline void oz_store(const OzArgs& a, int64_t i, int64_t j, double v)
 constexpr float kOzMagic = 12582912.0f;
 constexpr unsigned kOzMagicBits = 0x4B400000u;
 
-// Adds T_g of 8 columns (from column q0 on) to the integer sums.
-template <int N>
+// Adds T_g of 8 columns (from column q0 on) to the integer sums.  lo counts units of 2^-40
+// with 7 digits (T_6 rounded to it) and of 2^-48 with 8 (T_5 in two parts, T_7 rounded).
+template <int N, int D>
 __device__ inline void oz_add_slot(int g, int q0, const uint32_t* v, unsigned long long (&hi)[N],
                                    unsigned (&lo)[N]) {
     if (g == 0) {
@@ -377,10 +384,21 @@ __device__ inline void oz_add_slot(int g, int q0, const uint32_t* v, unsigned lo
             asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(hi[q0 + q]) : "r"(__float2int_rn(__uint_as_float(v[q]))), "r"(mul));
     } else if (g == 5) {
 #pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const int t = __float2int_rn(__uint_as_float(v[q]));
+            if (D == 7) {
+                lo[q0 + q] += (unsigned)t;
+            } else {
+                hi[q0 + q] += (unsigned long long)(long long)(t >> 8);
+                lo[q0 + q] += ((unsigned)t & 255u) << 8;
+            }
+        }
+    } else if (D == 8 && g == 6) {
+#pragma unroll
         for (int q = 0; q < 8; ++q) lo[q0 + q] += (unsigned)__float2int_rn(__uint_as_float(v[q]));
     } else {
 #pragma unroll
-        for (int q = 0; q < 8; ++q) lo[q0 + q] += __float_as_uint(fmaf(__uint_as_float(v[q]), 0.00390625f, kOzMagic));
+        for (int q = 0; q < 8; ++q) lo[q0 + q] += __float_as_uint(fmaf(__uint_as_float(v[q]), 0x1p-8f, kOzMagic));
     }
 }
 
@@ -405,11 +423,16 @@ __device__ inline bool oz_chunk_start(int group, int j) {
 // operands and copies share (142 of 128 KB per 1,000 clocks).  Tried and left out: copies
 // of A (or B) multicast to a cluster of two CTAs, which changed nothing once the copies
 // were long runs, and an L2 prefetch ahead of the copies, which slowed them by a third.
-template <int NC>
-__global__ void __launch_bounds__(OzShape<NC>::kThreads, 1)
+//
+// The wide form (D = 8) has 8 digits and accumulators and 36 digit products (12 MMAs and
+// 1,152 clocks a K block): 63 bits below a row's (column's) largest entry, where the 7-digit
+// form's 55 leave entries 1,000 times smaller than it fewer than FP64's 53.
+template <int NC, int D>
+__global__ void __launch_bounds__(OzShape<NC, D>::kThreads, 1)
     oz_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, OzArgs a) {
-    using S = OzShape<NC>;
+    using S = OzShape<NC, D>;
     constexpr int kSt = S::kStages;
+    constexpr int kFrac = D == 7 ? 8 : 16;  // lo counts units of 2^-kFrac of hi's
     extern __shared__ uint8_t dsm[];
     __shared__ __align__(8) uint64_t bars[2 * kSt + 5];
     __shared__ uint32_t s_tmem;
@@ -461,8 +484,8 @@ __global__ void __launch_bounds__(OzShape<NC>::kThreads, 1)
                 const uint32_t sA = base + (uint32_t)(st * S::kStage);
                 mbar_arrive_expect_tx(full(st), (uint32_t)S::kStage);
                 // (coordinates in groups of 16 rows)
-                tma_load_3d(sA, &tmA, 0, mt * (kOzM / 16), kb * kOzDig, full(st));
-                tma_load_3d(sA + S::kStageA, &tmB, 0, nt * (NC / 16), kb * kOzDig, full(st));
+                tma_load_3d(sA, &tmA, 0, mt * (kOzM / 16), kb * D, full(st));
+                tma_load_3d(sA + S::kStageA, &tmB, 0, nt * (NC / 16), kb * D, full(st));
                 if (issued < kSt) ++issued;
                 if (++st == kSt) {
                     st = 0;
@@ -531,11 +554,11 @@ __global__ void __launch_bounds__(OzShape<NC>::kThreads, 1)
                                              idesc_bf16(kOzM, (kOzLowSlots - p) * NC), (start && p == 0) ? 0u : 1u);
                             } else {
 #pragma unroll
-                                for (int p = 0; p < kOzDig; ++p) {  // slots max(4, p) .. 6
+                                for (int p = 0; p < D; ++p) {  // slots max(4, p) .. D - 1
                                     const int g0 = p < kOzLowSlots ? kOzLowSlots : p;
                                     mma_bf16(tmem + (uint32_t)(g0 * NC), a0 + (uint64_t)(p * (kOzPlaneA >> 4)),
                                              b0 + (uint64_t)((g0 - p) * (S::kPlaneB >> 4)),
-                                             idesc_bf16(kOzM, (kOzSlots - g0) * NC), (start && p == 0) ? 0u : 1u);
+                                             idesc_bf16(kOzM, (D - g0) * NC), (start && p == 0) ? 0u : 1u);
                                 }
                                 commit(empty(s));
                             }
@@ -575,8 +598,7 @@ __global__ void __launch_bounds__(OzShape<NC>::kThreads, 1)
         for (int left = (int)(hi - lo); left > 0 && ok; ++seg, ++mt) {
             const int nk = min(KB - kb, left);
             // integer sums of the digit products: hi in units of 2^-32 of the leading one
-            // (p + q <= 4, exact), lo in units of 2^-40 (p + q = 5 exact, 6 rounded), both
-            // biased by the magic bits of the chunks added
+            // (p + q <= 4, exact), lo below them (oz_add_slot), both biased by the magic bits of the chunks added
             unsigned long long hi64[CW];
             unsigned lo32[CW];
 #pragma unroll
@@ -604,11 +626,11 @@ __global__ void __launch_bounds__(OzShape<NC>::kThreads, 1)
                 fence_after();
                 // Slot g holds T_g, an integer within 2^24.  8 columns are converted while the
                 // next 8 are read; the group goes back to the MMA thread as soon as its last
-                // columns are in registers.  T_0 (at most 2^22) and T_6, rounded to 2^-40,
-                // convert on the FP32 pipe, the others by F2I.  The loop over slots stays
+                // columns are in registers.  T_0 (at most 2^22) and the last T_g, rounded to the
+                // unit of lo, convert on the FP32 pipe, the others by F2I.  The loop over slots stays
                 // rolled: unrolled, the scheduler gathers so many conversions that the sums
                 // no longer fit the 168 registers of a thread.
-                const int g1 = h == 0 ? kOzLowSlots : kOzSlots;
+                const int g1 = h == 0 ? kOzLowSlots : D;
                 uint32_t buf[2][8];
                 const int g0 = h == 0 ? 0 : kOzLowSlots;
                 tmem_ld8_async(t0 + g0 * NC, buf[0]);
@@ -628,7 +650,7 @@ __global__ void __launch_bounds__(OzShape<NC>::kThreads, 1)
                             __syncwarp();
                             if (lane == 0) mbar_arrive(acce(h));
                         }
-                        oz_add_slot<CW>(g, q, buf[b], hi64, lo32);
+                        oz_add_slot<CW, D>(g, q, buf[b], hi64, lo32);
                         if (CW == 8 && !lastg) {
                             tmem_ld8_async(t0 + (g + 1) * NC, buf[0]);
                             tmem_wait8(buf[0]);
@@ -650,10 +672,10 @@ __global__ void __launch_bounds__(OzShape<NC>::kThreads, 1)
                     if (++nfold == kOzFoldChunks) {
                         nfold = 0;
 #pragma unroll
-                        for (int q = 0; q < CW; ++q) {  // hi + lo 2^-8 unchanged
+                        for (int q = 0; q < CW; ++q) {  // hi + lo 2^-kFrac unchanged
                             const int t = (int)(lo32[q] - (unsigned)kOzFoldChunks * kOzMagicBits);
-                            hi64[q] += (unsigned long long)(long long)(t >> 8);
-                            lo32[q] = (unsigned)(t & 255);
+                            hi64[q] += (unsigned long long)(long long)(t >> kFrac);
+                            lo32[q] = (unsigned)(t & ((1 << kFrac) - 1));
                         }
                     }
                 }
@@ -682,8 +704,8 @@ __global__ void __launch_bounds__(OzShape<NC>::kThreads, 1)
                     if (row < a.M && col < a.N) {
                         const bool two = col + 1 < a.N;
                         double2 w = make_double2(0.0, 0.0);
-                        w.x = oz_value((long long)(hi64[0] - bias), (int)(lo32[0] - lobias), ea, eb0);
-                        if (two) w.y = oz_value((long long)(hi64[1] - bias), (int)(lo32[1] - lobias), ea, eb1);
+                        w.x = oz_value<kFrac>((long long)(hi64[0] - bias), (int)(lo32[0] - lobias), ea, eb0);
+                        if (two) w.y = oz_value<kFrac>((long long)(hi64[1] - bias), (int)(lo32[1] - lobias), ea, eb1);
                         double* oq = o + cc;
                         if (pair && two) {
                             if (direct) {
@@ -823,20 +845,20 @@ OzPlan oz_plan(int64_t M, int64_t N, int64_t K) {
     return p;
 }
 
-inline size_t oz_planes_bytes(int64_t rows, int64_t K) {
-    return align256((size_t)kOzDig * (size_t)oz_ra(rows) * (size_t)oz_k16(K) * 2);
+inline size_t oz_planes_bytes(int64_t rows, int64_t K, int dig) {
+    return align256((size_t)dig * (size_t)oz_ra(rows) * (size_t)oz_k16(K) * 2);
 }
 
-// 3-D tensor map of one operand: dims {16 rows = 256 elements, groups of 16 rows, 7 x K
-// blocks}, box 512 bytes x box_rows / 16 x 7, copied byte for byte.  Groups past
+// 3-D tensor map of one operand: dims {16 rows = 256 elements, groups of 16 rows, digits x
+// K blocks}, box 512 bytes x box_rows / 16 x digits, copied byte for byte.  Groups past
 // `rows` read zeros; the rows past it in the last group hold anything, and only reach output
 // rows (columns) that do not exist.
-bool make_oz_map(CUtensorMap* map, const void* planes, int64_t rows, int64_t Ra, int64_t K, int box_rows) {
+bool make_oz_map(CUtensorMap* map, const void* planes, int64_t rows, int64_t Ra, int64_t K, int box_rows, int dig) {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
-    const cuuint64_t dims[3] = {256, (cuuint64_t)(oz_ra(rows) / 16), (cuuint64_t)(kOzDig * (oz_k16(K) / 16))};
+    const cuuint64_t dims[3] = {256, (cuuint64_t)(oz_ra(rows) / 16), (cuuint64_t)(dig * (oz_k16(K) / 16))};
     const cuuint64_t strides[2] = {512, (cuuint64_t)Ra * 32};
-    const cuuint32_t box[3] = {256u, (cuuint32_t)(box_rows / 16), (cuuint32_t)kOzDig};
+    const cuuint32_t box[3] = {256u, (cuuint32_t)(box_rows / 16), (cuuint32_t)dig};
     const cuuint32_t estr[3] = {1, 1, 1};
     return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(planes), dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -859,7 +881,8 @@ int oz_slice_rows(tsvd_handle* h, int64_t R, int64_t K, const double* S, int64_t
     if (R == 0) return TSVD_OK;
     const int64_t blocks = std::min<int64_t>((R + 7) / 8, (int64_t)h->sm_count * 16);
     h->launches++;
-    oz_slice_rows_kernel<<<(unsigned)blocks, 256, 0, st>>>(R, K, S, lds, planes, oz_ra(R), eexp);
+    const auto kern = h->oz_dig == kOzWideDig ? oz_slice_rows_kernel<kOzWideDig> : oz_slice_rows_kernel<kOzDig>;
+    kern<<<(unsigned)blocks, 256, 0, st>>>(R, K, S, lds, planes, oz_ra(R), eexp);
     TSVD_TRY_CUDA(cudaGetLastError());
     return TSVD_OK;
 }
@@ -879,22 +902,24 @@ int oz_slice_cols(tsvd_handle* h, int64_t K, int64_t R, const double* S, int64_t
                                                                                            upper ? 1 : 0, rows_per,
                                                                                            eexp);
     const dim3 sg((unsigned)((oz_k16(K) + 63) / 64), gx);
-    oz_slice_cols_kernel<<<sg, 256, 0, st>>>(K, R, S, lds, upper ? 1 : 0, eexp, planes, Ra, r0);
+    const auto kern = h->oz_dig == kOzWideDig ? oz_slice_cols_kernel<kOzWideDig> : oz_slice_cols_kernel<kOzDig>;
+    kern<<<sg, 256, 0, st>>>(K, R, S, lds, upper ? 1 : 0, eexp, planes, Ra, r0);
     TSVD_TRY_CUDA(cudaGetLastError());
     return TSVD_OK;
 }
 
-template <int NC>
+template <int NC, int D>
 int oz_launch(tsvd_handle* h, int grid, const CUtensorMap& mA, const CUtensorMap& mB, const OzArgs& a,
               cudaStream_t st) {
-    using S = OzShape<NC>;
+    using S = OzShape<NC, D>;
     static thread_local int configured = -1;
     if (configured != h->device) {
-        TSVD_TRY_CUDA(cudaFuncSetAttribute(oz_gemm_kernel<NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kSmem));
+        TSVD_TRY_CUDA(cudaFuncSetAttribute(oz_gemm_kernel<NC, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           S::kSmem));
         configured = h->device;
     }
     h->launches++;
-    oz_gemm_kernel<NC><<<grid, S::kThreads, S::kSmem, st>>>(mA, mB, a);
+    oz_gemm_kernel<NC, D><<<grid, S::kThreads, S::kSmem, st>>>(mA, mB, a);
     TSVD_TRY_CUDA(cudaGetLastError());
     return TSVD_OK;
 }
@@ -902,9 +927,10 @@ int oz_launch(tsvd_handle* h, int grid, const CUtensorMap& mA, const CUtensorMap
 int oz_run(tsvd_handle* h, const OzPlan& p, const OzView& va, const OzView& vb, double* partial, double* out,
            int64_t ldo, double alpha, double beta, bool symmetric, int* status, cudaStream_t st) {
     if (p.tiles > 65535) return TSVD_ERR_UNSUPPORTED;
+    const int dig = h->oz_dig;
     CUtensorMap mA, mB;
-    if (!make_oz_map(&mA, va.planes, p.M, va.Ra, p.K, kOzM)) return TSVD_ERR_CUDA;
-    if (!make_oz_map(&mB, vb.planes, p.N, vb.Ra, p.K, p.tilen)) return TSVD_ERR_CUDA;
+    if (!make_oz_map(&mA, va.planes, p.M, va.Ra, p.K, kOzM, dig)) return TSVD_ERR_CUDA;
+    if (!make_oz_map(&mB, vb.planes, p.N, vb.Ra, p.K, p.tilen, dig)) return TSVD_ERR_CUDA;
     OzArgs a{};
     a.M = p.M;
     a.N = p.N;
@@ -924,12 +950,10 @@ int oz_run(tsvd_handle* h, const OzPlan& p, const OzView& va, const OzView& vb, 
     a.partial = partial;
     a.status = status;
     a.max_wait = h->max_wait;
-    if (p.tilen == 16)
-        TSVD_TRY(oz_launch<16>(h, p.G, mA, mB, a, st));
-    else if (p.tilen == 32)
-        TSVD_TRY(oz_launch<32>(h, p.G, mA, mB, a, st));
-    else
-        TSVD_TRY(oz_launch<64>(h, p.G, mA, mB, a, st));
+    constexpr int kD = kOzDig, kW = kOzWideDig;
+    const auto launch = dig == kW ? (p.tilen == 16 ? oz_launch<16, kW> : (p.tilen == 32 ? oz_launch<32, kW> : oz_launch<64, kW>))
+                                  : (p.tilen == 16 ? oz_launch<16, kD> : (p.tilen == 32 ? oz_launch<32, kD> : oz_launch<64, kD>));
+    TSVD_TRY(launch(h, p.G, mA, mB, a, st));
     const unsigned parts = p.KB > kOzHighChunk * kOzFlushChunks ? (unsigned)p.MT : (unsigned)(p.Gg - 1);
     if (parts > 0) {
         h->launches++;
@@ -948,15 +972,27 @@ bool oz_worth(int64_t M, int64_t N, int64_t K) {
     return M > 0 && N > 0 && K >= 32 && tiles <= 65535 && N <= 65535 * 32 && 2.0 * (double)M * N * K >= 3.0e7;
 }
 
-size_t oz_ws_bound(int64_t qmax, int64_t smax, int64_t bmax) {
+size_t oz_ws_bound(int64_t qmax, int64_t smax, int64_t bmax, int dig) {
     // planes and exponents of the largest operands of either product, and split-K
     // partial tiles for at most (tiles + 2 per CTA of one wave) tiles
-    const size_t tn = oz_planes_bytes(smax, qmax) + oz_planes_bytes(bmax, qmax);
-    const size_t nn = oz_planes_bytes(qmax, smax) + oz_planes_bytes(bmax, smax);
+    const size_t tn = oz_planes_bytes(smax, qmax, dig) + oz_planes_bytes(bmax, qmax, dig);
+    const size_t nn = oz_planes_bytes(qmax, smax, dig) + oz_planes_bytes(bmax, smax, dig);
     const size_t ex = align256(sizeof(int) * (size_t)(qmax + smax)) + align256(sizeof(int) * (size_t)(smax + bmax));
     const int64_t tiles = ((smax + kOzM - 1) / kOzM) * ((bmax + kOzN - 1) / kOzN);
     const size_t part = align256(sizeof(double) * (size_t)(tiles + 2 * kOzWave) * kOzM * kOzN);
     return std::max(tn, nn) + ex + part + 4096;
+}
+
+size_t oz_standalone_ws(int64_t q, int64_t s, int b) {
+    constexpr int kW = kOzWideDig;
+    size_t bytes = oz_ws_bound(q, b, b, kW);
+    if (s > 0) {
+        bytes += oz_cache_bytes(q, s, true, kW) + oz_cache_bytes(q, s, false, kW);
+        bytes += std::max(oz_tn_ws(q, s, b, false, true, kW), oz_nn_ws(q, s, b, true, kW));
+    }
+    // worth it only if one of the products is
+    const bool worth = oz_worth(b, b, q) || oz_worth(q, b, b) || (s > 0 && (oz_worth(s, b, q) || oz_worth(q, b, s)));
+    return worth && bytes <= kOzStandaloneMax ? bytes : 0;
 }
 
 namespace {
@@ -974,29 +1010,29 @@ OzView view_of_cache(const OzCache& c, int64_t s) {
 
 }  // namespace
 
-size_t oz_tn_ws(int64_t q, int64_t s, int64_t b, bool symmetric, bool cached_x) {
+size_t oz_tn_ws(int64_t q, int64_t s, int64_t b, bool symmetric, bool cached_x, int dig) {
     const OzPlan p = oz_plan(s, b, q);
     Arena ar;
     if (!cached_x) {
-        ar.take<char>(oz_planes_bytes(p.M, p.K));
+        ar.take<char>(oz_planes_bytes(p.M, p.K, dig));
         ar.take<int>((size_t)p.M);
     }
     if (!symmetric || cached_x) {
-        ar.take<char>(oz_planes_bytes(p.N, p.K));
+        ar.take<char>(oz_planes_bytes(p.N, p.K, dig));
         ar.take<int>((size_t)p.N);
     }
     ar.take<char>(oz_partial_bytes(p));
     return ar.off;
 }
 
-size_t oz_nn_ws(int64_t q, int64_t s, int64_t b, bool cached_x) {
+size_t oz_nn_ws(int64_t q, int64_t s, int64_t b, bool cached_x, int dig) {
     const OzPlan p = oz_plan(q, b, s);
     Arena ar;
     if (!cached_x) {
-        ar.take<char>(oz_planes_bytes(p.M, p.K));
+        ar.take<char>(oz_planes_bytes(p.M, p.K, dig));
         ar.take<int>((size_t)p.M);
     }
-    ar.take<char>(oz_planes_bytes(p.N, p.K));
+    ar.take<char>(oz_planes_bytes(p.N, p.K, dig));
     ar.take<int>((size_t)p.N);
     ar.take<char>(oz_partial_bytes(p));
     return ar.off;
@@ -1015,7 +1051,7 @@ int oz_gemm_tn(tsvd_handle* h, int64_t q, int64_t s, int64_t b, const double* X,
     if (xc) {
         va = view_of_cache(*xc, s);
     } else {
-        __nv_bfloat16* pa = reinterpret_cast<__nv_bfloat16*>(ar.take<char>(oz_planes_bytes(p.M, p.K)));
+        __nv_bfloat16* pa = reinterpret_cast<__nv_bfloat16*>(ar.take<char>(oz_planes_bytes(p.M, p.K, h->oz_dig)));
         int* ea = ar.take<int>((size_t)p.M);
         if (!ar.fits()) return TSVD_ERR_WORKSPACE;
         TSVD_TRY(oz_slice_cols(h, q, s, X, ldx, false, pa, ea, st));
@@ -1024,7 +1060,7 @@ int oz_gemm_tn(tsvd_handle* h, int64_t q, int64_t s, int64_t b, const double* X,
     if (symmetric && !xc) {
         vb = va;
     } else {
-        __nv_bfloat16* pb = reinterpret_cast<__nv_bfloat16*>(ar.take<char>(oz_planes_bytes(p.N, p.K)));
+        __nv_bfloat16* pb = reinterpret_cast<__nv_bfloat16*>(ar.take<char>(oz_planes_bytes(p.N, p.K, h->oz_dig)));
         int* eb = ar.take<int>((size_t)p.N);
         if (!ar.fits()) return TSVD_ERR_WORKSPACE;
         TSVD_TRY(oz_slice_cols(h, q, b, Z, ldz, false, pb, eb, st));
@@ -1045,13 +1081,13 @@ int oz_gemm_nn(tsvd_handle* h, int64_t q, int64_t s, int64_t b, double alpha, co
     if (xc) {
         va = view_of_cache(*xc, s);
     } else {
-        __nv_bfloat16* pa = reinterpret_cast<__nv_bfloat16*>(ar.take<char>(oz_planes_bytes(p.M, p.K)));
+        __nv_bfloat16* pa = reinterpret_cast<__nv_bfloat16*>(ar.take<char>(oz_planes_bytes(p.M, p.K, h->oz_dig)));
         int* ea = ar.take<int>((size_t)p.M);
         if (!ar.fits()) return TSVD_ERR_WORKSPACE;
         TSVD_TRY(oz_slice_rows(h, q, s, X, ldx, pa, ea, st));
         va = view_of(pa, q, s, ea);
     }
-    __nv_bfloat16* pb = reinterpret_cast<__nv_bfloat16*>(ar.take<char>(oz_planes_bytes(p.N, p.K)));
+    __nv_bfloat16* pb = reinterpret_cast<__nv_bfloat16*>(ar.take<char>(oz_planes_bytes(p.N, p.K, h->oz_dig)));
     int* eb = ar.take<int>((size_t)p.N);
     const size_t pbytes = oz_partial_bytes(p);
     double* part = pbytes ? reinterpret_cast<double*>(ar.take<char>(pbytes)) : nullptr;
@@ -1061,15 +1097,15 @@ int oz_gemm_nn(tsvd_handle* h, int64_t q, int64_t s, int64_t b, double alpha, co
 }
 
 // ---- caches of operands that many products read ----------------------------------
-size_t oz_cache_bytes(int64_t rows, int64_t cols, bool cols_layout) {
+size_t oz_cache_bytes(int64_t rows, int64_t cols, bool cols_layout, int dig) {
     Arena ar;
     OzCache c;
-    oz_cache_carve(c, ar, nullptr, 0, rows, cols, cols_layout, false);
+    oz_cache_carve(c, ar, nullptr, 0, rows, cols, cols_layout, false, dig);
     return ar.off;
 }
 
 void oz_cache_carve(OzCache& c, Arena& ar, const double* src, int64_t ld, int64_t rows, int64_t cols,
-                    bool cols_layout, bool grows) {
+                    bool cols_layout, bool grows, int dig) {
     c = OzCache{};
     c.src = src;
     c.ld = ld;
@@ -1078,7 +1114,7 @@ void oz_cache_carve(OzCache& c, Arena& ar, const double* src, int64_t ld, int64_
     c.cols_layout = cols_layout;
     c.grows = grows;
     const int64_t srows = cols_layout ? cols : rows, K = cols_layout ? rows : cols;
-    c.planes = reinterpret_cast<__nv_bfloat16*>(ar.take<char>(oz_planes_bytes(srows, K)));
+    c.planes = reinterpret_cast<__nv_bfloat16*>(ar.take<char>(oz_planes_bytes(srows, K, dig)));
     c.exps = ar.take<int>((size_t)srows);
     c.valid = 0;
 }

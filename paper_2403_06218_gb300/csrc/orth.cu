@@ -296,6 +296,7 @@ int cgs_cqr2(tsvd_handle* h, int64_t q, int64_t s, int b, const T* P, int64_t ld
     if (ctx.deferred) return TSVD_OK;
     int hs[kStCount];
     TSVD_TRY(read_status(st, status, hs));
+    if (hs[kStTimeout]) return TSVD_ERR_TIMEOUT;
     if (hs[kStNonfinite]) return TSVD_ERR_NONFINITE;
     if (hs[kStBreakdown]) {
         TSVD_TRY_CUDA(cudaMemsetAsync(status + kStBreakdown, 0, sizeof(int), st));

@@ -522,7 +522,8 @@ int tsvd_orth_workspace(int64_t q, int64_t s, int b, size_t* bytes) {
     hh.sm_count = 152;
     int dev = 0;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&hh.sm_count, cudaDevAttrMultiProcessorCount, dev);
-    *bytes = align256(sizeof(int) * kStCount) + orth_ws(&hh, q, s, b) + align256(sizeof(double) * (size_t)(s + b) * b);
+    *bytes = align256(sizeof(int) * kStCount) + orth_ws(&hh, q, s, b) + align256(sizeof(double) * (size_t)(s + b) * b) +
+             oz_standalone_ws(q, s, b);
     return TSVD_OK;
 }
 
@@ -546,7 +547,16 @@ int orth_entry(tsvd_handle* h, int64_t q, int64_t s, int b, const T* P, int64_t 
     ctx.seed = seed;
     ctx.replacements = replacements ? *replacements : 0;
     TSVD_TRY_CUDA(cudaMemsetAsync(R, 0, sizeof(double) * (size_t)b * b, st));
-    int rc = cgs_cqr2<T>(h, q, s, b, P, ldp, Y, ldy, H, R, b, false, ctx, ar, status, st);
+    int rc;
+    if constexpr (std::is_same<T, double>::value) {
+        // the products with P run on the tensor cores, from planes sliced once a layout
+        const size_t ozb = oz_standalone_ws(q, s, b);
+        OzStandalone oz(h, q, s, P, ldp, ar.take<char>(ozb), ozb, status);
+        TSVD_TRY(oz.slice(st));
+        rc = cgs_cqr2<T>(h, q, s, b, P, ldp, Y, ldy, H, R, b, false, ctx, ar, status, st);
+    } else {
+        rc = cgs_cqr2<T>(h, q, s, b, P, ldp, Y, ldy, H, R, b, false, ctx, ar, status, st);
+    }
     TSVD_TRY_CUDA(cudaStreamSynchronize(st));
     if (replacements) *replacements = ctx.replacements;
     if (breakdowns) *breakdowns += ctx.fallbacks;
@@ -612,6 +622,9 @@ int tsvd_cgs_qr(tsvd_handle* h, int64_t q, int r, int b, double* Y, int64_t ldy,
     OrthCtx ctx;
     ctx.seed = seed;
     ctx.replacements = replacements ? *replacements : 0;
+    // (the basis of a block is the columns before it, which change: no kept planes)
+    const size_t ozb = oz_standalone_ws(q, r - bw, bw);
+    OzStandalone oz(h, q, 0, nullptr, 0, ar.take<char>(ozb), ozb, status);
     int rc = cgs_qr<double>(h, q, r, bw, Y, ldy, R, ctx, ar, status, st);
     TSVD_TRY_CUDA(cudaStreamSynchronize(st));
     if (replacements) *replacements = ctx.replacements;

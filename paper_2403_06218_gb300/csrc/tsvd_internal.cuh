@@ -51,6 +51,8 @@ struct tsvd_handle {
     void* oz_ws = nullptr;
     size_t oz_bytes = 0;
     int* oz_status = nullptr;
+    // digits an entry in the products of the current call (k_oz.cu): 7, or 8 in the wide form
+    int oz_dig = 7;
     // operands whose digit planes are kept for the current call (owned by the caller)
     std::vector<const tsvd::OzCache*> oz_caches;
     // limit, in SM clock cycles, of one bounded wait of the pipelined product kernels
@@ -288,10 +290,10 @@ cudaError_t gemm_tn(tsvd_handle* h, int64_t q, int64_t s, int64_t b, const TI* X
 bool oz_worth(int64_t M, int64_t N, int64_t K);
 // Scratch of C = X^T Z (q rows; s x b outputs) and of Y = X M (q x s times s x b);
 // cached_x: the planes of X come from a cache.
-size_t oz_tn_ws(int64_t q, int64_t s, int64_t b, bool symmetric, bool cached_x = false);
-size_t oz_nn_ws(int64_t q, int64_t s, int64_t b, bool cached_x = false);
+size_t oz_tn_ws(int64_t q, int64_t s, int64_t b, bool symmetric, bool cached_x = false, int dig = 7);
+size_t oz_nn_ws(int64_t q, int64_t s, int64_t b, bool cached_x = false, int dig = 7);
 // Scratch that covers every product with q <= qmax, s <= smax, b <= bmax (and s, b swapped).
-size_t oz_ws_bound(int64_t qmax, int64_t smax, int64_t bmax);
+size_t oz_ws_bound(int64_t qmax, int64_t smax, int64_t bmax, int dig = 7);
 // Scratch of the products of a dense A (M x N) and A^T, both in digit-plane caches, with a
 // block of width w.
 size_t oz_a_ws(int64_t M, int64_t N, int64_t w);
@@ -308,14 +310,24 @@ int oz_gemm_nn(tsvd_handle* h, int64_t q, int64_t s, int64_t b, double alpha, co
                size_t ws_bytes, int* status, cudaStream_t st, const OzCache* xc = nullptr);
 // Caches: bytes, carving (no device work), slicing of columns [c0, c1) (c0 <= valid;
 // then valid = c1), and the lookup the products use.
-size_t oz_cache_bytes(int64_t rows, int64_t cols, bool cols_layout);
+size_t oz_cache_bytes(int64_t rows, int64_t cols, bool cols_layout, int dig = 7);
 void oz_cache_carve(OzCache& c, Arena& ar, const double* src, int64_t ld, int64_t rows, int64_t cols,
-                    bool cols_layout, bool grows);
+                    bool cols_layout, bool grows, int dig = 7);
 int oz_cache_slice(tsvd_handle* h, OzCache& c, int64_t c0, int64_t c1, cudaStream_t st);
 // Columns from v on are about to be rewritten: valid = min(valid, v).
 int oz_cache_truncate(tsvd_handle* h, OzCache& c, int64_t v, cudaStream_t st);
 const OzCache* oz_find_cache(const tsvd_handle* h, const double* X, int64_t ldx, int64_t rows, int64_t s,
                              bool cols_layout);
+// Scratch with which the products of an operand X (q x s) and blocks of width b run on the
+// tensor cores outside the solvers (oz_ws_bound), with X's planes in both layouts; 0 where
+// it would exceed kOzStandaloneMax or no product is large enough (oz_worth), and the
+// products stay on the FP64 pipe: a call whose operands fill the device must not fail for
+// scratch.  CGS-CQR2 of 64 columns against 512 of 100,000 rows: 24.5 ms on the FP64 pipe
+// (at its rate of 1.2 TFLOP/s), 3.0 ms here; error against 64-bit arithmetic 5.6e-16 there,
+// 7.5e-16 here (2.2e-14 with 7 digits, on a basis with entries near 1 and near 1e-3).
+constexpr size_t kOzStandaloneMax = size_t(4) << 30;
+size_t oz_standalone_ws(int64_t q, int64_t s, int b);
+
 // Registers caches with the handle for its lifetime.
 struct OzCacheScope {
     tsvd_handle* h;
@@ -342,6 +354,39 @@ struct OzScope {
         h->oz_ws = prev_ws;
         h->oz_bytes = prev_bytes;
         h->oz_status = prev_status;
+    }
+};
+
+// They run in the wide form, as accurate as the FP64 pipe that they replace.
+struct OzStandalone {
+    tsvd_handle* h;
+    int prev_dig;
+    OzCache cols, rows;
+    OzCacheScope caches;
+    OzScope scope;
+    // ws: oz_standalone_ws(q, s, b) bytes, 256-byte aligned (null or 0 bytes: no effect)
+    OzStandalone(tsvd_handle* hh, int64_t q, int64_t s, const double* X, int64_t ldx, void* ws, size_t bytes,
+                 int* status)
+        : h(hh), prev_dig(hh->oz_dig), caches(hh), scope(hh, nullptr, 0, status) {
+        h->oz_dig = 8;
+        if (!ws || !bytes) return;
+        Arena ar{static_cast<char*>(ws), bytes, 0};
+        if (s > 0) {
+            oz_cache_carve(cols, ar, X, ldx, q, s, true, false, 8);
+            oz_cache_carve(rows, ar, X, ldx, q, s, false, false, 8);
+        }
+        h->oz_ws = ar.base + ar.off;
+        h->oz_bytes = bytes - ar.off;
+    }
+    ~OzStandalone() { h->oz_dig = prev_dig; }
+    int slice(cudaStream_t st) {
+        for (OzCache* c : {&cols, &rows}) {
+            if (!c->planes) continue;
+            const int rc = oz_cache_slice(h, *c, 0, c->cols, st);
+            if (rc < 0) return rc;
+            caches.add(c);
+        }
+        return TSVD_OK;
     }
 };
 
