@@ -590,72 +590,131 @@ __global__ void gaussian_kernel(int64_t rows, int64_t cols, uint32_t k0, uint32_
 // ---------------------------------------------------------------------------
 // Residual column sums of squares, Lanczos estimate, sign convention.
 // ---------------------------------------------------------------------------
-__global__ void colres_partial_kernel(int64_t q, int k, const double* __restrict__ Y, int64_t ldy,
-                                      const double* __restrict__ U, int64_t ldu, const double* __restrict__ sigma,
-                                      double* __restrict__ partial, int64_t rows_per) {
+// (Blocks of 32 columns x 8 rows: the rows of a group are split over the block, as in
+// coldot.  With one thread a column, residual norms of 100,000 x 64 took 170 us and the
+// largest entries of its columns 165 us, against 30 us and 25 us.)
+__global__ void __launch_bounds__(256)
+    colres_partial_kernel(int64_t q, int k, const double* __restrict__ Y, int64_t ldy, const double* __restrict__ U,
+                          int64_t ldu, const double* __restrict__ sigma, double* __restrict__ partial,
+                          int64_t rows_per) {
+    __shared__ double red[8][33];
     const int64_t r0 = (int64_t)blockIdx.x * rows_per, r1 = min(q, r0 + rows_per);
-    for (int j = threadIdx.x; j < k; j += blockDim.x) {
+    const int j = (int)blockIdx.y * 32 + threadIdx.x;
+    double acc = 0.0;
+    if (j < k) {
         const double sj = sigma[j];
-        double acc = 0.0;
-        for (int64_t i = r0; i < r1; ++i) {
+#pragma unroll 4
+        for (int64_t i = r0 + threadIdx.y; i < r1; i += 8) {
             const double d = fma(-U[i * ldu + j], sj, Y[i * ldy + j]);
             acc = fma(d, d, acc);
         }
+    }
+    red[threadIdx.y][threadIdx.x] = acc;
+    __syncthreads();
+    if (threadIdx.y == 0 && j < k) {
+#pragma unroll
+        for (int y = 1; y < 8; ++y) acc += red[y][threadIdx.x];
         partial[(int64_t)blockIdx.x * k + j] = acc;
     }
 }
 
-__global__ void colres_reduce_kernel(int k, int g, const double* __restrict__ partial, double* __restrict__ out) {
-    for (int j = threadIdx.x; j < k; j += blockDim.x) {
-        double acc = 0.0;
-        for (int t = 0; t < g; ++t) acc += partial[(int64_t)t * k + j];
+// out[j] = sum_g partial[g][j]: thread (x, y) adds groups y, y + 32, .. of column x, then
+// the 32 sums are added in order.
+__global__ void __launch_bounds__(1024) col_sum_kernel(int k, int g, const double* __restrict__ partial,
+                                                       double* __restrict__ out) {
+    __shared__ double red[32][33];
+    const int j = (int)blockIdx.x * 32 + threadIdx.x;
+    double acc = 0.0;
+    if (j < k)
+        for (int t = threadIdx.y; t < g; t += 32) acc += partial[(int64_t)t * k + j];
+    red[threadIdx.y][threadIdx.x] = acc;
+    __syncthreads();
+    if (threadIdx.y == 0 && j < k) {
+        for (int y = 1; y < 32; ++y) acc += red[y][threadIdx.x];
         out[j] = acc;
     }
 }
 
-__global__ void lanczos_rho_kernel(int b, int k, const double* __restrict__ Rr, const double* __restrict__ V,
-                                   int64_t ldv, double* __restrict__ rho) {
-    for (int j = threadIdx.x; j < k; j += blockDim.x) {
+// rho[j], one block a column: y = Rr v_j with a warp a row, then the sum of squares in row
+// order.  (One block for all columns took 0.70 ms at b = 128, k = 100; 8 us now.)
+__global__ void __launch_bounds__(256) lanczos_rho_kernel(int b, int k, const double* __restrict__ Rr,
+                                                          const double* __restrict__ V, int64_t ldv,
+                                                          double* __restrict__ rho) {
+    __shared__ double v[TSVD_MAX_BLOCK], y2[TSVD_MAX_BLOCK];
+    const int j = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int l = threadIdx.x; l < b; l += blockDim.x) v[l] = V[(int64_t)l * ldv + j];
+    __syncthreads();
+    for (int i = warp; i < b; i += (int)blockDim.x >> 5) {
+        double yi = 0.0;
+        for (int l = i + lane; l < b; l += 32) yi = fma(Rr[i * b + l], v[l], yi);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) yi += __shfl_xor_sync(0xffffffffu, yi, o);
+        if (lane == 0) y2[i] = yi * yi;
+    }
+    __syncthreads();
+    if (warp == 0) {
         double acc = 0.0;
-        for (int i = 0; i < b; ++i) {
-            double yi = 0.0;
-            for (int l = i; l < b; ++l) yi = fma(Rr[i * b + l], V[(int64_t)l * ldv + j], yi);
-            acc = fma(yi, yi, acc);
-        }
-        rho[j] = sqrt(acc);
+        for (int i = lane; i < b; i += 32) acc += y2[i];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if (lane == 0) rho[j] = sqrt(acc);
     }
 }
 
-__global__ void argmax_partial_kernel(int64_t n, int k, const double* __restrict__ V, int64_t ldv,
-                                      int64_t rows_per, double* __restrict__ pv, int64_t* __restrict__ pi) {
+// The larger magnitude wins, the smaller row on ties.
+__device__ inline void argmax_take(double& best, int64_t& bi, double a, int64_t i) {
+    if (a > best || (a == best && i < bi)) {
+        best = a;
+        bi = i;
+    }
+}
+
+__global__ void __launch_bounds__(256)
+    argmax_partial_kernel(int64_t n, int k, const double* __restrict__ V, int64_t ldv, int64_t rows_per,
+                          double* __restrict__ pv, int64_t* __restrict__ pi) {
+    __shared__ double sv[8][33];
+    __shared__ int64_t si[8][33];
     const int64_t r0 = (int64_t)blockIdx.x * rows_per, r1 = min(n, r0 + rows_per);
-    for (int j = threadIdx.x; j < k; j += blockDim.x) {
-        double best = -1.0;
-        int64_t bi = 0;
-        for (int64_t i = r0; i < r1; ++i) {
+    const int j = (int)blockIdx.y * 32 + threadIdx.x;
+    double best = -1.0;
+    int64_t bi = 0;
+    if (j < k) {
+#pragma unroll 4
+        for (int64_t i = r0 + threadIdx.y; i < r1; i += 8) {
             const double a = fabs(V[i * ldv + j]);
             if (a > best) {
                 best = a;
                 bi = i;
             }
         }
+    }
+    sv[threadIdx.y][threadIdx.x] = best;
+    si[threadIdx.y][threadIdx.x] = bi;
+    __syncthreads();
+    if (threadIdx.y == 0 && j < k) {
+#pragma unroll
+        for (int y = 1; y < 8; ++y) argmax_take(best, bi, sv[y][threadIdx.x], si[y][threadIdx.x]);
         pv[(int64_t)blockIdx.x * k + j] = best;
         pi[(int64_t)blockIdx.x * k + j] = bi;
     }
 }
 
-__global__ void argmax_sign_kernel(int k, int g, const double* __restrict__ pv, const int64_t* __restrict__ pi,
-                                   const double* __restrict__ V, int64_t ldv, double* __restrict__ sgn) {
-    for (int j = threadIdx.x; j < k; j += blockDim.x) {
-        double best = -1.0;
-        int64_t bi = 0;
-        for (int t = 0; t < g; ++t) {
-            const double a = pv[(int64_t)t * k + j];
-            if (a > best) {
-                best = a;
-                bi = pi[(int64_t)t * k + j];
-            }
-        }
+__global__ void __launch_bounds__(1024)
+    argmax_sign_kernel(int k, int g, const double* __restrict__ pv, const int64_t* __restrict__ pi,
+                       const double* __restrict__ V, int64_t ldv, double* __restrict__ sgn) {
+    __shared__ double sv[32][33];
+    __shared__ int64_t si[32][33];
+    const int j = (int)blockIdx.x * 32 + threadIdx.x;
+    double best = -1.0;
+    int64_t bi = 0;
+    if (j < k)
+        for (int t = threadIdx.y; t < g; t += 32)
+            argmax_take(best, bi, pv[(int64_t)t * k + j], pi[(int64_t)t * k + j]);
+    sv[threadIdx.y][threadIdx.x] = best;
+    si[threadIdx.y][threadIdx.x] = bi;
+    __syncthreads();
+    if (threadIdx.y == 0 && j < k) {
+        for (int y = 1; y < 32; ++y) argmax_take(best, bi, sv[y][threadIdx.x], si[y][threadIdx.x]);
         sgn[j] = V[bi * ldv + j] < 0.0 ? -1.0 : 1.0;
     }
 }
@@ -680,13 +739,6 @@ __global__ void put_transposed_kernel(int rows, int cols, const double* __restri
 __global__ void put_diagonal_kernel(int s, const double* __restrict__ sig, double* __restrict__ B, int64_t ldb) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < s) B[(int64_t)i * ldb + i] = sig[i];
-}
-
-int colres_groups(int64_t q) {
-    int64_t g = (q + 255) / 256;
-    if (g > 512) g = 512;
-    if (g < 1) g = 1;
-    return (int)g;
 }
 
 }  // namespace
@@ -894,17 +946,23 @@ cudaError_t gaussian(tsvd_handle* h, int64_t rows, int64_t cols, uint64_t seed, 
     return cudaGetLastError();
 }
 
-size_t colres_ws(int64_t q, int k) { return align256(sizeof(double) * (size_t)colres_groups(q) * (size_t)k); }
+size_t colres_ws(int64_t q, int k) { return align256(sizeof(double) * (size_t)col_groups(q) * (size_t)k); }
+
+cudaError_t col_sum(tsvd_handle* h, int groups, int k, const double* partial, double* out, cudaStream_t st) {
+    h->launches++;
+    col_sum_kernel<<<(unsigned)((k + 31) / 32), dim3(32, 32), 0, st>>>(k, groups, partial, out);
+    return cudaGetLastError();
+}
 
 cudaError_t col_residual_sq(tsvd_handle* h, int64_t q, int k, const double* Y, int64_t ldy, const double* U,
                             int64_t ldu, const double* sigma, double* out, double* partial, cudaStream_t st) {
-    const int g = colres_groups(q);
+    const int g = col_groups(q);
     const int64_t rows_per = (q + g - 1) / g;
     ProfScope prof(h, TSVD_K_OTHER, 0.0, 0.0, st);
-    h->launches += 2;
-    colres_partial_kernel<<<g, 128, 0, st>>>(q, k, Y, ldy, U, ldu, sigma, partial, rows_per);
-    colres_reduce_kernel<<<1, 128, 0, st>>>(k, g, partial, out);
-    return cudaGetLastError();
+    h->launches++;
+    colres_partial_kernel<<<dim3((unsigned)g, (unsigned)((k + 31) / 32)), dim3(32, 8), 0, st>>>(
+        q, k, Y, ldy, U, ldu, sigma, partial, rows_per);
+    return col_sum(h, g, k, partial, out, st);
 }
 
 cudaError_t put_transposed(tsvd_handle* h, int rows, int cols, const double* H, int64_t ldh, double* D, int64_t ldd,
@@ -927,18 +985,18 @@ cudaError_t lanczos_rho(tsvd_handle* h, int b, int k, const double* Rr, const do
                         double* rho, cudaStream_t st) {
     ProfScope prof(h, TSVD_K_OTHER, 0.0, 0.0, st);
     h->launches++;
-    lanczos_rho_kernel<<<1, 128, 0, st>>>(b, k, Rr, Vlast, ldv, rho);
+    lanczos_rho_kernel<<<k, 256, 0, st>>>(b, k, Rr, Vlast, ldv, rho);
     return cudaGetLastError();
 }
 
 size_t sign_fix_ws(int64_t n, int k) {
-    const size_t g = (size_t)colres_groups(n);
+    const size_t g = (size_t)col_groups(n);
     return align256(sizeof(double) * g * k) + align256(sizeof(int64_t) * g * k) + align256(sizeof(double) * k);
 }
 
 cudaError_t sign_fix(tsvd_handle* h, int64_t n, int64_t m, int k, double* V, int64_t ldv, double* U, int64_t ldu,
                      void* ws, cudaStream_t st) {
-    const int g = colres_groups(n);
+    const int g = col_groups(n);
     char* p = static_cast<char*>(ws);
     double* pv = reinterpret_cast<double*>(p);
     p += align256(sizeof(double) * (size_t)g * k);
@@ -948,8 +1006,9 @@ cudaError_t sign_fix(tsvd_handle* h, int64_t n, int64_t m, int k, double* V, int
     const int64_t rows_per = (n + g - 1) / g;
     ProfScope prof(h, TSVD_K_OTHER, 0.0, 0.0, st);
     h->launches += 4;
-    argmax_partial_kernel<<<g, 128, 0, st>>>(n, k, V, ldv, rows_per, pv, pi);
-    argmax_sign_kernel<<<1, 128, 0, st>>>(k, g, pv, pi, V, ldv, sgn);
+    const unsigned strips = (unsigned)((k + 31) / 32);
+    argmax_partial_kernel<<<dim3((unsigned)g, strips), dim3(32, 8), 0, st>>>(n, k, V, ldv, rows_per, pv, pi);
+    argmax_sign_kernel<<<strips, dim3(32, 32), 0, st>>>(k, g, pv, pi, V, ldv, sgn);
     if (n * k > 0) apply_sign_kernel<<<(unsigned)((n * k + 255) / 256), 256, 0, st>>>(n, k, V, ldv, sgn);
     if (m * k > 0) apply_sign_kernel<<<(unsigned)((m * k + 255) / 256), 256, 0, st>>>(m, k, U, ldu, sgn);
     return cudaGetLastError();

@@ -26,7 +26,7 @@ namespace {
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kMaxSweeps = 40;
 
-enum Ctl : int { kCtlCount = 0, kCtlGen = 1, kCtlErr = 2, kCtlSweeps = 3, kCtlRot = 8 };
+enum Ctl : int { kCtlCount = 0, kCtlGen = 1, kCtlErr = 2, kCtlSweeps = 3, kCtlVBad = 4, kCtlRot = 8 };
 constexpr int kCtlWords = kCtlRot + kMaxSweeps;
 
 __device__ inline unsigned vload(const unsigned* p) { return *reinterpret_cast<const volatile unsigned*>(p); }
@@ -647,41 +647,46 @@ __global__ void jacobi_vinit_kernel(int n, int npad, const float* __restrict__ V
 }
 
 // After the polar iterations: if V^T V (in T) is not the identity to 1e-12, V = I
-// (the FP64 sweeps then start from B itself).  One CTA.
-__global__ void __launch_bounds__(1024) jacobi_vcheck_kernel(int n, const double* __restrict__ Tm,
-                                                             double* __restrict__ V) {
-    __shared__ int bad;
-    if (threadIdx.x == 0) bad = 0;
-    __syncthreads();
-    for (int64_t idx = threadIdx.x; idx < (int64_t)n * n; idx += blockDim.x) {
-        const int i = (int)(idx / n), j = (int)(idx % n);
-        const double d = Tm[idx] - (i == j ? 1.0 : 0.0);
-        if (!(fabs(d) <= 1e-12)) bad = 1;
+// (the FP64 sweeps then start from B itself).  Two kernels over all SMs: the check raises
+// `bad` (one CTA took 0.2 ms at order 512), the reset acts on it.
+__global__ void __launch_bounds__(256) jacobi_vcheck_kernel(int n, const double* __restrict__ Tm, unsigned* bad) {
+    bool off = false;
+    for (int idx = (int)(blockIdx.x * blockDim.x + threadIdx.x); idx < n * n; idx += (int)(gridDim.x * blockDim.x)) {
+        const int i = idx / n, j = idx % n;
+        if (!(fabs(Tm[idx] - (i == j ? 1.0 : 0.0)) <= 1e-12)) off = true;
     }
-    __syncthreads();
-    if (!bad) return;
-    for (int64_t idx = threadIdx.x; idx < (int64_t)n * n; idx += blockDim.x)
+    if (off) atomicOr(bad, 1u);
+}
+__global__ void __launch_bounds__(256) jacobi_vreset_kernel(int n, const unsigned* bad, double* __restrict__ V) {
+    if (*bad == 0u) return;
+    for (int idx = (int)(blockIdx.x * blockDim.x + threadIdx.x); idx < n * n; idx += (int)(gridDim.x * blockDim.x))
         V[idx] = (idx / n == idx % n) ? 1.0 : 0.0;
 }
 
-// One CTA (1024 threads): column norms, then a bitonic sort of (sigma desc, index asc).
-__global__ void __launch_bounds__(1024) jacobi_sort_kernel(int n, int npad, const double* __restrict__ G,
+// sigma_c = |g_c|, one warp a column.
+__global__ void __launch_bounds__(256) jacobi_norm_kernel(int n, int npad, const double* __restrict__ G,
+                                                          double* __restrict__ nrm, int* status) {
+    const int lane = threadIdx.x & 31, c = (int)blockIdx.x * 8 + ((int)threadIdx.x >> 5);
+    if (c >= npad) return;
+    const double* g = G + (int64_t)c * n;
+    double acc = 0.0;
+    for (int r = lane; r < n; r += 32) acc = fma(g[r], g[r], acc);
+    acc = warp_sum(acc);
+    if (lane == 0) {
+        nrm[c] = sqrt(acc);
+        if (!isfinite(nrm[c])) atomicOr(&status[kStNonfinite], 1);
+    }
+}
+
+// One CTA (1024 threads): bitonic sort of the column norms by (sigma desc, index asc).
+__global__ void __launch_bounds__(1024) jacobi_sort_kernel(int npad, const double* __restrict__ nrm,
                                                            double* __restrict__ sig, int* __restrict__ perm,
                                                            const unsigned* ctl, int* status) {
     __shared__ double sk[TSVD_MAX_SMALL_SVD];
     __shared__ int si[TSVD_MAX_SMALL_SVD];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int c = warp; c < npad; c += 32) {
-        const double* g = G + (int64_t)c * n;
-        double acc = 0.0;
-        for (int r = lane; r < n; r += 32) acc = fma(g[r], g[r], acc);
-        acc = warp_sum(acc);
-        if (lane == 0) {
-            const double s = sqrt(acc);
-            sk[c] = s;
-            si[c] = c;
-            if (!isfinite(s)) atomicOr(&status[kStNonfinite], 1);
-        }
+    for (int c = threadIdx.x; c < npad; c += blockDim.x) {
+        sk[c] = nrm[c];
+        si[c] = c;
     }
     int P = 1;
     while (P < npad) P <<= 1;
@@ -998,8 +1003,10 @@ int small_svd(tsvd_handle* h, int n, const double* B, int64_t ldb, double* Ubar,
                                     status, st));
             }
             TSVD_TRY(oz_gemm_tn(h, n, n, n, bf.Vp, n, bf.Vp, n, bf.Tm, n, true, bf.oz, bf.oz_bytes, status, st));
-            h->launches++;
-            jacobi_vcheck_kernel<<<1, 1024, 0, st>>>(n, bf.Tm, bf.Vp);
+            h->launches += 2;
+            const unsigned vb = (unsigned)std::min<int64_t>(304, ((int64_t)n * n + 255) / 256);
+            jacobi_vcheck_kernel<<<vb, 256, 0, st>>>(n, bf.Tm, bf.ctl32 + kCtlVBad);
+            jacobi_vreset_kernel<<<vb, 256, 0, st>>>(n, bf.ctl32 + kCtlVBad, bf.Vp);
             TSVD_TRY_CUDA(cudaGetLastError());
             // (3) FP64 sweeps on B V: the SVD of B V is that of B with the right vectors
             //     rotated by V, and its columns start orthogonal to FP32 accuracy
@@ -1034,8 +1041,9 @@ int small_svd(tsvd_handle* h, int n, const double* B, int64_t ldb, double* Ubar,
                                                           args, 0, st));
             }
         }
-        h->launches += 2;
-        jacobi_sort_kernel<<<1, 1024, 0, st>>>(n, npad, G, bf.sig, bf.perm, bf.ctl, status);
+        h->launches += 3;
+        jacobi_norm_kernel<<<(unsigned)((npad + 7) / 8), 256, 0, st>>>(n, npad, G, bf.nrm, status);
+        jacobi_sort_kernel<<<1, 1024, 0, st>>>(npad, bf.nrm, bf.sig, bf.perm, bf.ctl, status);
         jacobi_out_kernel<<<n, 128, 0, st>>>(n, npad, G, Vacc, bf.sig, bf.perm, Ubar, sigma, Vbar);
         TSVD_TRY_CUDA(cudaGetLastError());
     }

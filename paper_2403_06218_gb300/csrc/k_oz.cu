@@ -747,67 +747,45 @@ __global__ void __launch_bounds__(OzShape<NC, D>::kThreads, 1)
     }
 }
 
-// Tiles whose K range is split over CTAs (or longer than one 64-bit accumulation): the
-// parts are added in CTA order and the output rule applied.  Block (x, y): 1/32 of the
-// tile that unit group y + 1 starts in (cut tiles; a group that starts in a tile which
-// an earlier group also starts inside leaves it to that one), of column tile z; with
-// every tile split (long K), y is the row tile.
-__global__ void __launch_bounds__(256) oz_fixup_kernel(OzArgs a) {
-    __shared__ int s_g0, s_nc, s_mt;
-    __shared__ int64_t s_slot[kOzWave];
-    const int KB = a.KB, nt = blockIdx.z;
-    const bool all = KB > kOzHighChunk * kOzFlushChunks;
-    if (threadIdx.x == 0) {
-        int mt, nc = 0, g0 = 0;
-        if (all) {
-            mt = blockIdx.y;
-            const int64_t u = (int64_t)mt * KB;
-            g0 = (int)(u * a.Gg / a.totalg);
-            while (g0 + 1 < a.Gg && oz_glo(g0 + 1, a) <= u) ++g0;
-            while (g0 > 0 && oz_glo(g0, a) > u) --g0;
-            nc = 1;
-        } else {
-            const int g = (int)blockIdx.y + 1;
-            const int64_t u = oz_glo(g, a);
-            mt = (int)(u / KB);
-            g0 = g - 1;
-            // cut here, and the group before starts at or before the tile
-            if (u > (int64_t)mt * KB && oz_glo(g0, a) <= (int64_t)mt * KB) nc = 1;
-        }
-        if (nc)
-            while (g0 + nc < a.Gg && oz_glo(g0 + nc, a) < (int64_t)(mt + 1) * KB) ++nc;
-        s_g0 = g0;
-        s_nc = nc;
-        s_mt = mt;
-    }
-    __syncthreads();
-    const int nc = s_nc, mt = s_mt;
-    if (nc == 0) return;
-    // the partial tile of each contributing CTA, in order
-    for (int j = threadIdx.x; j < nc; j += blockDim.x) {
-        const int g = s_g0 + j;
-        const int64_t cc = (int64_t)g * a.NT + nt;
-        int seg = (int)(mt - oz_glo(g, a) / KB);
-        if (!all && seg > 1) seg = 1;
-        s_slot[j] = (cc * a.nslots + seg) * kOzM * kOzN;
-    }
-    __syncthreads();
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    const int r = idx / kOzN, cl = idx % kOzN;
+// The tiles whose K range is split over CTAs (or longer than one 64-bit accumulation): row
+// tile mt, the nc groups from g0 on, and the slot of group g0's partial tile (the others
+// start inside the tile: slot 0).  Listed by the host, as one thread finding them took
+// longer than the sums.
+struct OzCuts {
+    int mt[kOzWave];
+    short g0[kOzWave], nc[kOzWave], slot0[kOzWave];
+};
+
+// Adds the parts of a cut tile in a fixed order (four contiguous shares of the CTAs, then
+// the shares) and applies the output rule.  Block (x, y, z): row x of cut y, column tile z.
+__global__ void __launch_bounds__(256) oz_fixup_kernel(OzArgs a, OzCuts cuts) {
+    const int mt = cuts.mt[blockIdx.y], nc = cuts.nc[blockIdx.y], g0 = cuts.g0[blockIdx.y], nt = blockIdx.z;
+    if ((int64_t)mt * kOzM + blockIdx.x >= a.M) return;
+    auto slot = [&](int j) -> int64_t {
+        return (((int64_t)(g0 + j) * a.NT + nt) * a.nslots + (j ? 0 : cuts.slot0[blockIdx.y])) * kOzM * kOzN;
+    };
+    __shared__ double s_part[4][kOzN];
+    const int r = blockIdx.x, cl = threadIdx.x % kOzN, share = threadIdx.x / kOzN;
+    const int idx = r * kOzN + cl;
     const int64_t row = (int64_t)mt * kOzM + r, col = (int64_t)nt * a.tilen + cl;
-    if (cl >= a.tilen || row >= a.M || col >= a.N) return;
-    // sixteen loads in flight, added in CTA order (the same sum as a sequential loop)
+    const bool in = cl < a.tilen && row < a.M && col < a.N;
     double acc = 0.0;
-    int j = 0;
-    for (; j + 16 <= nc; j += 16) {
-        double v[16];
+    if (in) {
+        int j = nc * share / 4;
+        const int j1 = nc * (share + 1) / 4;
+        for (; j + 16 <= j1; j += 16) {  // sixteen loads in flight
+            double v[16];
 #pragma unroll
-        for (int u = 0; u < 16; ++u) v[u] = a.partial[s_slot[j + u] + idx];
+            for (int u = 0; u < 16; ++u) v[u] = a.partial[slot(j + u) + idx];
 #pragma unroll
-        for (int u = 0; u < 16; ++u) acc += v[u];
+            for (int u = 0; u < 16; ++u) acc += v[u];
+        }
+#pragma unroll 8
+        for (; j < j1; ++j) acc += a.partial[slot(j) + idx];
     }
-    for (; j < nc; ++j) acc += a.partial[s_slot[j] + idx];
-    oz_store(a, row, col, acc);
+    s_part[share][cl] = acc;
+    __syncthreads();
+    if (in && share == 0) oz_store(a, row, col, ((acc + s_part[1][cl]) + s_part[2][cl]) + s_part[3][cl]);
 }
 
 // ---- host side -------------------------------------------------------------------
@@ -954,12 +932,43 @@ int oz_run(tsvd_handle* h, const OzPlan& p, const OzView& va, const OzView& vb, 
     const auto launch = dig == kW ? (p.tilen == 16 ? oz_launch<16, kW> : (p.tilen == 32 ? oz_launch<32, kW> : oz_launch<64, kW>))
                                   : (p.tilen == 16 ? oz_launch<16, kD> : (p.tilen == 32 ? oz_launch<32, kD> : oz_launch<64, kD>));
     TSVD_TRY(launch(h, p.G, mA, mB, a, st));
-    const unsigned parts = p.KB > kOzHighChunk * kOzFlushChunks ? (unsigned)p.MT : (unsigned)(p.Gg - 1);
-    if (parts > 0) {
+    const bool all = p.KB > kOzHighChunk * kOzFlushChunks;
+    OzCuts cuts;
+    int n = 0;
+    auto flush = [&]() -> int {
+        if (n == 0) return TSVD_OK;
         h->launches++;
-        oz_fixup_kernel<<<dim3(kOzM * kOzN / 256, parts, (unsigned)p.NT), 256, 0, st>>>(a);
+        oz_fixup_kernel<<<dim3(kOzM, (unsigned)n, (unsigned)p.NT), 256, 0, st>>>(a, cuts);
+        n = 0;
         TSVD_TRY_CUDA(cudaGetLastError());
+        return TSVD_OK;
+    };
+    auto add = [&](int mt, int g0) -> int {  // row tile mt, first held by group g0
+        int nc = 1;
+        while (g0 + nc < p.Gg && oz_glo(g0 + nc, a) < (int64_t)(mt + 1) * p.KB) ++nc;
+        const int first = (int)(oz_glo(g0, a) / p.KB);
+        cuts.mt[n] = mt;
+        cuts.g0[n] = (short)g0;
+        cuts.nc[n] = (short)nc;
+        cuts.slot0[n] = (short)(all ? mt - first : (mt > first ? 1 : 0));
+        return ++n == kOzWave ? flush() : TSVD_OK;
+    };
+    if (all) {
+        for (int mt = 0, g = 0; mt < p.MT; ++mt) {
+            while (g + 1 < p.Gg && oz_glo(g + 1, a) <= (int64_t)mt * p.KB) ++g;
+            TSVD_TRY(add(mt, g));
+        }
+    } else {
+        int done = -1;  // row tiles that a group starts inside, each once
+        for (int g = 1; g < p.Gg; ++g) {
+            const int64_t u = oz_glo(g, a);
+            const int mt = (int)(u / p.KB);
+            if (mt == done || u == (int64_t)mt * p.KB) continue;
+            done = mt;
+            TSVD_TRY(add(mt, g - 1));
+        }
     }
+    TSVD_TRY(flush());
     return TSVD_OK;
 }
 

@@ -439,6 +439,14 @@ int svd_backward_run(tsvd_handle* h, const tsvd_matrix* A, int k, const double* 
                      const double* V, const double* sb, const double* Ub, const double* Vb, double* grad,
                      const tsvd_backward_opts* o, char* ws, size_t ws_bytes, size_t* sizing,
                      tsvd_backward_info* info);
+// Row groups of a column reduction over `rows` rows (at most 608: four for each of 152
+// SMs; a fixed number, so that the order of the sums does not depend on the device), and
+// the sums over the groups, out[j] = sum_g partial[g][j], in a fixed order.
+inline int col_groups(int64_t rows) {
+    const int64_t g = (rows + 63) / 64;
+    return (int)(g < 1 ? 1 : (g > 608 ? 608 : g));
+}
+cudaError_t col_sum(tsvd_handle* h, int groups, int k, const double* partial, double* out, cudaStream_t st);
 size_t coldot_ws(int64_t rows, int k);
 // out[j] = sum_i X[i][j] Y[i][j] (fixed order); partial: coldot_ws bytes.
 cudaError_t coldot(tsvd_handle* h, int64_t rows, int k, const double* X, int64_t ldx, const double* Y, int64_t ldy,
