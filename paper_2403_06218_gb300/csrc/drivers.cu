@@ -321,8 +321,7 @@ int setup_op(tsvd_handle* h, const tsvd_matrix* A, int wmax, Arena& ar, Op<T>& o
             oz_cache_carve(op.ozA[1], ar, op.dA64, op.lda64, M, N, true, false);
             if (run) {
                 if (!ar.fits()) return TSVD_ERR_WORKSPACE;
-                TSVD_TRY(oz_cache_slice(h, op.ozA[0], 0, N, st));
-                TSVD_TRY(oz_cache_slice(h, op.ozA[1], 0, N, st));
+                TSVD_TRY(oz_cache_slice_both(h, op.ozA[0], op.ozA[1], st));
             }
         }
     }

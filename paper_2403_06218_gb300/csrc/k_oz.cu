@@ -106,9 +106,12 @@ __device__ inline int oz_exp(double x) {
 
 __device__ inline int oz_norm_exp(int e) { return e <= kOzZeroExp ? 0 : e; }
 
-// round(x 2^(8 D - 1 - e)) (ties away from zero) as D balanced base-256 digits.
+// F = round(x 2^(T - e)) (ties away from zero; T = 8 D - 1) plus
+// sum_p 128 256^p over the D digits: digit p of F is then byte D - 1 - p of the sum less 128
+// (the leading one may need a ninth bit: with 8 digits it is lost, and 128 reads as -128).
 template <int D>
-__device__ inline void oz_digits(double x, int e, int (&d)[D]) {
+__device__ inline unsigned long long oz_biased(double x, int e) {
+    constexpr int T = 8 * D - 1;
     const uint64_t u = (uint64_t)__double_as_longlong(x);
     const int be = (int)((u >> 52) & 0x7FF);
     uint64_t m = u & ((1ull << 52) - 1);
@@ -117,28 +120,24 @@ __device__ inline void oz_digits(double x, int e, int (&d)[D]) {
         m |= 1ull << 52;
         q = be - 1075;
     }
-    int64_t F = 0;
-    if (be != 0x7FF && e < kOzNanExp && m != 0) {
-        const int sh = q + 8 * D - 1 - e;  // <= 8 D - 54 when |x| < 2^e
-        if (sh >= 0) {
-            F = (int64_t)(m << sh);
-        } else if (sh > -54) {
-            F = (int64_t)((m + (1ull << (-sh - 1))) >> (-sh));
-        }
-        if (u >> 63) F = -F;
-    }
-    int64_t r = F;
-#pragma unroll
-    for (int p = D - 1; p >= 1; --p) {
-        const int lo = (int)(((unsigned)r + 128u) & 255u) - 128;
-        d[p] = lo;
-        r = (r - lo) >> 8;
-    }
-    d[0] = (int)r;
+    // a row holding Inf or NaN has an exponent that shifts everything out
+    const int sh = q + T - e;  // <= T - 53 when |x| < 2^e
+    uint64_t F = 0;
+    if (sh >= 0)
+        F = m << sh;
+    else if (sh > -54)
+        F = (m + (1ull << (-sh - 1))) >> (-sh);
+    if (u >> 63) F = 0ull - F;
+    return F + (D == 7 ? 0x80808080808080ull : 0x8080808080808080ull);
 }
 
-__device__ inline __nv_bfloat162 oz_pack(int d0, int d1) {
-    return __floats2bfloat162_rn((float)d0, (float)d1);  // exact: |d| <= 128
+// Digit p as a float: the byte becomes the low mantissa bits of 2^23.
+template <int D>
+__device__ inline float oz_digit(unsigned long long w, int p) {
+    const int i = D - 1 - p;
+    const unsigned half = i < 4 ? (unsigned)w : (unsigned)(w >> 32);
+    const unsigned sel = D == 7 && p == 0 ? 0x7432u : 0x7540u | (unsigned)(i & 3);
+    return __uint_as_float(__byte_perm(half, 0x4B000000u, sel)) - 8388736.0f;  // 2^23 + 128
 }
 
 // Global layout of the digit planes: K-block major, and within a block the very bytes that
@@ -157,51 +156,40 @@ __host__ __device__ inline int64_t oz_off(int64_t Ra, int64_t r, int64_t k, int 
 __host__ __device__ inline int64_t oz_k16(int64_t K) { return (K + 15) / 16 * 16; }
 inline int64_t oz_ra(int64_t rows) { return (rows + 15) / 16 * 16; }
 
-// Stores the digits of (x0, x1) at columns (k, k + 1), k even, of stored row r.
+// Stores the digits of (x0, x1) at columns (k, k + 1), k even, of stored row r.  The slicers
+// give 8 lanes to the 16 columns of a K block and the 4 groups of 8 to consecutive stored
+// rows, so that a warp's store of one digit is 128 contiguous bytes.
 template <int D>
-__device__ inline void oz_store_pair(__nv_bfloat16* planes, int64_t Ra, int64_t r, int64_t k, const int (&da)[D],
-                                     const int (&db)[D]) {
+__device__ inline void oz_store_pair(__nv_bfloat16* planes, int64_t Ra, int64_t r, int64_t k, double x0, double x1,
+                                     int e) {
+    const unsigned long long a = oz_biased<D>(x0, e), b = oz_biased<D>(x1, e);
     __nv_bfloat162* dst = reinterpret_cast<__nv_bfloat162*>(planes + oz_off<D>(Ra, r, k, 0));
 #pragma unroll
-    for (int p = 0; p < D; ++p) dst[p * Ra * 8] = oz_pack(da[p], db[p]);  // plane step Ra*16 elements
-}
-
-// Rows slicer: row i of S (R x K, lds) -> stored row i; one warp per row.
-template <int D>
-__global__ void __launch_bounds__(256, 4) oz_slice_rows_kernel(int64_t R, int64_t K, const double* __restrict__ S,
-                                                            int64_t lds, __nv_bfloat16* __restrict__ planes,
-                                                            int64_t Ra, int* __restrict__ eexp) {
-    const int lane = threadIdx.x & 31;
-    const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
-    const int64_t K16 = oz_k16(K);
-    for (int64_t i = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < R; i += nw) {
-        const double* src = S + i * lds;
-        int e = kOzZeroExp;
-        for (int64_t k = lane; k < K; k += 32) e = max(e, oz_exp(src[k]));
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
-        e = oz_norm_exp(e);
-        if (lane == 0) eexp[i] = e;
-        for (int64_t k = 2 * lane; k < K16; k += 64) {
-            int da[D], db[D];
-            oz_digits(k < K ? src[k] : 0.0, e, da);
-            oz_digits(k + 1 < K ? src[k + 1] : 0.0, e, db);
-            oz_store_pair(planes, Ra, i, k, da, db);
+    for (int p = 0; p < D; ++p) {  // exact: |digit| <= 128; plane step Ra * 16 elements
+        float da = oz_digit<D>(a, p), db = oz_digit<D>(b, p);
+        if (D == 8 && p == 0) {  // the leading digit has the entry's sign
+            da = x0 > 0.0 ? fabsf(da) : da;
+            db = x1 > 0.0 ? fabsf(db) : db;
         }
+        dst[p * Ra * 8] = __floats2bfloat162_rn(da, db);
     }
 }
 
-// Rows slicer of a matrix that grows by columns (a Lanczos basis): columns [c0, c1) of S
-// (R rows, lds), zeros from c1 to the next multiple of 16; G lanes a row.  A row's exponent
-// is one above its largest entry when it was set (at c0 = 0, or when a later entry does
-// not fit it: the row's earlier columns are then sliced again), so that new columns rarely
-// raise it.  That keeps 55 bits below the row's largest entry; one exponent for all rows of
-// an orthonormal basis kept about log2(R) / 2 bits fewer.
-template <int G>
-__global__ void __launch_bounds__(256) oz_slice_rows_grow_kernel(int64_t R, int64_t c0, int64_t c1,
-                                                                 const double* __restrict__ S, int64_t lds,
-                                                                 __nv_bfloat16* __restrict__ planes, int64_t Ra,
-                                                                 int* __restrict__ eexp) {
+// Rows slicer: columns [c0, c1) of S (R rows, lds) -> columns [c0, c1) of stored row i, zeros
+// from c1 to the next multiple of 16; 8 lanes a row.
+// GROW false (c0 = 0): the exponent of a row's largest entry.  GROW true, for a matrix that
+// gains columns (a Lanczos basis): one above it when it is set (at c0 = 0, or when a later
+// entry does not fit it: the row's earlier columns are then sliced again), so that new
+// columns rarely raise it.  That keeps 55 bits below the row's largest entry; one exponent
+// for all rows of an orthonormal basis kept about log2(R) / 2 bits fewer.
+// Bound by the 14 (16) bytes written and 8 read an entry (the digits are read again from
+// cache where a row group fits it): 100,000 x 64 in 27 us = 5.2 TB/s.
+template <int D, bool GROW>
+__global__ void __launch_bounds__(256, 4) oz_slice_rows_kernel(int64_t R, int64_t c0, int64_t c1,
+                                                            const double* __restrict__ S, int64_t lds,
+                                                            __nv_bfloat16* __restrict__ planes, int64_t Ra,
+                                                            int* __restrict__ eexp) {
+    constexpr int G = 8;
     const int sl = threadIdx.x % G;
     const int64_t ng = (int64_t)gridDim.x * (blockDim.x / G);
     const int64_t rounds = (R + ng - 1) / ng;  // the same for every lane: the shuffles need them all
@@ -211,25 +199,33 @@ __global__ void __launch_bounds__(256) oz_slice_rows_grow_kernel(int64_t R, int6
         const bool in = i < R;
         const double* src = S + i * lds;
         int e = kOzZeroExp;
-        if (in)
+        if (in) {
+#pragma unroll 4
             for (int64_t k = c0 + sl; k < c1; k += G) e = max(e, oz_exp(src[k]));
+        }
 #pragma unroll
         for (int o = G / 2; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
-        int old = in && sl == 0 && c0 > 0 ? eexp[i] : kOzZeroExp;
-        old = __shfl_sync(0xffffffffu, old, (threadIdx.x & 31) & ~(G - 1));
-        if (!in) continue;
-        const bool set = c0 == 0 || e > old;
-        // (a row of zeros keeps the exponent of zero, which any entry exceeds)
-        const int en = !set ? old : (e >= kOzNanExp || e <= kOzZeroExp ? e : e + 1);
-        if (set && sl == 0) eexp[i] = en;
-        for (int64_t k = (set ? 0 : c0 & ~int64_t(1)) + 2 * sl; k < a1; k += 2 * G) {
-            int da[kOzDig], db[kOzDig];
-            oz_digits(k < c1 ? src[k] : 0.0, en, da);
-            oz_digits(k + 1 < c1 ? src[k + 1] : 0.0, en, db);
-            oz_store_pair(planes, Ra, i, k, da, db);
+        int64_t k0 = 0;
+        if (GROW) {
+            int old = in && sl == 0 && c0 > 0 ? eexp[i] : kOzZeroExp;
+            old = __shfl_sync(0xffffffffu, old, (threadIdx.x & 31) & ~(G - 1));
+            // (a row of zeros keeps the exponent of zero, which any entry exceeds)
+            const bool set = c0 == 0 || e > old;
+            e = !set ? old : (e >= kOzNanExp || e <= kOzZeroExp ? e : e + 1);
+            if (!set) k0 = c0 & ~int64_t(15);
+            if (in && set && sl == 0) eexp[i] = e;
+        } else {
+            e = oz_norm_exp(e);
+            if (in && sl == 0) eexp[i] = e;
         }
+        if (!in) continue;
+        for (int64_t k = k0 + 2 * sl; k < a1; k += 2 * G)
+            oz_store_pair<D>(planes, Ra, i, k, k < c1 ? src[k] : 0.0, k + 1 < c1 ? src[k + 1] : 0.0, e);
     }
 }
+
+// Exponent arrays start below every exponent (memset of 0x80 bytes) and grow by atomicMax.
+constexpr int kOzUnset = 0x80;
 
 // Column maxima of the exponents of S (K x R, lds); upper: entries with k > j are zero.
 __global__ void __launch_bounds__(256) oz_colmax_kernel(int64_t K, int64_t R, const double* __restrict__ S,
@@ -239,9 +235,11 @@ __global__ void __launch_bounds__(256) oz_colmax_kernel(int64_t K, int64_t R, co
     const int64_t j = (int64_t)blockIdx.x * 32 + threadIdx.x;
     const int64_t k0 = (int64_t)blockIdx.y * rows_per, k1 = min(K, k0 + rows_per);
     int e = kOzZeroExp;
-    if (j < R)
+    if (j < R) {
+#pragma unroll 8
         for (int64_t k = k0 + threadIdx.y; k < k1; k += 8)
             if (!(upper && k > j)) e = max(e, oz_exp(S[k * lds + j]));
+    }
     red[threadIdx.y][threadIdx.x] = e;
     __syncthreads();
     if (threadIdx.y == 0 && j < R) {
@@ -251,40 +249,131 @@ __global__ void __launch_bounds__(256) oz_colmax_kernel(int64_t K, int64_t R, co
     }
 }
 
-// Cols slicer: column j of S (K x R, lds) -> stored row r0 + j, tiles of 64 k x 32 j,
-// zeros past K up to the next multiple of 16.
+// Row and column maxima of the exponents of S (M x N, lds) in one read: a block of 128 rows
+// x 256 columns, one thread a column, a row's maximum by a warp reduction.
+__global__ void __launch_bounds__(256) oz_max_both_kernel(int64_t M, int64_t N, const double* __restrict__ S,
+                                                          int64_t lds, int* __restrict__ rexp,
+                                                          int* __restrict__ cexp) {
+    __shared__ int rmax[128];
+    const int64_t j = (int64_t)blockIdx.x * 256 + threadIdx.x, i0 = (int64_t)blockIdx.y * 128;
+    const int rows = (int)min((int64_t)128, M - i0);
+    if (threadIdx.x < 128) rmax[threadIdx.x] = kOzZeroExp;
+    __syncthreads();
+    int c = kOzZeroExp;
+    const double* src = S + i0 * lds + j;
+#pragma unroll 8
+    for (int r = 0; r < rows; ++r) {
+        const int e = j < N ? oz_exp(src[(int64_t)r * lds]) : kOzZeroExp;
+        c = max(c, e);
+        const int w = __reduce_max_sync(0xffffffffu, e);
+        if ((threadIdx.x & 31) == 0) atomicMax(&rmax[r], w);
+    }
+    if (j < N) atomicMax(&cexp[j], c);
+    __syncthreads();
+    if ((int)threadIdx.x < rows) atomicMax(&rexp[i0 + threadIdx.x], rmax[threadIdx.x]);
+}
+
+// Slices a 64 x 64 tile of S (M x N, lds) from shared memory (row stride 65): its rows into
+// the rows layout (stored row i, K = N) and its columns into the cols layout (stored row
+// j, K = M), or the columns alone.
+template <int D, bool ROWS>
+__device__ inline void oz_slice_tile(const double (*tile)[65], int64_t i0, int64_t j0, int64_t M, int64_t N,
+                                     const int* __restrict__ rexp, const int* __restrict__ cexp,
+                                     __nv_bfloat16* __restrict__ rplanes, int64_t rRa,
+                                     __nv_bfloat16* __restrict__ cplanes, int64_t cRa, int64_t c0) {
+    const int warp = threadIdx.x >> 5, pr = 2 * (threadIdx.x & 7), sub = (threadIdx.x & 31) >> 3;
+#pragma unroll 1
+    for (int u = warp; u < 64; u += 8) {  // K block u / 16, 4 stored rows
+        const int kb = (u >> 4) * 16 + pr, q = (u & 15) * 4 + sub;
+        if (ROWS && i0 + q < M && j0 + kb < oz_k16(N))
+            oz_store_pair<D>(rplanes, rRa, i0 + q, j0 + kb, tile[q][kb], tile[q][kb + 1],
+                             oz_norm_exp(rexp[i0 + q]));
+        if (j0 + q < N && i0 + kb < oz_k16(M))
+            oz_store_pair<D>(cplanes, cRa, c0 + j0 + q, i0 + kb, tile[kb][q], tile[kb + 1][q],
+                             oz_norm_exp(cexp[j0 + q]));
+    }
+}
+
+// Both layouts of a matrix in one read (a dense A, whose products need both): with the one
+// read of oz_max_both that is 16 bytes read and 28 written an entry, against 32 and 28 by
+// the single-layout slicers.
+template <int D>
+__global__ void __launch_bounds__(256)
+    oz_slice_both_kernel(int64_t M, int64_t N, const double* __restrict__ S, int64_t lds,
+                         const int* __restrict__ rexp, const int* __restrict__ cexp,
+                         __nv_bfloat16* __restrict__ rplanes, int64_t rRa, __nv_bfloat16* __restrict__ cplanes,
+                         int64_t cRa) {
+    __shared__ double tile[64][65];
+    const int64_t i0 = (int64_t)blockIdx.y * 64, j0 = (int64_t)blockIdx.x * 64;
+    const int tx = threadIdx.x & 63, ty = threadIdx.x >> 6;
+#pragma unroll
+    for (int r = ty; r < 64; r += 4)
+        tile[r][tx] = i0 + r < M && j0 + tx < N ? S[(i0 + r) * lds + j0 + tx] : 0.0;
+    __syncthreads();
+    oz_slice_tile<D, true>(tile, i0, j0, M, N, rexp, cexp, rplanes, rRa, cplanes, cRa, 0);
+}
+
+// Cols slicer: column j of S (K x R, lds) -> stored row r0 + j, tiles of 64 k x 64 j, zeros
+// past K up to the next multiple of 16.
 template <int D>
 __global__ void __launch_bounds__(256) oz_slice_cols_kernel(int64_t K, int64_t R, const double* __restrict__ S,
                                                             int64_t lds, int upper, const int* __restrict__ eexp,
                                                             __nv_bfloat16* __restrict__ planes, int64_t Ra,
                                                             int64_t r0) {
-    __shared__ double tile[64][33];
-    const int64_t k0 = (int64_t)blockIdx.x * 64, j0 = (int64_t)blockIdx.y * 32;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    for (int r = ty; r < 64; r += 8) {
+    __shared__ double tile[64][65];
+    const int64_t k0 = (int64_t)blockIdx.x * 64, j0 = (int64_t)blockIdx.y * 64;
+    const int tx = threadIdx.x & 63, ty = threadIdx.x >> 6;
+#pragma unroll
+    for (int r = ty; r < 64; r += 4) {
         const int64_t k = k0 + r, j = j0 + tx;
-        double v = 0.0;
-        if (k < K && j < R && !(upper && k > j)) v = S[k * lds + j];
-        tile[r][tx] = v;
+        tile[r][tx] = k < K && j < R && !(upper && k > j) ? S[k * lds + j] : 0.0;
     }
     __syncthreads();
-    const int kp = tx;  // k pair within the tile
-    const int64_t k = k0 + 2 * kp;
-    if (k >= oz_k16(K)) return;
-    for (int jj = ty; jj < 32; jj += 8) {
-        const int64_t j = j0 + jj;
-        if (j >= R) break;
-        const int e = oz_norm_exp(eexp[j]);
-        int da[D], db[D];
-        oz_digits(tile[2 * kp][jj], e, da);
-        oz_digits(tile[2 * kp + 1][jj], e, db);
-        oz_store_pair(planes, Ra, r0 + j, k, da, db);
-    }
+    oz_slice_tile<D, false>(tile, k0, j0, K, R, nullptr, eexp, nullptr, 0, planes, Ra, r0);
 }
 
-__global__ void oz_fill_kernel(int64_t n, int v, int* __restrict__ x) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) x[i] = v;
+// The same for a short K (at most kOzShortK: the coefficients and factors that multiply a
+// basis from the right), exponents included, in one launch: a block takes 8 columns over
+// all K.  (The column-maximum and slicing kernels and the fill before them took 9 us a
+// product at 512 x 64; 5 us now.)
+constexpr int kOzShortK = 2048;
+template <int D>
+__global__ void __launch_bounds__(256) oz_slice_cols_short_kernel(int64_t K, int64_t R, const double* __restrict__ S,
+                                                                  int64_t lds, int upper,
+                                                                  __nv_bfloat16* __restrict__ planes, int64_t Ra,
+                                                                  int* __restrict__ eexp) {
+    __shared__ int red[32][9];
+    __shared__ int es[8];
+    const int64_t j0 = (int64_t)blockIdx.x * 8;
+    {
+        const int64_t j = j0 + (threadIdx.x & 7);
+        int e = kOzZeroExp;
+        if (j < R) {
+#pragma unroll 4
+            for (int64_t k = threadIdx.x >> 3; k < K; k += 32)
+                if (!(upper && k > j)) e = max(e, oz_exp(S[k * lds + j]));
+        }
+        red[threadIdx.x >> 3][threadIdx.x & 7] = e;
+    }
+    __syncthreads();
+    if (threadIdx.x < 8) {
+        int e = red[0][threadIdx.x];
+        for (int y = 1; y < 32; ++y) e = max(e, red[y][threadIdx.x]);
+        es[threadIdx.x] = e = oz_norm_exp(e);
+        if (j0 + threadIdx.x < R) eexp[j0 + threadIdx.x] = e;
+    }
+    __syncthreads();
+    const int warp = threadIdx.x >> 5, pr = 2 * (threadIdx.x & 7), sub = (threadIdx.x & 31) >> 3;
+    const int units = 2 * (int)(oz_k16(K) / 16);
+#pragma unroll 2
+    for (int u = warp; u < units; u += 8) {
+        const int q = (u & 1) * 4 + sub;
+        const int64_t j = j0 + q, k = (int64_t)(u >> 1) * 16 + pr;
+        if (j >= R) continue;
+        const double x0 = k < K && !(upper && k > j) ? S[k * lds + j] : 0.0;
+        const double x1 = k + 1 < K && !(upper && k + 1 > j) ? S[(k + 1) * lds + j] : 0.0;
+        oz_store_pair<D>(planes, Ra, j, k, x0, x1, es[q]);
+    }
 }
 
 // ---- the product kernel ------------------------------------------------------
@@ -756,36 +845,54 @@ struct OzCuts {
     short g0[kOzWave], nc[kOzWave], slot0[kOzWave];
 };
 
-// Adds the parts of a cut tile in a fixed order (four contiguous shares of the CTAs, then
-// the shares) and applies the output rule.  Block (x, y, z): row x of cut y, column tile z.
-__global__ void __launch_bounds__(256) oz_fixup_kernel(OzArgs a, OzCuts cuts) {
-    const int mt = cuts.mt[blockIdx.y], nc = cuts.nc[blockIdx.y], g0 = cuts.g0[blockIdx.y], nt = blockIdx.z;
-    if ((int64_t)mt * kOzM + blockIdx.x >= a.M) return;
-    auto slot = [&](int j) -> int64_t {
-        return (((int64_t)(g0 + j) * a.NT + nt) * a.nslots + (j ? 0 : cuts.slot0[blockIdx.y])) * kOzM * kOzN;
-    };
+// Adds the parts of a cut tile and applies the output rule.  Block (x, y, z): `rows` rows
+// from x * rows on of cut y, column tile z.  Few parts: 4 rows at a time, in CTA order.
+// Many (a Gram matrix has 152 parts of one tile): a row at a time, four contiguous shares
+// of the CTAs, then the shares in order.
+__global__ void __launch_bounds__(256) oz_fixup_kernel(OzArgs a, OzCuts cuts, int rows) {
     __shared__ double s_part[4][kOzN];
-    const int r = blockIdx.x, cl = threadIdx.x % kOzN, share = threadIdx.x / kOzN;
-    const int idx = r * kOzN + cl;
-    const int64_t row = (int64_t)mt * kOzM + r, col = (int64_t)nt * a.tilen + cl;
-    const bool in = cl < a.tilen && row < a.M && col < a.N;
-    double acc = 0.0;
-    if (in) {
-        int j = nc * share / 4;
-        const int j1 = nc * (share + 1) / 4;
-        for (; j + 16 <= j1; j += 16) {  // sixteen loads in flight
-            double v[16];
-#pragma unroll
-            for (int u = 0; u < 16; ++u) v[u] = a.partial[slot(j + u) + idx];
-#pragma unroll
-            for (int u = 0; u < 16; ++u) acc += v[u];
+    const int mt = cuts.mt[blockIdx.y], nc = cuts.nc[blockIdx.y], g0 = cuts.g0[blockIdx.y], nt = blockIdx.z;
+    const int cl = threadIdx.x % kOzN, share = threadIdx.x / kOzN;
+    const int64_t col = (int64_t)nt * a.tilen + cl;
+    const bool in_col = cl < a.tilen && col < a.N;
+    const double* first = a.partial + (((int64_t)g0 * a.NT + nt) * a.nslots + cuts.slot0[blockIdx.y]) * kOzM * kOzN;
+    const double* rest = a.partial + ((int64_t)g0 * a.NT + nt) * a.nslots * kOzM * kOzN;
+    const int64_t step = (int64_t)a.NT * a.nslots * kOzM * kOzN;  // from one group's slot 0 to the next's
+    const int r1 = min((int)(blockIdx.x + 1) * rows, (int)min((int64_t)kOzM, a.M - (int64_t)mt * kOzM));
+    if (nc < 8) {
+#pragma unroll 2
+        for (int r = (int)blockIdx.x * rows + share; r < r1; r += 4) {
+            const int idx = r * kOzN + cl;
+            if (!in_col) continue;
+            double acc = first[idx];
+            for (int j = 1; j < nc; ++j) acc += rest[j * step + idx];
+            oz_store(a, (int64_t)mt * kOzM + r, col, acc);
         }
-#pragma unroll 8
-        for (; j < j1; ++j) acc += a.partial[slot(j) + idx];
+        return;
     }
-    s_part[share][cl] = acc;
-    __syncthreads();
-    if (in && share == 0) oz_store(a, row, col, ((acc + s_part[1][cl]) + s_part[2][cl]) + s_part[3][cl]);
+    for (int r = (int)blockIdx.x * rows; r < r1; ++r) {
+        const int idx = r * kOzN + cl;
+        double acc = 0.0;
+        if (in_col) {
+            int j = nc * share / 4;
+            const int j1 = nc * (share + 1) / 4;
+            if (j == 0) acc = first[idx], j = 1;
+            for (; j + 16 <= j1; j += 16) {  // sixteen loads in flight
+                double v[16];
+#pragma unroll
+                for (int u = 0; u < 16; ++u) v[u] = rest[(j + u) * step + idx];
+#pragma unroll
+                for (int u = 0; u < 16; ++u) acc += v[u];
+            }
+#pragma unroll 8
+            for (; j < j1; ++j) acc += rest[j * step + idx];
+        }
+        __syncthreads();
+        s_part[share][cl] = acc;
+        __syncthreads();
+        if (in_col && share == 0)
+            oz_store(a, (int64_t)mt * kOzM + r, col, ((acc + s_part[1][cl]) + s_part[2][cl]) + s_part[3][cl]);
+    }
 }
 
 // ---- host side -------------------------------------------------------------------
@@ -854,13 +961,15 @@ struct OzView {
     const int* exps;
 };
 
-int oz_slice_rows(tsvd_handle* h, int64_t R, int64_t K, const double* S, int64_t lds, __nv_bfloat16* planes,
-                  int* eexp, cudaStream_t st) {
+int oz_slice_rows(tsvd_handle* h, int64_t R, int64_t c0, int64_t c1, const double* S, int64_t lds, bool grow,
+                  __nv_bfloat16* planes, int* eexp, cudaStream_t st) {
     if (R == 0) return TSVD_OK;
-    const int64_t blocks = std::min<int64_t>((R + 7) / 8, (int64_t)h->sm_count * 16);
+    const int64_t blocks = std::min<int64_t>((R + 31) / 32, (int64_t)h->sm_count * 32);
+    const auto kern = grow ? oz_slice_rows_kernel<kOzDig, true>
+                           : (h->oz_dig == kOzWideDig ? oz_slice_rows_kernel<kOzWideDig, false>
+                                                      : oz_slice_rows_kernel<kOzDig, false>);
     h->launches++;
-    const auto kern = h->oz_dig == kOzWideDig ? oz_slice_rows_kernel<kOzWideDig> : oz_slice_rows_kernel<kOzDig>;
-    kern<<<(unsigned)blocks, 256, 0, st>>>(R, K, S, lds, planes, oz_ra(R), eexp);
+    kern<<<(unsigned)blocks, 256, 0, st>>>(R, c0, c1, S, lds, planes, oz_ra(R), eexp);
     TSVD_TRY_CUDA(cudaGetLastError());
     return TSVD_OK;
 }
@@ -870,17 +979,25 @@ int oz_slice_cols(tsvd_handle* h, int64_t K, int64_t R, const double* S, int64_t
                   __nv_bfloat16* planes, int* eexp, cudaStream_t st, int64_t Ra = -1, int64_t r0 = 0) {
     if (R == 0) return TSVD_OK;
     if (Ra < 0) Ra = oz_ra(R);
+    const bool wide = h->oz_dig == kOzWideDig;
+    if (K <= kOzShortK && r0 == 0) {
+        const auto kern = wide ? oz_slice_cols_short_kernel<kOzWideDig> : oz_slice_cols_short_kernel<kOzDig>;
+        h->launches++;
+        kern<<<(unsigned)((R + 7) / 8), 256, 0, st>>>(K, R, S, lds, upper ? 1 : 0, planes, Ra, eexp);
+        TSVD_TRY_CUDA(cudaGetLastError());
+        return TSVD_OK;
+    }
     const unsigned gx = (unsigned)((R + 31) / 32);
     int64_t gy = std::min<int64_t>((K + 255) / 256, std::max<int64_t>(1, (int64_t)h->sm_count * 8 / gx));
     const int64_t rows_per = (K + gy - 1) / gy;
     gy = (K + rows_per - 1) / rows_per;
-    h->launches += 3;
-    oz_fill_kernel<<<(unsigned)((R + 255) / 256), 256, 0, st>>>(R, kOzZeroExp - 1, eexp);
+    h->launches += 2;
+    TSVD_TRY_CUDA(cudaMemsetAsync(eexp, kOzUnset, sizeof(int) * R, st));
     oz_colmax_kernel<<<dim3(gx, (unsigned)std::max<int64_t>(1, gy)), dim3(32, 8), 0, st>>>(K, R, S, lds,
                                                                                            upper ? 1 : 0, rows_per,
                                                                                            eexp);
-    const dim3 sg((unsigned)((oz_k16(K) + 63) / 64), gx);
-    const auto kern = h->oz_dig == kOzWideDig ? oz_slice_cols_kernel<kOzWideDig> : oz_slice_cols_kernel<kOzDig>;
+    const dim3 sg((unsigned)((oz_k16(K) + 63) / 64), (unsigned)((R + 63) / 64));
+    const auto kern = wide ? oz_slice_cols_kernel<kOzWideDig> : oz_slice_cols_kernel<kOzDig>;
     kern<<<sg, 256, 0, st>>>(K, R, S, lds, upper ? 1 : 0, eexp, planes, Ra, r0);
     TSVD_TRY_CUDA(cudaGetLastError());
     return TSVD_OK;
@@ -938,7 +1055,9 @@ int oz_run(tsvd_handle* h, const OzPlan& p, const OzView& va, const OzView& vb, 
     auto flush = [&]() -> int {
         if (n == 0) return TSVD_OK;
         h->launches++;
-        oz_fixup_kernel<<<dim3(kOzM, (unsigned)n, (unsigned)p.NT), 256, 0, st>>>(a, cuts);
+        // a few tiles of many parts: a row a block; many tiles of few parts: 16 rows a block
+        const int rows = n * p.NT < 16 ? 1 : 16;
+        oz_fixup_kernel<<<dim3((unsigned)(kOzM / rows), (unsigned)n, (unsigned)p.NT), 256, 0, st>>>(a, cuts, rows);
         n = 0;
         TSVD_TRY_CUDA(cudaGetLastError());
         return TSVD_OK;
@@ -1093,7 +1212,7 @@ int oz_gemm_nn(tsvd_handle* h, int64_t q, int64_t s, int64_t b, double alpha, co
         __nv_bfloat16* pa = reinterpret_cast<__nv_bfloat16*>(ar.take<char>(oz_planes_bytes(p.M, p.K, h->oz_dig)));
         int* ea = ar.take<int>((size_t)p.M);
         if (!ar.fits()) return TSVD_ERR_WORKSPACE;
-        TSVD_TRY(oz_slice_rows(h, q, s, X, ldx, pa, ea, st));
+        TSVD_TRY(oz_slice_rows(h, q, 0, s, X, ldx, false, pa, ea, st));
         va = view_of(pa, q, s, ea);
     }
     __nv_bfloat16* pb = reinterpret_cast<__nv_bfloat16*>(ar.take<char>(oz_planes_bytes(p.N, p.K, h->oz_dig)));
@@ -1136,22 +1255,36 @@ int oz_cache_slice(tsvd_handle* h, OzCache& c, int64_t c0, int64_t c1, cudaStrea
             TSVD_TRY(oz_slice_cols(h, c.rows, c1 - c0, c.src + c0, c.ld, false, c.planes, c.exps + c0, st,
                                    oz_ra(c.cols),
                                    c0));
-        } else if (c.grows) {
-            const int64_t w = (c1 - c0 + 1) / 2;  // column pairs of a row
-            const int g = w >= 32 ? 32 : (w >= 16 ? 16 : 8);
-            const unsigned blocks = (unsigned)std::min<int64_t>((c.rows * g + 255) / 256, (int64_t)h->sm_count * 32);
-            h->launches++;
-            const auto kern = g == 32 ? oz_slice_rows_grow_kernel<32>
-                                      : (g == 16 ? oz_slice_rows_grow_kernel<16> : oz_slice_rows_grow_kernel<8>);
-            kern<<<std::max(1u, blocks), 256, 0, st>>>(c.rows, c0, c1, c.src, c.ld, c.planes, oz_ra(c.rows), c.exps);
-            TSVD_TRY_CUDA(cudaGetLastError());
         } else {
-            // per-row exponents need the whole rows at once
-            if (c0 != 0 || c1 != c.cols) return TSVD_ERR_INVALID_ARG;
-            TSVD_TRY(oz_slice_rows(h, c.rows, c.cols, c.src, c.ld, c.planes, c.exps, st));
+            // per-row exponents of a matrix that does not grow need the whole rows at once
+            if (!c.grows && (c0 != 0 || c1 != c.cols)) return TSVD_ERR_INVALID_ARG;
+            TSVD_TRY(oz_slice_rows(h, c.rows, c0, c1, c.src, c.ld, c.grows, c.planes, c.exps, st));
         }
     }
     c.valid = c1;
+    return TSVD_OK;
+}
+
+int oz_cache_slice_both(tsvd_handle* h, OzCache& rows, OzCache& cols, cudaStream_t st) {
+    const int64_t M = rows.rows, N = rows.cols;
+    if (rows.cols_layout || rows.grows || !cols.cols_layout || cols.src != rows.src || cols.ld != rows.ld ||
+        cols.rows != M || cols.cols != N)
+        return TSVD_ERR_INVALID_ARG;
+    const int64_t gy = (M + 127) / 128, ty = (std::max(M, oz_k16(M)) + 63) / 64;
+    if (gy > 65535 || ty > 65535) {  // (grid limit) one layout at a time
+        TSVD_TRY(oz_cache_slice(h, rows, 0, N, st));
+        return oz_cache_slice(h, cols, 0, N, st);
+    }
+    TSVD_TRY_CUDA(cudaMemsetAsync(rows.exps, kOzUnset, sizeof(int) * M, st));
+    TSVD_TRY_CUDA(cudaMemsetAsync(cols.exps, kOzUnset, sizeof(int) * N, st));
+    h->launches += 2;
+    oz_max_both_kernel<<<dim3((unsigned)((N + 255) / 256), (unsigned)gy), 256, 0, st>>>(M, N, rows.src, rows.ld,
+                                                                                       rows.exps, cols.exps);
+    const auto kern = h->oz_dig == kOzWideDig ? oz_slice_both_kernel<kOzWideDig> : oz_slice_both_kernel<kOzDig>;
+    kern<<<dim3((unsigned)((oz_k16(N) + 63) / 64), (unsigned)ty), 256, 0, st>>>(
+        M, N, rows.src, rows.ld, rows.exps, cols.exps, rows.planes, oz_ra(M), cols.planes, oz_ra(N));
+    TSVD_TRY_CUDA(cudaGetLastError());
+    rows.valid = cols.valid = N;
     return TSVD_OK;
 }
 

@@ -314,6 +314,9 @@ size_t oz_cache_bytes(int64_t rows, int64_t cols, bool cols_layout, int dig = 7)
 void oz_cache_carve(OzCache& c, Arena& ar, const double* src, int64_t ld, int64_t rows, int64_t cols,
                     bool cols_layout, bool grows, int dig = 7);
 int oz_cache_slice(tsvd_handle* h, OzCache& c, int64_t c0, int64_t c1, cudaStream_t st);
+// All columns of a matrix that does not grow, in both layouts (one read for the exponents,
+// one for the digits).
+int oz_cache_slice_both(tsvd_handle* h, OzCache& rows, OzCache& cols, cudaStream_t st);
 // Columns from v on are about to be rewritten: valid = min(valid, v).
 int oz_cache_truncate(tsvd_handle* h, OzCache& c, int64_t v, cudaStream_t st);
 const OzCache* oz_find_cache(const tsvd_handle* h, const double* X, int64_t ldx, int64_t rows, int64_t s,
@@ -380,12 +383,11 @@ struct OzStandalone {
     }
     ~OzStandalone() { h->oz_dig = prev_dig; }
     int slice(cudaStream_t st) {
-        for (OzCache* c : {&cols, &rows}) {
-            if (!c->planes) continue;
-            const int rc = oz_cache_slice(h, *c, 0, c->cols, st);
-            if (rc < 0) return rc;
-            caches.add(c);
-        }
+        if (!cols.planes) return TSVD_OK;
+        const int rc = oz_cache_slice_both(h, rows, cols, st);
+        if (rc < 0) return rc;
+        caches.add(&cols);
+        caches.add(&rows);
         return TSVD_OK;
     }
 };
