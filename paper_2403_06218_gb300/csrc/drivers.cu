@@ -303,13 +303,10 @@ int setup_op(tsvd_handle* h, const tsvd_matrix* A, int wmax, Arena& ar, Op<T>& o
             op.tcws = ar.take<char>(std::max(tc_mm_ws(M, N, wmax), tc_mm_ws(N, M, wmax)));
             if (run) {
                 if (!ar.fits()) return TSVD_ERR_WORKSPACE;
-                if (in64) {
-                    TSVD_TRY_CUDA(bf16x3_split<double>(h, M, N, (const double*)a, lda, false, pa, st));
-                    TSVD_TRY_CUDA(bf16x3_split<double>(h, M, N, (const double*)a, lda, true, pat, st));
-                } else {
-                    TSVD_TRY_CUDA(bf16x3_split<float>(h, M, N, (const float*)a, lda, false, pa, st));
-                    TSVD_TRY_CUDA(bf16x3_split<float>(h, M, N, (const float*)a, lda, true, pat, st));
-                }
+                if (in64)
+                    TSVD_TRY_CUDA(bf16x3_split<double>(h, M, N, (const double*)a, lda, pa, pat, st));
+                else
+                    TSVD_TRY_CUDA(bf16x3_split<float>(h, M, N, (const float*)a, lda, pa, pat, st));
             }
             op.pA = pa;
             op.pAt = pat;

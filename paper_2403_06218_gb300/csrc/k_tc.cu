@@ -295,60 +295,77 @@ __global__ void tc_fixup_kernel(int64_t M, int w, int Npad, int64_t KB, int64_t 
     Y[row * ldy + col] = acc;
 }
 
-// Three-way BF16 split: p0 = bf16(v), p1 = bf16(v - p0), p2 = bf16(v - p0 - p1);
-// each difference is exact in the source precision.
-template <typename T>
-__device__ inline void split3(T v, __nv_bfloat16& p0, __nv_bfloat16& p1, __nv_bfloat16& p2) {
-    if constexpr (std::is_same<T, double>::value) {
-        p0 = __double2bfloat16(v);
-        const double r1 = v - (double)__bfloat162float(p0);
-        p1 = __double2bfloat16(r1);
-        const double r2 = r1 - (double)__bfloat162float(p1);
-        p2 = __double2bfloat16(r2);
+// Three-way BF16 split: p0 = bf16(v), p1 = bf16(v - p0), p2 = bf16(v - p0 - p1), to 2^-27 of
+// v.  An FP64 value enters as v = f + t, f its leading 24 bits and t the other 29 to FP32
+// accuracy, taken from the bits: the FP64 pipe (2 instructions a clock and SM) needed 5 ms
+// for 20,000^2 entries in either layout.
+__device__ inline void split3(float f, float t, __nv_bfloat16& p0, __nv_bfloat16& p1, __nv_bfloat16& p2) {
+    p0 = __float2bfloat16_rn(f);
+    const float r1 = f - __bfloat162float(p0);  // exact
+    p1 = __float2bfloat16_rn(r1 + t);
+    const float r2 = r1 - __bfloat162float(p1);  // exact
+    p2 = __float2bfloat16_rn(r2 + t);
+}
+__device__ inline void split3(float v, __nv_bfloat16& p0, __nv_bfloat16& p1, __nv_bfloat16& p2) {
+    split3(v, 0.0f, p0, p1, p2);
+}
+__device__ inline void split3(double v, __nv_bfloat16& p0, __nv_bfloat16& p1, __nv_bfloat16& p2) {
+    const uint64_t u = (uint64_t)__double_as_longlong(v);
+    const int e = (int)((u >> 52) & 0x7FF) - 1023;  // exponent of a normal value
+    if (e >= -74 && e <= 126) {  // 2^(e - 52) is a normal FP32 value too
+        const unsigned sign = (unsigned)(u >> 32) & 0x80000000u;
+        const float f = __uint_as_float(sign | (unsigned)(e + 127) << 23 | ((unsigned)(u >> 29) & 0x7FFFFFu));
+        // t = low 29 bits 2^(e - 52), signed
+        const float t = (float)((unsigned)u & 0x1FFFFFFFu) * __uint_as_float(sign | (unsigned)(e + 75) << 23);
+        split3(f, t, p0, p1, p2);
+        return;
+    }
+    // zeros and values at the ends of the FP32 range
+    p0 = __double2bfloat16(v);
+    const double r1 = v - (double)__bfloat162float(p0);
+    p1 = __double2bfloat16(r1);
+    const double r2 = r1 - (double)__bfloat162float(p1);
+    p2 = __double2bfloat16(r2);
+}
+
+__device__ inline void store_pair(__nv_bfloat16* dst, __nv_bfloat16 a, __nv_bfloat16 b, int pairs, bool second) {
+    if (pairs) {
+        *reinterpret_cast<__nv_bfloat162*>(dst) = __halves2bfloat162(a, b);
     } else {
-        p0 = __float2bfloat16_rn(v);
-        const float r1 = v - __bfloat162float(p0);
-        p1 = __float2bfloat16_rn(r1);
-        const float r2 = r1 - __bfloat162float(p1);
-        p2 = __float2bfloat16_rn(r2);
+        dst[0] = a;
+        if (second) dst[1] = b;
     }
 }
 
-// Pieces of S (rows x cols, lds) or of its transpose: out[p][i][j] with the output
-// rows x cols = (trans ? cols x rows : rows x cols), leading dimension ldo.
+// Pieces of S (rows x cols, lds) and of its transpose, [3][rows][ld] and [3][cols][ldt] (a
+// null output is left out): one read and one split of every entry, tiles of 64 x 64 through
+// shared memory, pairs of a row stored together where the output is 4-byte aligned (`pairs`).
+// (A pair at an odd end writes one element of the row's padding, which nothing reads: the
+// tensor maps stop at the last column.)  One-dimensional grid, column tiles fastest.
 template <typename T>
-__global__ void split3_kernel(int64_t rows, int64_t cols, const T* __restrict__ S, int64_t lds, int trans,
-                              __nv_bfloat16* __restrict__ out, int64_t ldo, int64_t piece) {
-    __shared__ T tile[32][33];
-    const int64_t r0 = (int64_t)blockIdx.y * 32, c0 = (int64_t)blockIdx.x * 32;
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    if (!trans) {
-        for (int k = ty; k < 32; k += 8) {
-            const int64_t r = r0 + k, cc = c0 + tx;
-            if (r < rows && cc < cols) {
-                __nv_bfloat16 a, b, d;
-                split3(S[r * lds + cc], a, b, d);
-                out[r * ldo + cc] = a;
-                out[piece + r * ldo + cc] = b;
-                out[2 * piece + r * ldo + cc] = d;
-            }
-        }
-        return;
-    }
-    for (int k = ty; k < 32; k += 8) {
-        const int64_t r = r0 + k, cc = c0 + tx;
-        tile[k][tx] = (r < rows && cc < cols) ? S[r * lds + cc] : T(0);
+__global__ void __launch_bounds__(256) split3_kernel(int64_t rows, int64_t cols, const T* __restrict__ S, int64_t lds,
+                                                     __nv_bfloat16* __restrict__ out, int64_t ld,
+                                                     __nv_bfloat16* __restrict__ outt, int64_t ldt, unsigned ct,
+                                                     int pairs) {
+    __shared__ __nv_bfloat16 tile[3][64][66];
+    const int64_t r0 = (int64_t)(blockIdx.x / ct) * 64, c0 = (int64_t)(blockIdx.x % ct) * 64;
+    const int tx = threadIdx.x & 63, ty = threadIdx.x >> 6;
+#pragma unroll 4
+    for (int r = ty; r < 64; r += 4) {
+        const T v = r0 + r < rows && c0 + tx < cols ? S[(r0 + r) * lds + c0 + tx] : T(0);
+        split3(v, tile[0][r][tx], tile[1][r][tx], tile[2][r][tx]);
     }
     __syncthreads();
-    for (int k = ty; k < 32; k += 8) {
-        const int64_t orow = c0 + k, ocol = r0 + tx;  // output (transposed) coordinates
-        if (orow < cols && ocol < rows) {
-            __nv_bfloat16 a, b, d;
-            split3(tile[tx][k], a, b, d);
-            out[orow * ldo + ocol] = a;
-            out[piece + orow * ldo + ocol] = b;
-            out[2 * piece + orow * ldo + ocol] = d;
-        }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll 1
+    for (int u = warp; u < 3 * 64; u += 8) {
+        const int p = u >> 6, q = u & 63;
+        if (out && r0 + q < rows && c0 + 2 * lane < cols)
+            store_pair(out + (p * rows + r0 + q) * ld + c0 + 2 * lane, tile[p][q][2 * lane], tile[p][q][2 * lane + 1],
+                       pairs, c0 + 2 * lane + 1 < cols);
+        if (outt && c0 + q < cols && r0 + 2 * lane < rows)
+            store_pair(outt + (p * cols + c0 + q) * ldt + r0 + 2 * lane, tile[p][2 * lane][q],
+                       tile[p][2 * lane + 1][q], pairs, r0 + 2 * lane + 1 < rows);
     }
 }
 
@@ -382,22 +399,20 @@ int64_t bf16x3_ld(int64_t cols) { return (cols + 7) / 8 * 8; }
 size_t bf16x3_bytes(int64_t rows, int64_t cols) { return align256((size_t)3 * rows * bf16x3_ld(cols) * 2); }
 
 template <typename T>
-cudaError_t bf16x3_split(tsvd_handle* h, int64_t rows, int64_t cols, const T* S, int64_t lds, bool trans, void* out,
+cudaError_t bf16x3_split(tsvd_handle* h, int64_t rows, int64_t cols, const T* S, int64_t lds, void* out, void* outt,
                          cudaStream_t st) {
-    const int64_t orow = trans ? cols : rows, ocol = trans ? rows : cols;
-    if (orow == 0 || ocol == 0) return cudaSuccess;
-    const int64_t ldo = bf16x3_ld(ocol);
-    const int64_t piece = orow * ldo;
-    // the K padding of a row (ldo > ocol) is never read: the tensor maps stop at ocol
+    if (rows == 0 || cols == 0) return cudaSuccess;
     h->launches++;
-    const dim3 grid((unsigned)((cols + 31) / 32), (unsigned)((rows + 31) / 32));
-    split3_kernel<T><<<grid, dim3(32, 8), 0, st>>>(rows, cols, S, lds, trans ? 1 : 0,
-                                                   static_cast<__nv_bfloat16*>(out), ldo, piece);
+    const int64_t ct = (cols + 63) / 64;
+    const int pairs = ((reinterpret_cast<uintptr_t>(out) | reinterpret_cast<uintptr_t>(outt)) & 3) == 0;
+    split3_kernel<T><<<(unsigned)(ct * ((rows + 63) / 64)), 256, 0, st>>>(
+        rows, cols, S, lds, static_cast<__nv_bfloat16*>(out), bf16x3_ld(cols), static_cast<__nv_bfloat16*>(outt),
+        bf16x3_ld(rows), (unsigned)ct, pairs);
     return cudaGetLastError();
 }
-template cudaError_t bf16x3_split<double>(tsvd_handle*, int64_t, int64_t, const double*, int64_t, bool, void*,
+template cudaError_t bf16x3_split<double>(tsvd_handle*, int64_t, int64_t, const double*, int64_t, void*, void*,
                                           cudaStream_t);
-template cudaError_t bf16x3_split<float>(tsvd_handle*, int64_t, int64_t, const float*, int64_t, bool, void*,
+template cudaError_t bf16x3_split<float>(tsvd_handle*, int64_t, int64_t, const float*, int64_t, void*, void*,
                                          cudaStream_t);
 
 size_t tc_mm_ws(int64_t rows, int64_t cols, int w) {
@@ -431,7 +446,7 @@ cudaError_t tc_mm(tsvd_handle* h, int64_t rows, int64_t cols, const void* pieces
         uint8_t* xp = static_cast<uint8_t*>(ws);
         float* part = reinterpret_cast<float*>(xp + bf16x3_bytes(np, cols));
         // X^T pieces: wp x cols (K-major), rows wp..np-1 come from the map's zero fill
-        cudaError_t e = bf16x3_split<float>(h, cols, wp, X + c0, ldx, true, xp, st);
+        cudaError_t e = bf16x3_split<float>(h, cols, wp, X + c0, ldx, nullptr, xp, st);
         if (e != cudaSuccess) return e;
         CUtensorMap mA, mX;
         if (!make_map(&mA, pieces, cols, rows, lda, kTcM)) return cudaErrorInvalidValue;

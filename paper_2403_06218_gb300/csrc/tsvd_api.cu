@@ -488,7 +488,7 @@ int tsvd_bf16x3_split(tsvd_handle* h, int trans, int64_t m, int64_t n, const dou
                       void* stream) {
     if (!h || m < 0 || n < 0 || lda < n || (m * n > 0 && (!A || !pieces))) return TSVD_ERR_INVALID_ARG;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    TSVD_TRY_CUDA(bf16x3_split<double>(h, m, n, A, lda, trans != 0, pieces, st));
+    TSVD_TRY_CUDA(bf16x3_split<double>(h, m, n, A, lda, trans ? nullptr : pieces, trans ? pieces : nullptr, st));
     TSVD_TRY_CUDA(cudaStreamSynchronize(st));
     return TSVD_OK;
 }

@@ -255,9 +255,9 @@ cudaError_t launch_gemm_tn_f32(dim3 grid, cudaStream_t st, int64_t q, int64_t s,
 // stored [3][rows][bf16x3_ld(cols)] as BF16.
 int64_t bf16x3_ld(int64_t cols);
 size_t bf16x3_bytes(int64_t rows, int64_t cols);
-// Pieces of S (rows x cols) or, with trans, of S^T.
+// Pieces of S (rows x cols) to `out` and of S^T to `outt`, in one pass; either may be null.
 template <typename T>
-cudaError_t bf16x3_split(tsvd_handle* h, int64_t rows, int64_t cols, const T* S, int64_t lds, bool trans, void* out,
+cudaError_t bf16x3_split(tsvd_handle* h, int64_t rows, int64_t cols, const T* S, int64_t lds, void* out, void* outt,
                          cudaStream_t st);
 // Y (rows x w, FP32) = P X, P given by its pieces (rows x cols), X cols x w (FP32).
 size_t tc_mm_ws(int64_t rows, int64_t cols, int w);
