@@ -16,6 +16,8 @@
 // rotates nothing (or kMaxSweeps).  Then sigma_j = |g_j|, columns are sorted by
 // (sigma descending, index ascending), Ubar_j = g_j / sigma_j, Vbar_j = v_j, and
 // each pair is sign-flipped so the largest-magnitude entry of Vbar_j is positive.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 
 #include "tsvd_internal.cuh"
@@ -26,43 +28,54 @@ namespace {
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kMaxSweeps = 40;
 
-enum Ctl : int { kCtlCount = 0, kCtlGen = 1, kCtlErr = 2, kCtlSweeps = 3, kCtlVBad = 4, kCtlRot = 8 };
+enum Ctl : int { kCtlCount = 0, kCtlErr = 1, kCtlSweeps = 3, kCtlVBad = 4, kCtlNeed = 5, kCtlRot = 8 };
 constexpr int kCtlWords = kCtlRot + kMaxSweeps;
 
 __device__ inline unsigned vload(const unsigned* p) { return *reinterpret_cast<const volatile unsigned*>(p); }
 
-// Grid-wide barrier for a cooperative launch (all CTAs co-resident); one wait
-// gives up after max_wait SM clock cycles (the handle's limit, about 1 s by
-// default).  Returns false once any CTA has timed out; the answer is read once
-// per CTA (by thread 0, through shared memory), so every thread of a CTA takes
-// the same branch and none is left at a later __syncthreads.
-__device__ bool grid_sync(unsigned* ctl, long long max_wait) {
+__device__ inline void arrive_release(unsigned* p) {
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p) : "memory");
+}
+__device__ inline unsigned load_acquire(const unsigned* p) {
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+// Words 0 and 1 at p (8-byte aligned), read together.
+__device__ inline uint2 load2_acquire(const unsigned* p) {
+    unsigned long long v;
+    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return make_uint2((unsigned)v, (unsigned)(v >> 32));
+}
+
+// Grid-wide barrier for a cooperative launch (all CTAs co-resident): a count that only grows,
+// `epoch` times gridDim.x once every CTA has come (kept by each CTA, 0 at the start); one wait
+// gives up after max_wait SM clock cycles (the handle's limit, about 1 s by default).
+// Returns false once any CTA has timed out; the answer is read once per CTA (by thread 0,
+// through shared memory), so every thread of a CTA takes the same branch and none is left at
+// a later __syncthreads.  (A count that the last CTA resets, with a generation word to release
+// the others, added two more trips to memory to every barrier.)
+__device__ bool grid_sync(unsigned* ctl, long long max_wait, unsigned& epoch) {
     if (gridDim.x == 1) {
         __syncthreads();
         return true;
     }
     __shared__ int s_ok;
     __syncthreads();
+    ++epoch;
     if (threadIdx.x == 0) {
-        const unsigned g = vload(&ctl[kCtlGen]);
-        __threadfence();
-        const unsigned prev = atomicAdd(&ctl[kCtlCount], 1u);
-        if (prev == gridDim.x - 1) {
-            atomicExch(&ctl[kCtlCount], 0u);
-            __threadfence();
-            atomicAdd(&ctl[kCtlGen], 1u);
-        } else {
-            // busy-wait (naps wake late), bounded by the SM clock
-            const long long t0 = clock64();
-            while (vload(&ctl[kCtlGen]) == g) {
-                if (clock64() - t0 > max_wait) {
-                    atomicOr(&ctl[kCtlErr], 1u);
-                    break;
-                }
+        arrive_release(&ctl[kCtlCount]);
+        // busy-wait (naps wake late), bounded by the SM clock
+        const long long t0 = clock64();
+        uint2 v;  // count and error word in one read
+        while (v = load2_acquire(ctl), v.x < epoch * gridDim.x) {
+            if (clock64() - t0 > max_wait) {
+                atomicOr(&ctl[kCtlErr], 1u);
+                v.y = 1u;
+                break;
             }
         }
-        __threadfence();
-        s_ok = vload(&ctl[kCtlErr]) == 0u ? 1 : 0;
+        s_ok = v.y == 0u ? 1 : 0;
     }
     __syncthreads();
     return s_ok != 0;
@@ -105,6 +118,7 @@ __global__ void jacobi_sweep_kernel(int n, int npad, double* __restrict__ G, dou
                                     double* __restrict__ nrm, unsigned* ctl, double tol, int ppb,
                                     long long max_wait) {
     const double tol2 = tol * tol;
+    unsigned epoch = 0;
     __shared__ double s_gam[kMaxSlots], s_c[kMaxSlots], s_s[kMaxSlots];
     __shared__ int s_rot[kMaxSlots];
     __shared__ int s_any;
@@ -123,7 +137,7 @@ __global__ void jacobi_sweep_kernel(int n, int npad, double* __restrict__ G, dou
             if (lane == 0) nrm[c] = acc;
         }
         if (threadIdx.x == 0) s_any = 0;
-        if (!grid_sync(ctl, max_wait)) return;
+        if (!grid_sync(ctl, max_wait, epoch)) return;
         for (int rnd = 0; rnd < npad - 1; ++rnd) {
             for (int slot = warp; slot < cnt; slot += wpb) {                     // (A)
                 const int pi = base + slot;
@@ -194,10 +208,10 @@ __global__ void jacobi_sweep_kernel(int n, int npad, double* __restrict__ G, dou
                     }
                 }
             }
-            if (!grid_sync(ctl, max_wait)) return;
+            if (!grid_sync(ctl, max_wait, epoch)) return;
         }
         if (threadIdx.x == 0 && s_any) atomicAdd(&ctl[kCtlRot + sweep], 1u);
-        if (!grid_sync(ctl, max_wait)) return;
+        if (!grid_sync(ctl, max_wait, epoch)) return;
         if (vload(&ctl[kCtlRot + sweep]) == 0u) {
             if (blockIdx.x == 0 && threadIdx.x == 0) ctl[kCtlSweeps] = (unsigned)(sweep + 1);
             return;
@@ -231,7 +245,7 @@ constexpr int kJGThreads = 256;  // threads of the block kernel
 // FP64: zeta = (beta - alpha) / (2 gamma) with the difference in FP64 (it may cancel),
 // the ratio and t in FP32 (relative accuracy 1e-7 keeps the convergence quadratic),
 // c = 1/sqrt(1 + t^2) and s = c t in FP64 so that c^2 + s^2 = 1 to FP64 rounding and
-// the rotation stays orthogonal.  FP32 (the preconditioning sweeps): all in FP32.
+// the rotation stays orthogonal.
 __device__ inline bool rot_params(double al, double be, double ga, double tol2, double& c, double& sn, double& t) {
     const double big = fmax(al, be);
     if (!(ga != 0.0 && big > 0.0)) return false;
@@ -247,20 +261,6 @@ __device__ inline bool rot_params(double al, double be, double ga, double tol2, 
     sn = c * t;
     return true;
 }
-__device__ inline bool rot_params(float al, float be, float ga, float tol2, float& c, float& sn, float& t) {
-    const float big = fmaxf(al, be);
-    if (!(ga != 0.0f && big > 0.0f)) return false;
-    const int e = ilogbf(big);
-    const float as = scalbnf(al, -e), bs = scalbnf(be, -e), gs = scalbnf(ga, -e);
-    if (!(gs * gs > tol2 * as * bs)) return false;
-    const float zf = (bs - as) / (2.0f * gs);
-    const float az = fabsf(zf);
-    t = az > 1e18f ? 0.5f / zf : copysignf(1.0f, zf) / (az + sqrtf(fmaf(az, az, 1.0f)));
-    c = rsqrtf(fmaf(t, t, 1.0f));
-    sn = c * t;
-    return true;
-}
-
 template <typename T>
 __device__ inline T warp_sum_t(T v) {
 #pragma unroll
@@ -527,7 +527,12 @@ __global__ void __launch_bounds__(kJGThreads, 1) jacobi_gram_kernel(int n, int n
     __shared__ T s_c[W], s_s[W];
     __shared__ int s_rot[W], s_pp[W], s_pq[W];
     __shared__ int s_any, s_rnd;
+    if (vload(&ctl[kCtlNeed]) == 0u) {  // every column pair is orthogonal to tol already
+        if (blockIdx.x == 0 && threadIdx.x == 0) ctl[kCtlSweeps] = 1u;
+        return;
+    }
     const T tol2 = tol * tol;
+    unsigned epoch = 0;
     const int ld = gram_ld(n);
     const int nblk = npad / W;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -602,10 +607,10 @@ __global__ void __launch_bounds__(kJGThreads, 1) jacobi_gram_kernel(int n, int n
                     }
                 }
             }
-            if (!grid_sync(ctl, max_wait)) return;
+            if (!grid_sync(ctl, max_wait, epoch)) return;
         }
         if (threadIdx.x == 0 && s_any) atomicAdd(&ctl[kCtlRot + sweep], 1u);
-        if (!grid_sync(ctl, max_wait)) return;
+        if (!grid_sync(ctl, max_wait, epoch)) return;
         if (vload(&ctl[kCtlRot + sweep]) == 0u) {
             if (blockIdx.x == 0 && threadIdx.x == 0) ctl[kCtlSweeps] = (unsigned)(sweep + 1);
             return;
@@ -615,15 +620,328 @@ __global__ void __launch_bounds__(kJGThreads, 1) jacobi_gram_kernel(int n, int n
 }
 
 
-// FP32 copy of B in the Jacobi layout: column c of G32 (ld n) = column c of B
-// (B row-major), padded columns zero; V32 (npad x npad, column-major) = I.
+// ---- FP32 preconditioning sweeps -------------------------------------------------------
+// The block method above in FP32 with blocks of 16 columns, its rows shared by a cluster:
+// G (n x npad) and V (npad x npad) are row-major, cluster c of the grid owns the round's
+// block pair (I, J), and CTA k of a cluster's C keeps the k-th part of the rows of G and V.
+// A round: the 32 columns of the CTA's rows to shared memory; the Gram matrix of its rows of G,
+// sent to every CTA of the cluster; the sum of the C partial matrices in rank order, so that
+// every CTA has the same M bit for bit; the rotations on M and Z, the same in every CTA; its
+// rows times Z; a barrier with the CTAs of its rank in the other clusters, the only ones that
+// read its rows.
+// The rotations of a mini-round (16 disjoint pairs) are one step of all 256 threads: thread
+// (k, l) holds the 2 x 2 block of M at the rows of pair k and the columns of pair l, and two
+// rows of Z at the columns of pair l; thread (k, k) computes pair k's rotation.  From one
+// mini-round to the next, columns q move by one position between lanes and rows q through
+// shared memory.
+// Bound by the latency of that chain (16 mini-rounds a round, 15 more in a sweep's first) and
+// of the round's loads, cluster exchange and barrier.  One CTA a block pair, with the rotations
+// in the registers of one warp, held 16 SMs at order 512 and took 13.8 ms.
+constexpr int kJ32W = 16;          // columns of a block
+constexpr int kJ32Ld = 36;         // row stride (floats) of the 32 columns and of Z: float4 rows
+constexpr int kJ32LdM = 48;        // of M: consecutive rows half the banks apart
+constexpr int kJ32Threads = 256;
+constexpr int kJ32Tiles = 36;      // 4 x 4 tiles on and above the diagonal of M
+constexpr int kJ32Tri = 16 * kJ32Tiles;
+constexpr int kJ32Slices = kJ32Threads / kJ32Tiles;  // row slices of a CTA's Gram matrix
+// A sweep whose largest |cos| is below 2e-3 is the last one: it leaves couplings near its square,
+// below the rounding of the accumulated V (5e-6 a pair at order 512).
+constexpr float kJ32Again = 4e-6f;
+// Control words: the error word, then for every rank a barrier count (a 128-byte line each) and
+// its own record of the sweeps to repeat.
+constexpr int kJ32Count = 32, kJ32Rot = kJ32Count + 8 * 32, kJ32Words = kJ32Rot + 8 * kMaxSweeps;
+
+// Rotation of a pair in FP32; false when |gamma| <= tol sqrt(alpha beta).  With d = beta -
+// alpha and g = 2 gamma: t = g / (d + sign(d) sqrt(d^2 + g^2)), c = 1 / sqrt(1 + t^2), s = c t.
+// (Values are scaled, so the approximate instructions see normal numbers only.)
+__device__ inline float rsqrt_approx(float x) {
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ inline float rcp_approx(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ inline bool rot32(float al, float be, float ga, float tol2, float& c, float& sn) {
+    const float big = fmaxf(al, be);
+    if (!(ga != 0.0f && big > 0.0f)) return false;
+    // by a power of two, so that neither the test nor the root over- or underflows
+    const float f = __int_as_float(max((254 << 23) - (__float_as_int(big) & 0x7F800000), 1 << 23));
+    const float as = al * f, bs = be * f, gs = ga * f;
+    if (!(gs * gs > tol2 * as * bs)) return false;
+    const float d = bs - as, g = 2.0f * gs;
+    const float h2 = fmaf(d, d, g * g);
+    const float h = h2 * rsqrt_approx(h2);
+    const float t = g * rcp_approx(d >= 0.0f ? d + h : d - h);
+    c = rsqrt_approx(fmaf(t, t, 1.0f));
+    sn = c * t;
+    return true;
+}
+
+enum J32State : int { kJ32Go = 0, kJ32Done = 1, kJ32Fail = 2 };
+
+__host__ __device__ inline size_t j32_smem(int n, int npad, int C) {
+    return sizeof(float) * kJ32Ld * (size_t)((n + C - 1) / C + (npad + C - 1) / C);
+}
+
+// The 2 x 2 block (a b; c d) between the pairs with rotations R (rows) and S (columns).
+__device__ inline void rot_block(float2 R, float2 S, float& a, float& b, float& c, float& d) {
+    const float a1 = fmaf(R.x, a, -R.y * c), c1 = fmaf(R.y, a, R.x * c);
+    const float b1 = fmaf(R.x, b, -R.y * d), d1 = fmaf(R.y, b, R.x * d);
+    a = fmaf(S.x, a1, -S.y * b1), b = fmaf(S.y, a1, S.x * b1);
+    c = fmaf(S.x, c1, -S.y * d1), d = fmaf(S.y, c1, S.x * d1);
+}
+__device__ inline void rot_row(float2 S, float& x, float& y) {
+    const float u = fmaf(S.x, x, -S.y * y);
+    y = fmaf(S.y, x, S.x * y);
+    x = u;
+}
+
+template <int C>
+__global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(kJ32Threads, 2)
+    jacobi32_kernel(int n, int npad, float* G, float* V, unsigned* ctl, float tol, long long max_wait) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    extern __shared__ __align__(16) float buf[];  // own rows of G, then of V; 32 columns, stride kJ32Ld
+    __shared__ __align__(16) float s_part[kJ32Slices][kJ32Tri];  // Gram matrices of row slices (upper tiles)
+    __shared__ __align__(16) float s_in[C][kJ32Tri];             // and of the cluster's CTAs
+    __shared__ __align__(16) float M[32][kJ32LdM], Z[32][kJ32Ld];
+    __shared__ float2 s_cs[kJ32W];
+    __shared__ int s_state[2][C], s_ok;
+    float(*s_q)[2][kJ32W][kJ32W] = reinterpret_cast<float(*)[2][kJ32W][kJ32W]>(&s_part[0][0]);  // rows q, twice
+    static_assert(4 * kJ32W * kJ32W <= kJ32Slices * kJ32Tri, "the rotations' exchange fits the partial sums");
+    const int tid = threadIdx.x;
+    if ((int)cl.num_blocks() != C || (int)gridDim.x != C * (npad / (2 * kJ32W))) {  // not the launch it is built for
+        if (blockIdx.x == 0 && tid == 0) atomicOr(&ctl[kCtlErr], 1u);
+        return;
+    }
+    const int rank = (int)cl.block_rank(), pair = (int)blockIdx.x / C, nb = (int)gridDim.x / C;
+    const int nblk = npad / kJ32W;
+    const float tol2 = tol * tol;
+    const int g0 = n * rank / C, ng = n * (rank + 1) / C - g0;
+    const int v0 = npad * rank / C, nr = ng + npad * (rank + 1) / C - v0;
+    const int q4 = 4 * (tid & 7);              // this thread's 4 of the 32 columns in copies and products
+    const int k = tid >> 4, l = tid & 15;      // its pairs in the rotations
+    const int k1 = (k + 1) & 15, l1 = (l + 1) & 15;
+    // its 4 x 4 tile (ti <= tj) and row slice in the Gram matrix
+    const int slice = tid / kJ32Tiles;
+    int ti = 0, tj = tid % kJ32Tiles;
+    while (tj >= 8 - ti) tj -= 8 - ti, ++ti;
+    tj += ti;
+    int state = kJ32Go, sweeps = kMaxSweeps, parity = 0;
+    unsigned epoch = 0;
+    for (int sweep = 0; sweep < kMaxSweeps; ++sweep) {
+        bool again = false;
+        for (int rnd = 0; rnd < nblk - 1; ++rnd, parity ^= 1) {
+            const int bi = rr_player(pair, rnd, nblk), bj = rr_player(nblk - 1 - pair, rnd, nblk);
+            const int col = q4 < kJ32W ? bi * kJ32W + q4 : bj * kJ32W + q4 - kJ32W;
+#pragma unroll 4
+            for (int r = tid >> 3; r < nr; r += kJ32Threads / 8) {
+                const float* src = r < ng ? G + (int64_t)(g0 + r) * npad : V + (int64_t)(v0 + r - ng) * npad;
+                *reinterpret_cast<float4*>(buf + r * kJ32Ld + q4) = __ldcg(reinterpret_cast<const float4*>(src + col));
+            }
+            __syncthreads();
+            if (slice < kJ32Slices) {  // upper tiles of the Gram matrix of the own rows
+                float acc[4][4] = {};
+#pragma unroll 2
+                for (int r = slice; r < ng; r += kJ32Slices) {
+                    const float4 x = *reinterpret_cast<const float4*>(buf + r * kJ32Ld + 4 * ti);
+                    const float4 y = *reinterpret_cast<const float4*>(buf + r * kJ32Ld + 4 * tj);
+                    const float xa[4] = {x.x, x.y, x.z, x.w}, ya[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+                    for (int a = 0; a < 4; ++a)
+#pragma unroll
+                        for (int b = 0; b < 4; ++b) acc[a][b] = fmaf(xa[a], ya[b], acc[a][b]);
+                }
+#pragma unroll
+                for (int a = 0; a < 4; ++a)
+                    *reinterpret_cast<float4*>(&s_part[slice][16 * (tid % kJ32Tiles) + 4 * a]) =
+                        make_float4(acc[a][0], acc[a][1], acc[a][2], acc[a][3]);
+            }
+            __syncthreads();
+            if (tid < kJ32Tri / 4) {
+                float4 t = *reinterpret_cast<const float4*>(&s_part[0][4 * tid]);
+#pragma unroll
+                for (int p = 1; p < kJ32Slices; ++p) {
+                    const float4 v = *reinterpret_cast<const float4*>(&s_part[p][4 * tid]);
+                    t.x += v.x, t.y += v.y, t.z += v.z, t.w += v.w;
+                }
+#pragma unroll
+                for (int c = 0; c < C; ++c)
+                    *reinterpret_cast<float4*>(cl.map_shared_rank(&s_in[rank][4 * tid], c)) = t;
+            } else if (tid < kJ32Tri / 4 + C) {
+                *cl.map_shared_rank(&s_state[parity][rank], tid - kJ32Tri / 4) = state;
+            }
+            cl.sync();
+            if (tid < kJ32Tri / 4) {
+                float4 t = *reinterpret_cast<const float4*>(&s_in[0][4 * tid]);
+#pragma unroll
+                for (int c = 1; c < C; ++c) {
+                    const float4 v = *reinterpret_cast<const float4*>(&s_in[c][4 * tid]);
+                    t.x += v.x, t.y += v.y, t.z += v.z, t.w += v.w;
+                }
+                // row tid % 4 of tile tid / 4
+                int a = 0, b = tid >> 2;
+                while (b >= 8 - a) b -= 8 - a, ++a;
+                b += a;
+                const int row = 4 * a + (tid & 3);
+                *reinterpret_cast<float4*>(&M[row][4 * b]) = t;
+                if (a != b) {
+                    M[4 * b][row] = t.x;
+                    M[4 * b + 1][row] = t.y;
+                    M[4 * b + 2][row] = t.z;
+                    M[4 * b + 3][row] = t.w;
+                }
+            }
+            // A CTA whose barrier timed out, or that saw a last sweep, leaves together with its
+            // cluster: no shared memory is written after its CTA has left.  (Two sets of state
+            // words: a CTA may be a round ahead of one that still reads.)
+            const int fail = __syncthreads_or(tid < C && s_state[parity][tid] == kJ32Fail);
+            if (fail || state == kJ32Done) {
+                sweeps = sweep;
+                goto out;
+            }
+            bool any = false;
+            float zp[2], zq[2];  // rows k and k + 16 of Z at columns p and q of pair l
+#pragma unroll
+            for (int e = 0; e < 2; ++e) zp[e] = k + 16 * e == l, zq[e] = k + 16 * e == l + 16;
+            if (rnd == 0) {  // rotations inside I and J: round-robin on 16 players in each, 8 pairs a block
+                for (int e = tid; e < 32 * 32; e += kJ32Threads) Z[e >> 5][e & 31] = (e >> 5) == (e & 31);
+                __syncthreads();
+                for (int m = 0; m < kJ32W - 1; ++m) {
+                    const int ak = rr_player(k & 7, m, kJ32W), bk = rr_player(15 - (k & 7), m, kJ32W);
+                    const int al = rr_player(l & 7, m, kJ32W), bl = rr_player(15 - (l & 7), m, kJ32W);
+                    const int pk = 2 * (k & 8) + min(ak, bk), qk = 2 * (k & 8) + max(ak, bk);
+                    const int pl = 2 * (l & 8) + min(al, bl), ql = 2 * (l & 8) + max(al, bl);
+                    float a = M[pk][pl], b = M[pk][ql], c = M[qk][pl], d = M[qk][ql];
+                    float x0 = Z[k][pl], y0 = Z[k][ql], x1 = Z[k + 16][pl], y1 = Z[k + 16][ql];
+                    int rot = 0;
+                    if (k == l) {
+                        float cc = 1.0f, sn = 0.0f;
+                        if (rot32(a, d, b, tol2, cc, sn)) {
+                            rot = 1;
+                            again |= b * b > kJ32Again * a * d;
+                        }
+                        s_cs[k] = make_float2(cc, sn);
+                    }
+                    if (!__syncthreads_or(rot)) continue;
+                    any = true;
+                    const float2 R = s_cs[k], S = s_cs[l];
+                    rot_block(R, S, a, b, c, d);
+                    rot_row(S, x0, y0);
+                    rot_row(S, x1, y1);
+                    M[pk][pl] = a, M[pk][ql] = b, M[qk][pl] = c, M[qk][ql] = d;
+                    Z[k][pl] = x0, Z[k][ql] = y0, Z[k + 16][pl] = x1, Z[k + 16][ql] = y1;
+                    __syncthreads();
+                }
+#pragma unroll
+                for (int e = 0; e < 2; ++e) zp[e] = Z[k + 16 * e][l], zq[e] = Z[k + 16 * e][l + 16];
+            }
+            {  // rotations between I and J: pair k is (k, 16 + (k + m) mod 16)
+                float a = M[k][l], b = M[k][l + 16], c = M[k + 16][l], d = M[k + 16][l + 16];
+#pragma unroll 2
+                for (int m = 0; m < kJ32W; ++m) {
+                    int rot = 0;
+                    if (k == l) {
+                        float cc = 1.0f, sn = 0.0f;
+                        if (rot32(a, d, b, tol2, cc, sn)) {
+                            rot = 1;
+                            again |= b * b > kJ32Again * a * d;
+                        }
+                        s_cs[k] = make_float2(cc, sn);
+                    }
+                    if (__syncthreads_or(rot)) {
+                        any = true;
+                        const float2 R = s_cs[k], S = s_cs[l];
+                        rot_block(R, S, a, b, c, d);
+                        rot_row(S, zp[0], zq[0]);
+                        rot_row(S, zp[1], zq[1]);
+                    }
+                    s_q[m & 1][0][k][l] = c;
+                    s_q[m & 1][1][k][l] = d;
+                    const int next = (tid & 16) | l1;  // the lane of pair l + 1
+                    b = __shfl_sync(kFull, b, next);
+                    zq[0] = __shfl_sync(kFull, zq[0], next);
+                    zq[1] = __shfl_sync(kFull, zq[1], next);
+                    __syncthreads();
+                    c = s_q[m & 1][0][k1][l];
+                    d = s_q[m & 1][1][k1][l1];
+                }
+            }
+            if (any) {
+#pragma unroll
+                for (int e = 0; e < 2; ++e) Z[k + 16 * e][l] = zp[e], Z[k + 16 * e][l + 16] = zq[e];
+                __syncthreads();
+                for (int r0 = tid >> 3; r0 < nr; r0 += kJ32Threads / 2) {  // four rows share the reads of Z
+                    float acc[4][4] = {};
+                    const float* x[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) x[u] = buf + min(r0 + u * (kJ32Threads / 8), nr - 1) * kJ32Ld;
+#pragma unroll 2
+                    for (int kk = 0; kk < 32; kk += 4) {
+                        float4 z[4];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) z[e] = *reinterpret_cast<const float4*>(&Z[kk + e][q4]);
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const float4 v = *reinterpret_cast<const float4*>(x[u] + kk);
+                            const float xs[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                acc[u][0] = fmaf(xs[e], z[e].x, acc[u][0]);
+                                acc[u][1] = fmaf(xs[e], z[e].y, acc[u][1]);
+                                acc[u][2] = fmaf(xs[e], z[e].z, acc[u][2]);
+                                acc[u][3] = fmaf(xs[e], z[e].w, acc[u][3]);
+                            }
+                        }
+                    }
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int r = r0 + u * (kJ32Threads / 8);
+                        if (r >= nr) break;
+                        float* dst = r < ng ? G + (int64_t)(g0 + r) * npad : V + (int64_t)(v0 + r - ng) * npad;
+                        *reinterpret_cast<float4*>(dst + col) = make_float4(acc[u][0], acc[u][1], acc[u][2], acc[u][3]);
+                    }
+                }
+            }
+            if (rnd == nblk - 2 && again) atomicOr(&ctl[kJ32Rot + rank * kMaxSweeps + sweep], 1u);
+            // barrier with the CTAs of this rank; bounded as grid_sync is
+            __syncthreads();
+            ++epoch;
+            if (tid == 0) {
+                unsigned* cnt = ctl + kJ32Count + 32 * rank;
+                arrive_release(cnt);
+                const long long t0 = clock64();
+                int ok = 1;
+                while (load_acquire(cnt) < epoch * (unsigned)nb) {
+                    if (clock64() - t0 > max_wait) {
+                        atomicOr(&ctl[kCtlErr], 1u);
+                        ok = 0;
+                        break;
+                    }
+                }
+                s_ok = ok;
+            }
+            __syncthreads();
+            if (!s_ok) state = kJ32Fail;
+        }
+        if (state == kJ32Go && vload(&ctl[kJ32Rot + rank * kMaxSweeps + sweep]) == 0u) state = kJ32Done;
+    }
+out:
+    if (blockIdx.x == 0 && tid == 0) ctl[kCtlSweeps] = (unsigned)sweeps;
+    cl.sync();
+}
+
+// FP32 copy of B (n x npad row-major, padded columns zero) and V (npad x npad) = I.
 __global__ void jacobi_init32_kernel(int n, int npad, const double* __restrict__ B, int64_t ldb,
                                      float* __restrict__ G, float* __restrict__ V) {
     const int64_t tot = (int64_t)npad * n, totv = (int64_t)npad * npad;
     for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < tot + totv;
          idx += (int64_t)gridDim.x * blockDim.x) {
         if (idx < tot) {
-            const int c = (int)(idx / n), r = (int)(idx % n);
+            const int r = (int)(idx / npad), c = (int)(idx % npad);
             G[idx] = c < n ? (float)B[(int64_t)r * ldb + c] : 0.0f;
         } else {
             const int64_t k = idx - tot;
@@ -641,7 +959,7 @@ __global__ void jacobi_vinit_kernel(int n, int npad, const float* __restrict__ V
     for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < tot;
          idx += (int64_t)gridDim.x * blockDim.x) {
         const int r = (int)(idx / n), c = (int)(idx % n);
-        V[idx] = (double)V32[(int64_t)c * npad + r];
+        V[idx] = (double)V32[(int64_t)r * npad + c];
     }
     if (blockIdx.x == 0 && threadIdx.x == 0 && ctl32[kCtlErr]) atomicOr(&status[kStTimeout], 1);
 }
@@ -661,6 +979,92 @@ __global__ void __launch_bounds__(256) jacobi_vreset_kernel(int n, const unsigne
     if (*bad == 0u) return;
     for (int idx = (int)(blockIdx.x * blockDim.x + threadIdx.x); idx < n * n; idx += (int)(gridDim.x * blockDim.x))
         V[idx] = (idx / n == idx % n) ? 1.0 : 0.0;
+}
+
+// ---- all column pairs at once -----------------------------------------------------------
+// With the columns of Y nearly orthogonal and M = Y^T Y, the rotations of all pairs together
+// are Q = I + E + E^2/2 + E^3/8, E skew with the tangents t_pq of the pairs' rotations:
+// Q^T Q = I - E^6/64, orthogonal to FP64 rounding while |E|_2 <= 2^-7.8, and a coupling of
+// relative size kappa falls to about kappa^2 / gap.  A column far smaller than the others has
+// tangents in proportion, so Y + Y (Q - I) keeps its relative accuracy.
+// The first two steps, on V, take Q = the polar factor of I + E by Newton-Schulz iterations
+// instead (exact for a pair of close singular values apart from the others).  |E|_2 <= 0.95 needs
+// six, |E|_2 <= 0.5 four: the three after the first step and four after the second are enough.
+// The bound: |E|_2 <= L + S, S = |E_small|_F / sqrt(2) of the tangents up to `small` and L the
+// largest row sum of the others (a few close pairs).  Tangents above `all` are left out, if the
+// bound fails those above `mid`, else those above `small`, else all; they stay for the sweeps.
+struct TanLimits {
+    double all, mid, small, norm;
+};
+constexpr TanLimits kJTanV1{0.7, 0.35, 0.03, 0.95}, kJTanV2{0.45, 0.2, 0.03, 0.5};
+constexpr TanLimits kJTanY{4e-3, 2e-3, 0x1p-10, 4.48e-3};
+
+// Block i: row i of E from M (null E: only the test), its sum of squares up to lim.small, its
+// sums from there to lim.mid and to lim.all, and `need` if a coupling of the row exceeds tol.
+__global__ void __launch_bounds__(128) jacobi_tan_kernel(int n, const double* __restrict__ M, double tol,
+                                                         TanLimits lim, double* __restrict__ E,
+                                                         double* __restrict__ rows, unsigned* need) {
+    __shared__ double red[3][4];
+    const int i = blockIdx.x;
+    const double tol2 = tol * tol;
+    bool over = false;
+    double sq = 0.0, mid = 0.0, all = 0.0;
+    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+        const int p = min(i, j), q = max(i, j);
+        double c, sn, t = 0.0;
+        const bool rot = p != q && rot_params(M[p * n + p], M[q * n + q], M[p * n + q], tol2, c, sn, t);
+        if (rot) over = true;
+        if (!rot || fabs(t) > lim.all) t = 0.0;
+        if (E) E[i * n + j] = i < j ? t : -t;
+        const double v = fabs(t);
+        if (v <= lim.small) sq = fma(v, v, sq);
+        else all += v;
+        if (v > lim.small && v <= lim.mid) mid += v;
+    }
+    if (need && __syncthreads_or(over) && threadIdx.x == 0) atomicOr(need, 1u);
+    if (!E) return;
+    sq = warp_sum(sq), mid = warp_sum(mid), all = warp_sum(all);
+    const int warp = threadIdx.x >> 5;
+    if ((threadIdx.x & 31) == 0) red[0][warp] = sq, red[1][warp] = mid, red[2][warp] = all;
+    __syncthreads();
+    if (threadIdx.x < 3) {
+        const double* r = red[threadIdx.x];
+        rows[threadIdx.x * n + i] = (r[0] + r[1]) + (r[2] + r[3]);
+    }
+}
+
+// Block i: row i of E without the tangents that the norm bound leaves out; H = E (null: not wanted).
+__global__ void __launch_bounds__(128) jacobi_guard_kernel(int n, const double* __restrict__ rows, TanLimits lim,
+                                                           double* __restrict__ E, double* __restrict__ H) {
+    __shared__ double red[3][4];
+    double sq = 0.0, mid = 0.0, all = 0.0;
+    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+        sq += rows[j];
+        mid = fmax(mid, rows[n + j]);
+        all = fmax(all, rows[2 * n + j]);
+    }
+    sq = warp_sum(sq);
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+        mid = fmax(mid, __shfl_xor_sync(kFull, mid, d));
+        all = fmax(all, __shfl_xor_sync(kFull, all, d));
+    }
+    const int warp = threadIdx.x >> 5;
+    if ((threadIdx.x & 31) == 0) red[0][warp] = sq, red[1][warp] = mid, red[2][warp] = all;
+    __syncthreads();
+    const double S = sqrt(0.5 * ((red[0][0] + red[0][1]) + (red[0][2] + red[0][3])));
+    mid = fmax(fmax(red[1][0], red[1][1]), fmax(red[1][2], red[1][3]));
+    all = fmax(fmax(red[2][0], red[2][1]), fmax(red[2][2], red[2][3]));
+    const double keep = S + all <= lim.norm   ? lim.all
+                        : S + mid <= lim.norm ? lim.mid
+                        : S <= lim.norm       ? lim.small
+                                              : -1.0;
+    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+        const int idx = (int)blockIdx.x * n + j;
+        const double t = E[idx], v = fabs(t) <= keep ? t : 0.0;
+        E[idx] = v;
+        if (H) H[idx] = v;
+    }
 }
 
 // sigma_c = |g_c|, one warp a column.
@@ -832,15 +1236,11 @@ static int block_width(int n) {
     while (w < 8 && (n + 2 * w - 1) / (2 * w) > 152) w *= 2;
     return w;
 }
-// Block width of the FP32 preconditioning sweeps: the widest blocks (fewest rounds;
-// FP32 work is cheap next to the rounds' latency).
-constexpr int kJW32 = 16;
-
 static int pad_to(int n, int w) { return (n + 2 * w - 1) / (2 * w) * (2 * w); }
 
 // Buffers of one small SVD, carved identically by the sizing and the run.
 struct SvdBufs {
-    double *G, *V, *nrm, *sig, *part;
+    double *G, *V, *nrm, *sig, *part, *rows_n;
     int* perm;
     unsigned *ctl, *ctl32;
     float *G32, *V32;
@@ -859,13 +1259,14 @@ static SvdBufs carve_svd(Arena& ar, int n, int npad, int nv, bool precond) {
     b.ctl = ar.take<unsigned>(kCtlWords);
     b.part = ar.take<double>(gemm_tn_ws(nullptr, n, n, nv > 0 ? nv : 1, false) / sizeof(double) + 1);
     if (precond) {
-        const int np32 = pad_to(n, kJW32);
-        b.ctl32 = ar.take<unsigned>(kCtlWords);
+        const int np32 = pad_to(n, kJ32W);
+        b.ctl32 = ar.take<unsigned>(kJ32Words);
         b.G32 = ar.take<float>((size_t)n * np32);
         b.V32 = ar.take<float>((size_t)np32 * np32);
         b.Vp = ar.take<double>((size_t)n * n);
         b.Tm = ar.take<double>((size_t)n * n);
         b.Y = ar.take<double>((size_t)n * n);
+        b.rows_n = ar.take<double>((size_t)3 * n);
         b.oz_bytes = std::max(oz_tn_ws(n, n, n, true), oz_nn_ws(n, n, n));
         b.oz = ar.take<char>(b.oz_bytes);
     }
@@ -942,11 +1343,47 @@ static int run_block_sweeps(tsvd_handle* h, int n, int npad, int w, T* G, unsign
         default: return TSVD_ERR_UNSUPPORTED;
     }
 }
-template <>
-int run_block_sweeps<float>(tsvd_handle* h, int n, int npad, int w, float* G, unsigned* ctl, float tol,
-                            cudaStream_t st, float* V) {
-    if (w != kJW32) return TSVD_ERR_UNSUPPORTED;
-    return launch_gram<float, kJW32>(h, n, npad, G, ctl, tol, st, V);
+// Cooperative launch of the FP32 sweeps with clusters of C CTAs; false if the chip does not hold
+// all of them at once.
+template <int C>
+static int launch_jacobi32(tsvd_handle* h, int n, int npad, float* G, float* V, unsigned* ctl, float tol,
+                           cudaStream_t st, bool& fits) {
+    const int nb = npad / (2 * kJ32W);
+    static thread_local int configured = -1;
+    if (configured != h->device) {
+        TSVD_TRY_CUDA(cudaFuncSetAttribute(jacobi32_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)j32_smem(1024, 1024, C)));
+        configured = h->device;
+    }
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(nb * C));
+    cfg.blockDim = dim3(kJ32Threads);
+    cfg.dynamicSmemBytes = j32_smem(n, npad, C);
+    cfg.stream = st;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = C;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    int fit = 0;
+    TSVD_TRY_CUDA(cudaOccupancyMaxActiveClusters(&fit, jacobi32_kernel<C>, &cfg));
+    fits = fit >= nb;
+    if (!fits) return TSVD_OK;
+    long long mw = h->max_wait;
+    void* args[] = {(void*)&n, (void*)&npad, (void*)&G, (void*)&V, (void*)&ctl, (void*)&tol, (void*)&mw};
+    h->launches++;
+    TSVD_TRY_CUDA(cudaLaunchCooperativeKernel((const void*)jacobi32_kernel<C>, cfg.gridDim, cfg.blockDim, args,
+                                              cfg.dynamicSmemBytes, st));
+    return TSVD_OK;
+}
+static int run_jacobi32(tsvd_handle* h, int n, int npad, float* G, float* V, unsigned* ctl, float tol,
+                        cudaStream_t st) {
+    bool fits = false;
+    TSVD_TRY(launch_jacobi32<8>(h, n, npad, G, V, ctl, tol, st, fits));
+    if (!fits) TSVD_TRY(launch_jacobi32<4>(h, n, npad, G, V, ctl, tol, st, fits));
+    if (!fits) TSVD_TRY(launch_jacobi32<2>(h, n, npad, G, V, ctl, tol, st, fits));
+    return fits ? TSVD_OK : TSVD_ERR_UNSUPPORTED;
 }
 
 int small_svd(tsvd_handle* h, int n, const double* B, int64_t ldb, double* Ubar, double* sigma, double* Vbar, int nv,
@@ -983,35 +1420,65 @@ int small_svd(tsvd_handle* h, int n, const double* B, int64_t ldb, double* Ubar,
             //     columns orthogonal to about eps32 sigma_1 / sigma_j, where the right
             //     vectors from the orthogonalised columns of B^T would leave couplings of
             //     eps32 (sigma_1 / sigma_j)^2 and more FP64 sweeps)
-            const int np32 = pad_to(n, kJW32);
-            TSVD_TRY_CUDA(cudaMemsetAsync(bf.ctl32, 0, sizeof(unsigned) * kCtlWords, st));
+            const int np32 = pad_to(n, kJ32W);
+            TSVD_TRY_CUDA(cudaMemsetAsync(bf.ctl32, 0, sizeof(unsigned) * kJ32Words, st));
             h->launches += 2;
             jacobi_init32_kernel<<<(unsigned)std::min<int64_t>(4096, ((int64_t)(n + np32) * np32 + 255) / 256), 256, 0,
                                    st>>>(n, np32, B, ldb, bf.G32, bf.V32);
             TSVD_TRY_CUDA(cudaGetLastError());
             const float tol32 = (float)(n > 16 ? n : 16) * 5.9604645e-08f;  // n 2^-24
-            TSVD_TRY(run_block_sweeps<float>(h, n, np32, kJW32, bf.G32, bf.ctl32, tol32, st, bf.V32));
+            TSVD_TRY(run_jacobi32(h, n, np32, bf.G32, bf.V32, bf.ctl32, tol32, st));
             jacobi_vinit_kernel<<<(unsigned)std::min<int64_t>(4096, ((int64_t)n * n + 255) / 256), 256, 0, st>>>(
                 n, np32, bf.V32, bf.Vp, bf.ctl32, status);
             TSVD_TRY_CUDA(cudaGetLastError());
-            // (2) V orthogonal to FP64 rounding: two polar (Newton-Schulz) steps
-            //     V <- V (3 I - V^T V) / 2 with FP64-accurate tensor-core products, then a
-            //     check that falls back to V = I if V^T V is not the identity to 1e-12
-            for (int itn = 0; itn < 2; ++itn) {
-                TSVD_TRY(oz_gemm_tn(h, n, n, n, bf.Vp, n, bf.Vp, n, bf.Tm, n, true, bf.oz, bf.oz_bytes, status, st));
-                TSVD_TRY(oz_gemm_nn(h, n, n, n, -0.5, bf.Vp, n, bf.Tm, n, 1.5, bf.Vp, n, false, bf.oz, bf.oz_bytes,
-                                    status, st));
+            // (2) V orthogonal to FP64 rounding by polar (Newton-Schulz) steps V <- V (3 I - V^T V) / 2
+            //     with FP64-accurate tensor-core products.  After the first (orthogonal to 1e-8) and
+            //     after three more all pairs are rotated at once, V <- V (I + E) with E from
+            //     (B V)^T (B V); after the last four, a check that falls back to V = I if V^T V is not
+            //     the identity to 1e-12.
+            // (3) Y = B V: the SVD of B V is that of B with the right vectors rotated by V.  Two more
+            //     rounds of all rotations at once, on Y (E in Vp, H in V: both free here), take its
+            //     couplings to FP64 rounding unless singular values nearly coincide.
+            // (4) The test that a sweep would make: the FP64 sweeps run only if it finds a pair.
+            const auto tn = [&](const double* X) {  // Tm = X^T X
+                return oz_gemm_tn(h, n, n, n, X, n, X, n, bf.Tm, n, true, bf.oz, bf.oz_bytes, status, st);
+            };
+            const auto nn = [&](double alpha, const double* X, int64_t ldx, const double* Mm, double beta, double* Yo) {
+                return oz_gemm_nn(h, n, n, n, alpha, X, ldx, Mm, n, beta, Yo, n, false, bf.oz, bf.oz_bytes, status, st);
+            };
+            const auto tangents = [&](const TanLimits& lim, double* E, double* H, unsigned* need) {
+                h->launches += E ? 2 : 1;
+                jacobi_tan_kernel<<<n, 128, 0, st>>>(n, bf.Tm, tol, lim, E, bf.rows_n, need);
+                if (E) jacobi_guard_kernel<<<n, 128, 0, st>>>(n, bf.rows_n, lim, E, H);
+                return cudaGetLastError();
+            };
+            double* const H = bf.V;
+            for (int itn = 0; itn < 8; ++itn) {
+                TSVD_TRY(tn(bf.Vp));
+                TSVD_TRY(nn(-0.5, bf.Vp, n, bf.Tm, 1.5, bf.Vp));
+                if (itn == 0 || itn == 3) {
+                    TSVD_TRY(nn(1.0, B, ldb, bf.Vp, 0.0, bf.Y));
+                    TSVD_TRY(tn(bf.Y));
+                    TSVD_TRY_CUDA(tangents(itn == 0 ? kJTanV1 : kJTanV2, H, nullptr, nullptr));
+                    TSVD_TRY(nn(1.0, bf.Vp, n, H, 1.0, bf.Vp));
+                }
             }
-            TSVD_TRY(oz_gemm_tn(h, n, n, n, bf.Vp, n, bf.Vp, n, bf.Tm, n, true, bf.oz, bf.oz_bytes, status, st));
+            TSVD_TRY(tn(bf.Vp));
             h->launches += 2;
             const unsigned vb = (unsigned)std::min<int64_t>(304, ((int64_t)n * n + 255) / 256);
             jacobi_vcheck_kernel<<<vb, 256, 0, st>>>(n, bf.Tm, bf.ctl32 + kCtlVBad);
             jacobi_vreset_kernel<<<vb, 256, 0, st>>>(n, bf.ctl32 + kCtlVBad, bf.Vp);
             TSVD_TRY_CUDA(cudaGetLastError());
-            // (3) FP64 sweeps on B V: the SVD of B V is that of B with the right vectors
-            //     rotated by V, and its columns start orthogonal to FP32 accuracy
-            TSVD_TRY(oz_gemm_nn(h, n, n, n, 1.0, B, ldb, bf.Vp, n, 0.0, bf.Y, n, false, bf.oz, bf.oz_bytes, status,
-                                st));
+            TSVD_TRY(nn(1.0, B, ldb, bf.Vp, 0.0, bf.Y));
+            for (int itn = 0; itn < 2; ++itn) {
+                TSVD_TRY(tn(bf.Y));
+                TSVD_TRY_CUDA(tangents(kJTanY, bf.Vp, H, nullptr));
+                TSVD_TRY(nn(0.125, bf.Vp, n, bf.Vp, 0.5, H));   // H = E / 2 + E^2 / 8
+                TSVD_TRY(nn(1.0, bf.Vp, n, H, 1.0, bf.Vp));     // E + E H = Q - I
+                TSVD_TRY(nn(1.0, bf.Y, n, bf.Vp, 1.0, bf.Y));
+            }
+            TSVD_TRY(tn(bf.Y));
+            TSVD_TRY_CUDA(tangents(kJTanY, nullptr, nullptr, bf.ctl + kCtlNeed));
             h->launches++;
             jacobi_init_kernel<<<ib, 256, 0, st>>>(n, npad, bf.Y, n, G, V);
             TSVD_TRY_CUDA(cudaGetLastError());

@@ -176,7 +176,8 @@ __device__ inline void oz_store_pair(__nv_bfloat16* planes, int64_t Ra, int64_t 
 }
 
 // Rows slicer: columns [c0, c1) of S (R rows, lds) -> columns [c0, c1) of stored row i, zeros
-// from c1 to the next multiple of 16; 8 lanes a row.
+// from c1 to the next multiple of 16; G lanes a row: 8, or 32 where the rows are few (512 x 512
+// took 45 us with 8, 4,096 lanes in all).
 // GROW false (c0 = 0): the exponent of a row's largest entry.  GROW true, for a matrix that
 // gains columns (a Lanczos basis): one above it when it is set (at c0 = 0, or when a later
 // entry does not fit it: the row's earlier columns are then sliced again), so that new
@@ -184,12 +185,11 @@ __device__ inline void oz_store_pair(__nv_bfloat16* planes, int64_t Ra, int64_t 
 // for all rows of an orthonormal basis kept about log2(R) / 2 bits fewer.
 // Bound by the 14 (16) bytes written and 8 read an entry (the digits are read again from
 // cache where a row group fits it): 100,000 x 64 in 27 us = 5.2 TB/s.
-template <int D, bool GROW>
+template <int D, bool GROW, int G>
 __global__ void __launch_bounds__(256, 4) oz_slice_rows_kernel(int64_t R, int64_t c0, int64_t c1,
                                                             const double* __restrict__ S, int64_t lds,
                                                             __nv_bfloat16* __restrict__ planes, int64_t Ra,
                                                             int* __restrict__ eexp) {
-    constexpr int G = 8;
     const int sl = threadIdx.x % G;
     const int64_t ng = (int64_t)gridDim.x * (blockDim.x / G);
     const int64_t rounds = (R + ng - 1) / ng;  // the same for every lane: the shuffles need them all
@@ -964,10 +964,16 @@ struct OzView {
 int oz_slice_rows(tsvd_handle* h, int64_t R, int64_t c0, int64_t c1, const double* S, int64_t lds, bool grow,
                   __nv_bfloat16* planes, int* eexp, cudaStream_t st) {
     if (R == 0) return TSVD_OK;
-    const int64_t blocks = std::min<int64_t>((R + 31) / 32, (int64_t)h->sm_count * 32);
-    const auto kern = grow ? oz_slice_rows_kernel<kOzDig, true>
-                           : (h->oz_dig == kOzWideDig ? oz_slice_rows_kernel<kOzWideDig, false>
-                                                      : oz_slice_rows_kernel<kOzDig, false>);
+    // 8 lanes a row; 32 where that leaves fewer warps than the chip has room for
+    const bool few = R <= (int64_t)h->sm_count * 32;
+    const int64_t rows = few ? 8 : 32;  // of a block
+    const int64_t blocks = std::min<int64_t>((R + rows - 1) / rows, (int64_t)h->sm_count * 32);
+    const bool wide = h->oz_dig == kOzWideDig;
+    const auto kern = grow   ? (few ? oz_slice_rows_kernel<kOzDig, true, 32> : oz_slice_rows_kernel<kOzDig, true, 8>)
+                      : wide ? (few ? oz_slice_rows_kernel<kOzWideDig, false, 32>
+                                    : oz_slice_rows_kernel<kOzWideDig, false, 8>)
+                             : (few ? oz_slice_rows_kernel<kOzDig, false, 32>
+                                    : oz_slice_rows_kernel<kOzDig, false, 8>);
     h->launches++;
     kern<<<(unsigned)blocks, 256, 0, st>>>(R, c0, c1, S, lds, planes, oz_ra(R), eexp);
     TSVD_TRY_CUDA(cudaGetLastError());
