@@ -479,7 +479,7 @@ int tsvd_cgs_qr(tsvd_handle* h, int64_t q, int r, int b, double* Y, int64_t ldy,
  * computes only the leading nv columns of Vbar, as B^T ubar_j / sigma_j (the
  * other columns of Vbar are left undefined, and only the leading nv columns of
  * Ubar follow the sign convention); this is what the methods use, and for
- * 64 < n <= 1024 it runs the block-Jacobi kernel.  Sign convention: the
+ * 48 < n <= 1024 it runs the block-Jacobi kernel.  Sign convention: the
  * largest-magnitude entry of each defined Vbar column is positive.
  * *sweeps (may be NULL) receives the sweep count.
  * Requires 1 <= n <= TSVD_MAX_SMALL_SVD. */

@@ -18,6 +18,8 @@
 // are reduced in a fixed order so results are bitwise reproducible.
 #include <cooperative_groups.h>
 
+#include <algorithm>
+
 #include "tsvd_internal.cuh"
 
 namespace tsvd {
@@ -42,7 +44,7 @@ __device__ inline void decode_upper(int lin, int nr, int& ri, int& rj) {
 
 // TI: input element type (also the accumulation type within a slab); TW: type written.
 template <typename TI, typename TW>
-__global__ void __launch_bounds__(128) gemm_tn_kernel(int64_t q, int64_t s, int64_t b,
+__global__ void __launch_bounds__(128, 7) gemm_tn_kernel(int64_t q, int64_t s, int64_t b,
                                                       const TI* __restrict__ X, int64_t ldx,
                                                       const TI* __restrict__ Z, int64_t ldz,
                                                       TW* __restrict__ out, int64_t ldo,
@@ -62,7 +64,9 @@ __global__ void __launch_bounds__(128) gemm_tn_kernel(int64_t q, int64_t s, int6
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int wr = warp >> 1, wc = warp & 1;
     const int i = lane >> 1, jg = (lane & 1) * 8;
-    const bool active = !(symmetric && ri == rj && wr > wc);
+    // (a sub-tile below the diagonal or wholly past the last row or column has no work)
+    const bool active = !(symmetric && ri == rj && wr > wc) && (int64_t)ri * kTnR + wr * 16 < s &&
+                        (int64_t)rj * kTnR + wc * 16 < b;
     TI acc[8];
 #pragma unroll
     for (int t = 0; t < 8; ++t) acc[t] = TI(0);
@@ -77,8 +81,9 @@ __global__ void __launch_bounds__(128) gemm_tn_kernel(int64_t q, int64_t s, int6
         }
         __syncthreads();
         if (active) {
+            const int kn = (int)min((int64_t)kTnKc, r1 - k0);
 #pragma unroll 4
-            for (int kk = 0; kk < kTnKc; ++kk) {
+            for (int kk = 0; kk < kn; ++kk) {
                 const TI x = Xs[kk][wr * 16 + i];
                 const TI* zr = &Zs[kk][wc * 16 + jg];
 #pragma unroll
@@ -144,7 +149,13 @@ struct TnPlan {
 constexpr int64_t kTnWave = 152 * 7;
 constexpr int64_t kTnWaveF32 = 152 * 16;
 
-TnPlan tn_plan(int64_t q, int64_t s, int64_t b, bool symmetric, int elem_bytes) {
+// More slabs (of 16 rows and up) for a product that would leave half the SMs without a CTA:
+// its time is that of one CTA's rows, 32 x 32 x 32 FP64 steps taking 8 us of an SM
+// (512 x 64 by 512 x 16: 107 us in 2 slabs of 256 rows).  Only while the partial sums stay
+// within kTnExtra bytes, which every FP64 workspace has room for.
+constexpr size_t kTnExtra = 1 << 20;
+
+TnPlan tn_plan(int64_t q, int64_t s, int64_t b, bool symmetric, int elem_bytes, bool extra) {
     TnPlan p;
     p.nreg_s = (int)((s + kTnR - 1) / kTnR);
     p.nreg_b = (int)((b + kTnR - 1) / kTnR);
@@ -154,9 +165,18 @@ TnPlan tn_plan(int64_t q, int64_t s, int64_t b, bool symmetric, int elem_bytes) 
     if (slabs > max_slabs) slabs = max_slabs;
     if (slabs > 65535) slabs = 65535;
     if (slabs < 1) slabs = 1;
+    int64_t align = kTnKc;
+    if (extra && elem_bytes == 8 && p.regions * slabs < 76) {
+        const int64_t fit = (int64_t)(kTnExtra / sizeof(double)) / (s * b);
+        const int64_t more = std::min<int64_t>(std::min<int64_t>((q + 15) / 16, (152 + p.regions - 1) / p.regions), fit);
+        if (more > slabs) {
+            slabs = more;
+            align = 16;
+        }
+    }
     int64_t rows = (q + slabs - 1) / slabs;
-    rows = (rows + kTnKc - 1) / kTnKc * kTnKc;
-    if (rows < kTnKc) rows = kTnKc;
+    rows = (rows + align - 1) / align * align;
+    if (rows < align) rows = align;
     p.slab_rows = rows;
     p.slabs = (int)((q + rows - 1) / rows);
     if (p.slabs < 1) p.slabs = 1;
@@ -165,7 +185,8 @@ TnPlan tn_plan(int64_t q, int64_t s, int64_t b, bool symmetric, int elem_bytes) 
 
 // ---------------------------------------------------------------------------
 // gemm_nn: CTA = 4 warps, 32 rows; lane = row, warp w owns CW columns of the
-// current panel (4*CW columns).  X tile and M chunk staged in shared memory,
+// current panel (4*CW columns); CTAs (x, y), (x, y + gridDim.y) ... of a row of the grid
+// share the panels.  X tile and M chunk staged in shared memory,
 // output staged for coalesced stores.
 // ---------------------------------------------------------------------------
 // Accumulation in TX (the precision of the tall operand); M is converted to TX on load.
@@ -179,7 +200,7 @@ __global__ void __launch_bounds__(128) gemm_nn_kernel(int64_t q, int64_t s, int6
     __shared__ TX Ms[32][PW + 1];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int64_t r0 = (int64_t)blockIdx.x * 32;
-    for (int64_t c0 = 0; c0 < b; c0 += PW) {
+    for (int64_t c0 = (int64_t)blockIdx.y * PW; c0 < b; c0 += (int64_t)gridDim.y * PW) {
         TX acc[CW];
 #pragma unroll
         for (int c = 0; c < CW; ++c) acc[c] = TX(0);
@@ -199,9 +220,10 @@ __global__ void __launch_bounds__(128) gemm_nn_kernel(int64_t q, int64_t s, int6
                 Ms[kk][cc] = in ? (TX)M[k * ldm + col] : TX(0);
             }
             __syncthreads();
-            if (!(upper && k0 > jw_hi)) {
+            if (!(upper && k0 > jw_hi) && c0 + warp * CW < b) {
+                const int kn = (int)min((int64_t)32, kmax - k0);
 #pragma unroll 4
-                for (int kk = 0; kk < 32; ++kk) {
+                for (int kk = 0; kk < kn; ++kk) {
                     const TX x = Xs[lane][kk];
                     const TX* mr = &Ms[kk][warp * CW];
 #pragma unroll
@@ -745,18 +767,23 @@ __global__ void put_diagonal_kernel(int s, const double* __restrict__ sig, doubl
 
 // ---------------------------------------------------------------------------
 size_t gemm_tn_ws(tsvd_handle* h, int64_t q, int64_t s, int64_t b, bool symmetric, int elem_bytes) {
+    const size_t least = gemm_tn_ws_min(h, q, s, b, symmetric, elem_bytes);
+    return elem_bytes == 8 ? std::max(least, kTnExtra) : least;
+}
+size_t gemm_tn_ws_min(tsvd_handle* h, int64_t q, int64_t s, int64_t b, bool symmetric, int elem_bytes) {
     (void)h;
-    const TnPlan p = tn_plan(q, s, b, symmetric, elem_bytes);
+    const TnPlan p = tn_plan(q, s, b, symmetric, elem_bytes, false);
     if (p.slabs == 1 && !symmetric) return 0;
     return align256(sizeof(double) * (size_t)p.slabs * (size_t)s * (size_t)b);
 }
 
 template <typename TI, typename TC>
 cudaError_t gemm_tn(tsvd_handle* h, int64_t q, int64_t s, int64_t b, const TI* X, int64_t ldx, const TI* Z,
-                    int64_t ldz, TC* C, int64_t ldc, bool symmetric, double* partial, cudaStream_t st) {
+                    int64_t ldz, TC* C, int64_t ldc, bool symmetric, double* partial, cudaStream_t st,
+                    size_t partial_bytes, bool fp64_pipe) {
     if (s == 0 || b == 0) return cudaSuccess;
     constexpr bool kF32 = std::is_same<TI, float>::value;
-    const TnPlan p = tn_plan(q, s, b, symmetric, (int)sizeof(TI));
+    const TnPlan p = tn_plan(q, s, b, symmetric, (int)sizeof(TI), partial_bytes >= kTnExtra);
     if (q == 0) {
         for (int64_t i = 0; i < s; ++i) {
             cudaError_t e = cudaMemsetAsync(C + i * ldc, 0, sizeof(TC) * b, st);
@@ -771,7 +798,7 @@ cudaError_t gemm_tn(tsvd_handle* h, int64_t q, int64_t s, int64_t b, const TI* X
                    (double)sizeof(TI) * (double)q * (symmetric ? b : s + b) + (double)sizeof(TC) * s * b, st);
     if constexpr (std::is_same<TI, double>::value && std::is_same<TC, double>::value) {
         const OzCache* xc = h->oz_ws ? oz_find_cache(h, X, ldx, q, s, true) : nullptr;
-        if (h->oz_ws && oz_worth(s, b, q) && oz_tn_ws(q, s, b, symmetric, xc != nullptr, h->oz_dig) <= h->oz_bytes) {
+        if (!fp64_pipe && h->oz_ws && oz_worth(s, b, q) && oz_tn_ws(q, s, b, symmetric, xc != nullptr, h->oz_dig) <= h->oz_bytes) {
             const int rc = oz_gemm_tn(h, q, s, b, X, ldx, Z, ldz, C, ldc, symmetric, h->oz_ws, h->oz_bytes,
                                       h->oz_status, st, xc);
             return rc == TSVD_OK ? cudaSuccess : cudaErrorUnknown;
@@ -852,15 +879,16 @@ cudaError_t update_gram(tsvd_handle* h, int64_t q, int64_t s, int64_t b, double 
 }
 
 template cudaError_t gemm_tn<double, double>(tsvd_handle*, int64_t, int64_t, int64_t, const double*, int64_t,
-                                             const double*, int64_t, double*, int64_t, bool, double*, cudaStream_t);
+                                             const double*, int64_t, double*, int64_t, bool, double*, cudaStream_t, size_t, bool);
 template cudaError_t gemm_tn<float, double>(tsvd_handle*, int64_t, int64_t, int64_t, const float*, int64_t,
-                                            const float*, int64_t, double*, int64_t, bool, double*, cudaStream_t);
+                                            const float*, int64_t, double*, int64_t, bool, double*, cudaStream_t, size_t, bool);
 template cudaError_t gemm_tn<float, float>(tsvd_handle*, int64_t, int64_t, int64_t, const float*, int64_t,
-                                           const float*, int64_t, float*, int64_t, bool, double*, cudaStream_t);
+                                           const float*, int64_t, float*, int64_t, bool, double*, cudaStream_t, size_t, bool);
 
 template <typename TX, typename TM, typename TY>
 cudaError_t gemm_nn(tsvd_handle* h, int64_t q, int64_t s, int64_t b, double alpha, const TX* X, int64_t ldx,
-                    const TM* M, int64_t ldm, double beta, TY* Y, int64_t ldy, bool upper, cudaStream_t st) {
+                    const TM* M, int64_t ldm, double beta, TY* Y, int64_t ldy, bool upper, cudaStream_t st,
+                    bool fp64_pipe) {
     if (q == 0 || b == 0) return cudaSuccess;
     const unsigned grid = (unsigned)((q + 31) / 32);
     ProfScope prof(h, TSVD_K_GEMM_NN, upper ? (double)q * b * (b + 1) : 2.0 * q * s * b,
@@ -869,7 +897,7 @@ cudaError_t gemm_nn(tsvd_handle* h, int64_t q, int64_t s, int64_t b, double alph
     if constexpr (std::is_same<TX, double>::value && std::is_same<TM, double>::value &&
                   std::is_same<TY, double>::value) {
         const OzCache* xc = h->oz_ws ? oz_find_cache(h, X, ldx, q, s, false) : nullptr;
-        if (h->oz_ws && s > 0 && oz_worth(q, b, s) && oz_nn_ws(q, s, b, xc != nullptr, h->oz_dig) <= h->oz_bytes) {
+        if (!fp64_pipe && h->oz_ws && s > 0 && oz_worth(q, b, s) && oz_nn_ws(q, s, b, xc != nullptr, h->oz_dig) <= h->oz_bytes) {
             const int rc = oz_gemm_nn(h, q, s, b, alpha, X, ldx, M, ldm, beta, Y, ldy, upper, h->oz_ws, h->oz_bytes,
                                       h->oz_status, st, xc);
             return rc == TSVD_OK ? cudaSuccess : cudaErrorUnknown;
@@ -879,21 +907,41 @@ cudaError_t gemm_nn(tsvd_handle* h, int64_t q, int64_t s, int64_t b, double alph
     if constexpr (std::is_same<TX, float>::value) {
         if (b <= 128) return launch_gemm_nn_f32<TM, TY>(st, q, s, b, alpha, X, ldx, M, ldm, beta, Y, ldy, upper);
     }
-    if (b <= 32) {
-        gemm_nn_kernel<8, TX, TM, TY><<<grid, 128, 0, st>>>(q, s, b, alpha, X, ldx, M, ldm, beta, Y, ldy, upper ? 1 : 0);
-    } else if (b <= 64) {
-        gemm_nn_kernel<16, TX, TM, TY><<<grid, 128, 0, st>>>(q, s, b, alpha, X, ldx, M, ldm, beta, Y, ldy,
-                                                             upper ? 1 : 0);
-    } else {
-        gemm_nn_kernel<32, TX, TM, TY><<<grid, 128, 0, st>>>(q, s, b, alpha, X, ldx, M, ldm, beta, Y, ldy,
-                                                             upper ? 1 : 0);
+    // Columns of a CTA: all of them (up to 128) where X is read from memory once that way;
+    // fewer while the grid leaves SMs without a CTA (the FP64 pipe of an SM then bounds the
+    // time: 512 x 64 by 64 x 16 took 31 us on 16 SMs), but not in place, where one CTA reads
+    // all of its rows before it writes them.
+    int cw = b <= 16 ? 4 : (b <= 32 ? 8 : (b <= 64 ? 16 : 32));
+    if constexpr (!std::is_same<TX, double>::value) cw = std::max(cw, 8);
+    const uintptr_t x0 = reinterpret_cast<uintptr_t>(X), x1 = reinterpret_cast<uintptr_t>(X + q * ldx);
+    const uintptr_t y0 = reinterpret_cast<uintptr_t>(Y), y1 = reinterpret_cast<uintptr_t>(Y + q * ldy);
+    unsigned gy = 1;
+    if (std::is_same<TX, double>::value && (x1 <= y0 || y1 <= x0)) {
+        while (cw > 1 && (int64_t)grid * ((b + 4 * cw - 1) / (4 * cw)) < 152) cw /= 2;
+        if ((int64_t)grid < 152) gy = (unsigned)std::min<int64_t>((b + 4 * cw - 1) / (4 * cw), 65535);
+    }
+    const dim3 g(grid, gy);
+    const int up = upper ? 1 : 0;
+    if (cw == 32) {
+        gemm_nn_kernel<32, TX, TM, TY><<<g, 128, 0, st>>>(q, s, b, alpha, X, ldx, M, ldm, beta, Y, ldy, up);
+    } else if (cw == 16) {
+        gemm_nn_kernel<16, TX, TM, TY><<<g, 128, 0, st>>>(q, s, b, alpha, X, ldx, M, ldm, beta, Y, ldy, up);
+    } else if (cw == 8) {
+        gemm_nn_kernel<8, TX, TM, TY><<<g, 128, 0, st>>>(q, s, b, alpha, X, ldx, M, ldm, beta, Y, ldy, up);
+    } else if constexpr (std::is_same<TX, double>::value) {
+        if (cw == 4)
+            gemm_nn_kernel<4, TX, TM, TY><<<g, 128, 0, st>>>(q, s, b, alpha, X, ldx, M, ldm, beta, Y, ldy, up);
+        else if (cw == 2)
+            gemm_nn_kernel<2, TX, TM, TY><<<g, 128, 0, st>>>(q, s, b, alpha, X, ldx, M, ldm, beta, Y, ldy, up);
+        else
+            gemm_nn_kernel<1, TX, TM, TY><<<g, 128, 0, st>>>(q, s, b, alpha, X, ldx, M, ldm, beta, Y, ldy, up);
     }
     return cudaGetLastError();
 }
 
 #define TSVD_INST_NN(TX, TM, TY)                                                                                  \
     template cudaError_t gemm_nn<TX, TM, TY>(tsvd_handle*, int64_t, int64_t, int64_t, double, const TX*, int64_t, \
-                                             const TM*, int64_t, double, TY*, int64_t, bool, cudaStream_t);
+                                             const TM*, int64_t, double, TY*, int64_t, bool, cudaStream_t, bool);
 TSVD_INST_NN(double, double, double)
 TSVD_INST_NN(float, double, float)
 TSVD_INST_NN(float, float, float)

@@ -1229,9 +1229,10 @@ __global__ void __launch_bounds__(128) jacobi_vfix_kernel(int n, const double* _
 
 // Block width of the FP64 block-Jacobi kernel for an order-n SVD without V (at most
 // one wave of 152 CTAs, each owning a pair of blocks), or 0 when the per-pair kernel
-// is used (small n, or V accumulated).
+// is used (V accumulated, or n <= 48: its FP64 rotations of all columns by one SM take 3.9 ms at
+// order 64, growing as n^3, the block path 1 ms).
 static int block_width(int n) {
-    if (n <= 64 || n > 1024) return 0;
+    if (n <= 48 || n > 1024) return 0;
     int w = 1;
     while (w < 8 && (n + 2 * w - 1) / (2 * w) > 152) w *= 2;
     return w;
@@ -1257,7 +1258,8 @@ static SvdBufs carve_svd(Arena& ar, int n, int npad, int nv, bool precond) {
     b.sig = ar.take<double>(npad);
     b.perm = ar.take<int>(npad);
     b.ctl = ar.take<unsigned>(kCtlWords);
-    b.part = ar.take<double>(gemm_tn_ws(nullptr, n, n, nv > 0 ? nv : 1, false) / sizeof(double) + 1);
+    b.part = ar.take<double>(std::max(gemm_tn_ws(nullptr, n, n, nv > 0 ? nv : 1, false),
+                                      gemm_tn_ws(nullptr, n, n, n, true)) / sizeof(double) + 1);
     if (precond) {
         const int np32 = pad_to(n, kJ32W);
         b.ctl32 = ar.take<unsigned>(kJ32Words);
@@ -1267,7 +1269,7 @@ static SvdBufs carve_svd(Arena& ar, int n, int npad, int nv, bool precond) {
         b.Tm = ar.take<double>((size_t)n * n);
         b.Y = ar.take<double>((size_t)n * n);
         b.rows_n = ar.take<double>((size_t)3 * n);
-        b.oz_bytes = std::max(oz_tn_ws(n, n, n, true), oz_nn_ws(n, n, n));
+        b.oz_bytes = std::max(std::max(oz_tn_ws(n, n, n, true), oz_nn_ws(n, n, n)), sizeof(double) * n * n);
         b.oz = ar.take<char>(b.oz_bytes);
     }
     return b;
@@ -1440,15 +1442,37 @@ int small_svd(tsvd_handle* h, int n, const double* B, int64_t ldb, double* Ubar,
             //     rounds of all rotations at once, on Y (E in Vp, H in V: both free here), take its
             //     couplings to FP64 rounding unless singular values nearly coincide.
             // (4) The test that a sweep would make: the FP64 sweeps run only if it finds a pair.
+            // Up to order 256 the products are shorter on the FP64 pipe (15 us each at order 64, 110 us
+            // with slices and cut tiles; 29 and 60 us at order 256).
+            const bool pipe = n <= 256;
             const auto tn = [&](const double* X) {  // Tm = X^T X
+                if (pipe)
+                    return gemm_tn<double, double>(h, n, n, n, X, n, X, n, bf.Tm, n, true, bf.part, st, ~size_t(0),
+                                                   true) == cudaSuccess
+                               ? TSVD_OK
+                               : TSVD_ERR_CUDA;
                 return oz_gemm_tn(h, n, n, n, X, n, X, n, bf.Tm, n, true, bf.oz, bf.oz_bytes, status, st);
             };
             const auto nn = [&](double alpha, const double* X, int64_t ldx, const double* Mm, double beta, double* Yo) {
+                if (pipe) {
+                    if (X == Yo || Mm == Yo) {  // in place through a copy
+                        double* const cp = static_cast<double*>(bf.oz);
+                        if (cudaMemcpyAsync(cp, Yo, sizeof(double) * n * n, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
+                            return (int)TSVD_ERR_CUDA;
+                        if (X == Yo) X = cp;
+                        if (Mm == Yo) Mm = cp;
+                    }
+                    return gemm_nn<double, double, double>(h, n, n, n, alpha, X, ldx, Mm, n, beta, Yo, n, false, st,
+                                                           true) == cudaSuccess
+                               ? (int)TSVD_OK
+                               : (int)TSVD_ERR_CUDA;
+                }
                 return oz_gemm_nn(h, n, n, n, alpha, X, ldx, Mm, n, beta, Yo, n, false, bf.oz, bf.oz_bytes, status, st);
             };
             const auto tangents = [&](const TanLimits& lim, double* E, double* H, unsigned* need) {
+                // (the steps take out couplings below tol too, as a sweep's other rotations would)
                 h->launches += E ? 2 : 1;
-                jacobi_tan_kernel<<<n, 128, 0, st>>>(n, bf.Tm, tol, lim, E, bf.rows_n, need);
+                jacobi_tan_kernel<<<n, 128, 0, st>>>(n, bf.Tm, E ? 2 * kEps : tol, lim, E, bf.rows_n, need);
                 if (E) jacobi_guard_kernel<<<n, 128, 0, st>>>(n, bf.rows_n, lim, E, H);
                 return cudaGetLastError();
             };

@@ -38,7 +38,7 @@ extern "C" int tsvd_dense_mm_t_noalloc(tsvd_handle* h, int64_t m, int64_t n, con
                                        const double* X, int64_t ldx, double* Y, int64_t ldy, void* stream) {
     if (!h || m < 0 || n < 0 || w < 0 || lda < n || !A || !X || !Y || ldx < w || ldy < w)
         return TSVD_ERR_INVALID_ARG;
-    const size_t need = tsvd::gemm_tn_ws(h, m, n, w, false);
+    const size_t need = tsvd::gemm_tn_ws_min(h, m, n, w, false);
     if (need > kNoAllocScratchBytes) return TSVD_ERR_UNSUPPORTED;
     tsvd::DeviceGuard dg(h->device);
     if (!dg.ok()) return TSVD_ERR_CUDA;
@@ -47,7 +47,8 @@ extern "C" int tsvd_dense_mm_t_noalloc(tsvd_handle* h, int64_t m, int64_t n, con
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // Every partial-sum slot the reduction reads is written first by the same
     // call, so nothing in the scratch has to start at zero.
-    TSVD_TRY_CUDA(tsvd::gemm_tn(h, m, n, w, A, lda, X, ldx, Y, ldy, false, static_cast<double*>(scratch), st));
+    TSVD_TRY_CUDA(tsvd::gemm_tn(h, m, n, w, A, lda, X, ldx, Y, ldy, false, static_cast<double*>(scratch), st,
+                                kNoAllocScratchBytes));
     TSVD_TRY_CUDA(cudaStreamSynchronize(st));
     return TSVD_OK;
 }

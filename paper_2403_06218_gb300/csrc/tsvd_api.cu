@@ -412,11 +412,12 @@ int tsvd_dense_mm(tsvd_handle* h, int trans, int64_t m, int64_t n, const double*
                   const double* X, int64_t ldx, double* Y, int64_t ldy, void* ws, size_t ws_bytes, void* stream) {
     if (!h || m < 0 || n < 0 || w < 0 || lda < n || !A || !X || !Y) return TSVD_ERR_INVALID_ARG;
     if (ldx < w || ldy < w) return TSVD_ERR_INVALID_ARG;
-    size_t need = trans ? gemm_tn_ws(h, m, n, w, false) : 0;
+    size_t need = trans ? gemm_tn_ws_min(h, m, n, w, false) : 0;
     TSVD_TRY(check_ws(ws, ws_bytes, need));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (trans)
-        TSVD_TRY_CUDA((gemm_tn<double, double>(h, m, n, w, A, lda, X, ldx, Y, ldy, false, static_cast<double*>(ws), st)));
+        TSVD_TRY_CUDA((gemm_tn<double, double>(h, m, n, w, A, lda, X, ldx, Y, ldy, false, static_cast<double*>(ws), st,
+                                               ws ? ws_bytes : 0)));
     else
         TSVD_TRY_CUDA((gemm_nn<double, double, double>(h, m, n, w, 1.0, A, lda, X, ldx, 0.0, Y, ldy, false, st)));
     TSVD_TRY_CUDA(cudaStreamSynchronize(st));

@@ -246,6 +246,9 @@ cudaError_t convert_to_float(tsvd_handle* h, int64_t n, const double* x, float* 
 // partial sums are FP64; TC is the output type.
 // Split-K scratch of gemm_tn for inputs of elem_bytes (8: FP64 inputs, 4: FP32 inputs).
 size_t gemm_tn_ws(tsvd_handle* h, int64_t q, int64_t s, int64_t b, bool symmetric, int elem_bytes = 8);
+// The least that gemm_tn runs with (partial_bytes); with gemm_tn_ws it may split a small product
+// over more CTAs.  fp64_pipe: never on the tensor cores.
+size_t gemm_tn_ws_min(tsvd_handle* h, int64_t q, int64_t s, int64_t b, bool symmetric, int elem_bytes = 8);
 // Register-tiled FP32 kernels (k_f32.cu) behind gemm_tn<float, *> and gemm_nn<float, *, *>.
 template <typename TW>
 cudaError_t launch_gemm_tn_f32(dim3 grid, cudaStream_t st, int64_t q, int64_t s, int64_t b, const float* X,
@@ -283,7 +286,7 @@ cudaError_t launch_update_gram_f32(cudaStream_t st, int slabs, int64_t slab_rows
 template <typename TI, typename TC>
 cudaError_t gemm_tn(tsvd_handle* h, int64_t q, int64_t s, int64_t b, const TI* X, int64_t ldx,
                     const TI* Z, int64_t ldz, TC* C, int64_t ldc, bool symmetric,
-                    double* partial_ws, cudaStream_t st);
+                    double* partial_ws, cudaStream_t st, size_t partial_bytes = ~size_t(0), bool fp64_pipe = false);
 
 // ---- FP64-accurate tensor-core products (k_oz.cu) -------------------------------
 // Worth running on the tensor cores rather than the FP64 pipe (M x N outputs, K deep).
@@ -399,7 +402,7 @@ struct OzStandalone {
 template <typename TX, typename TM, typename TY>
 cudaError_t gemm_nn(tsvd_handle* h, int64_t q, int64_t s, int64_t b, double alpha, const TX* X,
                     int64_t ldx, const TM* M, int64_t ldm, double beta, TY* Y, int64_t ldy,
-                    bool upper, cudaStream_t st);
+                    bool upper, cudaStream_t st, bool fp64_pipe = false);
 
 // Cholesky W = L L^T of a b x b SPD matrix (ld b) in one CTA; writes
 // Lt = L^T and Mt = L^{-T} (both upper, ld b).  Sets kStBreakdown on a pivot
