@@ -791,7 +791,7 @@ cudaError_t gemm_tn(tsvd_handle* h, int64_t q, int64_t s, int64_t b, const TI* X
         }
         return cudaSuccess;
     }
-    const dim3 grid((unsigned)p.regions, (unsigned)p.slabs);
+    dim3 grid((unsigned)p.regions, (unsigned)p.slabs);
     // algorithmic work: 2qsb flops (the upper half, q b (b+1), for a Gram matrix);
     // compulsory traffic: X and Z read once, C written once
     ProfScope prof(h, TSVD_K_GEMM_TN, symmetric ? (double)q * b * (b + 1) : 2.0 * q * s * b,
@@ -804,8 +804,24 @@ cudaError_t gemm_tn(tsvd_handle* h, int64_t q, int64_t s, int64_t b, const TI* X
             return rc == TSVD_OK ? cudaSuccess : cudaErrorUnknown;
         }
     }
-    if (p.slabs == 1 && !symmetric) {
+    int slabs = p.slabs;
+    int64_t slab_rows = p.slab_rows;
+    bool wide = false;
+    if constexpr (kF32) {
+        // one CTA an SM, in no more slabs than the partial sums have room for
+        const int regions = symmetric ? 0 : wide_f32_regions(q, s, b);
+        wide = regions > 0;
+        if (wide) {
+            slabs = std::min(slabs, std::max(1, 152 / regions));
+            slab_rows = ((q + slabs - 1) / slabs + 31) / 32 * 32;
+            slabs = (int)((q + slab_rows - 1) / slab_rows);
+            grid = dim3((unsigned)regions, (unsigned)slabs);
+        }
+    }
+    if (slabs == 1 && !symmetric) {
         h->launches++;
+        if constexpr (kF32)
+            if (wide) return launch_gemm_tn_wide_f32<TC>(grid, st, q, s, b, X, ldx, Z, ldz, C, ldc, 0, slab_rows);
         if constexpr (kF32)
             return launch_gemm_tn_f32<TC>(grid, st, q, s, b, X, ldx, Z, ldz, C, ldc, 0, p.slab_rows, 0, p.nreg_s,
                                           p.nreg_b);
@@ -816,7 +832,9 @@ cudaError_t gemm_tn(tsvd_handle* h, int64_t q, int64_t s, int64_t b, const TI* X
     const int64_t stride = s * b;
     h->launches += 2;
     if constexpr (kF32) {
-        cudaError_t e = launch_gemm_tn_f32<double>(grid, st, q, s, b, X, ldx, Z, ldz, partial, b, stride, p.slab_rows,
+        cudaError_t e = wide ? launch_gemm_tn_wide_f32<double>(grid, st, q, s, b, X, ldx, Z, ldz, partial, b, stride,
+                                                               slab_rows)
+                             : launch_gemm_tn_f32<double>(grid, st, q, s, b, X, ldx, Z, ldz, partial, b, stride, p.slab_rows,
                                                    symmetric ? 1 : 0, p.nreg_s, p.nreg_b);
         if (e != cudaSuccess) return e;
     } else {
@@ -824,7 +842,7 @@ cudaError_t gemm_tn(tsvd_handle* h, int64_t q, int64_t s, int64_t b, const TI* X
                                                          symmetric ? 1 : 0, p.nreg_s, p.nreg_b);
     }
     const int64_t tot = s * b;
-    gemm_tn_reduce_kernel<TC><<<(unsigned)((tot + 31) / 32), dim3(32, 8), 0, st>>>(s, b, p.slabs, partial, stride, C,
+    gemm_tn_reduce_kernel<TC><<<(unsigned)((tot + 31) / 32), dim3(32, 8), 0, st>>>(s, b, slabs, partial, stride, C,
                                                                                   ldc, symmetric ? 1 : 0);
     return cudaGetLastError();
 }

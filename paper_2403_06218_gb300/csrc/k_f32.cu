@@ -86,6 +86,145 @@ __global__ void __launch_bounds__(64, 16) gemm_tn_f32_kernel(int64_t q, int64_t 
     }
 }
 
+// The wide form: 128 x NB outputs a CTA, an 8 x 8 (8 x 4 for NB = 64) tile a thread, so that two
+// (three) 16-byte loads feed 32 packed FMAs (two FP32 FMAs an instruction): the FP32 pipe bounds
+// it, where the 4 x 4 tiles above were bound by shared-memory reads (500,003 x 512 by 500,003 x
+// 128: 3.32 ms = 20 TFLOP/s; here 1.16 ms = 57 TFLOP/s).  Two groups of 256 threads take alternate chunks of 16
+// rows, each with its own three buffers filled by asynchronous copies, and their sums are added
+// in FP64: half the run of FP32 additions, and one partial matrix a CTA.
+constexpr int kWideS = 128, kWideK = 16, kWideStages = 3;
+template <int NB>
+constexpr int kWideSmem = 2 * kWideStages * kWideK * (kWideS + NB) * (int)sizeof(float);
+
+__device__ inline void cp_async16(uint32_t dst, const float* src, int bytes) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+__device__ inline void cp_async4(uint32_t dst, const float* src, int bytes) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+using f32x2 = unsigned long long;
+__device__ inline f32x2 pack2(float lo, float hi) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ inline float2 unpack2(f32x2 v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ inline f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
+// 16 rows x COLS columns from column c0 of S (row0 on; zeros past row r1 or column `cols`) to dst
+// (row-major) by 256 threads; VEC: 16-byte aligned rows.
+template <int COLS, bool VEC>
+__device__ inline void wide_copy(uint32_t dst, const float* __restrict__ S, int64_t ld, int64_t row0, int64_t r1,
+                                 int64_t c0, int64_t cols, int tid) {
+    if constexpr (VEC) {
+#pragma unroll
+        for (int u = 0; u < kWideK * COLS / 4 / 256; ++u) {
+            const int idx = tid + 256 * u, rr = idx / (COLS / 4), cc = idx % (COLS / 4) * 4;
+            const int64_t left = cols - c0 - cc;
+            const int bytes = row0 + rr < r1 ? 4 * (int)max((int64_t)0, min((int64_t)4, left)) : 0;
+            cp_async16(dst + 16u * (uint32_t)idx, bytes ? S + (row0 + rr) * ld + c0 + cc : S, bytes);
+        }
+    } else {
+#pragma unroll
+        for (int u = 0; u < kWideK * COLS / 256; ++u) {
+            const int idx = tid + 256 * u, rr = idx / COLS, cc = idx % COLS;
+            const bool in = row0 + rr < r1 && c0 + cc < cols;
+            cp_async4(dst + 4u * (uint32_t)idx, in ? S + (row0 + rr) * ld + c0 + cc : S, in ? 4 : 0);
+        }
+    }
+}
+
+template <int NB, bool VEC, typename TW>
+__global__ void __launch_bounds__(512, 1) gemm_tn_wide_f32_kernel(int64_t q, int64_t s, int64_t b,
+                                                                  const float* __restrict__ X, int64_t ldx,
+                                                                  const float* __restrict__ Z, int64_t ldz,
+                                                                  TW* __restrict__ out, int64_t ldo,
+                                                                  int64_t slab_stride, int64_t slab_rows, int nreg_b) {
+    extern __shared__ __align__(16) float wsm[];
+    constexpr int ST = kWideK * (kWideS + NB), NZ = NB / 64;  // floats of a stage; groups of 4 columns of a thread
+    const int g = threadIdx.x >> 8, tid = threadIdx.x & 255, ty = tid >> 4, tx = tid & 15;
+    const int64_t xc0 = (int64_t)(blockIdx.x / nreg_b) * kWideS, zc0 = (int64_t)(blockIdx.x % nreg_b) * NB;
+    const int64_t r0 = (int64_t)blockIdx.y * slab_rows, r1 = min(q, r0 + slab_rows);
+    const int chunks = (int)((r1 - r0 + kWideK - 1) / kWideK);
+    const int mine = (chunks - g + 1) / 2;  // chunks g, g + 2, ...
+    float* const sm = wsm + g * kWideStages * ST;
+    const uint32_t sm32 = (uint32_t)__cvta_generic_to_shared(sm);
+    const auto issue = [&](int t) {
+        if (t < mine) {
+            const uint32_t d = sm32 + (uint32_t)(t % kWideStages * ST) * 4u;
+            const int64_t row = r0 + (int64_t)(2 * t + g) * kWideK;
+            wide_copy<kWideS, VEC>(d, X, ldx, row, r1, xc0, s, tid);
+            wide_copy<NB, VEC>(d + 4u * kWideK * kWideS, Z, ldz, row, r1, zc0, b, tid);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    f32x2 acc[8][2 * NZ];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 2 * NZ; ++j) acc[i][j] = 0ull;
+    issue(0);
+    issue(1);
+    for (int t = 0; t < mine; ++t) {
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        asm volatile("bar.sync %0, 256;" ::"r"(g + 1) : "memory");  // chunk t is here, buffer of t - 1 is free
+        issue(t + 2);
+        const float* xs = sm + t % kWideStages * ST + 4 * ty;
+        const float* zs = sm + t % kWideStages * ST + kWideK * kWideS + 4 * tx;
+#pragma unroll 4
+        for (int kk = 0; kk < kWideK; ++kk) {
+            const float4 x0 = *reinterpret_cast<const float4*>(xs + kk * kWideS);
+            const float4 x1 = *reinterpret_cast<const float4*>(xs + kk * kWideS + 64);
+            const float xa[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+            ulonglong2 z[NZ];
+#pragma unroll
+            for (int p = 0; p < NZ; ++p) z[p] = *reinterpret_cast<const ulonglong2*>(zs + kk * NB + 64 * p);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const f32x2 xx = pack2(xa[i], xa[i]);
+#pragma unroll
+                for (int p = 0; p < NZ; ++p) {
+                    acc[i][2 * p] = fma2(xx, z[p].x, acc[i][2 * p]);
+                    acc[i][2 * p + 1] = fma2(xx, z[p].y, acc[i][2 * p + 1]);
+                }
+            }
+        }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    // the second group's sums to the first through shared memory, thread by thread
+    f32x2* ex = reinterpret_cast<f32x2*>(wsm);
+    if (g == 1) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int j = 0; j < 2 * NZ; ++j) ex[(i * 2 * NZ + j) * 256 + tid] = acc[i][j];
+    }
+    __syncthreads();
+    if (g == 1) return;
+    TW* o = out + (int64_t)blockIdx.y * slab_stride;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int64_t row = xc0 + 4 * ty + (i & 3) + 64 * (i >> 2);
+        if (row >= s) continue;
+#pragma unroll
+        for (int j = 0; j < 2 * NZ; ++j) {
+            const float2 u = unpack2(acc[i][j]), v = unpack2(ex[(i * 2 * NZ + j) * 256 + tid]);
+            const int64_t col = zc0 + 4 * tx + 2 * (j & 1) + 64 * (j >> 1);
+            if (col < b) o[row * ldo + col] = (TW)((double)u.x + (double)v.x);
+            if (col + 1 < b) o[row * ldo + col + 1] = (TW)((double)u.y + (double)v.y);
+        }
+    }
+}
+
 // 256 threads: thread (ty, tx) in 16 x 16 owns rows 4ty..4ty+3 of a 64-row tile and
 // columns {4tx..4tx+3} + 64 p, p < NP, of the output (NP = 1: b <= 64, NP = 2: b <= 128).
 // All panels are accumulated before any store, so Y may alias X (s == b).
@@ -353,6 +492,49 @@ template cudaError_t launch_gemm_tn_f32<double>(dim3, cudaStream_t, int64_t, int
                                                 int);
 template cudaError_t launch_gemm_tn_f32<float>(dim3, cudaStream_t, int64_t, int64_t, int64_t, const float*, int64_t,
                                                const float*, int64_t, float*, int64_t, int64_t, int64_t, int, int, int);
+
+// Regions of 128 x NB outputs pay where little of them lies outside the matrix: at most half more
+// outputs than in the 32 x 32 regions of the other kernel.
+int wide_f32_regions(int64_t q, int64_t s, int64_t b) {
+    const int64_t nb = b <= 64 ? 64 : 128;
+    const int64_t wide = (s + 127) / 128 * 128 * ((b + nb - 1) / nb * nb);
+    const int64_t tiled = (s + 31) / 32 * 32 * ((b + 31) / 32 * 32);
+    return q >= 1024 && 2 * wide <= 3 * tiled ? (int)(wide / (128 * nb)) : 0;
+}
+
+template <int NB, bool VEC, typename TW>
+static cudaError_t launch_wide(dim3 grid, cudaStream_t st, int64_t q, int64_t s, int64_t b, const float* X,
+                               int64_t ldx, const float* Z, int64_t ldz, TW* out, int64_t ldo, int64_t slab_stride,
+                               int64_t slab_rows) {
+    static thread_local int configured = -1;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess && configured != dev) {
+        e = cudaFuncSetAttribute(gemm_tn_wide_f32_kernel<NB, VEC, TW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 kWideSmem<NB>);
+        if (e == cudaSuccess) configured = dev;
+    }
+    if (e != cudaSuccess) return e;
+    gemm_tn_wide_f32_kernel<NB, VEC, TW><<<grid, 512, kWideSmem<NB>, st>>>(
+        q, s, b, X, ldx, Z, ldz, out, ldo, slab_stride, slab_rows, (int)((b + NB - 1) / NB));
+    return cudaGetLastError();
+}
+
+template <typename TW>
+cudaError_t launch_gemm_tn_wide_f32(dim3 grid, cudaStream_t st, int64_t q, int64_t s, int64_t b, const float* X,
+                                    int64_t ldx, const float* Z, int64_t ldz, TW* out, int64_t ldo,
+                                    int64_t slab_stride, int64_t slab_rows) {
+    const bool vec = (ldx | ldz) % 4 == 0 &&
+                     ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(Z)) & 15) == 0;
+    const auto go = b <= 64 ? (vec ? launch_wide<64, true, TW> : launch_wide<64, false, TW>)
+                            : (vec ? launch_wide<128, true, TW> : launch_wide<128, false, TW>);
+    return go(grid, st, q, s, b, X, ldx, Z, ldz, out, ldo, slab_stride, slab_rows);
+}
+template cudaError_t launch_gemm_tn_wide_f32<double>(dim3, cudaStream_t, int64_t, int64_t, int64_t, const float*,
+                                                     int64_t, const float*, int64_t, double*, int64_t, int64_t,
+                                                     int64_t);
+template cudaError_t launch_gemm_tn_wide_f32<float>(dim3, cudaStream_t, int64_t, int64_t, int64_t, const float*,
+                                                    int64_t, const float*, int64_t, float*, int64_t, int64_t, int64_t);
 
 template <typename TM, typename TY>
 cudaError_t launch_gemm_nn_f32(cudaStream_t st, int64_t q, int64_t s, int64_t b, double alpha, const float* X,

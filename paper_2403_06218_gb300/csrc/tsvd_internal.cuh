@@ -266,6 +266,12 @@ cudaError_t bf16x3_split(tsvd_handle* h, int64_t rows, int64_t cols, const T* S,
 size_t tc_mm_ws(int64_t rows, int64_t cols, int w);
 cudaError_t tc_mm(tsvd_handle* h, int64_t rows, int64_t cols, const void* pieces, int w, const float* X, int64_t ldx,
                   float* Y, int64_t ldy, void* ws, int* status, cudaStream_t st);
+// Regions of the wide kernel (128 x 128, or 128 x 64 for b <= 64), 0 where it does not pay.
+int wide_f32_regions(int64_t q, int64_t s, int64_t b);
+template <typename TW>
+cudaError_t launch_gemm_tn_wide_f32(dim3 grid, cudaStream_t st, int64_t q, int64_t s, int64_t b, const float* X,
+                                    int64_t ldx, const float* Z, int64_t ldz, TW* out, int64_t ldo,
+                                    int64_t slab_stride, int64_t slab_rows);
 template <typename TM, typename TY>
 cudaError_t launch_gemm_nn_f32(cudaStream_t st, int64_t q, int64_t s, int64_t b, double alpha, const float* X,
                                int64_t ldx, const TM* M, int64_t ldm, double beta, TY* Y, int64_t ldy, bool upper);
