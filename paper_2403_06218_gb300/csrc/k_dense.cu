@@ -365,51 +365,90 @@ __global__ void __launch_bounds__(256) chol_inv_kernel(int b, const double* __re
 }
 
 // ---------------------------------------------------------------------------
-// chol_inv on a cluster of kCholCluster CTAs (b >= kCholClusterMin): the same
-// factorisation and inverse with the FP64 work spread over 8 SMs (one SM's FP64
-// pipe, 2 DFMA/clk, bounds the single-CTA kernel above).  Every CTA keeps a full
-// b x b copy in its shared memory; row i belongs to CTA i mod 8.  Per panel of 16
-// columns:
-//   1. every CTA factors the 16 x 16 diagonal block (warp 0; the same numbers and
-//      code in every CTA, so every CTA takes the same breakdown decision);
-//   2. each CTA solves its rows of the panel, L[i][P] = A[i][P] L11^{-T}, and writes
-//      them into every CTA's copy (distributed shared memory); cluster barrier;
-//   3. each CTA applies the rank-16 update A[i][k] -= L[i][P] L[k][P]^T to its rows
-//      (k <= i), then writes its rows of the next diagonal block into every copy;
-//      cluster barrier.
-// Afterwards every copy holds all of L; the inverse is split by columns (column c of
-// L^{-1} on CTA c mod 8, no exchange), and each CTA writes its rows of Lt and Mt.
-// The trailing updates sum 16 products per panel before subtracting (the one-CTA
-// kernel subtracts them one at a time), so results agree to rounding, not bits.
+// chol_inv on a cluster of kCholCluster CTAs (b >= kCholClusterMin): forward elimination of
+// [A | I], which leaves L^T's columns and M = L^{-1}, with the FP64 work spread over 8 SMs (one
+// SM's FP64 pipe, 2 DFMA/clk, bounds the one-CTA kernel above).  Row i belongs to CTA i mod 8,
+// column c of M's panel rows to CTA c mod 8.  Per panel of 16 columns:
+//   1. warp 0 of every CTA factors the 16 x 16 diagonal block, a row in the registers of each of
+//      lanes 0-15 (the same numbers and code in every CTA, so every CTA takes the same breakdown
+//      decision), while lanes 16-31 take its own 16 rows below through the same steps, which is
+//      their substitution L[i][P] = A[i][P] L11^{-T};
+//   2. warp 1 substitutes its own columns of the panel's rows of M, a column a lane;
+//   3. both go to every CTA (distributed shared memory); cluster barrier;
+//   4. rank-16 update of the own rows below, A[i][k] -= L[i][P] L[k][P]^T and M[i][c] -=
+//      L[i][P] M[P][c], 16 threads a row; the next panel's rows go out: its diagonal block to
+//      every CTA, its rows of M to their columns' owners; cluster barrier.
+// Bound by the chain of the pivots (16 steps of 1/sqrt, scale, update a panel) and, at b = 128,
+// by the FP64 pipe in the updates.  With the pivot steps through shared memory, a chain of 136
+// dependent FMAs a row for its substitution, and the inverse in a pass of its own at the end,
+// b = 128 took 296 us and b = 64 131 us.
+// The updates sum 16 products per panel before subtracting (the one-CTA kernel subtracts them
+// one at a time), so results agree to rounding, not bits.
 // ---------------------------------------------------------------------------
 constexpr int kCholCluster = 8;
 constexpr int kCholPanel = 16;
 constexpr int kCholClusterMin = 64;
+constexpr int kCholRows = TSVD_MAX_BLOCK / kCholCluster;  // own rows (and own columns of M) at most
+constexpr int kCholLd = TSVD_MAX_BLOCK + 4, kCholLdP = kCholPanel + 1;
+static_assert(kCholRows == kCholPanel && kCholPanel % kCholCluster == 0, "two own rows a panel, one lane a row");
 
-__global__ void __cluster_dims__(kCholCluster, 1, 1) __launch_bounds__(256)
+struct CholSmem {
+    double A[kCholRows][kCholLd];        // own rows of A (columns <= i), then of L
+    double M[kCholRows][kCholLd];        // own rows of M (columns < i)
+    double Lp[TSVD_MAX_BLOCK][kCholLdP];  // the panel's columns of L, all rows
+    double Mp[kCholPanel][kCholLd];      // the panel's rows of M, all columns
+    double D[kCholPanel][kCholLdP];      // the diagonal block, then its L
+    double Mq[kCholPanel][kCholLdP];     // the panel's rows of M before substitution, own columns
+    double dinv[kCholPanel];
+    double thresh;
+    int bad;
+};
+
+// 1/sqrt(d) for finite d > 0 with a short chain: FP32 estimate y (2^-22), then
+// y (1 + e / 2 + 3 e^2 / 8), e = 1 - d y^2, to beyond 53 bits; d scaled to [1, 4) by its bits.
+__device__ inline double rsqrt_fp64_short(double d) {
+    const int hi = __double2hiint(d);
+    const int ex = ((hi >> 20) - 1023) & ~1;
+    if ((hi >> 20) == 0) return rsqrt_fp64(d);  // subnormal
+    const double dd = __hiloint2double(hi - (ex << 20), __double2loint(d));
+    const double y = (double)rsqrtf((float)dd);
+    const double e = fma(-dd, y * y, 1.0);
+    const double z = fma(y * e, fma(e, 0.375, 0.5), y);
+    return __hiloint2double(__double2hiint(z) - ((ex >> 1) << 20), __double2loint(z));
+}
+
+__global__ void __cluster_dims__(kCholCluster, 1, 1) __launch_bounds__(256, 1)
     chol_inv_cluster_kernel(int b, const double* __restrict__ W, double* __restrict__ Lt, double* __restrict__ Mt,
                             int* status) {
     namespace cg = cooperative_groups;
-    constexpr int C = kCholCluster;
+    constexpr int C = kCholCluster, P = kCholPanel;
     cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)cl.block_rank();
-    extern __shared__ double sm[];
-    const int ld = b + 1;
-    double* A = sm;                     // lower: L; upper (transposed): own columns of L^{-1}
-    double* dinv = sm + (size_t)b * ld;  // 1 / L_jj
-    __shared__ double s_thresh;
-    __shared__ int s_bad;
-    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
-    for (int idx = tid; idx < b * b; idx += nt) {
-        const int i = idx / b, j = idx % b;
-        A[i * ld + j] = (j <= i) ? W[idx] : 0.0;
+    extern __shared__ __align__(16) unsigned char chol_raw[];
+    CholSmem& sm = *reinterpret_cast<CholSmem*>(chol_raw);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tr = tid >> 4, tx = tid & 15;       // own row and column group in the updates
+    const int ti = rank + C * tr;                 // that row
+    for (int idx = tid; idx < kCholRows * kCholLd; idx += 256) {
+        const int r = idx / kCholLd, k = idx % kCholLd, i = rank + C * r;
+        sm.A[r][k] = i < b && k <= i ? W[(size_t)i * b + k] : 0.0;
+        sm.M[r][k] = 0.0;
     }
-    __syncthreads();
-    if (tid < 32) {  // max of the diagonal and a non-finite flag, over warp 0
+    {
+        const int i = tid >> 4, k = tid & 15;  // b >= 64: the first block is whole
+        sm.D[i][k] = k <= i ? W[(size_t)i * b + k] : 0.0;
+        sm.Mq[i][k] = 0.0;
+    }
+    for (int row = rank; row < b; row += C)  // zeros left of the panel that holds the diagonal
+        for (int j = tid; j < row / P * P; j += 256) {
+            Lt[(size_t)row * b + j] = 0.0;
+            Mt[(size_t)row * b + j] = 0.0;
+        }
+    if (warp == 0) {  // max of the diagonal and a non-finite flag
         double wmax = 0.0;
         int bad = 0;
         for (int i = lane; i < b; i += 32) {
-            const double d = A[i * ld + i];
+            const double d = W[(size_t)i * b + i];
             if (!isfinite(d)) bad = 2;
             if (d > wmax) wmax = d;
         }
@@ -420,135 +459,125 @@ __global__ void __cluster_dims__(kCholCluster, 1, 1) __launch_bounds__(256)
         }
         if (lane == 0) {
             if (bad == 0 && !(wmax > 0.0)) bad = 1;
-            s_bad = bad;
-            s_thresh = (double)b * kEps * wmax;
+            sm.bad = bad;
+            sm.thresh = (double)b * kEps * wmax;
         }
     }
-    __syncthreads();
-    cl.sync();  // every copy is loaded before any CTA writes into another's
-    for (int p0 = 0; p0 < b; p0 += kCholPanel) {
-        if (s_bad) break;  // the same in every CTA
-        const int p1 = min(b, p0 + kCholPanel), pw = p1 - p0;
-        // 1. the diagonal block
-        if (tid < 32) {
-            for (int j = p0; j < p1; ++j) {
-                if (lane == 0) {
-                    const double d = A[j * ld + j];
-                    if (!isfinite(d) || !(d > s_thresh)) {
-                        s_bad = isfinite(d) ? 1 : 2;
-                    } else {
-                        const double y = rsqrt_fp64(d);
-                        A[j * ld + j] = d * y;
-                        dinv[j] = y;
-                    }
+    cl.sync();
+    int bad = sm.bad;  // the same in every CTA
+    for (int p0 = 0; p0 < b && bad == 0; p0 += P) {
+        const int p1 = p0 + P, pw = min(P, b - p0);
+        const int r1 = p1 / C;  // own rows from here on lie below the panel
+        if (warp == 0) {        // 1.
+            double v[P];
+            const int r = lane - 16;
+            const bool below = r >= r1 && rank + C * r < b;
+#pragma unroll
+            for (int k = 0; k < P; ++k) v[k] = lane < 16 ? sm.D[lane][k] : (below ? sm.A[max(r, 0)][p0 + k] : 0.0);
+            int wrong = 0;
+#pragma unroll
+            for (int j = 0; j < P; ++j) {
+                const double d = __shfl_sync(0xffffffffu, v[j], j);
+                if (j < pw && wrong == 0) {
+                    if (!isfinite(d) || !(d > sm.thresh)) wrong = isfinite(d) ? 1 : 2;
+                    const double y = wrong == 0 ? rsqrt_fp64_short(d) : 0.0;
+                    v[j] *= y;
+                    if (lane == 0) sm.dinv[j] = y;
+#pragma unroll
+                    for (int k = j + 1; k < P; ++k) v[k] = fma(-v[j], __shfl_sync(0xffffffffu, v[j], k), v[k]);
+                } else if (lane == 0) {
+                    sm.dinv[j] = 1.0;
                 }
-                __syncwarp();
-                if (s_bad) break;
-                const double inv = dinv[j];
-                for (int i = j + 1 + lane; i < p1; i += 32) A[i * ld + j] *= inv;
-                __syncwarp();
-                const int nn = p1 - j - 1;
-                for (int idx = lane; idx < nn * (nn + 1) / 2; idx += 32) {
-                    int ii, kk;
-                    tri_decode(idx, ii, kk);
-                    const int i = j + 1 + ii, k = j + 1 + kk;
-                    A[i * ld + k] = fma(-A[i * ld + j], A[k * ld + j], A[i * ld + k]);
-                }
-                __syncwarp();
+            }
+            if (lane == 0) sm.bad = wrong;
+            if (lane < 16) {
+#pragma unroll
+                for (int k = 0; k < P; ++k) sm.D[lane][k] = k <= lane ? v[k] : 0.0;
+            } else if (below) {
+#pragma unroll
+                for (int k = 0; k < P; ++k) sm.A[r][p0 + k] = v[k];
             }
         }
         __syncthreads();
-        if (s_bad) break;
-        // 2. this CTA's rows below the block (one thread a row), then every CTA's
-        //    copy of them (all threads, one remote store each)
-        const int first = p1 + ((rank - p1 % C) % C + C) % C;
-        const int nown = first < b ? (b - first + C - 1) / C : 0;
-        for (int i = first + C * tid; i < b; i += C * nt) {
-            double x[kCholPanel];
+        bad = sm.bad;
+        if (bad) break;
+        if (warp == 1 && lane < P) {  // 2.
+            const int c = rank + C * lane;
+            if (c < p1) {
+                double m[P];
 #pragma unroll
-            for (int l = 0; l < kCholPanel; ++l) {
-                if (l < pw) {
-                    double a = A[i * ld + p0 + l];
+                for (int i = 0; i < P; ++i) m[i] = c < p0 ? sm.Mq[i][lane] : (c - p0 == i ? 1.0 : 0.0);
 #pragma unroll
-                    for (int m = 0; m < l; ++m) a = fma(-x[m], A[(p0 + l) * ld + p0 + m], a);
-                    x[l] = a * dinv[p0 + l];
+                for (int j = 0; j < P; ++j) {
+                    m[j] *= sm.dinv[j];
+#pragma unroll
+                    for (int i = j + 1; i < P; ++i) m[i] = fma(-sm.D[i][j], m[j], m[i]);
                 }
-            }
 #pragma unroll
-            for (int l = 0; l < kCholPanel; ++l)
-                if (l < pw) A[i * ld + p0 + l] = x[l];
+                for (int i = 0; i < P; ++i) sm.Mq[i][lane] = m[i];
+            }
         }
         __syncthreads();
-        for (int idx = tid; idx < nown * pw * (C - 1); idx += nt) {
-            const int r = (rank + 1 + idx % (C - 1)) % C, rest = idx / (C - 1);
-            const int i = first + C * (rest / pw), col = p0 + rest % pw;
-            cl.map_shared_rank(A, r)[i * ld + col] = A[i * ld + col];
+        // 3. thread (tr, tx): entry tx of own row tr of L, and row tr of own column tx of M
+        if (tr >= r1 && ti < b) {
+            const double x = sm.A[tr][p0 + tx];
+#pragma unroll
+            for (int c = 0; c < C; ++c) cl.map_shared_rank(&sm.Lp[0][0], c)[ti * kCholLdP + tx] = x;
+            Lt[(size_t)(p0 + tx) * b + ti] = x;
         }
+        {
+            const int c = rank + C * tx;
+            if (c < p1 && c < b) {
+                const double x = sm.Mq[tr][tx];
+#pragma unroll
+                for (int u = 0; u < C; ++u) cl.map_shared_rank(&sm.Mp[0][0], u)[tr * kCholLd + c] = x;
+                if (p0 + tr < b) Mt[(size_t)c * b + p0 + tr] = x;
+            }
+        }
+        if (rank == 0 && tr < pw && tx < pw) Lt[(size_t)(p0 + tx) * b + p0 + tr] = sm.D[tr][tx];
+        if (p1 >= b) break;
         cl.sync();
-        // 3. rank-pw update of this CTA's rows i >= p1, columns p1 <= k <= i: 16
-        //    threads a row, each over k = p1 + (tid % 16) + 16 m
-        for (int t = tid / 16; t < nown; t += nt / 16) {
-            const int i = first + C * t;
-            double li[kCholPanel];
+        // 4.
+        if (tr >= r1 && ti < b) {
+            double li[P];
 #pragma unroll
-            for (int l = 0; l < kCholPanel; ++l) li[l] = l < pw ? A[i * ld + p0 + l] : 0.0;
-            for (int k = p1 + (tid % 16); k <= i; k += 16) {
+            for (int l = 0; l < P; ++l) li[l] = sm.A[tr][p0 + l];
+            for (int k = tx; k < p1; k += 16) {
                 double acc = 0.0;
 #pragma unroll
-                for (int l = 0; l < kCholPanel; ++l)
-                    if (l < pw) acc = fma(li[l], A[k * ld + p0 + l], acc);
-                A[i * ld + k] -= acc;
+                for (int l = 0; l < P; ++l) acc = fma(li[l], sm.Mp[l][k], acc);
+                sm.M[tr][k] -= acc;
+            }
+            for (int k = p1 + tx; k <= ti; k += 16) {
+                double acc = 0.0;
+#pragma unroll
+                for (int l = 0; l < P; ++l) acc = fma(li[l], sm.Lp[k][l], acc);
+                sm.A[tr][k] -= acc;
             }
         }
         __syncthreads();
-        // this CTA's rows of the next diagonal block into every other copy, one remote
-        // store per thread: (row t, column p1 + kk <= row, rank)
-        const int p2 = min(b, p1 + kCholPanel);
-        const int nnext = first < p2 ? (p2 - first + C - 1) / C : 0;
-        for (int idx = tid; idx < nnext * kCholPanel * (C - 1); idx += nt) {
-            const int r = (rank + 1 + idx % (C - 1)) % C, rest = idx / (C - 1);
-            const int i = first + C * (rest / kCholPanel), k = p1 + rest % kCholPanel;
-            if (k <= i) cl.map_shared_rank(A, r)[i * ld + k] = A[i * ld + k];
+        {  // the two own rows of the next panel
+            const int half = tid >> 7, e = tid & 127, r = r1 + half, i = rank + C * r;
+            const bool in = r < kCholRows && i < b;
+            // diagonal block: entry e / 8 for CTA e % 8
+            const int k = e >> 3;
+            if (r < kCholRows)
+                cl.map_shared_rank(&sm.D[0][0], e & 7)[(i - p1) * kCholLdP + k] = in && p1 + k <= i ? sm.A[r][p1 + k] : 0.0;
+            // M: column e to its owner
+            if (r < kCholRows && e < p1)
+                cl.map_shared_rank(&sm.Mq[0][0], e & 7)[(i - p1) * kCholLdP + (e >> 3)] = in ? sm.M[r][e] : 0.0;
         }
         cl.sync();
     }
-    if (s_bad) {
-        if (rank == 0 && tid == 0) atomicOr(&status[s_bad == 2 ? kStNonfinite : kStBreakdown], 1);
-        for (int idx = rank * nt + tid; idx < b * b; idx += C * nt) {
+    // (the copies of one's rows end at a barrier; after a last panel nobody writes to another CTA's
+    // memory but in step 3, so wait for that too)
+    cl.sync();
+    if (bad) {
+        if (rank == 0 && tid == 0) atomicOr(&status[bad == 2 ? kStNonfinite : kStBreakdown], 1);
+        for (int idx = rank * 256 + tid; idx < b * b; idx += C * 256) {
             const double v = (idx / b == idx % b) ? 1.0 : 0.0;
             Lt[idx] = v;
             Mt[idx] = v;
-        }
-        return;
-    }
-    // Lt = L^T (rows i = rank + C u)
-    for (int row = rank; row < b; row += C)
-        for (int j = tid; j < b; j += nt) Lt[(size_t)row * b + j] = (j >= row) ? A[j * ld + row] : 0.0;
-    // X = L^{-1}, column c = rank + C u by one warp (no barriers): forward substitution
-    // L x = e_c with the running sums of rows c + lane + 32 t in registers; x_k =
-    // acc_k / L_kk comes from the lane holding row k, then rows i > k take
-    // acc_i -= L[i][k] x_k.  Row c of Mt = L^{-T} is x (zero left of c).
-    constexpr int kRowsPerLane = TSVD_MAX_BLOCK / 32;
-    const int warp = tid >> 5, nwarps = nt >> 5;
-    for (int c = rank + C * warp; c < b; c += C * nwarps) {
-        double acc[kRowsPerLane];
-#pragma unroll
-        for (int t = 0; t < kRowsPerLane; ++t) acc[t] = (c + lane + 32 * t == c) ? 1.0 : 0.0;
-        double* mrow = Mt + (size_t)c * b;
-        for (int j = lane; j < c; j += 32) mrow[j] = 0.0;
-#pragma unroll
-        for (int tt = 0; tt < kRowsPerLane; ++tt) {
-            for (int ll = 0; ll < 32; ++ll) {
-                const int k = c + 32 * tt + ll;
-                if (k >= b) break;  // uniform over the warp
-                const double xk = __shfl_sync(0xffffffffu, acc[tt], ll) * dinv[k];
-                if (lane == 0) mrow[k] = xk;
-#pragma unroll
-                for (int t = tt; t < kRowsPerLane; ++t) {
-                    const int i = c + lane + 32 * t;
-                    if (i > k && i < b) acc[t] = fma(-A[i * ld + k], xk, acc[t]);
-                }
-            }
         }
     }
 }
@@ -974,17 +1003,17 @@ cudaError_t chol_inv(tsvd_handle* h, int b, const double* W, double* Lt, double*
     static thread_local int configured_device = -1;
     if (configured_device != h->device) {
         cudaError_t e = cudaFuncSetAttribute(chol_inv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)chol_smem(TSVD_MAX_BLOCK));
+                                             (int)chol_smem(kCholClusterMin - 1));
         if (e != cudaSuccess) return e;
         e = cudaFuncSetAttribute(chol_inv_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)chol_smem(TSVD_MAX_BLOCK));
+                                 (int)sizeof(CholSmem));
         if (e != cudaSuccess) return e;
         configured_device = h->device;
     }
     ProfScope prof(h, TSVD_K_CHOL, 2.0 * b * b * (double)b / 3.0, 24.0 * b * b, st);
     h->launches++;
     if (b >= kCholClusterMin)
-        chol_inv_cluster_kernel<<<kCholCluster, 256, smem, st>>>(b, W, Lt, Mt, status);
+        chol_inv_cluster_kernel<<<kCholCluster, 256, sizeof(CholSmem), st>>>(b, W, Lt, Mt, status);
     else
         chol_inv_kernel<<<1, 256, smem, st>>>(b, W, Lt, Mt, status);
     return cudaGetLastError();
