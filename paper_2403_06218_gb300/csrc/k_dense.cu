@@ -369,19 +369,23 @@ __global__ void __launch_bounds__(256) chol_inv_kernel(int b, const double* __re
 // [A | I], which leaves L^T's columns and M = L^{-1}, with the FP64 work spread over 8 SMs (one
 // SM's FP64 pipe, 2 DFMA/clk, bounds the one-CTA kernel above).  Row i belongs to CTA i mod 8,
 // column c of M's panel rows to CTA c mod 8.  Per panel of 16 columns:
-//   1. warp 0 of every CTA factors the 16 x 16 diagonal block, a row in the registers of each of
-//      lanes 0-15 (the same numbers and code in every CTA, so every CTA takes the same breakdown
-//      decision), while lanes 16-31 take its own 16 rows below through the same steps, which is
-//      their substitution L[i][P] = A[i][P] L11^{-T};
-//   2. warp 1 substitutes its own columns of the panel's rows of M, a column a lane;
+//   1. warps 0-3 of every CTA factor the 16 x 16 diagonal block, lanes 0-15 a row each and warp w
+//      columns w, w + 4, ... (the same numbers and code in every CTA, so every CTA takes the same
+//      breakdown decision), while lanes 16-31 take its own 16 rows below through the same steps,
+//      which is their substitution L[i][P] = A[i][P] L11^{-T}.  One CTA barrier a pivot; the next
+//      pivot's warp updates that column before its others;
+//   2. a step behind, warps 4-7 substitute the own columns of the panel's rows of M, a column a
+//      lane and rows w, w + 4, ... a warp;
 //   3. both go to every CTA (distributed shared memory); cluster barrier;
 //   4. rank-16 update of the own rows below, A[i][k] -= L[i][P] L[k][P]^T and M[i][c] -=
 //      L[i][P] M[P][c], 16 threads a row; the next panel's rows go out: its diagonal block to
 //      every CTA, its rows of M to their columns' owners; cluster barrier.
 // Bound by the chain of the pivots (16 steps of 1/sqrt, scale, update a panel) and, at b = 128,
-// by the FP64 pipe in the updates.  With the pivot steps through shared memory, a chain of 136
-// dependent FMAs a row for its substitution, and the inverse in a pass of its own at the end,
-// b = 128 took 296 us and b = 64 131 us.
+// by the FP64 pipe in the updates.  One warp has a quarter of the SM's FP64 pipe (64 clocks an
+// instruction), hence the four warps: with steps 1 and 2 in a warp each, b = 128 took 218 us and
+// b = 64 100 us (1,700 clocks a pivot); before, with the pivot steps through shared memory, a
+// chain of 136 dependent FMAs a row for its substitution and the inverse in a pass of its own,
+// 296 us and 131 us.
 // The updates sum 16 products per panel before subtracting (the one-CTA kernel subtracts them
 // one at a time), so results agree to rounding, not bits.
 // ---------------------------------------------------------------------------
@@ -399,19 +403,24 @@ struct CholSmem {
     double Mp[kCholPanel][kCholLd];      // the panel's rows of M, all columns
     double D[kCholPanel][kCholLdP];      // the diagonal block, then its L
     double Mq[kCholPanel][kCholLdP];     // the panel's rows of M before substitution, own columns
+    double col[3][32], mrow[2][kCholPanel];  // a pivot's column of L (16 + 16 rows), its row of M
     double dinv[kCholPanel];
     double thresh;
     int bad;
 };
 
-// 1/sqrt(d) for finite d > 0 with a short chain: FP32 estimate y (2^-22), then
-// y (1 + e / 2 + 3 e^2 / 8), e = 1 - d y^2, to beyond 53 bits; d scaled to [1, 4) by its bits.
+// 1/sqrt(d) for a normal finite d > 0 with a short chain on the FP64 pipe: FP32 estimate y
+// (2^-21) of d scaled to [1, 4), both conversions by bits, then y (1 + e / 2 + 3 e^2 / 8),
+// e = 1 - d y^2, to beyond 53 bits.
 __device__ inline double rsqrt_fp64_short(double d) {
-    const int hi = __double2hiint(d);
+    const int hi = __double2hiint(d), lo = __double2loint(d);
     const int ex = ((hi >> 20) - 1023) & ~1;
     if ((hi >> 20) == 0) return rsqrt_fp64(d);  // subnormal
-    const double dd = __hiloint2double(hi - (ex << 20), __double2loint(d));
-    const double y = (double)rsqrtf((float)dd);
+    const int h = hi - (ex << 20);  // exponent field 1023 or 1024
+    const double dd = __hiloint2double(h, lo);
+    const float f = __int_as_float(((h >> 20) - 896) << 23 | (h & 0xFFFFF) << 3 | (int)((unsigned)lo >> 29));
+    const int yb = __float_as_int(rsqrtf(f));  // in (1/2, 1]
+    const double y = __hiloint2double((yb >> 3) + (896 << 20), yb << 29);
     const double e = fma(-dd, y * y, 1.0);
     const double z = fma(y * e, fma(e, 0.375, 0.5), y);
     return __hiloint2double(__double2hiint(z) - ((ex >> 1) << 20), __double2loint(z));
@@ -468,56 +477,79 @@ __global__ void __cluster_dims__(kCholCluster, 1, 1) __launch_bounds__(256, 1)
     for (int p0 = 0; p0 < b && bad == 0; p0 += P) {
         const int p1 = p0 + P, pw = min(P, b - p0);
         const int r1 = p1 / C;  // own rows from here on lie below the panel
-        if (warp == 0) {        // 1.
-            double v[P];
+        const auto pivot_sync = [] { asm volatile("bar.sync 1, 256;" ::: "memory"); };  // from both branches
+        if (warp < 4) {         // 1.
+            double v[4];
             const int r = lane - 16;
             const bool below = r >= r1 && rank + C * r < b;
 #pragma unroll
-            for (int k = 0; k < P; ++k) v[k] = lane < 16 ? sm.D[lane][k] : (below ? sm.A[max(r, 0)][p0 + k] : 0.0);
-            int wrong = 0;
+            for (int t = 0; t < 4; ++t)
+                v[t] = lane < 16 ? sm.D[lane][warp + 4 * t] : (below ? sm.A[max(r, 0)][p0 + warp + 4 * t] : 0.0);
+            const auto pivot = [&](int j, double& x) {  // by the warp of column j
+                const double d = __shfl_sync(0xffffffffu, x, j);
+                double y = 1.0;
+                if (j < pw) {
+                    const bool finite = (__double2hiint(d) & 0x7FF00000) != 0x7FF00000;
+                    if (finite && __double_as_longlong(d) > __double_as_longlong(sm.thresh)) {  // both >= 0, or d < 0
+                        y = rsqrt_fp64_short(d);
+                    } else if (lane == 0 && sm.bad == 0) {
+                        sm.bad = finite ? 1 : 2;  // the steps run on: every warp comes to every barrier
+                    }
+                }
+                x *= y;
+                sm.col[j % 3][lane] = x;
+                if (lane == 0) sm.dinv[j] = y;
+            };
+            if (warp == 0) pivot(0, v[0]);
 #pragma unroll
             for (int j = 0; j < P; ++j) {
-                const double d = __shfl_sync(0xffffffffu, v[j], j);
-                if (j < pw && wrong == 0) {
-                    if (!isfinite(d) || !(d > sm.thresh)) wrong = isfinite(d) ? 1 : 2;
-                    const double y = wrong == 0 ? rsqrt_fp64_short(d) : 0.0;
-                    v[j] *= y;
-                    if (lane == 0) sm.dinv[j] = y;
+                pivot_sync();
+                const double l = sm.col[j % 3][lane];
+                const bool mine = warp == ((j + 1) & 3);
+                if (j + 1 < P && mine) {
+                    v[(j + 1) >> 2] = fma(-l, sm.col[j % 3][j + 1], v[(j + 1) >> 2]);
+                    pivot(j + 1, v[(j + 1) >> 2]);
+                }
 #pragma unroll
-                    for (int k = j + 1; k < P; ++k) v[k] = fma(-v[j], __shfl_sync(0xffffffffu, v[j], k), v[k]);
-                } else if (lane == 0) {
-                    sm.dinv[j] = 1.0;
+                for (int t = 0; t < 4; ++t)
+                    if (warp + 4 * t > j && !(mine && t == (j + 1) >> 2))
+                        v[t] = fma(-l, sm.col[j % 3][warp + 4 * t], v[t]);
+            }
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const int k = warp + 4 * t;
+                if (lane < 16)
+                    sm.D[lane][k] = k <= lane ? v[t] : 0.0;
+                else if (below)
+                    sm.A[r][p0 + k] = v[t];
+            }
+        } else {                // 2.
+            double m[4];
+            const int w = warp - 4, u = lane & 15, c = rank + C * u;
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+                m[t] = c < p0 ? sm.Mq[w + 4 * t][u] : (c - p0 == w + 4 * t ? 1.0 : 0.0);
+#pragma unroll
+            for (int j = 0; j < P; ++j) {
+                pivot_sync();
+                if (j > 0) {  // the update of pivot j - 1
+                    const double x = sm.mrow[(j - 1) & 1][u];
+#pragma unroll
+                    for (int t = 0; t < 4; ++t)
+                        if (w + 4 * t >= j) m[t] = fma(-sm.col[(j - 1) % 3][w + 4 * t], x, m[t]);
+                }
+                if (w == (j & 3)) {
+                    m[j >> 2] *= sm.dinv[j];
+                    if (lane < 16) sm.mrow[j & 1][u] = m[j >> 2];
                 }
             }
-            if (lane == 0) sm.bad = wrong;
-            if (lane < 16) {
+            if (lane < 16)
 #pragma unroll
-                for (int k = 0; k < P; ++k) sm.D[lane][k] = k <= lane ? v[k] : 0.0;
-            } else if (below) {
-#pragma unroll
-                for (int k = 0; k < P; ++k) sm.A[r][p0 + k] = v[k];
-            }
+                for (int t = 0; t < 4; ++t) sm.Mq[w + 4 * t][u] = m[t];
         }
         __syncthreads();
         bad = sm.bad;
         if (bad) break;
-        if (warp == 1 && lane < P) {  // 2.
-            const int c = rank + C * lane;
-            if (c < p1) {
-                double m[P];
-#pragma unroll
-                for (int i = 0; i < P; ++i) m[i] = c < p0 ? sm.Mq[i][lane] : (c - p0 == i ? 1.0 : 0.0);
-#pragma unroll
-                for (int j = 0; j < P; ++j) {
-                    m[j] *= sm.dinv[j];
-#pragma unroll
-                    for (int i = j + 1; i < P; ++i) m[i] = fma(-sm.D[i][j], m[j], m[i]);
-                }
-#pragma unroll
-                for (int i = 0; i < P; ++i) sm.Mq[i][lane] = m[i];
-            }
-        }
-        __syncthreads();
         // 3. thread (tr, tx): entry tx of own row tr of L, and row tr of own column tx of M
         if (tr >= r1 && ti < b) {
             const double x = sm.A[tr][p0 + tx];
