@@ -35,6 +35,10 @@ struct VecLoad<double, 2> {
         o[0] = v.x;
         o[1] = v.y;
     }
+    __device__ static void put(double* p, const double* v) {
+        p[0] = v[0];
+        p[1] = v[1];
+    }
 };
 template <>
 struct VecLoad<float, 4> {
@@ -45,81 +49,157 @@ struct VecLoad<float, 4> {
         o[2] = v.z;
         o[3] = v.w;
     }
+    __device__ static void put(float* p, const float* v) {
+        *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+    }
 };
 template <typename T>
 struct VecLoad<T, 1> {
     __device__ static void get(const T* p, T* o) { o[0] = __ldg(p); }
+    __device__ static void put(T* p, const T* v) { p[0] = v[0]; }
 };
 
 // One output row y = sum over the entries [beg, end) of a_e x_{col(e)}, written to
-// out[0 .. w), by a sub-warp of G lanes: lane sl owns VW consecutive columns of each
-// panel of VW G columns and gathers them with one vector load per entry (the
-// entry's (col, val) is read by all G lanes: a broadcast).  Each y_ij is
-// accumulated in CSR order with FMA, so the result is deterministic.
+// out[0 .. w) (nothing if out is null), by a sub-warp of G lanes: lane sl owns VW consecutive
+// columns of each panel of VW G columns.  Each y_ij is accumulated in CSR order with FMA, so the
+// result is deterministic.
+// FP32: the lanes read G entries' (col, val) at once and pass them around by shuffles, so that
+// four gathers are in flight; with one entry's column, value and gather after the other the kernel
+// waited for memory (500,000 x 250,000 power-law, 12 M entries, 100 columns: 1.39 ms, now 0.84).
+// FP64: one entry after the other; the FP64 pipe bounds that, and the shuffles only delay it
+// (100,000 rows of 10 entries, 128 columns: 325 us against 371 us).
 template <typename T, int VW, int G>
 __device__ inline void spmm_segment(int64_t beg, int64_t end, int64_t n, const int32_t* __restrict__ ci,
                                     const T* __restrict__ va, int w, const T* __restrict__ X, int64_t ldx,
                                     T* __restrict__ out, int* status, int sl) {
+    if constexpr (sizeof(T) == 8) {
+        if (!out) return;
+        for (int c0 = 0; c0 < w; c0 += VW * G) {
+            const int col = c0 + VW * sl;
+            if (col >= w) continue;  // lanes past the last column of a narrow panel
+            const bool full = col + VW <= w;
+            T acc[VW];
+#pragma unroll
+            for (int q = 0; q < VW; ++q) acc[q] = T(0);
+            for (int64_t e = beg; e < end; ++e) {
+                const int c = __ldg(ci + e);  // read by all G lanes: a broadcast
+                const T a = __ldg(va + e);
+                if ((uint64_t)(int64_t)c >= (uint64_t)n) {  // skipped, and reported
+                    if (sl == 0) atomicOr(&status[kStBadCsr], 1);
+                    continue;
+                }
+                const T* xr = X + (int64_t)c * ldx + col;
+                T x[VW];
+                if (full) {
+                    VecLoad<T, VW>::get(xr, x);
+                } else {
+#pragma unroll
+                    for (int q = 0; q < VW; ++q) x[q] = (col + q < w) ? __ldg(xr + q) : T(0);
+                }
+#pragma unroll
+                for (int q = 0; q < VW; ++q) acc[q] = fma(a, x[q], acc[q]);
+            }
+#pragma unroll
+            for (int q = 0; q < VW; ++q)
+                if (col + q < w) out[col + q] = acc[q];
+        }
+        return;
+    }
+    int len = (int)min((int64_t)INT_MAX, max((int64_t)0, end - beg));
+    if (G < 32) len = __reduce_max_sync(kFull, len);  // the warp's sub-warps stay together
     for (int c0 = 0; c0 < w; c0 += VW * G) {
         const int col = c0 + VW * sl;
-        if (col >= w) continue;  // lanes past the last column of a narrow panel
-        const bool full = col + VW <= w;
+        const int have = min(VW, w - col);  // columns of this lane (none or fewer past a panel's end)
         T acc[VW];
 #pragma unroll
         for (int q = 0; q < VW; ++q) acc[q] = T(0);
-        for (int64_t e = beg; e < end; ++e) {
-            const int c = __ldg(ci + e);
-            const T a = __ldg(va + e);
-            if ((uint64_t)(int64_t)c >= (uint64_t)n) {  // skipped, and reported
-                if (sl == 0) atomicOr(&status[kStBadCsr], 1);
-                continue;
+        for (int o = 0; o < len; o += G) {
+            int mc = -1;
+            T ma = T(0);
+            if (beg + o + sl < end) {
+                const int64_t e = beg + o + sl;
+                mc = __ldg(ci + e);
+                ma = __ldg(va + e);
+                if ((uint64_t)(int64_t)mc >= (uint64_t)n) {  // skipped, and reported
+                    atomicOr(&status[kStBadCsr], 1);
+                    mc = -1;
+                }
             }
-            const T* xr = X + (int64_t)c * ldx + col;
-            T x[VW];
-            if (full) {
-                VecLoad<T, VW>::get(xr, x);
-            } else {
+            __syncwarp();
+            const int cnt = min(G, len - o);
+            for (int t = 0; t < cnt; t += 4) {
+                int c[4];
+                T a[4], x[4][VW];
 #pragma unroll
-                for (int q = 0; q < VW; ++q) x[q] = (col + q < w) ? __ldg(xr + q) : T(0);
+                for (int u = 0; u < 4; ++u) {
+                    c[u] = __shfl_sync(kFull, mc, t + u, G);
+                    a[u] = __shfl_sync(kFull, ma, t + u, G);
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const T* xr = X + (int64_t)c[u] * ldx + col;
+                    if (c[u] >= 0 && have == VW) {
+                        VecLoad<T, VW>::get(xr, x[u]);
+                    } else {
+#pragma unroll
+                        for (int q = 0; q < VW; ++q) x[u][q] = c[u] >= 0 && q < have ? __ldg(xr + q) : T(0);
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    // an entry that is not there adds 0 * 0
+                    const T v = c[u] >= 0 ? a[u] : T(0);
+                    if (t + u < cnt)
+#pragma unroll
+                        for (int q = 0; q < VW; ++q) acc[q] = fma(v, x[u][q], acc[q]);
+                }
             }
-#pragma unroll
-            for (int q = 0; q < VW; ++q) acc[q] = fma(a, x[q], acc[q]);
         }
+        if (!out) continue;
+        if (VW * sizeof(T) == 16 && have == VW && (reinterpret_cast<uintptr_t>(out + col) & 15) == 0) {
+            VecLoad<T, VW>::put(out + col, acc);
+        } else {
 #pragma unroll
-        for (int q = 0; q < VW; ++q)
-            if (col + q < w) out[col + q] = acc[q];
+            for (int q = 0; q < VW; ++q)
+                if (q < have) out[col + q] = acc[q];
+        }
     }
 }
 
-// Sub-warp of G lanes per row; rows longer than `split` entries are left to the chunk kernels.
+// Sub-warp of G lanes per row or chunk.  The first blocks take the chunks of the rows longer than
+// `split` entries (a chunk: entries [rp[row] + j C, min(rp[row + 1], rp[row] + (j + 1) C)), into
+// partial[chunk][0 .. w)), so that they run beside the rows; the others the rows up to `split`.
 template <typename T, int VW, int G>
-__global__ void __launch_bounds__(256) spmm_rows_kernel(int64_t m, int64_t n, const int32_t* __restrict__ rp,
+__global__ void __launch_bounds__(256, sizeof(T) == 8 ? 6 : 0) spmm_rows_kernel(int64_t m, int64_t n, const int32_t* __restrict__ rp,
                                                         const int32_t* __restrict__ ci, const T* __restrict__ va,
                                                         int w, const T* __restrict__ X, int64_t ldx,
-                                                        T* __restrict__ Y, int64_t ldy, int64_t split, int* status) {
-    const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
-    const int sl = threadIdx.x % G;
-    if (row >= m) return;
-    const int64_t beg = rp[row], end = rp[row + 1];
-    if (end - beg > split) return;
-    spmm_segment<T, VW, G>(beg, end, n, ci, va, w, X, ldx, Y + row * ldy, status, sl);
-}
-
-// Sub-warp per chunk of a long row: entries [rp[row] + j C, min(rp[row + 1], rp[row] + (j+1) C))
-// into partial[chunk][0 .. w).
-template <typename T, int VW, int G>
-__global__ void __launch_bounds__(256) spmm_chunks_kernel(int64_t nchunks, const int4* __restrict__ chunks,
-                                                          int64_t n, const int32_t* __restrict__ rp,
-                                                          const int32_t* __restrict__ ci, const T* __restrict__ va,
-                                                          int w, const T* __restrict__ X, int64_t ldx,
-                                                          T* __restrict__ partial, int64_t ldp, int* status) {
-    const int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
-    const int sl = threadIdx.x % G;
-    if (c >= nchunks) return;
-    const int4 d = chunks[c];
-    const int64_t beg = (int64_t)rp[d.x] + (int64_t)d.y * kSpmmChunk;
-    const int64_t end = min((int64_t)rp[d.x + 1], beg + kSpmmChunk);
-    spmm_segment<T, VW, G>(beg, end, n, ci, va, w, X, ldx, partial + c * ldp, status, sl);
+                                                        T* __restrict__ Y, int64_t ldy, int64_t split,
+                                                        int64_t nchunks, const int4* __restrict__ chunks,
+                                                        T* __restrict__ partial, int64_t ldp, int* status) {
+    constexpr int per = 256 / G;
+    const int64_t cb = (nchunks + per - 1) / per;
+    const int sl = threadIdx.x % G, sub = threadIdx.x / G;
+    int64_t beg = 0, end = 0;
+    T* out = nullptr;
+    if ((int64_t)blockIdx.x < cb) {
+        const int64_t c = (int64_t)blockIdx.x * per + sub;
+        if (c < nchunks) {
+            const int4 d = chunks[c];
+            beg = (int64_t)rp[d.x] + (int64_t)d.y * kSpmmChunk;
+            end = min((int64_t)rp[d.x + 1], beg + kSpmmChunk);
+            out = partial + c * ldp;
+        }
+    } else {
+        const int64_t row = ((int64_t)blockIdx.x - cb) * per + sub;
+        if (row < m) {
+            beg = rp[row], end = rp[row + 1];
+            if (end - beg <= split)
+                out = Y + row * ldy;
+            else
+                end = beg;
+        }
+    }
+    spmm_segment<T, VW, G>(beg, end, n, ci, va, w, X, ldx, out, status, sl);
 }
 
 // Y[row] = sum of the row's chunk partials in chunk order (the first chunk's warp does the row).
@@ -416,14 +496,14 @@ template <typename T, int VW, int G>
 static void spmm_launch_all(int64_t m, int64_t n, const int32_t* rp, const int32_t* ci, const T* va, int w, const T* X,
                             int64_t ldx, T* Y, int64_t ldy, const SpmmPlan* plan, int* status, cudaStream_t st) {
     const bool split = plan && plan->nchunks > 0;
-    const int64_t per_block = 256 / G;
-    spmm_rows_kernel<T, VW, G><<<(unsigned)((m + per_block - 1) / per_block), 256, 0, st>>>(
-        m, n, rp, ci, va, w, X, ldx, Y, ldy, split ? (int64_t)kSpmmChunk : INT64_MAX, status);
-    if (!split) return;
-    T* part = static_cast<T*>(plan->partial);
+    const int64_t per_block = 256 / G, nchunks = split ? plan->nchunks : 0;
+    T* part = split ? static_cast<T*>(plan->partial) : nullptr;
     const int64_t ldp = spmm_partial_ld(w);
-    spmm_chunks_kernel<T, VW, G><<<(unsigned)((plan->nchunks + per_block - 1) / per_block), 256, 0, st>>>(
-        plan->nchunks, plan->chunks, n, rp, ci, va, w, X, ldx, part, ldp, status);
+    const int64_t blocks = (m + per_block - 1) / per_block + (nchunks + per_block - 1) / per_block;
+    spmm_rows_kernel<T, VW, G><<<(unsigned)blocks, 256, 0, st>>>(
+        m, n, rp, ci, va, w, X, ldx, Y, ldy, split ? (int64_t)kSpmmChunk : INT64_MAX, nchunks,
+        split ? plan->chunks : nullptr, part, ldp, status);
+    if (!split) return;
     spmm_chunk_sum_kernel<T><<<(unsigned)((plan->nchunks + 7) / 8), 256, 0, st>>>(plan->nchunks, plan->chunks, w,
                                                                                   part, ldp, Y, ldy);
 }
@@ -455,7 +535,7 @@ cudaError_t launch_spmm(tsvd_handle* h, int64_t m, int64_t n, int64_t nnz, const
                    (4.0 + es) * nnz + 4.0 * (m + 1) + es * (double)n * w + es * (double)m * w, st);
     // 16-byte gathers need 16-byte aligned X rows
     const bool v16 = (ldx * sizeof(T)) % 16 == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
-    h->launches += (plan && plan->nchunks > 0) ? 3 : 1;
+    h->launches += (plan && plan->nchunks > 0) ? 2 : 1;
     if (v16)
         spmm_dispatch<T, 16 / sizeof(T)>(m, n, row_ptr, col_idx, val, w, X, ldx, Y, ldy, plan, status, st);
     else
