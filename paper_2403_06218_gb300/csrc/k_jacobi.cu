@@ -261,13 +261,6 @@ __device__ inline bool rot_params(double al, double be, double ga, double tol2, 
     sn = c * t;
     return true;
 }
-template <typename T>
-__device__ inline T warp_sum_t(T v) {
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(kFull, v, d);
-    return v;
-}
-
 // Column stride (elements) of the block's columns in shared memory: odd, so that
 // the same row of different columns falls in different banks.
 __host__ __device__ inline int gram_ld(int n) { return n | 1; }
@@ -284,7 +277,7 @@ __host__ __device__ constexpr size_t gram_smem(int n) {
 template <typename T, int W>
 __device__ inline void gram_form(const T* cols, int n, int ld, T (*M)[2 * W + 1]) {
     constexpr int W2 = 2 * W;
-    constexpr int TM = W2 >= 32 ? 8 : (W2 >= 8 ? 4 : 2);
+    constexpr int TM = W2 >= 8 ? 4 : 2;
     constexpr int NTS = W2 / TM;
     constexpr int NT = NTS * (NTS + 1) / 2;
     constexpr int S0 = kJGThreads / NT;
@@ -338,8 +331,7 @@ __device__ inline void gram_form(const T* cols, int n, int ld, T (*M)[2 * W + 1]
         }
 }
 
-// Row stride of Z: 16-byte rows, so that the C Z products read a row of Z four
-// floats (two doubles) at a time.
+// Row stride of Z: 16-byte rows, so that the C Z products read a row of Z two doubles at a time.
 template <typename T, int W>
 __host__ __device__ constexpr int gram_zs() {
     return 2 * W + (int)(16 / sizeof(T));
@@ -349,16 +341,7 @@ __host__ __device__ constexpr int gram_zs() {
 // to the warp).
 template <typename T, int W2>
 __device__ inline void gram_axpy_row(T x, const T* zk, T* acc) {
-    if constexpr (sizeof(T) == 4 && W2 % 4 == 0) {
-#pragma unroll
-        for (int j = 0; j < W2; j += 4) {
-            const float4 z = *reinterpret_cast<const float4*>(zk + j);
-            acc[j] = fma(x, (T)z.x, acc[j]);
-            acc[j + 1] = fma(x, (T)z.y, acc[j + 1]);
-            acc[j + 2] = fma(x, (T)z.z, acc[j + 2]);
-            acc[j + 3] = fma(x, (T)z.w, acc[j + 3]);
-        }
-    } else if constexpr (sizeof(T) == 8 && W2 % 2 == 0) {
+    if constexpr (W2 % 2 == 0) {
 #pragma unroll
         for (int j = 0; j < W2; j += 2) {
             const double2 z = *reinterpret_cast<const double2*>(zk + j);
@@ -516,10 +499,9 @@ __device__ inline bool gram_rounds_ij(T (*M)[2 * W + 1], T (*Z)[gram_zs<T, W>()]
 
 template <typename T, int W>
 __global__ void __launch_bounds__(kJGThreads, 1) jacobi_gram_kernel(int n, int npad, T* __restrict__ G,
-                                                                 T* __restrict__ V, unsigned* ctl, T tol,
-                                                                 long long max_wait) {
+                                                                 unsigned* ctl, T tol, long long max_wait) {
     constexpr int W2 = 2 * W;
-    static_assert(W2 <= 32 && (W == 1 || W % 2 == 0), "block width: 1 or even, at most 16");
+    static_assert(W2 <= 16 && (W == 1 || W % 2 == 0), "block width: 1 or even, at most 8");
     extern __shared__ __align__(16) unsigned char jsm_raw[];
     T* cols = reinterpret_cast<T*>(jsm_raw);  // 2W columns, stride ld
     __shared__ T M[W2][W2 + 1];
@@ -588,23 +570,6 @@ __global__ void __launch_bounds__(kJGThreads, 1) jacobi_gram_kernel(int n, int n
                     }
 #pragma unroll
                     for (int j = 0; j < W2; ++j) G[(int64_t)(j < W ? bi * W + j : bj * W + (j - W)) * n + r] = acc[j];
-                }
-                if (V) {
-                    // accumulated rotations (npad x npad, column-major): V <- V Z on the
-                    // block pair's columns, read from global memory row by row
-                    for (int r = threadIdx.x; r < npad; r += blockDim.x) {
-                        T acc[W2];
-#pragma unroll
-                        for (int j = 0; j < W2; ++j) acc[j] = T(0);
-#pragma unroll 4
-                        for (int k = 0; k < W2; ++k) {
-                            const T x = V[(int64_t)(k < W ? bi * W + k : bj * W + (k - W)) * npad + r];
-                            gram_axpy_row<T, W2>(x, Z[k], acc);
-                        }
-#pragma unroll
-                        for (int j = 0; j < W2; ++j)
-                            V[(int64_t)(j < W ? bi * W + j : bj * W + (j - W)) * npad + r] = acc[j];
-                    }
                 }
             }
             if (!grid_sync(ctl, max_wait, epoch)) return;
@@ -1312,7 +1277,7 @@ static int jacobi_grid(const tsvd_handle* h, int npairs, int& block) {
 // Cooperative launch of the block-Jacobi sweeps on G (n x npad, column-major) in T
 // with blocks of W columns.
 template <typename T, int W>
-static int launch_gram(tsvd_handle* h, int n, int npad, T* G, unsigned* ctl, T tol, cudaStream_t st, T* V) {
+static int launch_gram(tsvd_handle* h, int n, int npad, T* G, unsigned* ctl, T tol, cudaStream_t st) {
     const int nb = npad / W / 2;
     const size_t smem = gram_smem<T, W>(n);
     static thread_local int configured = -1;
@@ -1327,7 +1292,7 @@ static int launch_gram(tsvd_handle* h, int n, int npad, T* G, unsigned* ctl, T t
     int nn = n, np = npad;
     T t = tol;
     long long mw = h->max_wait;
-    void* args[] = {(void*)&nn, (void*)&np, (void*)&G, (void*)&V, (void*)&ctl, (void*)&t, (void*)&mw};
+    void* args[] = {(void*)&nn, (void*)&np, (void*)&G, (void*)&ctl, (void*)&t, (void*)&mw};
     h->launches++;
     TSVD_TRY_CUDA(cudaLaunchCooperativeKernel((const void*)jacobi_gram_kernel<T, W>, dim3(nb), dim3(kJGThreads), args,
                                               smem, st));
@@ -1335,13 +1300,12 @@ static int launch_gram(tsvd_handle* h, int n, int npad, T* G, unsigned* ctl, T t
 }
 
 template <typename T>
-static int run_block_sweeps(tsvd_handle* h, int n, int npad, int w, T* G, unsigned* ctl, T tol, cudaStream_t st,
-                            T* V = nullptr) {
+static int run_block_sweeps(tsvd_handle* h, int n, int npad, int w, T* G, unsigned* ctl, T tol, cudaStream_t st) {
     switch (w) {
-        case 1: return launch_gram<T, 1>(h, n, npad, G, ctl, tol, st, V);
-        case 2: return launch_gram<T, 2>(h, n, npad, G, ctl, tol, st, V);
-        case 4: return launch_gram<T, 4>(h, n, npad, G, ctl, tol, st, V);
-        case 8: return launch_gram<T, 8>(h, n, npad, G, ctl, tol, st, V);
+        case 1: return launch_gram<T, 1>(h, n, npad, G, ctl, tol, st);
+        case 2: return launch_gram<T, 2>(h, n, npad, G, ctl, tol, st);
+        case 4: return launch_gram<T, 4>(h, n, npad, G, ctl, tol, st);
+        case 8: return launch_gram<T, 8>(h, n, npad, G, ctl, tol, st);
         default: return TSVD_ERR_UNSUPPORTED;
     }
 }
