@@ -7,13 +7,15 @@
 // Rayleigh-Ritz step relies on).
 //
 // Kernel structure (sm_103a, one CTA per SM, 320 threads):
-//   warp 0     TMA producer: per 32-wide K block, one 3-D box of the three A
+//   warp 0     TMA producer: per 64-wide K block, one 3-D box of the three A
 //              pieces (128 rows) and one of the three X^T pieces (Npad rows),
-//              64-byte swizzled, into a 4-stage ring (48 KB a stage) guarded
-//              by mbarriers;
+//              128-byte swizzled, into a 2-stage ring (96 KB a stage) guarded
+//              by mbarriers (boxes 32 wide in 4 stages have twice as many and
+//              shorter runs; with the fix-up below 0.56 against 0.545 ms for a
+//              20,000^2 x 128 product);
 //   warp 1     owns the TMEM allocation (256 columns: two 128 x Npad FP32
 //              accumulators) and issues tcgen05.mma (M = 128, N = Npad, K = 16,
-//              BF16 x BF16 -> FP32) from one thread, 12 per K block.  Each
+//              BF16 x BF16 -> FP32) from one thread, 24 per K block.  Each
 //              accumulation covers only kTcChunk K blocks (48 MMAs), alternating
 //              between the two accumulators;
 //   warps 2-9  epilogue: tcgen05.ld of each finished accumulator (two warps per
@@ -47,14 +49,14 @@ namespace tsvd {
 namespace {
 
 constexpr int kTcM = 128;                          // A rows per tile = TMEM lanes
-constexpr int kTcBK = 32;                          // K per stage: 32 BF16 = one 64-byte row
+constexpr int kTcBK = 64;                          // K per stage: 64 BF16 = one 128-byte row
 constexpr int kTcRowB = kTcBK * 2;                 // bytes of one tile row
-constexpr int kTcStages = 4;
-constexpr int kTcPieceA = kTcM * kTcRowB;          // one A piece per stage: 8 KB
+constexpr int kTcStages = 2;
+constexpr int kTcPieceA = kTcM * kTcRowB;          // one A piece per stage: 16 KB
 constexpr int kTcMaxN = 128;
-constexpr int kTcStageBytes = 3 * kTcPieceA + 3 * kTcMaxN * kTcRowB;  // 48 KB
+constexpr int kTcStageBytes = 3 * kTcPieceA + 3 * kTcMaxN * kTcRowB;  // 96 KB
 constexpr int kTcSmem = kTcStages * kTcStageBytes + 1024;               // + alignment slack
-constexpr int kTcChunk = 4;                         // K blocks per tensor-memory accumulation
+constexpr int kTcChunk = 2;                         // K blocks per tensor-memory accumulation
 constexpr int kTcEpiWarps = 8;                      // two per TMEM lane quarter, half the columns each
 constexpr int kTcThreads = 64 + 32 * kTcEpiWarps;
 constexpr int kTcWave = 152;
@@ -118,20 +120,20 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     const uint32_t stage_tx = (uint32_t)(3 * kTcPieceA + 3 * Npad * kTcRowB);
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             // ---- TMA producer
-            int64_t it = 0;
+            int64_t it = 0, t = lo / KB, kb = lo - t * KB;
             bool ok = true;
             for (int64_t i = lo; i < hi && ok; ++i, ++it) {
                 const int st = (int)(it % kTcStages);
                 if (it >= kTcStages) ok = mbar_wait(empty(st), (uint32_t)(((it / kTcStages) - 1) & 1), abort_flag, max_wait);
                 if (!ok) break;
-                const int64_t t = i / KB;
-                const int kx = (int)((i - t * KB) * kTcBK);
+                const int kx = (int)(kb * kTcBK);
                 const uint32_t sA = base + (uint32_t)st * kTcStageBytes;
                 mbar_arrive_expect_tx(full(st), stage_tx);
                 tma_load_3d(sA, &tmA, kx, (int)(t * kTcM), 0, full(st));
                 tma_load_3d(sA + 3 * kTcPieceA, &tmX, kx, 0, 0, full(st));
+                if (++kb == KB) kb = 0, ++t;
             }
             if (!ok) {
                 atomicOr(&status[kStTimeout], 1);
@@ -147,7 +149,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         }
         __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             // ---- MMA issuer: one accumulation per chunk of kTcChunk K blocks, alternating
             // between the two accumulators so that the epilogue drains one while the
             // other fills
@@ -181,9 +183,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                         for (int kk = 0; kk < kTcBK / 16; ++kk) {
 #pragma unroll
                             for (int tm = 0; tm < 6; ++tm) {
-                                const uint64_t ad = sdesc_sw64(sA + (uint32_t)(kTermA[tm] * kTcPieceA + kk * 32));
+                                const uint64_t ad = sdesc_sw128(sA + (uint32_t)(kTermA[tm] * kTcPieceA + kk * 32));
                                 const uint64_t bd =
-                                    sdesc_sw64(sX + (uint32_t)(kTermX[tm] * Npad * kTcRowB + kk * 32));
+                                    sdesc_sw128(sX + (uint32_t)(kTermX[tm] * Npad * kTcRowB + kk * 32));
                                 mma_bf16(d, ad, bd, idesc, acc);
                                 acc = 1;
                             }
@@ -266,8 +268,11 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     }
 }
 
-// Y[t*128 + r][col] = sum over the CTAs covering tile t (in CTA order) of their partial tile.
-__global__ void tc_fixup_kernel(int64_t M, int w, int Npad, int64_t KB, int64_t total, int G, int maxseg,
+// Y[t*128 + r][col] = sum over the CTAs covering tile t (in CTA order) of their partial tile; a block
+// takes 32 rows (a block for 256 elements, each finding its CTAs by 64-bit divisions, took 32 us at
+// 20,000 x 128).
+constexpr int kTcFixRows = 32;
+__global__ void __launch_bounds__(256) tc_fixup_kernel(int64_t M, int w, int Npad, int64_t KB, int64_t total, int G, int maxseg,
                                 const float* __restrict__ partial, float* __restrict__ Y, int64_t ldy) {
     __shared__ int s_c0, s_c1;
     const int64_t t = blockIdx.y;
@@ -282,17 +287,16 @@ __global__ void tc_fixup_kernel(int64_t M, int w, int Npad, int64_t KB, int64_t 
         s_c1 = cta_of((t + 1) * KB - 1);
     }
     __syncthreads();
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (int64_t)kTcM * w) return;
-    const int r = (int)(idx / w), col = (int)(idx % w);
-    const int64_t row = t * kTcM + r;
-    if (row >= M) return;
-    float acc = 0.f;
-    for (int cc = s_c0; cc <= s_c1; ++cc) {
-        const int seg = (int)(t - tc_lo(cc, total, G) / KB);
-        acc += partial[((int64_t)(cc * maxseg + seg) * kTcM + r) * Npad + col];
+    const int r0 = (int)blockIdx.x * kTcFixRows, rows = (int)min((int64_t)kTcFixRows, M - t * kTcM - r0);
+    // the first CTA of the tile may come from an earlier one; the others begin with this tile
+    const int64_t first = ((int64_t)s_c0 * maxseg + (t - tc_lo(s_c0, total, G) / KB)) * kTcM;
+#pragma unroll 4
+    for (int idx = threadIdx.x; idx < rows * w; idx += 256) {
+        const int r = r0 + idx / w, col = idx % w;
+        float acc = partial[(first + r) * Npad + col];
+        for (int cc = s_c0 + 1; cc <= s_c1; ++cc) acc += partial[((int64_t)cc * maxseg * kTcM + r) * Npad + col];
+        Y[(t * kTcM + r) * ldy + col] = acc;
     }
-    Y[row * ldy + col] = acc;
 }
 
 // Three-way BF16 split: p0 = bf16(v), p1 = bf16(v - p0), p2 = bf16(v - p0 - p1), to 2^-27 of
@@ -370,7 +374,7 @@ __global__ void __launch_bounds__(256) split3_kernel(int64_t rows, int64_t cols,
 }
 
 // ---- host side ---------------------------------------------------------------
-// 3-D map over pieces [3][rows][ld] (BF16), box 32 (K) x box_rows x 3, 64-byte swizzle.
+// 3-D map over pieces [3][rows][ld] (BF16), box 64 (K) x box_rows x 3, 128-byte swizzle.
 bool make_map(CUtensorMap* map, const void* base, int64_t cols, int64_t rows, int64_t ld, int box_rows) {
     return make_plane_map(map, base, cols, rows, ld, box_rows, 3);
 }
@@ -456,7 +460,7 @@ cudaError_t tc_mm(tsvd_handle* h, int64_t rows, int64_t cols, const void* pieces
                                                             status, h->max_wait);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
-        const dim3 fg((unsigned)((kTcM * wp + 255) / 256), (unsigned)p.tiles);
+        const dim3 fg((unsigned)(kTcM / kTcFixRows), (unsigned)p.tiles);
         tc_fixup_kernel<<<fg, 256, 0, st>>>(rows, wp, np, p.kb, p.total, p.ctas, p.maxseg, part, Y + c0, ldy);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
@@ -483,14 +487,14 @@ EncodeTiledFn encode_fn() {
 bool make_plane_map(CUtensorMap* map, const void* base, int64_t cols, int64_t rows, int64_t ld, int box_rows,
                     int planes, int box_k, int64_t pstride) {
     EncodeTiledFn fn = encode_fn();
-    if (!fn || (box_k != 32 && box_k != 16)) return false;
+    if (!fn || (box_k != 64 && box_k != 16)) return false;
     if (pstride < 0) pstride = ld * rows;
     const cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)planes};
     const cuuint64_t strides[2] = {(cuuint64_t)ld * 2, (cuuint64_t)pstride * 2};
     const cuuint32_t box[3] = {(cuuint32_t)box_k, (cuuint32_t)box_rows, (cuuint32_t)planes};
     const cuuint32_t estr[3] = {1, 1, 1};
     return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, box_k == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, box_k == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_32B,
               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 

@@ -91,14 +91,15 @@ __device__ inline void tma_load_3d(uint32_t dst, const CUtensorMap* map, int x, 
 __device__ inline void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ inline void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// Shared-memory matrix descriptor: K-major operand, 64-byte swizzle, rows of
-// 64 bytes, 8-row groups 512 bytes apart (tile base 512-byte aligned).
-__device__ inline uint64_t sdesc_sw64(uint32_t addr) {
+// Shared-memory matrix descriptor: K-major operand, 128-byte swizzle, rows of
+// 128 bytes, 8-row groups 1,024 bytes apart (tile base 1,024-byte aligned); the next
+// K = 16 of a row starts 32 bytes further on.
+__device__ inline uint64_t sdesc_sw128(uint32_t addr) {
     return (uint64_t)((addr >> 4) & 0x3FFFu)  // start address / 16
            | ((uint64_t)1 << 16)              // leading byte offset (unused for swizzled K-major)
-           | ((uint64_t)(512 >> 4) << 32)     // stride byte offset: 8 rows x 64 B
+           | ((uint64_t)(1024 >> 4) << 32)    // stride byte offset: 8 rows x 128 B
            | ((uint64_t)1 << 46)              // descriptor version of tcgen05
-           | ((uint64_t)4 << 61);             // swizzle mode: 64 B
+           | ((uint64_t)2 << 61);             // swizzle mode: 128 B
 }
 
 // The same for rows of 32 bytes (16 BF16) with 32-byte swizzle: 8-row groups 256
@@ -178,11 +179,11 @@ EncodeTiledFn encode_fn();
 
 // 3-D map over `planes` BF16 matrices stored [planes][rows][ld] (ld in elements,
 // a multiple of 8), K extent `cols`; box box_k (K) x box_rows x planes with a
-// swizzle of 2 box_k bytes (box_k = 32: 64-byte swizzle, 16: 32-byte swizzle).
+// swizzle of 2 box_k bytes (box_k = 64: 128-byte swizzle, 16: 32-byte swizzle).
 // Loads beyond `cols` or `rows` read zeros.
 // pstride: elements between planes (default rows x ld).
 bool make_plane_map(CUtensorMap* map, const void* base, int64_t cols, int64_t rows, int64_t ld, int box_rows,
-                    int planes, int box_k = 32, int64_t pstride = -1);
+                    int planes, int box_k = 64, int64_t pstride = -1);
 
 }  // namespace tcx
 }  // namespace tsvd
