@@ -382,8 +382,8 @@ __global__ void __launch_bounds__(256) chol_inv_kernel(int b, const double* __re
 //      every CTA, its rows of M to their columns' owners; cluster barrier.
 // Bound by the chain of the pivots (16 steps of 1/sqrt, scale, update a panel) and, at b = 128,
 // by the FP64 pipe in the updates.  One warp has a quarter of the SM's FP64 pipe (64 clocks an
-// instruction), hence the four warps: with steps 1 and 2 in a warp each, b = 128 took 218 us and
-// b = 64 100 us (1,700 clocks a pivot); before, with the pivot steps through shared memory, a
+// instruction), hence the four warps: b = 128 takes 133 us and b = 64 56 us; with steps 1 and 2 in
+// a warp each they took 218 us and 100 us (1,700 clocks a pivot); before, with the pivot steps through shared memory, a
 // chain of 136 dependent FMAs a row for its substitution and the inverse in a pass of its own,
 // 296 us and 131 us.
 // The updates sum 16 products per panel before subtracting (the one-CTA kernel subtracts them

@@ -600,8 +600,9 @@ __global__ void __launch_bounds__(kJGThreads, 1) jacobi_gram_kernel(int n, int n
 // mini-round to the next, columns q move by one position between lanes and rows q through
 // shared memory.
 // Bound by the latency of that chain (16 mini-rounds a round, 15 more in a sweep's first) and
-// of the round's loads, cluster exchange and barrier.  One CTA a block pair, with the rotations
-// in the registers of one warp, held 16 SMs at order 512 and took 13.8 ms.
+// of the round's loads, cluster exchange and barrier: 24,000 clocks a round, 10,400 of them the
+// rotations, 3.1 ms at order 512.  One CTA a block pair, with the rotations in the registers of one
+// warp, held 16 SMs and took 13.8 ms.
 constexpr int kJ32W = 16;          // columns of a block
 constexpr int kJ32Ld = 36;         // row stride (floats) of the 32 columns and of Z: float4 rows
 constexpr int kJ32LdM = 48;        // of M: consecutive rows half the banks apart
