@@ -648,6 +648,10 @@ __device__ inline bool rot32(float al, float be, float ga, float tol2, float& c,
 
 enum J32State : int { kJ32Go = 0, kJ32Done = 1, kJ32Fail = 2 };
 
+// The two halves of a cluster barrier (every thread of every CTA; a release and an acquire).
+__device__ inline void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ inline void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
 __host__ __device__ inline size_t j32_smem(int n, int npad, int C) {
     return sizeof(float) * kJ32Ld * (size_t)((n + C - 1) / C + (npad + C - 1) / C);
 }
@@ -675,7 +679,7 @@ __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(kJ32Threads, 2)
     __shared__ __align__(16) float s_in[C][kJ32Tri];             // and of the cluster's CTAs
     __shared__ __align__(16) float M[32][kJ32LdM], Z[32][kJ32Ld];
     __shared__ float2 s_cs[kJ32W];
-    __shared__ int s_state[2][C], s_ok;
+    __shared__ int s_state[C], s_ok;
     float(*s_q)[2][kJ32W][kJ32W] = reinterpret_cast<float(*)[2][kJ32W][kJ32W]>(&s_part[0][0]);  // rows q, twice
     static_assert(4 * kJ32W * kJ32W <= kJ32Slices * kJ32Tri, "the rotations' exchange fits the partial sums");
     const int tid = threadIdx.x;
@@ -696,11 +700,12 @@ __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(kJ32Threads, 2)
     int ti = 0, tj = tid % kJ32Tiles;
     while (tj >= 8 - ti) tj -= 8 - ti, ++ti;
     tj += ti;
-    int state = kJ32Go, sweeps = kMaxSweeps, parity = 0;
+    int state = kJ32Go, sweeps = kMaxSweeps;
+    bool pending = false;  // an arrival at the cluster barrier that has not been waited for
     unsigned epoch = 0;
     for (int sweep = 0; sweep < kMaxSweeps; ++sweep) {
         bool again = false;
-        for (int rnd = 0; rnd < nblk - 1; ++rnd, parity ^= 1) {
+        for (int rnd = 0; rnd < nblk - 1; ++rnd) {
             const int bi = rr_player(pair, rnd, nblk), bj = rr_player(nblk - 1 - pair, rnd, nblk);
             const int col = q4 < kJ32W ? bi * kJ32W + q4 : bj * kJ32W + q4 - kJ32W;
 #pragma unroll 4
@@ -727,6 +732,9 @@ __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(kJ32Threads, 2)
                         make_float4(acc[a][0], acc[a][1], acc[a][2], acc[a][3]);
             }
             __syncthreads();
+            // the cluster's CTAs have read what the round before put into s_in and s_state (the
+            // barrier that ends a round joins CTAs of different clusters and does not say so)
+            if (pending) cluster_wait();
             if (tid < kJ32Tri / 4) {
                 float4 t = *reinterpret_cast<const float4*>(&s_part[0][4 * tid]);
 #pragma unroll
@@ -738,7 +746,7 @@ __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(kJ32Threads, 2)
                 for (int c = 0; c < C; ++c)
                     *reinterpret_cast<float4*>(cl.map_shared_rank(&s_in[rank][4 * tid], c)) = t;
             } else if (tid < kJ32Tri / 4 + C) {
-                *cl.map_shared_rank(&s_state[parity][rank], tid - kJ32Tri / 4) = state;
+                *cl.map_shared_rank(&s_state[rank], tid - kJ32Tri / 4) = state;
             }
             cl.sync();
             if (tid < kJ32Tri / 4) {
@@ -762,13 +770,15 @@ __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(kJ32Threads, 2)
                 }
             }
             // A CTA whose barrier timed out, or that saw a last sweep, leaves together with its
-            // cluster: no shared memory is written after its CTA has left.  (Two sets of state
-            // words: a CTA may be a round ahead of one that still reads.)
-            const int fail = __syncthreads_or(tid < C && s_state[parity][tid] == kJ32Fail);
-            if (fail || state == kJ32Done) {
+            // cluster (every CTA of which reads the same words): no shared memory is written
+            // after its CTA has left.
+            if (__syncthreads_or(tid < C && s_state[tid] != kJ32Go)) {
                 sweeps = sweep;
+                pending = false;
                 goto out;
             }
+            cluster_arrive();  // s_in and s_state have been read
+            pending = true;
             bool any = false;
             float zp[2], zq[2];  // rows k and k + 16 of Z at columns p and q of pair l
 #pragma unroll
@@ -897,6 +907,7 @@ __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(kJ32Threads, 2)
     }
 out:
     if (blockIdx.x == 0 && tid == 0) ctl[kCtlSweeps] = (unsigned)sweeps;
+    if (pending) cluster_wait();
     cl.sync();
 }
 
