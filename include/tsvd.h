@@ -193,6 +193,12 @@ int tsvd_destroy(tsvd_handle* h);
  * handle. */
 int tsvd_set_wait_limit(tsvd_handle* h, long long cycles);
 
+/* Largest thread-block cluster (8, 4 or 2 CTAs; 0 restores 8) that the small SVD's FP32
+ * sweeps take a pair of column blocks with.  They take the largest one of which the device
+ * holds enough at once; this is a test hook that reaches the smaller ones on any device.
+ * Results agree to rounding.  TSVD_ERR_INVALID_ARG for a NULL handle or another value. */
+int tsvd_set_svd_cluster(tsvd_handle* h, int ctas);
+
 /* Row-partitioned LancSVD (Alg. 2 with the rows of A, and of the left basis Pbar,
  * split over processes; Sec. 3.2's CholeskyQR2 exchanges only b x b Gram matrices).
  * After this call tsvd_blanczos on this handle treats its matrix argument A (m x n,

@@ -64,6 +64,20 @@ def wait_limit(cycles: int, device=None):
         capi.check(lib.tsvd_set_wait_limit(h, 0), "tsvd_set_wait_limit")
 
 
+@contextlib.contextmanager
+def svd_cluster(ctas: int, device=None):
+    """Within the block, the FP32 sweeps of the small SVDs run through this device's handle
+    share a pair of column blocks over clusters of at most ``ctas`` (8, 4 or 2) CTAs (a test
+    hook).  The default of 8 is restored on exit."""
+    lib = capi.load()
+    h = handle(device)
+    capi.check(lib.tsvd_set_svd_cluster(h, int(ctas)), "tsvd_set_svd_cluster")
+    try:
+        yield
+    finally:
+        capi.check(lib.tsvd_set_svd_cluster(h, 0), "tsvd_set_svd_cluster")
+
+
 def _stream_ptr(device) -> int:
     return torch.cuda.current_stream(device).cuda_stream
 

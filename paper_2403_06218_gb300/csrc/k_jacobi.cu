@@ -1358,8 +1358,8 @@ static int launch_jacobi32(tsvd_handle* h, int n, int npad, float* G, float* V, 
 static int run_jacobi32(tsvd_handle* h, int n, int npad, float* G, float* V, unsigned* ctl, float tol,
                         cudaStream_t st) {
     bool fits = false;
-    TSVD_TRY(launch_jacobi32<8>(h, n, npad, G, V, ctl, tol, st, fits));
-    if (!fits) TSVD_TRY(launch_jacobi32<4>(h, n, npad, G, V, ctl, tol, st, fits));
+    if (h->svd_cluster >= 8) TSVD_TRY(launch_jacobi32<8>(h, n, npad, G, V, ctl, tol, st, fits));
+    if (!fits && h->svd_cluster >= 4) TSVD_TRY(launch_jacobi32<4>(h, n, npad, G, V, ctl, tol, st, fits));
     if (!fits) TSVD_TRY(launch_jacobi32<2>(h, n, npad, G, V, ctl, tol, st, fits));
     return fits ? TSVD_OK : TSVD_ERR_UNSUPPORTED;
 }

@@ -207,6 +207,12 @@ int tsvd_set_wait_limit(tsvd_handle* h, long long cycles) {
     return TSVD_OK;
 }
 
+int tsvd_set_svd_cluster(tsvd_handle* h, int ctas) {
+    if (!h || (ctas != 0 && ctas != 2 && ctas != 4 && ctas != 8)) return TSVD_ERR_INVALID_ARG;
+    h->svd_cluster = ctas ? ctas : tsvd_handle{}.svd_cluster;
+    return TSVD_OK;
+}
+
 int tsvd_workspace_size(const tsvd_matrix* A, int method, int k, int a, int c, const tsvd_opts* opts, size_t* bytes) {
     if (!bytes) return TSVD_ERR_INVALID_ARG;
     tsvd_opts o;

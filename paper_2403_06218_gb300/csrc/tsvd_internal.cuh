@@ -58,6 +58,8 @@ struct tsvd_handle {
     // limit, in SM clock cycles, of one bounded wait of the pipelined product kernels
     // and of the Jacobi grid barrier (2e9, about 1 s; tsvd_set_wait_limit lowers it)
     long long max_wait = 2000000000LL;
+    // largest cluster of the small SVD's FP32 sweeps (tsvd_set_svd_cluster)
+    int svd_cluster = 8;
     // row partition (tsvd_set_row_partition): this process holds rows
     // [part_row0, part_row0 + m) of a part_rows x n matrix; part_fn sums host buffers
     // over the processes of the partition
