@@ -414,8 +414,12 @@ int tsvd_mm_bf16x6(tsvd_handle* h, int64_t rows, int64_t cols, const void* piece
                    void* ws, size_t ws_bytes, void* stream);
 
 /* Workspace bytes for the orthogonalisation entry points below on a q-row
- * block of width b against s earlier columns. */
+ * block of width b against s earlier columns.  tsvd_orth_workspace includes the
+ * scratch (at most 4 GiB) with which the FP64 products run on the tensor cores;
+ * with less, down to tsvd_orth_workspace_min, they run on the FP64 pipe.  FP32
+ * blocks need tsvd_orth_workspace_min and use no more. */
 int tsvd_orth_workspace(int64_t q, int64_t s, int b, size_t* bytes);
+int tsvd_orth_workspace_min(int64_t q, int64_t s, int b, size_t* bytes);
 
 /* CholeskyQR2, Alg. 4 (Sec. 3.2): in place Y (q x b, ldy) <- Q with Q^T Q = I and
  * R (b x b, row-major, ld = b, upper triangular, positive diagonal) with
@@ -448,7 +452,7 @@ int tsvd_cgs_cqr2(tsvd_handle* h, int64_t q, int64_t s, int b, const double* P, 
  * projection coefficients, Cholesky factors, H and R are FP64.  Each update
  * (Y - P H, and with s = 0 the first Y L^{-T}) runs as one fused pass with the
  * Gram matrix of its result (tsvd_update_gram_f32).  Workspace:
- * tsvd_orth_workspace(q, s, b).  Synchronises `stream` before returning. */
+ * tsvd_orth_workspace_min(q, s, b).  Synchronises `stream` before returning. */
 int tsvd_cgs_cqr2_f32(tsvd_handle* h, int64_t q, int64_t s, int b, const float* P, int64_t ldp,
                       float* Y, int64_t ldy, double* H, double* R,
                       uint64_t seed, int* replacements, int* breakdowns,
@@ -473,7 +477,10 @@ int tsvd_update_gram_f32(tsvd_handle* h, int64_t q, int64_t s, int b, double alp
 
 /* CGS-QR, Alg. 3 (Sec. 3.1): QR of Y (q x r) by column blocks of width b
  * (the last one narrower if b does not divide r): Y <- Q in place, R (r x r,
- * ld = r) upper triangular assembled from [H_j; R_j].  1 <= b <= TSVD_MAX_BLOCK. */
+ * ld = r) upper triangular assembled from [H_j; R_j].  1 <= b <= TSVD_MAX_BLOCK.
+ * tsvd_cgs_qr_workspace includes the tensor-core scratch; without it the call needs
+ * tsvd_orth_workspace_min(q, r, b') + 8 r b' (rounded up to 256) bytes, b' = min(b, r). */
+int tsvd_cgs_qr_workspace(int64_t q, int r, int b, size_t* bytes);
 int tsvd_cgs_qr(tsvd_handle* h, int64_t q, int r, int b, double* Y, int64_t ldy, double* R,
                 uint64_t seed, int* replacements, int* breakdowns,
                 void* ws, size_t ws_bytes, void* stream);

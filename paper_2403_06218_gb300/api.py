@@ -604,10 +604,23 @@ def mm_bf16x6(P: Bf16x3, X: torch.Tensor) -> torch.Tensor:
     return Y
 
 
-def _orth_ws(q, s, b, dev):
+def _bytes(query: str, *args) -> int:
     nb = C.c_size_t()
-    capi.check(capi.load().tsvd_orth_workspace(q, s, b, C.byref(nb)), "tsvd_orth_workspace")
-    return _ws(nb.value + 256 * 4 + 8 * (s + b) * b, dev)
+    capi.check(getattr(capi.load(), query)(*args, C.byref(nb)), query)
+    return nb.value
+
+
+def _ws_or(full: int, least: int, dev) -> torch.Tensor:
+    """A workspace of ``full`` bytes, or of ``least`` where the device has no room for it."""
+    try:
+        return _ws(full, dev)
+    except torch.cuda.OutOfMemoryError:
+        return _ws(least, dev)
+
+
+def _orth_ws(q, s, b, dev, f32=False):
+    least = _bytes("tsvd_orth_workspace_min", q, s, b)
+    return _ws_or(least if f32 else _bytes("tsvd_orth_workspace", q, s, b), least, dev)
 
 
 def cholqr2(Y: torch.Tensor, seed: int = 0):
@@ -658,7 +671,7 @@ def cgs_cqr2(Y: torch.Tensor, P: torch.Tensor, seed: int = 0):
     H = torch.empty((max(s, 1), b), dtype=torch.float64, device=dev)
     rep, bd = C.c_int(0), C.c_int(0)
     with torch.cuda.device(dev):
-        ws = _orth_ws(q, s, b, dev)
+        ws = _orth_ws(q, s, b, dev, Y.dtype == torch.float32)
         capi.check(fn(handle(dev), q, s, b, P.data_ptr(), max(P.stride(0), s), Q.data_ptr(), Q.stride(0),
                       H.data_ptr(), R.data_ptr(), C.c_uint64(seed), C.byref(rep), C.byref(bd),
                       ws.data_ptr(), ws.numel(), _stream_ptr(dev)), name)
@@ -714,7 +727,9 @@ def cgs_qr(Y: torch.Tensor, b: int, seed: int = 0):
     R = torch.empty((r, r), dtype=torch.float64, device=dev)
     rep, bd = C.c_int(0), C.c_int(0)
     with torch.cuda.device(dev):
-        ws = _orth_ws(q, r, min(b, r), dev)
+        bw = min(b, r)
+        ws = _ws_or(_bytes("tsvd_cgs_qr_workspace", q, r, b),
+                    _bytes("tsvd_orth_workspace_min", q, r, bw) + (8 * r * bw + 255) // 256 * 256, dev)
         capi.check(lib.tsvd_cgs_qr(handle(dev), q, r, b, Q.data_ptr(), Q.stride(0), R.data_ptr(), C.c_uint64(seed),
                                    C.byref(rep), C.byref(bd), ws.data_ptr(), ws.numel(), _stream_ptr(dev)),
                    "tsvd_cgs_qr")

@@ -910,7 +910,7 @@ template <typename F1, typename F2>
 int cg_side(tsvd_handle* h, int64_t rows, int k, const double* Q, const double* rhs, const double* s, F1 op1, F2 op2,
             double* X, const tsvd_backward_opts* o, CgBufs& b, cudaStream_t st, int* iters, double* resid) {
     const size_t bytes = sizeof(double) * (size_t)rows * k;
-    const size_t ozneed = oz_standalone_ws(rows, k, k);
+    const size_t ozneed = oz_standalone_ws(rows, k, k, true);
     OzStandalone oz(h, rows, k, Q, k, b.ozws, ozneed <= b.ozbytes ? ozneed : 0, b.status);
     TSVD_TRY(oz.slice(st));
     auto project = [&](double* Z) -> int {
@@ -1004,7 +1004,7 @@ int svd_backward_run(tsvd_handle* h, const tsvd_matrix* A, int k, const double* 
     b.part = ar.take<double>(tn_partial_max(h, mx, k, k) / sizeof(double) + 1);
     b.cpart = ar.take<double>(coldot_ws(mx, k) / sizeof(double) + 1);
     // the complement projections run on the tensor cores, from planes of U (then V) sliced once
-    b.ozbytes = std::max(oz_standalone_ws(m, k, k), oz_standalone_ws(n, k, k));
+    b.ozbytes = std::max(oz_standalone_ws(m, k, k, true), oz_standalone_ws(n, k, k, true));
     b.ozws = ar.take<char>(b.ozbytes);
     b.status = status;
     if (!run) {

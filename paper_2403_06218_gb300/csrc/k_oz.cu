@@ -1117,10 +1117,10 @@ size_t oz_ws_bound(int64_t qmax, int64_t smax, int64_t bmax, int dig) {
     return std::max(tn, nn) + ex + part + 4096;
 }
 
-size_t oz_standalone_ws(int64_t q, int64_t s, int b) {
+size_t oz_standalone_ws(int64_t q, int64_t s, int b, bool keep) {
     constexpr int kW = kOzWideDig;
-    size_t bytes = oz_ws_bound(q, b, b, kW);
-    if (s > 0) {
+    size_t bytes = oz_ws_bound(q, keep ? b : std::max<int64_t>(s, b), b, kW);
+    if (s > 0 && keep) {
         bytes += oz_cache_bytes(q, s, true, kW) + oz_cache_bytes(q, s, false, kW);
         bytes += std::max(oz_tn_ws(q, s, b, false, true, kW), oz_nn_ws(q, s, b, true, kW));
     }

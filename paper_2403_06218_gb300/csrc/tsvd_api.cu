@@ -523,14 +523,19 @@ int tsvd_mm_bf16x6(tsvd_handle* h, int64_t rows, int64_t cols, const void* piece
     return hs[kStTimeout] ? TSVD_ERR_TIMEOUT : TSVD_OK;
 }
 
-int tsvd_orth_workspace(int64_t q, int64_t s, int b, size_t* bytes) {
+int tsvd_orth_workspace_min(int64_t q, int64_t s, int b, size_t* bytes) {
     if (!bytes || q < 0 || s < 0 || b < 1) return TSVD_ERR_INVALID_ARG;
     tsvd_handle hh{};
     hh.sm_count = 152;
     int dev = 0;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&hh.sm_count, cudaDevAttrMultiProcessorCount, dev);
-    *bytes = align256(sizeof(int) * kStCount) + orth_ws(&hh, q, s, b) + align256(sizeof(double) * (size_t)(s + b) * b) +
-             oz_standalone_ws(q, s, b);
+    *bytes = align256(sizeof(int) * kStCount) + orth_ws(&hh, q, s, b) + align256(sizeof(double) * (size_t)(s + b) * b);
+    return TSVD_OK;
+}
+
+int tsvd_orth_workspace(int64_t q, int64_t s, int b, size_t* bytes) {
+    TSVD_TRY(tsvd_orth_workspace_min(q, s, b, bytes));
+    *bytes += oz_standalone_ws(q, s, b, true);
     return TSVD_OK;
 }
 
@@ -544,7 +549,7 @@ int orth_entry(tsvd_handle* h, int64_t q, int64_t s, int b, const T* P, int64_t 
     if (s > 0 && (!P || ldp < s)) return TSVD_ERR_INVALID_ARG;
     if (s + b > q) return TSVD_ERR_INVALID_ARG;
     size_t need = 0;
-    TSVD_TRY(tsvd_orth_workspace(q, s, b, &need));
+    TSVD_TRY(tsvd_orth_workspace_min(q, s, b, &need));
     TSVD_TRY(check_ws(ws, ws_bytes, need));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     Arena ar{static_cast<char*>(ws), ws_bytes, 0};
@@ -556,8 +561,9 @@ int orth_entry(tsvd_handle* h, int64_t q, int64_t s, int b, const T* P, int64_t 
     TSVD_TRY_CUDA(cudaMemsetAsync(R, 0, sizeof(double) * (size_t)b * b, st));
     int rc;
     if constexpr (std::is_same<T, double>::value) {
-        // the products with P run on the tensor cores, from planes sliced once a layout
-        const size_t ozb = oz_standalone_ws(q, s, b);
+        // with room for it, the products with P run on the tensor cores, from planes sliced once
+        // a layout
+        const size_t ozfull = oz_standalone_ws(q, s, b, true), ozb = ws_bytes >= need + ozfull ? ozfull : 0;
         OzStandalone oz(h, q, s, P, ldp, ar.take<char>(ozb), ozb, status);
         TSVD_TRY(oz.slice(st));
         rc = cgs_cqr2<T>(h, q, s, b, P, ldp, Y, ldy, H, R, b, false, ctx, ar, status, st);
@@ -613,13 +619,21 @@ int tsvd_update_gram_f32(tsvd_handle* h, int64_t q, int64_t s, int b, double alp
     return TSVD_OK;
 }
 
+int tsvd_cgs_qr_workspace(int64_t q, int r, int b, size_t* bytes) {
+    if (!bytes || r < 1 || b < 1 || q < r) return TSVD_ERR_INVALID_ARG;
+    const int bw = b < r ? b : r;
+    TSVD_TRY(tsvd_orth_workspace_min(q, r, bw, bytes));
+    *bytes += align256(sizeof(double) * (size_t)r * bw) + oz_standalone_ws(q, r - bw, bw, false);
+    return TSVD_OK;
+}
+
 int tsvd_cgs_qr(tsvd_handle* h, int64_t q, int r, int b, double* Y, int64_t ldy, double* R, uint64_t seed,
                 int* replacements, int* breakdowns, void* ws, size_t ws_bytes, void* stream) {
     if (!h || r < 1 || b < 1 || q < r || !Y || !R || ldy < r) return TSVD_ERR_INVALID_ARG;
     if (b > TSVD_MAX_BLOCK) return TSVD_ERR_UNSUPPORTED;
     const int bw = b < r ? b : r;
     size_t need = 0;
-    TSVD_TRY(tsvd_orth_workspace(q, r - bw, bw, &need));
+    TSVD_TRY(tsvd_orth_workspace_min(q, r - bw, bw, &need));
     need += align256(sizeof(double) * (size_t)r * bw);
     TSVD_TRY(check_ws(ws, ws_bytes, need));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -630,7 +644,7 @@ int tsvd_cgs_qr(tsvd_handle* h, int64_t q, int r, int b, double* Y, int64_t ldy,
     ctx.seed = seed;
     ctx.replacements = replacements ? *replacements : 0;
     // (the basis of a block is the columns before it, which change: no kept planes)
-    const size_t ozb = oz_standalone_ws(q, r - bw, bw);
+    const size_t ozfull = oz_standalone_ws(q, r - bw, bw, false), ozb = ws_bytes >= need + ozfull ? ozfull : 0;
     OzStandalone oz(h, q, 0, nullptr, 0, ar.take<char>(ozb), ozb, status);
     int rc = cgs_qr<double>(h, q, r, bw, Y, ldy, R, ctx, ar, status, st);
     TSVD_TRY_CUDA(cudaStreamSynchronize(st));

@@ -333,14 +333,14 @@ int oz_cache_truncate(tsvd_handle* h, OzCache& c, int64_t v, cudaStream_t st);
 const OzCache* oz_find_cache(const tsvd_handle* h, const double* X, int64_t ldx, int64_t rows, int64_t s,
                              bool cols_layout);
 // Scratch with which the products of an operand X (q x s) and blocks of width b run on the
-// tensor cores outside the solvers (oz_ws_bound), with X's planes in both layouts; 0 where
-// it would exceed kOzStandaloneMax or no product is large enough (oz_worth), and the
-// products stay on the FP64 pipe: a call whose operands fill the device must not fail for
-// scratch.  CGS-CQR2 of 64 columns against 512 of 100,000 rows: 24.5 ms on the FP64 pipe
+// tensor cores outside the solvers (oz_ws_bound), with X's planes in both layouts (`keep`), or
+// sliced for each product; 0 where it would exceed kOzStandaloneMax or no product is large
+// enough (oz_worth), and the products stay on the FP64 pipe.  So do those of a caller that
+// brings less: a call whose operands fill the device must not fail for scratch.  CGS-CQR2 of 64 columns against 512 of 100,000 rows: 24.5 ms on the FP64 pipe
 // (at its rate of 1.2 TFLOP/s), 3.0 ms here; error against 64-bit arithmetic 5.6e-16 there,
 // 7.5e-16 here (2.2e-14 with 7 digits, on a basis with entries near 1 and near 1e-3).
 constexpr size_t kOzStandaloneMax = size_t(4) << 30;
-size_t oz_standalone_ws(int64_t q, int64_t s, int b);
+size_t oz_standalone_ws(int64_t q, int64_t s, int b, bool keep);
 
 // Registers caches with the handle for its lifetime.
 struct OzCacheScope {
@@ -378,7 +378,7 @@ struct OzStandalone {
     OzCache cols, rows;
     OzCacheScope caches;
     OzScope scope;
-    // ws: oz_standalone_ws(q, s, b) bytes, 256-byte aligned (null or 0 bytes: no effect)
+    // ws: oz_standalone_ws(q, s, b, X != null) bytes, 256-byte aligned (null or 0 bytes: no effect)
     OzStandalone(tsvd_handle* hh, int64_t q, int64_t s, const double* X, int64_t ldx, void* ws, size_t bytes,
                  int* status)
         : h(hh), prev_dig(hh->oz_dig), caches(hh), scope(hh, nullptr, 0, status) {
