@@ -382,7 +382,10 @@ typedef struct tsvd_backward_info {
 } tsvd_backward_info;
 
 void tsvd_default_backward_opts(tsvd_backward_opts* opts);
+/* Workspace of tsvd_svd_backward: with the scratch of its tensor-core projections (at most
+ * 4 GiB), and the least, with which they run on the FP64 pipe. */
 int tsvd_svd_backward_workspace(const tsvd_matrix* A, int k, const tsvd_backward_opts* opts, size_t* bytes);
+int tsvd_svd_backward_workspace_min(const tsvd_matrix* A, int k, const tsvd_backward_opts* opts, size_t* bytes);
 int tsvd_svd_backward(tsvd_handle* h, const tsvd_matrix* A, int k, const double* sigma, const double* U,
                       const double* V, const double* sigma_bar, const double* U_bar, const double* V_bar,
                       double* grad, const tsvd_backward_opts* opts, void* ws, size_t ws_bytes,

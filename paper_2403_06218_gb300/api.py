@@ -498,10 +498,8 @@ def svd_backward(A, sigma: torch.Tensor, U: torch.Tensor, V: torch.Tensor, sigma
     info = capi.TsvdBackwardInfo()
     with torch.cuda.device(dev):
         opts.stream = _stream_ptr(dev)
-        nb = C.c_size_t()
-        capi.check(lib.tsvd_svd_backward_workspace(C.byref(desc), k, C.byref(opts), C.byref(nb)),
-                   "tsvd_svd_backward_workspace")
-        ws = _ws(nb.value, dev)
+        full, least = (_bytes(f"tsvd_svd_backward_workspace{s}", C.byref(desc), k, C.byref(opts)) for s in ("", "_min"))
+        ws = _ws_or(full, least, dev)
         rc = lib.tsvd_svd_backward(handle(dev), C.byref(desc), k, _ptr(s_), _ptr(U_), _ptr(V_),
                                    _ptr(sb) if sb is not None else None, _ptr(Ub) if Ub is not None else None,
                                    _ptr(Vb) if Vb is not None else None, grad.data_ptr(), C.byref(opts),

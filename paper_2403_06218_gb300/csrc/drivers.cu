@@ -965,6 +965,10 @@ int cg_side(tsvd_handle* h, int64_t rows, int k, const double* Q, const double* 
 
 }  // namespace
 
+size_t svd_backward_tc_ws(int64_t m, int64_t n, int k) {
+    return align256(std::max(oz_standalone_ws(m, k, k, true), oz_standalone_ws(n, k, k, true)));
+}
+
 int svd_backward_run(tsvd_handle* h, const tsvd_matrix* A, int k, const double* sigma, const double* U,
                      const double* V, const double* sb, const double* Ub, const double* Vb, double* grad,
                      const tsvd_backward_opts* o, char* ws, size_t ws_bytes, size_t* sizing,
@@ -1003,15 +1007,17 @@ int svd_backward_run(tsvd_handle* h, const tsvd_matrix* A, int k, const double* 
     for (double** v : {&b.rr, &b.rr_new, &b.pap, &b.bb, &b.alpha, &b.beta}) *v = ar.take<double>(k);
     b.part = ar.take<double>(tn_partial_max(h, mx, k, k) / sizeof(double) + 1);
     b.cpart = ar.take<double>(coldot_ws(mx, k) / sizeof(double) + 1);
-    // the complement projections run on the tensor cores, from planes of U (then V) sliced once
-    b.ozbytes = std::max(oz_standalone_ws(m, k, k, true), oz_standalone_ws(n, k, k, true));
-    b.ozws = ar.take<char>(b.ozbytes);
     b.status = status;
+    if (run && !ar.fits()) return TSVD_ERR_WORKSPACE;
+    // with room for it, the complement projections run on the tensor cores, from planes of U
+    // (then V) sliced once
+    b.ozbytes = svd_backward_tc_ws(m, n, k);
+    if (run && ar.off + b.ozbytes > ws_bytes) b.ozbytes = 0;
+    b.ozws = ar.take<char>(b.ozbytes);
     if (!run) {
         *sizing = ar.off + 256;
         return TSVD_OK;
     }
-    if (!ar.fits()) return TSVD_ERR_WORKSPACE;
     // products with A and A^T in the caller's orientation (op(A) may be A^T)
     auto amul = [&](const double* X, double* Yo, int64_t ldy) {
         return op.transposed ? op_tmul64(h, op, k, X, k, Yo, ldy, status, st) : op_mul64(h, op, k, X, k, Yo, ldy, status, st);

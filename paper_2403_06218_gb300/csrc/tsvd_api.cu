@@ -307,6 +307,12 @@ int tsvd_svd_backward_workspace(const tsvd_matrix* A, int k, const tsvd_backward
                             bytes, nullptr);
 }
 
+int tsvd_svd_backward_workspace_min(const tsvd_matrix* A, int k, const tsvd_backward_opts* opts, size_t* bytes) {
+    TSVD_TRY(tsvd_svd_backward_workspace(A, k, opts, bytes));
+    *bytes -= svd_backward_tc_ws(A->m, A->n, k);
+    return TSVD_OK;
+}
+
 int tsvd_svd_backward(tsvd_handle* h, const tsvd_matrix* A, int k, const double* sigma, const double* U,
                       const double* V, const double* sigma_bar, const double* U_bar, const double* V_bar,
                       double* grad, const tsvd_backward_opts* opts, void* ws, size_t ws_bytes,
@@ -317,7 +323,7 @@ int tsvd_svd_backward(tsvd_handle* h, const tsvd_matrix* A, int k, const double*
     if (opts) o = *opts;
     TSVD_TRY(check_backward_args(A, k, &o));
     size_t need = 0;
-    TSVD_TRY(tsvd_svd_backward_workspace(A, k, &o, &need));
+    TSVD_TRY(tsvd_svd_backward_workspace_min(A, k, &o, &need));
     TSVD_TRY(check_ws(ws, ws_bytes, need));
     DeviceGuard dg(h->device);
     if (!dg.ok()) return TSVD_ERR_CUDA;
