@@ -106,6 +106,18 @@ __device__ inline int oz_exp(double x) {
 
 __device__ inline int oz_norm_exp(int e) { return e <= kOzZeroExp ? 0 : e; }
 
+// Balanced triangular products (wide form): X M = (X D^-1)(D M), D the powers of two above the
+// columns of X.  c: exponent of D at a column from its column maximum (1 for a column of zeros
+// or with Inf or NaN); oz_exp_over: exponent of x / 2^c.
+__device__ inline int oz_balance(const int* cexp, int64_t k) {
+    const int e = cexp ? cexp[k] : 0;
+    return e <= kOzZeroExp || e >= kOzNanExp ? 0 : e;
+}
+__device__ inline int oz_exp_over(double x, int c) {
+    const int e = oz_exp(x);
+    return e <= kOzZeroExp || e >= kOzNanExp ? e : e - c;
+}
+
 // F = round(x 2^(T - e)) (ties away from zero; T = 8 D - 1) plus
 // sum_p 128 256^p over the D digits: digit p of F is then byte D - 1 - p of the sum less 128
 // (the leading one may need a ninth bit: with 8 digits it is lost, and 128 reads as -128).
@@ -161,8 +173,8 @@ inline int64_t oz_ra(int64_t rows) { return (rows + 15) / 16 * 16; }
 // rows, so that a warp's store of one digit is 128 contiguous bytes.
 template <int D>
 __device__ inline void oz_store_pair(__nv_bfloat16* planes, int64_t Ra, int64_t r, int64_t k, double x0, double x1,
-                                     int e) {
-    const unsigned long long a = oz_biased<D>(x0, e), b = oz_biased<D>(x1, e);
+                                     int e0, int e1) {
+    const unsigned long long a = oz_biased<D>(x0, e0), b = oz_biased<D>(x1, e1);
     __nv_bfloat162* dst = reinterpret_cast<__nv_bfloat162*>(planes + oz_off<D>(Ra, r, k, 0));
 #pragma unroll
     for (int p = 0; p < D; ++p) {  // exact: |digit| <= 128; plane step Ra * 16 elements
@@ -174,6 +186,11 @@ __device__ inline void oz_store_pair(__nv_bfloat16* planes, int64_t Ra, int64_t 
         dst[p * Ra * 8] = __floats2bfloat162_rn(da, db);
     }
 }
+template <int D>
+__device__ inline void oz_store_pair(__nv_bfloat16* planes, int64_t Ra, int64_t r, int64_t k, double x0, double x1,
+                                     int e) {
+    oz_store_pair<D>(planes, Ra, r, k, x0, x1, e, e);
+}
 
 // Rows slicer: columns [c0, c1) of S (R rows, lds) -> columns [c0, c1) of stored row i, zeros
 // from c1 to the next multiple of 16; G lanes a row: 8, or 32 where the rows are few (512 x 512
@@ -183,13 +200,14 @@ __device__ inline void oz_store_pair(__nv_bfloat16* planes, int64_t Ra, int64_t 
 // entry does not fit it: the row's earlier columns are then sliced again), so that new
 // columns rarely raise it.  That keeps 55 bits below the row's largest entry; one exponent
 // for all rows of an orthonormal basis kept about log2(R) / 2 bits fewer.
+// BAL: the entries over the powers of two above their columns (cexp, oz_balance).
 // Bound by the 14 (16) bytes written and 8 read an entry (the digits are read again from
 // cache where a row group fits it): 100,000 x 64 in 27 us = 5.2 TB/s.
-template <int D, bool GROW, int G>
+template <int D, bool GROW, int G, bool BAL = false>
 __global__ void __launch_bounds__(256, 4) oz_slice_rows_kernel(int64_t R, int64_t c0, int64_t c1,
                                                             const double* __restrict__ S, int64_t lds,
                                                             __nv_bfloat16* __restrict__ planes, int64_t Ra,
-                                                            int* __restrict__ eexp) {
+                                                            int* __restrict__ eexp, const int* __restrict__ cexp) {
     const int sl = threadIdx.x % G;
     const int64_t ng = (int64_t)gridDim.x * (blockDim.x / G);
     const int64_t rounds = (R + ng - 1) / ng;  // the same for every lane: the shuffles need them all
@@ -201,7 +219,8 @@ __global__ void __launch_bounds__(256, 4) oz_slice_rows_kernel(int64_t R, int64_
         int e = kOzZeroExp;
         if (in) {
 #pragma unroll 4
-            for (int64_t k = c0 + sl; k < c1; k += G) e = max(e, oz_exp(src[k]));
+            for (int64_t k = c0 + sl; k < c1; k += G)
+                e = max(e, BAL ? oz_exp_over(src[k], oz_balance(cexp, k)) : oz_exp(src[k]));
         }
 #pragma unroll
         for (int o = G / 2; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
@@ -219,8 +238,10 @@ __global__ void __launch_bounds__(256, 4) oz_slice_rows_kernel(int64_t R, int64_
             if (in && sl == 0) eexp[i] = e;
         }
         if (!in) continue;
-        for (int64_t k = k0 + 2 * sl; k < a1; k += 2 * G)
-            oz_store_pair<D>(planes, Ra, i, k, k < c1 ? src[k] : 0.0, k + 1 < c1 ? src[k + 1] : 0.0, e);
+        for (int64_t k = k0 + 2 * sl; k < a1; k += 2 * G) {
+            const int s0 = BAL && k < c1 ? oz_balance(cexp, k) : 0, s1 = BAL && k + 1 < c1 ? oz_balance(cexp, k + 1) : 0;
+            oz_store_pair<D>(planes, Ra, i, k, k < c1 ? src[k] : 0.0, k + 1 < c1 ? src[k + 1] : 0.0, e + s0, e + s1);
+        }
     }
 }
 
@@ -336,12 +357,13 @@ __global__ void __launch_bounds__(256) oz_slice_cols_kernel(int64_t K, int64_t R
 // basis from the right), exponents included, in one launch: a block takes 8 columns over
 // all K.  (The column-maximum and slicing kernels and the fill before them took 9 us a
 // product at 512 x 64; 5 us now.)
+// BAL: row k times the power of two that the left operand's column k was divided by.
 constexpr int kOzShortK = 2048;
-template <int D>
+template <int D, bool BAL>
 __global__ void __launch_bounds__(256) oz_slice_cols_short_kernel(int64_t K, int64_t R, const double* __restrict__ S,
                                                                   int64_t lds, int upper,
                                                                   __nv_bfloat16* __restrict__ planes, int64_t Ra,
-                                                                  int* __restrict__ eexp) {
+                                                                  int* __restrict__ eexp, const int* __restrict__ cexp) {
     __shared__ int red[32][9];
     __shared__ int es[8];
     const int64_t j0 = (int64_t)blockIdx.x * 8;
@@ -351,7 +373,8 @@ __global__ void __launch_bounds__(256) oz_slice_cols_short_kernel(int64_t K, int
         if (j < R) {
 #pragma unroll 4
             for (int64_t k = threadIdx.x >> 3; k < K; k += 32)
-                if (!(upper && k > j)) e = max(e, oz_exp(S[k * lds + j]));
+                if (!(upper && k > j))
+                    e = max(e, BAL ? oz_exp_over(S[k * lds + j], -oz_balance(cexp, k)) : oz_exp(S[k * lds + j]));
         }
         red[threadIdx.x >> 3][threadIdx.x & 7] = e;
     }
@@ -372,7 +395,8 @@ __global__ void __launch_bounds__(256) oz_slice_cols_short_kernel(int64_t K, int
         if (j >= R) continue;
         const double x0 = k < K && !(upper && k > j) ? S[k * lds + j] : 0.0;
         const double x1 = k + 1 < K && !(upper && k + 1 > j) ? S[(k + 1) * lds + j] : 0.0;
-        oz_store_pair<D>(planes, Ra, j, k, x0, x1, es[q]);
+        const int s0 = BAL && k < K ? oz_balance(cexp, k) : 0, s1 = BAL && k + 1 < K ? oz_balance(cexp, k + 1) : 0;
+        oz_store_pair<D>(planes, Ra, j, k, x0, x1, es[q] - s0, es[q] - s1);
     }
 }
 
@@ -961,8 +985,9 @@ struct OzView {
     const int* exps;
 };
 
+// cexp: balanced (wide form only).
 int oz_slice_rows(tsvd_handle* h, int64_t R, int64_t c0, int64_t c1, const double* S, int64_t lds, bool grow,
-                  __nv_bfloat16* planes, int* eexp, cudaStream_t st) {
+                  __nv_bfloat16* planes, int* eexp, cudaStream_t st, const int* cexp = nullptr) {
     if (R == 0) return TSVD_OK;
     // 8 lanes a row; 32 where that leaves fewer warps than the chip has room for
     const bool few = R <= (int64_t)h->sm_count * 32;
@@ -970,38 +995,53 @@ int oz_slice_rows(tsvd_handle* h, int64_t R, int64_t c0, int64_t c1, const doubl
     const int64_t blocks = std::min<int64_t>((R + rows - 1) / rows, (int64_t)h->sm_count * 32);
     const bool wide = h->oz_dig == kOzWideDig;
     const auto kern = grow   ? (few ? oz_slice_rows_kernel<kOzDig, true, 32> : oz_slice_rows_kernel<kOzDig, true, 8>)
+                      : cexp ? (few ? oz_slice_rows_kernel<kOzWideDig, false, 32, true>
+                                    : oz_slice_rows_kernel<kOzWideDig, false, 8, true>)
                       : wide ? (few ? oz_slice_rows_kernel<kOzWideDig, false, 32>
                                     : oz_slice_rows_kernel<kOzWideDig, false, 8>)
                              : (few ? oz_slice_rows_kernel<kOzDig, false, 32>
                                     : oz_slice_rows_kernel<kOzDig, false, 8>);
     h->launches++;
-    kern<<<(unsigned)blocks, 256, 0, st>>>(R, c0, c1, S, lds, planes, oz_ra(R), eexp);
+    kern<<<(unsigned)blocks, 256, 0, st>>>(R, c0, c1, S, lds, planes, oz_ra(R), eexp, cexp);
     TSVD_TRY_CUDA(cudaGetLastError());
     return TSVD_OK;
 }
 
-// Ra: allocated stored rows of `planes` (default R); r0: first stored row written.
-int oz_slice_cols(tsvd_handle* h, int64_t K, int64_t R, const double* S, int64_t lds, bool upper,
-                  __nv_bfloat16* planes, int* eexp, cudaStream_t st, int64_t Ra = -1, int64_t r0 = 0) {
-    if (R == 0) return TSVD_OK;
-    if (Ra < 0) Ra = oz_ra(R);
-    const bool wide = h->oz_dig == kOzWideDig;
-    if (K <= kOzShortK && r0 == 0) {
-        const auto kern = wide ? oz_slice_cols_short_kernel<kOzWideDig> : oz_slice_cols_short_kernel<kOzDig>;
-        h->launches++;
-        kern<<<(unsigned)((R + 7) / 8), 256, 0, st>>>(K, R, S, lds, upper ? 1 : 0, planes, Ra, eexp);
-        TSVD_TRY_CUDA(cudaGetLastError());
-        return TSVD_OK;
-    }
+// The column maxima of S alone.
+int oz_colmax(tsvd_handle* h, int64_t K, int64_t R, const double* S, int64_t lds, bool upper, int* eexp,
+              cudaStream_t st) {
     const unsigned gx = (unsigned)((R + 31) / 32);
     int64_t gy = std::min<int64_t>((K + 255) / 256, std::max<int64_t>(1, (int64_t)h->sm_count * 8 / gx));
     const int64_t rows_per = (K + gy - 1) / gy;
     gy = (K + rows_per - 1) / rows_per;
-    h->launches += 2;
+    h->launches++;
     TSVD_TRY_CUDA(cudaMemsetAsync(eexp, kOzUnset, sizeof(int) * R, st));
     oz_colmax_kernel<<<dim3(gx, (unsigned)std::max<int64_t>(1, gy)), dim3(32, 8), 0, st>>>(K, R, S, lds,
                                                                                            upper ? 1 : 0, rows_per,
                                                                                            eexp);
+    TSVD_TRY_CUDA(cudaGetLastError());
+    return TSVD_OK;
+}
+
+// Ra: allocated stored rows of `planes` (default R); r0: first stored row written; cexp:
+// balanced (wide form, K <= kOzShortK).
+int oz_slice_cols(tsvd_handle* h, int64_t K, int64_t R, const double* S, int64_t lds, bool upper,
+                  __nv_bfloat16* planes, int* eexp, cudaStream_t st, int64_t Ra = -1, int64_t r0 = 0,
+                  const int* cexp = nullptr) {
+    if (R == 0) return TSVD_OK;
+    if (Ra < 0) Ra = oz_ra(R);
+    const bool wide = h->oz_dig == kOzWideDig;
+    if (K <= kOzShortK && r0 == 0) {
+        const auto kern = cexp   ? oz_slice_cols_short_kernel<kOzWideDig, true>
+                          : wide ? oz_slice_cols_short_kernel<kOzWideDig, false>
+                                 : oz_slice_cols_short_kernel<kOzDig, false>;
+        h->launches++;
+        kern<<<(unsigned)((R + 7) / 8), 256, 0, st>>>(K, R, S, lds, upper ? 1 : 0, planes, Ra, eexp, cexp);
+        TSVD_TRY_CUDA(cudaGetLastError());
+        return TSVD_OK;
+    }
+    TSVD_TRY(oz_colmax(h, K, R, S, lds, upper, eexp, st));
+    h->launches++;
     const dim3 sg((unsigned)((oz_k16(K) + 63) / 64), (unsigned)((R + 63) / 64));
     const auto kern = wide ? oz_slice_cols_kernel<kOzWideDig> : oz_slice_cols_kernel<kOzDig>;
     kern<<<sg, 256, 0, st>>>(K, R, S, lds, upper ? 1 : 0, eexp, planes, Ra, r0);
@@ -1168,6 +1208,7 @@ size_t oz_nn_ws(int64_t q, int64_t s, int64_t b, bool cached_x, int dig) {
     }
     ar.take<char>(oz_planes_bytes(p.N, p.K, dig));
     ar.take<int>((size_t)p.N);
+    if (dig == kOzWideDig && !cached_x) ar.take<int>((size_t)p.K);
     ar.take<char>(oz_partial_bytes(p));
     return ar.off;
 }
@@ -1212,13 +1253,22 @@ int oz_gemm_nn(tsvd_handle* h, int64_t q, int64_t s, int64_t b, double alpha, co
     const OzPlan p = oz_plan(q, b, s);
     Arena ar{static_cast<char*>(ws), ws_bytes, 0};
     OzView va{};
+    // Wide form, triangular M (the normalisation Y L^-T of a block whose columns may differ by
+    // orders of magnitude): balanced by the columns of X, so that one exponent a row serves all
+    // of them.  Error of Q against 1e-28 arithmetic, 87,413 x 128 with columns from 1 to 1e-3:
+    // 4.6e-16 without, 1.1e-16 on the FP64 pipe.
+    const bool bal = h->oz_dig == kOzWideDig && upper && !xc && s <= kOzShortK;
+    int* cexp = nullptr;
     if (xc) {
         va = view_of_cache(*xc, s);
     } else {
         __nv_bfloat16* pa = reinterpret_cast<__nv_bfloat16*>(ar.take<char>(oz_planes_bytes(p.M, p.K, h->oz_dig)));
         int* ea = ar.take<int>((size_t)p.M);
+        if (h->oz_dig == kOzWideDig) cexp = ar.take<int>((size_t)p.K);
         if (!ar.fits()) return TSVD_ERR_WORKSPACE;
-        TSVD_TRY(oz_slice_rows(h, q, 0, s, X, ldx, false, pa, ea, st));
+        if (!bal) cexp = nullptr;
+        if (bal) TSVD_TRY(oz_colmax(h, q, s, X, ldx, false, cexp, st));
+        TSVD_TRY(oz_slice_rows(h, q, 0, s, X, ldx, false, pa, ea, st, cexp));
         va = view_of(pa, q, s, ea);
     }
     __nv_bfloat16* pb = reinterpret_cast<__nv_bfloat16*>(ar.take<char>(oz_planes_bytes(p.N, p.K, h->oz_dig)));
@@ -1226,7 +1276,7 @@ int oz_gemm_nn(tsvd_handle* h, int64_t q, int64_t s, int64_t b, double alpha, co
     const size_t pbytes = oz_partial_bytes(p);
     double* part = pbytes ? reinterpret_cast<double*>(ar.take<char>(pbytes)) : nullptr;
     if (!ar.fits()) return TSVD_ERR_WORKSPACE;
-    TSVD_TRY(oz_slice_cols(h, s, b, Mm, ldm, upper, pb, eb, st));
+    TSVD_TRY(oz_slice_cols(h, s, b, Mm, ldm, upper, pb, eb, st, -1, 0, cexp));
     return oz_run(h, p, va, view_of(pb, b, s, eb), part, Y, ldy, alpha, beta, false, status, st);
 }
 

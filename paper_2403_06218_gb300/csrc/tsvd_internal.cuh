@@ -336,9 +336,11 @@ const OzCache* oz_find_cache(const tsvd_handle* h, const double* X, int64_t ldx,
 // tensor cores outside the solvers (oz_ws_bound), with X's planes in both layouts (`keep`), or
 // sliced for each product; 0 where it would exceed kOzStandaloneMax or no product is large
 // enough (oz_worth), and the products stay on the FP64 pipe.  So do those of a caller that
-// brings less: a call whose operands fill the device must not fail for scratch.  CGS-CQR2 of 64 columns against 512 of 100,000 rows: 24.5 ms on the FP64 pipe
-// (at its rate of 1.2 TFLOP/s), 3.0 ms here; error against 64-bit arithmetic 5.6e-16 there,
-// 7.5e-16 here (2.2e-14 with 7 digits, on a basis with entries near 1 and near 1e-3).
+// brings less: a call whose operands fill the device must not fail for scratch.
+// CGS-CQR2 of 64 columns against 512 of 100,000 rows: 24.5 ms on the FP64 pipe (at its rate of
+// 1.2 TFLOP/s), 2.4 ms here.  Error of Q and H against 1e-28 arithmetic: 5.2e-16 and 7.4e-16
+// there, 1.2e-16 and 7.1e-17 here (with 7 digits 100 times more, on a basis with entries near 1
+// and near 1e-3).
 constexpr size_t kOzStandaloneMax = size_t(4) << 30;
 size_t oz_standalone_ws(int64_t q, int64_t s, int b, bool keep);
 
