@@ -55,6 +55,8 @@ struct tsvd_handle {
     int oz_dig = 7;
     // operands whose digit planes are kept for the current call (owned by the caller)
     std::vector<const tsvd::OzCache*> oz_caches;
+    // set by OzFreshRows: products slice their left operand afresh
+    bool oz_fresh_rows = false;
     // limit, in SM clock cycles, of one bounded wait of the pipelined product kernels
     // and of the Jacobi grid barrier (2e9, about 1 s; tsvd_set_wait_limit lowers it)
     long long max_wait = 2000000000LL;
@@ -351,6 +353,18 @@ struct OzCacheScope {
     explicit OzCacheScope(tsvd_handle* hh) : h(hh), n0(hh->oz_caches.size()) {}
     void add(const OzCache* c) { h->oz_caches.push_back(c); }
     ~OzCacheScope() { h->oz_caches.resize(n0); }
+};
+
+// Within its lifetime the FP64 products slice their left operand afresh, with one exponent a
+// row, instead of reading the rows-layout planes of a basis.  The exponents of a basis that
+// grows lie one above the row's largest entry, which doubles the error of a product.  In a
+// cycle the coefficients come from the same planes; the restart and Ritz products, whose
+// results the next cycle takes as exact, slice afresh (0.3 ms for 100,000 x 576).
+struct OzFreshRows {
+    tsvd_handle* h;
+    bool prev;
+    explicit OzFreshRows(tsvd_handle* hh) : h(hh), prev(hh->oz_fresh_rows) { h->oz_fresh_rows = true; }
+    ~OzFreshRows() { h->oz_fresh_rows = prev; }
 };
 
 // Makes the FP64 products of one call run on the tensor cores with `bytes` of
