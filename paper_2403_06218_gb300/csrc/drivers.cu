@@ -937,7 +937,10 @@ int cg_side(tsvd_handle* h, int64_t rows, int k, const double* Q, const double* 
         if (check) {
             TSVD_TRY_CUDA(cudaMemcpyAsync(hrr.data(), b.rr, sizeof(double) * k, cudaMemcpyDeviceToHost, st));
             TSVD_TRY_CUDA(cudaMemcpyAsync(hbb.data(), b.bb, sizeof(double) * k, cudaMemcpyDeviceToHost, st));
-            TSVD_TRY_CUDA(cudaStreamSynchronize(st));
+            // a product that gave up leaves its output unfinished: that is not the caller's data
+            int hs[kStCount];
+            TSVD_TRY(read_status(st, b.status, hs));
+            if (hs[kStTimeout]) return TSVD_ERR_TIMEOUT;
             bool done = true;
             worst = 0.0;
             for (int j = 0; j < k; ++j) {

@@ -303,7 +303,11 @@ int cgs_cqr2(tsvd_handle* h, int64_t q, int64_t s, int b, const T* P, int64_t ld
         TSVD_TRY_CUDA(copy_block(w.save, b, Y, ldy, q, b, st));
         ctx.fallbacks++;
         for (int64_t i = 0; i < b; ++i) TSVD_TRY_CUDA(cudaMemsetAsync(R + i * ldr, 0, sizeof(double) * b, st));
-        TSVD_TRY(cgs2_columns(h, q, s, b, P, ldp, Y, ldy, H, b, R, ldr, r_trans, ctx, w, st));
+        const int rc = cgs2_columns(h, q, s, b, P, ldp, Y, ldy, H, b, R, ldr, r_trans, ctx, w, st);
+        // (a product of the fallback that gave up, whatever its unfinished output looked like)
+        TSVD_TRY(read_status(st, status, hs));
+        if (hs[kStTimeout]) return TSVD_ERR_TIMEOUT;
+        return rc;
     }
     return TSVD_OK;
 }
