@@ -20,6 +20,7 @@
 
 #include <algorithm>
 
+#include "fp64_rsqrt.cuh"
 #include "tsvd_internal.cuh"
 
 namespace tsvd {
@@ -268,17 +269,6 @@ __device__ inline void tri_decode(int idx, int& ii, int& kk) {
     kk = idx - r * (r + 1) / 2;
 }
 
-// 1/sqrt(d) for finite d > 0: FP32 estimate of the scaled value, two Newton steps
-// y <- y (3 - d y^2) / 2 in FP64 (24 -> 48 -> beyond 53 bits), rescaled.
-__device__ inline double rsqrt_fp64(double d) {
-    const int e = ilogb(d) & ~1;  // even exponent: d = dd 2^e, dd in [1, 4)
-    const double dd = scalbn(d, -e);
-    double y = (double)rsqrtf((float)dd);
-    y = y * fma(-0.5 * dd, y * y, 1.5);
-    y = y * fma(-0.5 * dd, y * y, 1.5);
-    return scalbn(y, -e / 2);
-}
-
 __global__ void __launch_bounds__(256) chol_inv_kernel(int b, const double* __restrict__ W, double* __restrict__ Lt,
                                                        double* __restrict__ Mt, int* status) {
     extern __shared__ double sm[];
@@ -408,23 +398,6 @@ struct CholSmem {
     double thresh;
     int bad;
 };
-
-// 1/sqrt(d) for a normal finite d > 0 with a short chain on the FP64 pipe: FP32 estimate y
-// (2^-21) of d scaled to [1, 4), both conversions by bits, then y (1 + e / 2 + 3 e^2 / 8),
-// e = 1 - d y^2, to beyond 53 bits.
-__device__ inline double rsqrt_fp64_short(double d) {
-    const int hi = __double2hiint(d), lo = __double2loint(d);
-    const int ex = ((hi >> 20) - 1023) & ~1;
-    if ((hi >> 20) == 0) return rsqrt_fp64(d);  // subnormal
-    const int h = hi - (ex << 20);  // exponent field 1023 or 1024
-    const double dd = __hiloint2double(h, lo);
-    const float f = __int_as_float(((h >> 20) - 896) << 23 | (h & 0xFFFFF) << 3 | (int)((unsigned)lo >> 29));
-    const int yb = __float_as_int(rsqrtf(f));  // in (1/2, 1]
-    const double y = __hiloint2double((yb >> 3) + (896 << 20), yb << 29);
-    const double e = fma(-dd, y * y, 1.0);
-    const double z = fma(y * e, fma(e, 0.375, 0.5), y);
-    return __hiloint2double(__double2hiint(z) - ((ex >> 1) << 20), __double2loint(z));
-}
 
 __global__ void __cluster_dims__(kCholCluster, 1, 1) __launch_bounds__(256, 1)
     chol_inv_cluster_kernel(int b, const double* __restrict__ W, double* __restrict__ Lt, double* __restrict__ Mt,
