@@ -337,6 +337,11 @@ int tsvd_dense_mm_f64tc_workspace(int trans, int64_t m, int64_t n, int w, size_t
 int tsvd_dense_mm_f64tc(tsvd_handle* h, int trans, int64_t m, int64_t n, const double* A, int64_t lda,
                         int w, const double* X, int64_t ldx, double* Y, int64_t ldy,
                         void* ws, size_t ws_bytes, void* stream);
+/* Test hook: tsvd_dense_mm_f64tc runs with 8 digits an entry (the form of the standalone
+ * orthogonalisation and the gradient, 63 bits below a row's or column's largest entry and the
+ * 36 digit products of weight >= 2^-56) instead of 7, and needs 8/7 of the planes' scratch.
+ * digits: 7, 8, or 0 for the default of 7. */
+int tsvd_set_product_digits(tsvd_handle* h, int digits);
 
 /* The same products in FP32 (the mixed-precision form's kernels): A, X and Y
  * float32, products accumulated in FP32 within a row slab, and for trans = 1

@@ -101,6 +101,7 @@ SIGNATURES = [
     ("tsvd_destroy", _I, [_P]),
     ("tsvd_set_wait_limit", _I, [_P, C.c_longlong]),
     ("tsvd_set_svd_cluster", _I, [_P, _I]),
+    ("tsvd_set_product_digits", _I, [_P, _I]),
     ("tsvd_set_row_partition", _I, [_P, _I64, _I64, ALLREDUCE_FN, _P]),
     ("tsvd_status_string", C.c_char_p, [_I]),
     ("tsvd_workspace_size", _I, [C.POINTER(TsvdMatrix), _I, _I, _I, _I, C.POINTER(TsvdOpts), _PSZ]),

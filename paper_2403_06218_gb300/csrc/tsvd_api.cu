@@ -443,6 +443,12 @@ int tsvd_dense_mm_f64tc_workspace(int trans, int64_t m, int64_t n, int w, size_t
     return TSVD_OK;
 }
 
+int tsvd_set_product_digits(tsvd_handle* h, int digits) {
+    if (!h || (digits != 0 && digits != 7 && digits != 8)) return TSVD_ERR_INVALID_ARG;
+    h->mm_dig = digits ? digits : tsvd_handle{}.mm_dig;
+    return TSVD_OK;
+}
+
 int tsvd_dense_mm_f64tc(tsvd_handle* h, int trans, int64_t m, int64_t n, const double* A, int64_t lda, int w,
                         const double* X, int64_t ldx, double* Y, int64_t ldy, void* ws, size_t ws_bytes,
                         void* stream) {
@@ -450,9 +456,15 @@ int tsvd_dense_mm_f64tc(tsvd_handle* h, int trans, int64_t m, int64_t n, const d
     // empty operands may come with null pointers
     if ((m * n > 0 && !A) || ((trans ? m : n) * w > 0 && !X) || ((trans ? n : m) * w > 0 && !Y))
         return TSVD_ERR_INVALID_ARG;
-    size_t need = 0;
-    TSVD_TRY(tsvd_dense_mm_f64tc_workspace(trans, m, n, w, &need));
+    const size_t need =
+        256 + (trans ? oz_tn_ws(m, n, w, false, false, h->mm_dig) : oz_nn_ws(m, n, w, false, h->mm_dig));
     TSVD_TRY(check_ws(ws, ws_bytes, need));
+    struct Digits {  // of this call's product
+        tsvd_handle* h;
+        const int prev;
+        ~Digits() { h->oz_dig = prev; }
+    } digits{h, h->oz_dig};
+    h->oz_dig = h->mm_dig;
     DeviceGuard dg(h->device);
     if (!dg.ok()) return TSVD_ERR_CUDA;
     cudaStream_t st = static_cast<cudaStream_t>(stream);

@@ -53,6 +53,8 @@ struct tsvd_handle {
     int* oz_status = nullptr;
     // digits an entry in the products of the current call (k_oz.cu): 7, or 8 in the wide form
     int oz_dig = 7;
+    // the same for tsvd_dense_mm_f64tc (tsvd_set_product_digits)
+    int mm_dig = 7;
     // operands whose digit planes are kept for the current call (owned by the caller)
     std::vector<const tsvd::OzCache*> oz_caches;
     // set by OzFreshRows: products slice their left operand afresh
