@@ -75,6 +75,7 @@ struct Op {
     double* partial = nullptr;  // split-K scratch of dense A^T X
     // mixed form, dense A: BF16 pieces of A and of A^T for the tensor-core products
     SpmmPlan plan_a, plan_at;  // long-row split plans of CSR(A) and CSR(A^T)
+    size_t peak = 0;           // sizing: bytes up to the end of the transposition's scratch
     bool tc = false;
     const void* pA = nullptr;
     const void* pAt = nullptr;
@@ -224,7 +225,7 @@ int setup_op(tsvd_handle* h, const tsvd_matrix* A, int wmax, Arena& ar, Op<T>& o
         } else {
             Arena tmp = ar;
             tmp.take<char>(csr_transpose_ws(M, N, nnz));
-            ar.off = tmp.off;  // size the scratch (the run reuses it later)
+            op.peak = tmp.off;  // later buffers take its place
         }
         // values in both precisions
         if (in64) {
@@ -535,7 +536,7 @@ int rsvd_run(tsvd_handle* h, const tsvd_matrix* A, int k, int p, int q, int bq, 
         const size_t t2 = small_svd_ws(ell), t3 = final_tail_ws(h, m, n, k, kMixed);
         if (t2 > t1) t1 = t2;
         if (t3 > t1) t1 = t3;
-        *sizing = ar.off + t1 + 256;
+        *sizing = std::max(ar.off + t1, op.peak) + 256;
         return TSVD_OK;
     }
     if (!ar.fits()) return TSVD_ERR_WORKSPACE;
@@ -713,7 +714,7 @@ int blanczos_run(tsvd_handle* h, const tsvd_matrix* A, int k, int b, int r, uint
         if (t2 > t1) t1 = t2;
         if (t3 > t1) t1 = t3;
         if (t4 > t1) t1 = t4;
-        *sizing = ar.off + t1 + 256;
+        *sizing = std::max(ar.off + t1, op.peak) + 256;
         return TSVD_OK;
     }
     if (!ar.fits()) return TSVD_ERR_WORKSPACE;
@@ -972,14 +973,10 @@ int cg_side(tsvd_handle* h, int64_t rows, int k, const double* Q, const double* 
 
 }  // namespace
 
-size_t svd_backward_tc_ws(int64_t m, int64_t n, int k) {
-    return align256(std::max(oz_standalone_ws(m, k, k, true), oz_standalone_ws(n, k, k, true)));
-}
-
 int svd_backward_run(tsvd_handle* h, const tsvd_matrix* A, int k, const double* sigma, const double* U,
                      const double* V, const double* sb, const double* Ub, const double* Vb, double* grad,
                      const tsvd_backward_opts* o, char* ws, size_t ws_bytes, size_t* sizing,
-                     tsvd_backward_info* info) {
+                     tsvd_backward_info* info, size_t* least) {
     const bool run = sizing == nullptr;
     cudaStream_t st = static_cast<cudaStream_t>(o->stream);
     Arena ar{run ? ws : nullptr, ws_bytes, 0};
@@ -1018,13 +1015,14 @@ int svd_backward_run(tsvd_handle* h, const tsvd_matrix* A, int k, const double* 
     if (run && !ar.fits()) return TSVD_ERR_WORKSPACE;
     // with room for it, the complement projections run on the tensor cores, from planes of U
     // (then V) sliced once
-    b.ozbytes = svd_backward_tc_ws(m, n, k);
+    b.ozbytes = align256(std::max(oz_standalone_ws(m, k, k, true), oz_standalone_ws(n, k, k, true)));
     if (run && ar.off + b.ozbytes > ws_bytes) b.ozbytes = 0;
-    b.ozws = ar.take<char>(b.ozbytes);
     if (!run) {
-        *sizing = ar.off + 256;
+        if (least) *least = std::max(ar.off, op.peak) + 256;
+        *sizing = std::max(ar.off + b.ozbytes, op.peak) + 256;
         return TSVD_OK;
     }
+    b.ozws = ar.take<char>(b.ozbytes);
     // products with A and A^T in the caller's orientation (op(A) may be A^T)
     auto amul = [&](const double* X, double* Yo, int64_t ldy) {
         return op.transposed ? op_tmul64(h, op, k, X, k, Yo, ldy, status, st) : op_mul64(h, op, k, X, k, Yo, ldy, status, st);

@@ -296,21 +296,27 @@ static int check_backward_args(const tsvd_matrix* A, int k, const tsvd_backward_
     return TSVD_OK;
 }
 
-int tsvd_svd_backward_workspace(const tsvd_matrix* A, int k, const tsvd_backward_opts* opts, size_t* bytes) {
-    if (!A || !bytes) return TSVD_ERR_INVALID_ARG;
+extern "C++" {
+static int backward_sizes(const tsvd_matrix* A, int k, const tsvd_backward_opts* opts, size_t* full, size_t* least) {
+    if (!A || !full || !least) return TSVD_ERR_INVALID_ARG;
     tsvd_backward_opts o;
     tsvd_default_backward_opts(&o);
     if (opts) o = *opts;
     TSVD_TRY(check_backward_args(A, k, &o));
     tsvd_handle hh = sizing_handle();
     return svd_backward_run(&hh, A, k, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, &o, nullptr, 0,
-                            bytes, nullptr);
+                            full, nullptr, least);
+}
+}  // extern "C++"
+
+int tsvd_svd_backward_workspace(const tsvd_matrix* A, int k, const tsvd_backward_opts* opts, size_t* bytes) {
+    size_t least = 0;
+    return backward_sizes(A, k, opts, bytes, &least);
 }
 
 int tsvd_svd_backward_workspace_min(const tsvd_matrix* A, int k, const tsvd_backward_opts* opts, size_t* bytes) {
-    TSVD_TRY(tsvd_svd_backward_workspace(A, k, opts, bytes));
-    *bytes -= svd_backward_tc_ws(A->m, A->n, k);
-    return TSVD_OK;
+    size_t full = 0;
+    return backward_sizes(A, k, opts, &full, bytes);
 }
 
 int tsvd_svd_backward(tsvd_handle* h, const tsvd_matrix* A, int k, const double* sigma, const double* U,

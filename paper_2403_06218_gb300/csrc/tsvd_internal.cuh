@@ -469,10 +469,9 @@ cudaError_t col_residual_sq(tsvd_handle* h, int64_t q, int k, const double* Y, i
 int svd_backward_run(tsvd_handle* h, const tsvd_matrix* A, int k, const double* sigma, const double* U,
                      const double* V, const double* sb, const double* Ub, const double* Vb, double* grad,
                      const tsvd_backward_opts* o, char* ws, size_t ws_bytes, size_t* sizing,
-                     tsvd_backward_info* info);
-// The part of its workspace with which the projections run on the tensor cores (they run on
-// the FP64 pipe without it).
-size_t svd_backward_tc_ws(int64_t m, int64_t n, int k);
+                     tsvd_backward_info* info, size_t* least = nullptr);
+// (sizing: with the scratch of its projections on the tensor cores; least: without, for which
+// they run on the FP64 pipe)
 // Row groups of a column reduction over `rows` rows (at most 608: four for each of 152
 // SMs; a fixed number, so that the order of the sums does not depend on the device), and
 // the sums over the groups, out[j] = sum_g partial[g][j], in a fixed order.
