@@ -265,17 +265,17 @@ __device__ inline bool rot_params(double al, double be, double ga, double tol2, 
 // the same row of different columns falls in different banks.
 __host__ __device__ inline int gram_ld(int n) { return n | 1; }
 
-template <typename T, int W>
+template <int W>
 __host__ __device__ constexpr size_t gram_smem(int n) {
-    return sizeof(T) * (size_t)(2 * W) * (size_t)gram_ld(n);
+    return sizeof(double) * (size_t)(2 * W) * (size_t)gram_ld(n);
 }
 
 // M = C^T C for the 2W columns in shared memory (stride ld): the tiles on and
 // above the diagonal of TM x TM register tiles (the others mirrored), each tile's
 // rows split over S interleaved lane slices that a shuffle tree sums in a fixed
 // order.  A diagonal tile is symmetric bit for bit (x_a x_b = x_b x_a in every fma).
-template <typename T, int W>
-__device__ inline void gram_form(const T* cols, int n, int ld, T (*M)[2 * W + 1]) {
+template <int W>
+__device__ inline void gram_form(const double* cols, int n, int ld, double (*M)[2 * W + 1]) {
     constexpr int W2 = 2 * W;
     constexpr int TM = W2 >= 8 ? 4 : 2;
     constexpr int NTS = W2 / TM;
@@ -298,15 +298,15 @@ __device__ inline void gram_form(const T* cols, int n, int ld, T (*M)[2 * W + 1]
         ++ti;
     }
     const int tj = ti + u;
-    T acc[TM][TM];
+    double acc[TM][TM];
 #pragma unroll
     for (int a = 0; a < TM; ++a)
 #pragma unroll
-        for (int b = 0; b < TM; ++b) acc[a][b] = T(0);
-    const T* ca = cols + (size_t)(ti * TM) * ld;
-    const T* cb = cols + (size_t)(tj * TM) * ld;
+        for (int b = 0; b < TM; ++b) acc[a][b] = 0.0;
+    const double* ca = cols + (size_t)(ti * TM) * ld;
+    const double* cb = cols + (size_t)(tj * TM) * ld;
     for (int r = s; r < n; r += S) {
-        T x[TM], y[TM];
+        double x[TM], y[TM];
 #pragma unroll
         for (int a = 0; a < TM; ++a) {
             x[a] = ca[(size_t)a * ld + r];
@@ -321,7 +321,7 @@ __device__ inline void gram_form(const T* cols, int n, int ld, T (*M)[2 * W + 1]
     for (int a = 0; a < TM; ++a)
 #pragma unroll
         for (int b = 0; b < TM; ++b) {
-            T v = acc[a][b];
+            double v = acc[a][b];
 #pragma unroll
             for (int d = S / 2; d > 0; d >>= 1) v += __shfl_xor_sync(kFull, v, d);
             if (s == 0 && live) {
@@ -332,41 +332,37 @@ __device__ inline void gram_form(const T* cols, int n, int ld, T (*M)[2 * W + 1]
 }
 
 // Row stride of Z: 16-byte rows, so that the C Z products read a row of Z two doubles at a time.
-template <typename T, int W>
+template <int W>
 __host__ __device__ constexpr int gram_zs() {
-    return 2 * W + (int)(16 / sizeof(T));
+    return 2 * W + 2;
 }
 
 // acc[j] += x Z_k[j] for j < W2, Z_k a 16-byte aligned row (vector loads, broadcast
 // to the warp).
-template <typename T, int W2>
-__device__ inline void gram_axpy_row(T x, const T* zk, T* acc) {
-    if constexpr (W2 % 2 == 0) {
+template <int W2>
+__device__ inline void gram_axpy_row(double x, const double* zk, double* acc) {
+    static_assert(W2 % 2 == 0, "pairs of columns");
 #pragma unroll
-        for (int j = 0; j < W2; j += 2) {
-            const double2 z = *reinterpret_cast<const double2*>(zk + j);
-            acc[j] = fma(x, (T)z.x, acc[j]);
-            acc[j + 1] = fma(x, (T)z.y, acc[j + 1]);
-        }
-    } else {
-#pragma unroll
-        for (int j = 0; j < W2; ++j) acc[j] = fma(x, zk[j], acc[j]);
+    for (int j = 0; j < W2; j += 2) {
+        const double2 z = *reinterpret_cast<const double2*>(zk + j);
+        acc[j] = fma(x, z.x, acc[j]);
+        acc[j + 1] = fma(x, z.y, acc[j + 1]);
     }
 }
 
 // One mini-round on the block's Gram matrix by warp 0: npr disjoint pairs
 // (pp[k], pq[k]) rotated at once; M <- R^T M R and Z <- Z R.  Returns whether any
 // pair rotated (warp-uniform).
-template <typename T, int W>
-__device__ inline bool gram_mini_round(T (*M)[2 * W + 1], T (*Z)[gram_zs<T, W>()], const int* pp, const int* pq,
+template <int W>
+__device__ inline bool gram_mini_round(double (*M)[2 * W + 1], double (*Z)[gram_zs<W>()], const int* pp, const int* pq,
                                        int npr,
-                                       T tol2, T* s_c, T* s_s, int* s_rot) {
+                                       double tol2, double* s_c, double* s_s, int* s_rot) {
     constexpr int W2 = 2 * W;
     const int lane = threadIdx.x & 31;
     int rot = 0;
     if (lane < npr) {
         const int p = pp[lane], q = pq[lane];
-        T c = T(1), sn = T(0), t = T(0);
+        double c = 1.0, sn = 0.0, t = 0.0;
         rot = rot_params(M[p][p], M[q][q], M[p][q], tol2, c, sn, t) ? 1 : 0;
         s_c[lane] = c;
         s_s[lane] = sn;
@@ -379,11 +375,11 @@ __device__ inline bool gram_mini_round(T (*M)[2 * W + 1], T (*Z)[gram_zs<T, W>()
         for (int k = 0; k < npr; ++k) {
             if (!s_rot[k]) continue;
             const int p = pp[k], q = pq[k];
-            const T c = s_c[k], sn = s_s[k];
-            const T x = M[lane][p], y = M[lane][q];
+            const double c = s_c[k], sn = s_s[k];
+            const double x = M[lane][p], y = M[lane][q];
             M[lane][p] = fma(c, x, -sn * y);
             M[lane][q] = fma(sn, x, c * y);
-            const T u = Z[lane][p], v = Z[lane][q];
+            const double u = Z[lane][p], v = Z[lane][q];
             Z[lane][p] = fma(c, u, -sn * v);
             Z[lane][q] = fma(sn, u, c * v);
         }
@@ -393,8 +389,8 @@ __device__ inline bool gram_mini_round(T (*M)[2 * W + 1], T (*Z)[gram_zs<T, W>()
         for (int k = 0; k < npr; ++k) {
             if (!s_rot[k]) continue;
             const int p = pp[k], q = pq[k];
-            const T c = s_c[k], sn = s_s[k];
-            const T x = M[p][lane], y = M[q][lane];
+            const double c = s_c[k], sn = s_s[k];
+            const double x = M[p][lane], y = M[q][lane];
             M[p][lane] = fma(c, x, -sn * y);
             M[q][lane] = fma(sn, x, c * y);
         }
@@ -411,12 +407,12 @@ __device__ inline bool gram_mini_round(T (*M)[2 * W + 1], T (*Z)[gram_zs<T, W>()
 // M and Z within each lane, and on the rows of M between lane k and its partner
 // lane by shuffles.  M and Z enter and leave in shared memory.  Returns whether
 // any pair rotated (warp-uniform).
-template <typename T, int W>
-__device__ inline bool gram_rounds_ij(T (*M)[2 * W + 1], T (*Z)[gram_zs<T, W>()], T tol2) {
+template <int W>
+__device__ inline bool gram_rounds_ij(double (*M)[2 * W + 1], double (*Z)[gram_zs<W>()], double tol2) {
     constexpr int W2 = 2 * W;
     const int lane = threadIdx.x & 31;
     const int r = lane < W2 ? lane : 0;  // lanes past 2W mirror row 0 (their results are dropped)
-    T A[W], J[W], ZA[W], ZJ[W];
+    double A[W], J[W], ZA[W], ZJ[W];
 #pragma unroll
     for (int j = 0; j < W; ++j) {
         A[j] = M[r][j];
@@ -428,20 +424,20 @@ __device__ inline bool gram_rounds_ij(T (*M)[2 * W + 1], T (*Z)[gram_zs<T, W>()]
     for (int mr = 0; mr < W; ++mr) {
         // own diagonal entry: column r sits at A[r] (r < W) or at J[(r - W - mr) mod W]
         const int jpos = r < W ? r : (r - W - mr + 2 * W) % W;
-        T d = T(0), g = T(0);
+        double d = 0.0, g = 0.0;
 #pragma unroll
         for (int j = 0; j < W; ++j) {
             if (j == jpos) d = r < W ? A[j] : J[j];
             if (j == r) g = J[j];  // M[k][q_k] for the pair's I lane k = r
         }
         const int partner = r < W ? W + (r + mr) % W : jpos;
-        const T dq = __shfl_sync(kFull, d, partner);
-        T c = T(1), sn = T(0), t = T(0);
+        const double dq = __shfl_sync(kFull, d, partner);
+        double c = 1.0, sn = 0.0, t = 0.0;
         int rot = 0;
         if (lane < W) rot = rot_params(d, dq, g, tol2, c, sn, t) ? 1 : 0;
         if (!rot) {
-            c = T(1);
-            sn = T(0);
+            c = 1.0;
+            sn = 0.0;
         }
         if (!__any_sync(kFull, rot != 0)) {
             // no pair rotates: only the shift of the J halves
@@ -450,20 +446,20 @@ __device__ inline bool gram_rounds_ij(T (*M)[2 * W + 1], T (*Z)[gram_zs<T, W>()]
             // columns (p, q) = (k, W + (k + mr) mod W) of this lane's rows of M and Z
 #pragma unroll
             for (int k = 0; k < W; ++k) {
-                const T ck = __shfl_sync(kFull, c, k), sk = __shfl_sync(kFull, sn, k);
-                const T x = A[k], y = J[k];
+                const double ck = __shfl_sync(kFull, c, k), sk = __shfl_sync(kFull, sn, k);
+                const double x = A[k], y = J[k];
                 A[k] = fma(ck, x, -sk * y);
                 J[k] = fma(sk, x, ck * y);
-                const T u = ZA[k], v = ZJ[k];
+                const double u = ZA[k], v = ZJ[k];
                 ZA[k] = fma(ck, u, -sk * v);
                 ZJ[k] = fma(sk, u, ck * v);
             }
             // rows p and q of M: lane p (r < W) and lane q exchange their rows
             const int pair = r < W ? r : jpos;
-            const T cp = __shfl_sync(kFull, c, pair), sp = __shfl_sync(kFull, sn, pair);
+            const double cp = __shfl_sync(kFull, c, pair), sp = __shfl_sync(kFull, sn, pair);
 #pragma unroll
             for (int k = 0; k < W; ++k) {
-                const T oa = __shfl_sync(kFull, A[k], partner), oj = __shfl_sync(kFull, J[k], partner);
+                const double oa = __shfl_sync(kFull, A[k], partner), oj = __shfl_sync(kFull, J[k], partner);
                 if (r < W) {
                     A[k] = fma(cp, A[k], -sp * oa);
                     J[k] = fma(cp, J[k], -sp * oj);
@@ -474,7 +470,7 @@ __device__ inline bool gram_rounds_ij(T (*M)[2 * W + 1], T (*Z)[gram_zs<T, W>()]
             }
         }
         // next mini-round: position k of the J halves moves to column W + (k + mr + 1) mod W
-        const T j0 = J[0], z0 = ZJ[0];
+        const double j0 = J[0], z0 = ZJ[0];
 #pragma unroll
         for (int k = 0; k < W - 1; ++k) {
             J[k] = J[k + 1];
@@ -497,23 +493,23 @@ __device__ inline bool gram_rounds_ij(T (*M)[2 * W + 1], T (*Z)[gram_zs<T, W>()]
     return any;
 }
 
-template <typename T, int W>
-__global__ void __launch_bounds__(kJGThreads, 1) jacobi_gram_kernel(int n, int npad, T* __restrict__ G,
-                                                                 unsigned* ctl, T tol, long long max_wait) {
+template <int W>
+__global__ void __launch_bounds__(kJGThreads, 1) jacobi_gram_kernel(int n, int npad, double* __restrict__ G,
+                                                                 unsigned* ctl, double tol, long long max_wait) {
     constexpr int W2 = 2 * W;
-    static_assert(W2 <= 16 && (W == 1 || W % 2 == 0), "block width: 1 or even, at most 8");
+    static_assert(W == 1 || W == 2 || W == 4, "block width");
     extern __shared__ __align__(16) unsigned char jsm_raw[];
-    T* cols = reinterpret_cast<T*>(jsm_raw);  // 2W columns, stride ld
-    __shared__ T M[W2][W2 + 1];
-    __shared__ __align__(16) T Z[W2][gram_zs<T, W>()];
-    __shared__ T s_c[W], s_s[W];
+    double* cols = reinterpret_cast<double*>(jsm_raw);  // 2W columns, stride ld
+    __shared__ double M[W2][W2 + 1];
+    __shared__ __align__(16) double Z[W2][gram_zs<W>()];
+    __shared__ double s_c[W], s_s[W];
     __shared__ int s_rot[W], s_pp[W], s_pq[W];
     __shared__ int s_any, s_rnd;
     if (vload(&ctl[kCtlNeed]) == 0u) {  // every column pair is orthogonal to tol already
         if (blockIdx.x == 0 && threadIdx.x == 0) ctl[kCtlSweeps] = 1u;
         return;
     }
-    const T tol2 = tol * tol;
+    const double tol2 = tol * tol;
     unsigned epoch = 0;
     const int ld = gram_ld(n);
     const int nblk = npad / W;
@@ -523,17 +519,17 @@ __global__ void __launch_bounds__(kJGThreads, 1) jacobi_gram_kernel(int n, int n
         for (int rnd = 0; rnd < nblk - 1; ++rnd) {
             const int bi = rr_player(blockIdx.x, rnd, nblk), bj = rr_player(nblk - 1 - blockIdx.x, rnd, nblk);
             for (int r = threadIdx.x; r < n; r += blockDim.x) {  // all 2W loads in flight at once
-                T v[W2];
+                double v[W2];
 #pragma unroll
                 for (int k = 0; k < W2; ++k) v[k] = G[(int64_t)(k < W ? bi * W + k : bj * W + (k - W)) * n + r];
 #pragma unroll
                 for (int k = 0; k < W2; ++k) cols[(size_t)k * ld + r] = v[k];
             }
             __syncthreads();
-            gram_form<T, W>(cols, n, ld, M);
+            gram_form<W>(cols, n, ld, M);
             __syncthreads();
             if (warp == 0) {
-                for (int e = lane; e < W2 * W2; e += 32) Z[e / W2][e % W2] = (e / W2 == e % W2) ? T(1) : T(0);
+                for (int e = lane; e < W2 * W2; e += 32) Z[e / W2][e % W2] = (e / W2 == e % W2) ? 1.0 : 0.0;
                 __syncwarp();
                 bool any = false;
                 if (rnd == 0) {
@@ -546,11 +542,11 @@ __global__ void __launch_bounds__(kJGThreads, 1) jacobi_gram_kernel(int n, int n
                             s_pq[lane] = blk * W + max(a, b2);
                         }
                         __syncwarp();
-                        any |= gram_mini_round<T, W>(M, Z, s_pp, s_pq, W, tol2, s_c, s_s, s_rot);
+                        any |= gram_mini_round<W>(M, Z, s_pp, s_pq, W, tol2, s_c, s_s, s_rot);
                         __syncwarp();
                     }
                 }
-                any |= gram_rounds_ij<T, W>(M, Z, tol2);  // rotations between I and J
+                any |= gram_rounds_ij<W>(M, Z, tol2);  // rotations between I and J
                 if (lane == 0) {
                     s_rnd = any ? 1 : 0;
                     if (any) s_any = 1;
@@ -560,13 +556,13 @@ __global__ void __launch_bounds__(kJGThreads, 1) jacobi_gram_kernel(int n, int n
             if (s_rnd) {
                 // C Z: thread r computes row r of the 2W rotated columns (2W independent sums)
                 for (int r = threadIdx.x; r < n; r += blockDim.x) {
-                    T acc[W2];
+                    double acc[W2];
 #pragma unroll
-                    for (int j = 0; j < W2; ++j) acc[j] = T(0);
+                    for (int j = 0; j < W2; ++j) acc[j] = 0.0;
 #pragma unroll 2
                     for (int k = 0; k < W2; ++k) {
-                        const T x = cols[(size_t)k * ld + r];
-                        gram_axpy_row<T, W2>(x, Z[k], acc);
+                        const double x = cols[(size_t)k * ld + r];
+                        gram_axpy_row<W2>(x, Z[k], acc);
                     }
 #pragma unroll
                     for (int j = 0; j < W2; ++j) G[(int64_t)(j < W ? bi * W + j : bj * W + (j - W)) * n + r] = acc[j];
@@ -1211,7 +1207,7 @@ __global__ void __launch_bounds__(128) jacobi_vfix_kernel(int n, const double* _
 static int block_width(int n) {
     if (n <= 48 || n > 1024) return 0;
     int w = 1;
-    while (w < 8 && (n + 2 * w - 1) / (2 * w) > 152) w *= 2;
+    while ((n + 2 * w - 1) / (2 * w) > 152) w *= 2;  // up to 4
     return w;
 }
 static int pad_to(int n, int w) { return (n + 2 * w - 1) / (2 * w) * (2 * w); }
@@ -1286,38 +1282,37 @@ static int jacobi_grid(const tsvd_handle* h, int npairs, int& block) {
     return nb;
 }
 
-// Cooperative launch of the block-Jacobi sweeps on G (n x npad, column-major) in T
-// with blocks of W columns.
-template <typename T, int W>
-static int launch_gram(tsvd_handle* h, int n, int npad, T* G, unsigned* ctl, T tol, cudaStream_t st) {
+// Cooperative launch of the block-Jacobi sweeps on G (n x npad, column-major) with blocks of W
+// columns.
+template <int W>
+static int launch_gram(tsvd_handle* h, int n, int npad, double* G, unsigned* ctl, double tol, cudaStream_t st) {
     const int nb = npad / W / 2;
-    const size_t smem = gram_smem<T, W>(n);
+    const size_t smem = gram_smem<W>(n);
     static thread_local int configured = -1;
     if (configured != h->device) {
-        TSVD_TRY_CUDA(cudaFuncSetAttribute(jacobi_gram_kernel<T, W>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)gram_smem<T, W>(1024)));
+        TSVD_TRY_CUDA(cudaFuncSetAttribute(jacobi_gram_kernel<W>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)gram_smem<W>(1024)));
         configured = h->device;
     }
     int per_sm = 0;
-    TSVD_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, jacobi_gram_kernel<T, W>, kJGThreads, smem));
+    TSVD_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, jacobi_gram_kernel<W>, kJGThreads, smem));
     if (per_sm * h->sm_count < nb) return TSVD_ERR_UNSUPPORTED;
     int nn = n, np = npad;
-    T t = tol;
+    double t = tol;
     long long mw = h->max_wait;
     void* args[] = {(void*)&nn, (void*)&np, (void*)&G, (void*)&ctl, (void*)&t, (void*)&mw};
     h->launches++;
-    TSVD_TRY_CUDA(cudaLaunchCooperativeKernel((const void*)jacobi_gram_kernel<T, W>, dim3(nb), dim3(kJGThreads), args,
+    TSVD_TRY_CUDA(cudaLaunchCooperativeKernel((const void*)jacobi_gram_kernel<W>, dim3(nb), dim3(kJGThreads), args,
                                               smem, st));
     return TSVD_OK;
 }
 
-template <typename T>
-static int run_block_sweeps(tsvd_handle* h, int n, int npad, int w, T* G, unsigned* ctl, T tol, cudaStream_t st) {
+static int run_block_sweeps(tsvd_handle* h, int n, int npad, int w, double* G, unsigned* ctl, double tol,
+                            cudaStream_t st) {
     switch (w) {
-        case 1: return launch_gram<T, 1>(h, n, npad, G, ctl, tol, st);
-        case 2: return launch_gram<T, 2>(h, n, npad, G, ctl, tol, st);
-        case 4: return launch_gram<T, 4>(h, n, npad, G, ctl, tol, st);
-        case 8: return launch_gram<T, 8>(h, n, npad, G, ctl, tol, st);
+        case 1: return launch_gram<1>(h, n, npad, G, ctl, tol, st);
+        case 2: return launch_gram<2>(h, n, npad, G, ctl, tol, st);
+        case 4: return launch_gram<4>(h, n, npad, G, ctl, tol, st);
         default: return TSVD_ERR_UNSUPPORTED;
     }
 }
@@ -1482,7 +1477,7 @@ int small_svd(tsvd_handle* h, int n, const double* B, int64_t ldb, double* Ubar,
             h->launches++;
             jacobi_init_kernel<<<ib, 256, 0, st>>>(n, npad, bf.Y, n, G, V);
             TSVD_TRY_CUDA(cudaGetLastError());
-            TSVD_TRY(run_block_sweeps<double>(h, n, npad, w, G, bf.ctl, tol, st));
+            TSVD_TRY(run_block_sweeps(h, n, npad, w, G, bf.ctl, tol, st));
         } else {
             h->launches++;
             jacobi_init_kernel<<<ib, 256, 0, st>>>(n, npad, B, ldb, G, V);

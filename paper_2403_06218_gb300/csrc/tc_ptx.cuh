@@ -61,18 +61,6 @@ __device__ inline bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* ab
     }
     return true;
 }
-// The same with a short sleep between polls, for roles whose waits are long
-// (frees issue slots for the warps that share the SM sub-partition).
-__device__ inline bool mbar_wait_sleep(uint32_t bar, uint32_t parity, volatile int* abort_flag,
-                                       long long max_wait = kMaxWait) {
-    const long long t0 = clock64();
-    while (!mbar_try_wait(bar, parity)) {
-        if (*abort_flag) return false;
-        if (clock64() - t0 > max_wait) return false;
-        __nanosleep(64);
-    }
-    return true;
-}
 // Bounded wait that ignores the abort flag (draining copies or products in flight).
 __device__ inline void mbar_drain(uint32_t bar, uint32_t parity, long long max_wait = kMaxWait) {
     const long long t0 = clock64();
@@ -178,12 +166,10 @@ using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t
 EncodeTiledFn encode_fn();
 
 // 3-D map over `planes` BF16 matrices stored [planes][rows][ld] (ld in elements,
-// a multiple of 8), K extent `cols`; box box_k (K) x box_rows x planes with a
-// swizzle of 2 box_k bytes (box_k = 64: 128-byte swizzle, 16: 32-byte swizzle).
-// Loads beyond `cols` or `rows` read zeros.
-// pstride: elements between planes (default rows x ld).
+// a multiple of 8), K extent `cols`; box 64 (K) x box_rows x planes with 128-byte
+// swizzle.  Loads beyond `cols` or `rows` read zeros.
 bool make_plane_map(CUtensorMap* map, const void* base, int64_t cols, int64_t rows, int64_t ld, int box_rows,
-                    int planes, int box_k = 64, int64_t pstride = -1);
+                    int planes);
 
 }  // namespace tcx
 }  // namespace tsvd

@@ -59,3 +59,21 @@ def test_clusters_leave_when_a_wait_runs_out(tsvd, n, ctas):
         s = tsvd.small_svd(B, nv=n // 2)[1].cpu().numpy()
     ref = np.linalg.svd(B.cpu().numpy(), compute_uv=False)
     assert np.abs(s - ref).max() < 1e-12 * ref[0] * n
+
+
+@pytest.mark.parametrize("n,decades", [(100, 8), (256, 8), (512, 8), (100, 12), (256, 12), (512, 12)])
+def test_spectra_over_many_decades(tsvd, n, decades):
+    # (the sweeps finish before their limit of 40; values are held to sigma_1, as everywhere)
+    import torch
+    rng = np.random.default_rng(n + decades)
+    q = [np.linalg.qr(rng.standard_normal((n, n)))[0] for _ in range(2)]
+    B = (q[0] * np.logspace(0, -decades, n)) @ q[1].T
+    nv = n // 3
+    U, s, V, sweeps = tsvd.small_svd(torch.from_numpy(B).cuda(), nv=nv)
+    U, s, V = (x.cpu().numpy() for x in (U, s, V))
+    tol = 4 * n ** 1.5 * EPS
+    assert 1 <= sweeps < 40
+    assert np.abs(s - np.linalg.svd(B, compute_uv=False)).max() <= tol
+    assert np.abs(B @ V[:, :nv] - U[:, :nv] * s[:nv]).max() <= tol
+    assert np.abs(B.T @ U[:, :nv] - V[:, :nv] * s[:nv]).max() <= tol
+    assert np.abs(V[:, :nv].T @ V[:, :nv] - np.eye(nv)).max() <= 1e-12
