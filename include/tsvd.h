@@ -486,9 +486,10 @@ int tsvd_update_gram_f32(tsvd_handle* h, int64_t q, int64_t s, int b, double alp
 /* CGS-QR, Alg. 3 (Sec. 3.1): QR of Y (q x r) by column blocks of width b
  * (the last one narrower if b does not divide r): Y <- Q in place, R (r x r,
  * ld = r) upper triangular assembled from [H_j; R_j].  1 <= b <= TSVD_MAX_BLOCK.
- * tsvd_cgs_qr_workspace includes the tensor-core scratch; without it the call needs
- * tsvd_orth_workspace_min(q, r, b') + 8 r b' (rounded up to 256) bytes, b' = min(b, r). */
+ * tsvd_cgs_qr_workspace includes the tensor-core scratch, tsvd_cgs_qr_workspace_min does
+ * not. */
 int tsvd_cgs_qr_workspace(int64_t q, int r, int b, size_t* bytes);
+int tsvd_cgs_qr_workspace_min(int64_t q, int r, int b, size_t* bytes);
 int tsvd_cgs_qr(tsvd_handle* h, int64_t q, int r, int b, double* Y, int64_t ldy, double* R,
                 uint64_t seed, int* replacements, int* breakdowns,
                 void* ws, size_t ws_bytes, void* stream);

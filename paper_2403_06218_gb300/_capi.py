@@ -130,6 +130,7 @@ SIGNATURES = [
     ("tsvd_mm_bf16x6", _I, [_P, _I64, _I64, _P, _I, _P, _I64, _P, _I64, _P, _SZ, _P]),
     ("tsvd_orth_workspace", _I, [_I64, _I64, _I, _PSZ]),
     ("tsvd_orth_workspace_min", _I, [_I64, _I64, _I, _PSZ]),
+    ("tsvd_cgs_qr_workspace_min", _I, [_I64, _I, _I, _PSZ]),
     ("tsvd_cgs_qr_workspace", _I, [_I64, _I, _I, _PSZ]),
     ("tsvd_cholqr2", _I, [_P, _I64, _I, _P, _I64, _P, C.c_uint64, _PI, _PI, _P, _SZ, _P]),
     ("tsvd_cgs_cqr2", _I, [_P, _I64, _I64, _I, _P, _I64, _P, _I64, _P, _P, C.c_uint64, _PI, _PI, _P, _SZ, _P]),

@@ -725,9 +725,7 @@ def cgs_qr(Y: torch.Tensor, b: int, seed: int = 0):
     R = torch.empty((r, r), dtype=torch.float64, device=dev)
     rep, bd = C.c_int(0), C.c_int(0)
     with torch.cuda.device(dev):
-        bw = min(b, r)
-        ws = _ws_or(_bytes("tsvd_cgs_qr_workspace", q, r, b),
-                    _bytes("tsvd_orth_workspace_min", q, r, bw) + (8 * r * bw + 255) // 256 * 256, dev)
+        ws = _ws_or(_bytes("tsvd_cgs_qr_workspace", q, r, b), _bytes("tsvd_cgs_qr_workspace_min", q, r, b), dev)
         capi.check(lib.tsvd_cgs_qr(handle(dev), q, r, b, Q.data_ptr(), Q.stride(0), R.data_ptr(), C.c_uint64(seed),
                                    C.byref(rep), C.byref(bd), ws.data_ptr(), ws.numel(), _stream_ptr(dev)),
                    "tsvd_cgs_qr")

@@ -532,7 +532,7 @@ int rsvd_run(tsvd_handle* h, const tsvd_matrix* A, int k, int p, int q, int bq, 
     void* ozws = ar.take<char>(ozb);
     if (!run) {
         const int64_t qmax = m > n ? m : n;
-        size_t t1 = orth_ws(h, qmax, ell > bq ? ell - bq : 0, bq) + align256(sizeof(double) * (size_t)ell * bq);
+        size_t t1 = orth_ws(h, qmax, ell, bq, true) + align256(sizeof(double) * (size_t)ell * bq);
         const size_t t2 = small_svd_ws(ell), t3 = final_tail_ws(h, m, n, k, kMixed);
         if (t2 > t1) t1 = t2;
         if (t3 > t1) t1 = t3;
@@ -709,8 +709,8 @@ int blanczos_run(tsvd_handle* h, const tsvd_matrix* A, int k, int b, int r, uint
         return TSVD_OK;
     };
     if (!run) {
-        size_t t1 = orth_ws(h, m, rb, b);
-        const size_t t2 = orth_ws(h, n, rb, b), t3 = small_svd_ws(rb), t4 = final_tail_ws(h, m, n, k, kMixed);
+        size_t t1 = orth_ws(h, m, rb, b, true);
+        const size_t t2 = orth_ws(h, n, rb, b, true), t3 = small_svd_ws(rb), t4 = final_tail_ws(h, m, n, k, kMixed);
         if (t2 > t1) t1 = t2;
         if (t3 > t1) t1 = t3;
         if (t4 > t1) t1 = t4;

@@ -811,6 +811,19 @@ size_t gemm_tn_ws_min(tsvd_handle* h, int64_t q, int64_t s, int64_t b, bool symm
     return align256(sizeof(double) * (size_t)p.slabs * (size_t)s * (size_t)b);
 }
 
+size_t gemm_tn_ws_bound(int64_t q, int64_t s, int64_t b, bool symmetric, int elem_bytes) {
+    const int64_t wave = elem_bytes == 4 ? kTnWaveF32 : kTnWave;
+    const int64_t max_slabs = std::max<int64_t>(1, std::min<int64_t>((q + 255) / 256, 65535));
+    int64_t most = 0;  // doubles
+    for (int64_t i = 1; i <= (s + kTnR - 1) / kTnR; ++i)
+        for (int64_t j = symmetric ? i : 1; j <= (symmetric ? i : (b + kTnR - 1) / kTnR); ++j) {
+            const int64_t regions = symmetric ? i * (i + 1) / 2 : i * j;
+            const int64_t slabs = std::max<int64_t>(1, std::min(wave / regions, max_slabs));
+            most = std::max(most, slabs * std::min(s, i * kTnR) * std::min(b, j * kTnR));
+        }
+    return std::max(align256(sizeof(double) * (size_t)most), elem_bytes == 8 ? kTnExtra : 0);
+}
+
 template <typename TI, typename TC>
 cudaError_t gemm_tn(tsvd_handle* h, int64_t q, int64_t s, int64_t b, const TI* X, int64_t ldx, const TI* Z,
                     int64_t ldz, TC* C, int64_t ldc, bool symmetric, double* partial, cudaStream_t st,

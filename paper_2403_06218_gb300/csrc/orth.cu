@@ -69,8 +69,9 @@ struct OrthWs {
     double *fcol64, *fh, *fhacc, *fc, *fcacc, *fnrm;
 };
 
+// upto: the partial sums for every block before it too (sizing).
 template <typename T>
-OrthWs<T> carve(tsvd_handle* h, Arena& ar, int64_t q, int64_t s, int b) {
+OrthWs<T> carve(tsvd_handle* h, Arena& ar, int64_t q, int64_t s, int b, bool upto = false) {
     OrthWs<T> w{};
     const size_t bb = (size_t)b * b;
     w.W = ar.take<double>(bb);
@@ -91,6 +92,10 @@ OrthWs<T> carve(tsvd_handle* h, Arena& ar, int64_t q, int64_t s, int b) {
     }
     for (int j = 1; j <= b; ++j) upd(gemm_tn_ws(h, q, j, 1, false, eb));
     upd(gemm_tn_ws(h, q, 1, 1, true, eb));
+    if (upto) {
+        upd(gemm_tn_ws_bound(q, b, b, true, eb));
+        upd(gemm_tn_ws_bound(q, s > b ? s : b, b, false, eb));
+    }
     if (eb == 4) upd(update_gram_ws(q, b));
     w.partial = ar.take<double>(pbytes / sizeof(double) + 1);
     w.save = ar.take<T>((size_t)q * b);
@@ -254,10 +259,10 @@ int read_status(cudaStream_t st, const int* d_status, int* h_status) {
 
 // Covers both block types: FP32 blocks take half the copies but a wider split-K
 // plan and the fused update + Gram partials.
-size_t orth_ws(tsvd_handle* h, int64_t q, int64_t s, int b) {
+size_t orth_ws(tsvd_handle* h, int64_t q, int64_t s, int b, bool upto) {
     Arena a64, a32;
-    carve<double>(h, a64, q, s, b);
-    carve<float>(h, a32, q, s, b);
+    carve<double>(h, a64, q, s, b, upto);
+    carve<float>(h, a32, q, s, b, upto);
     return a64.off > a32.off ? a64.off : a32.off;
 }
 

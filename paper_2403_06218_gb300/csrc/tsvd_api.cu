@@ -643,11 +643,20 @@ int tsvd_update_gram_f32(tsvd_handle* h, int64_t q, int64_t s, int b, double alp
     return TSVD_OK;
 }
 
-int tsvd_cgs_qr_workspace(int64_t q, int r, int b, size_t* bytes) {
+int tsvd_cgs_qr_workspace_min(int64_t q, int r, int b, size_t* bytes) {
     if (!bytes || r < 1 || b < 1 || q < r) return TSVD_ERR_INVALID_ARG;
     const int bw = b < r ? b : r;
-    TSVD_TRY(tsvd_orth_workspace_min(q, r, bw, bytes));
-    *bytes += align256(sizeof(double) * (size_t)r * bw) + oz_standalone_ws(q, r - bw, bw, false);
+    tsvd_handle hh = sizing_handle();
+    // all blocks against all columns, and the coefficients of one
+    *bytes = align256(sizeof(int) * kStCount) + orth_ws(&hh, q, r, bw, true) +
+             2 * align256(sizeof(double) * (size_t)r * bw);
+    return TSVD_OK;
+}
+
+int tsvd_cgs_qr_workspace(int64_t q, int r, int b, size_t* bytes) {
+    TSVD_TRY(tsvd_cgs_qr_workspace_min(q, r, b, bytes));
+    const int bw = b < r ? b : r;
+    *bytes += oz_standalone_ws(q, r - bw, bw, false);
     return TSVD_OK;
 }
 

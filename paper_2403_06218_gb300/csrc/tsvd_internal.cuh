@@ -255,6 +255,10 @@ size_t gemm_tn_ws(tsvd_handle* h, int64_t q, int64_t s, int64_t b, bool symmetri
 // The least that gemm_tn runs with (partial_bytes); with gemm_tn_ws it may split a small product
 // over more CTAs.  fp64_pipe: never on the tensor cores.
 size_t gemm_tn_ws_min(tsvd_handle* h, int64_t q, int64_t s, int64_t b, bool symmetric, int elem_bytes = 8);
+// The most that a product with q' <= q, s' <= s and b' <= b needs.  (gemm_tn_ws is not monotone:
+// fewer regions of outputs are cut into more slabs, so 160 columns can take more partial sums
+// than 512.)
+size_t gemm_tn_ws_bound(int64_t q, int64_t s, int64_t b, bool symmetric, int elem_bytes);
 // Register-tiled FP32 kernels (k_f32.cu) behind gemm_tn<float, *> and gemm_nn<float, *, *>.
 template <typename TW>
 cudaError_t launch_gemm_tn_f32(dim3 grid, cudaStream_t st, int64_t q, int64_t s, int64_t b, const float* X,
@@ -544,8 +548,9 @@ struct OrthCtx {
 // handle, in place (a no-op without one).  TSVD_ERR_COMM when the exchange fails.
 int part_sum(tsvd_handle* h, double* d, int64_t rows, int64_t cols, int64_t ld, cudaStream_t st);
 
-// Workspace of one orthogonalisation (sized for double blocks, which covers float).
-size_t orth_ws(tsvd_handle* h, int64_t q, int64_t s, int b);
+// Workspace of one orthogonalisation (sized for double blocks, which covers float); upto: of
+// every one against at most s columns, of blocks of at most b.
+size_t orth_ws(tsvd_handle* h, int64_t q, int64_t s, int b, bool upto = false);
 // Y (q x b) <- Q; R (b x b, ld ldr, trans: write R^T); H (s x b, ld b) optional.
 // T = double or float (storage of P and Y); H and R are FP64.
 template <typename T>

@@ -28,7 +28,7 @@ def test_least_size_holds_no_copy_of_the_basis(tsvd, q, s, b):
     assert least <= 8 * q * (b + 2) + 8 * 152 * 16 * 1024 + (64 << 10) + 8 * (8 * b * b + 4 * (s + b) * b)
     assert least <= full <= least + (4 << 30)
     r = s + b
-    qr = _query(lib, "tsvd_cgs_qr_workspace", q, r, b) - _query(lib, "tsvd_orth_workspace_min", q, r, b)
+    qr = _query(lib, "tsvd_cgs_qr_workspace", q, r, b) - _query(lib, "tsvd_cgs_qr_workspace_min", q, r, b)
     # no kept planes: one layout of 8 two-byte digits at a time, and the block's
     assert qr <= 16 * (q + 16) * (r + b + 32) + 64 * 2 ** 20
 
@@ -69,10 +69,10 @@ def test_least_size_is_accepted(tsvd, q, s, b, f32):
 @pytest.mark.parametrize("r,b", [(300, 64), (160, 128), (129, 128), (130, 33), (64, 100)])
 def test_cgs_qr_with_and_without_its_scratch(tsvd, r, b):
     import torch
-    q, bw, lib = 20_000, min(b, r), tsvd.load()
+    q, lib = 20_000, tsvd.load()
     Y = torch.randn(q, r, generator=torch.Generator(device="cuda").manual_seed(r), dtype=torch.float64, device="cuda")
     full = _query(lib, "tsvd_cgs_qr_workspace", q, r, b)
-    least = _query(lib, "tsvd_orth_workspace_min", q, r, bw) + (8 * r * bw + 255) // 256 * 256
+    least = _query(lib, "tsvd_cgs_qr_workspace_min", q, r, b)
     for nbytes in (least, full):
         Q, R = Y.clone(), torch.empty(r, r, dtype=torch.float64, device="cuda")
         ws = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
@@ -82,3 +82,19 @@ def test_cgs_qr_with_and_without_its_scratch(tsvd, r, b):
         assert rc == _capi.TSVD_OK and bd.value == 0
         assert float((Q @ R - Y).norm() / Y.norm()) <= 8 * r * EPS
         assert float((Q.t() @ Q - torch.eye(r, device="cuda").double()).abs().max()) <= 100 * EPS
+
+
+def test_blocks_sized_for_the_last_one_hold_the_earlier_ones(tsvd):
+    # more rows, columns or width never take less, and the size for a basis of r columns covers
+    # every block of its orthogonalisation
+    lib = tsvd.load()
+    least = lambda *a: _query(lib, "tsvd_cgs_qr_workspace_min", *a)  # noqa: E731
+    for q in (5_000, 60_000, 200_000, 2_000_000):
+        for b in (16, 32, 33, 64, 100, 128):
+            row = [least(q, r, b) for r in range(b, 1_025, 16)]
+            assert row == sorted(row), (q, b)
+            for s in range(0, 1_024 - b, b):
+                assert _query(lib, "tsvd_orth_workspace_min", q, s, b) <= row[-1], (q, s, b)
+    for r, b in ((64, 64), (160, 32), (512, 64)):
+        row = [least(q, r, b) for q in range(1_000, 400_000, 7_001)]
+        assert row == sorted(row), (r, b)
