@@ -6,15 +6,17 @@
 // X row the row touches (float4 / double2), so G = w / (16 / sizeof(T)) lanes
 // cover a block of w columns and narrow blocks put several rows in a warp.  The
 // gathers (nnz w sizeof(T) bytes, from L2 for a block that fits there) bound the
-// kernel, not the compulsory HBM bytes: measured ~13 TB/s of gathered data on
-// GB300.  FP64 is also close to the FP64 pipe's rate (2 DFMA/clk/SM).  Every y_ij
-// is accumulated in CSR order with FMA, so the result is deterministic.
+// kernel, not the compulsory HBM bytes: 8 TB/s of gathered data and more on
+// GB300 where X stays in L2 (uniform 100,000 x 100,000, 10 entries a row, FP32, 64 columns: 256 MB
+// gathered in 31 us = 8.3 TB/s; power-law 2M x 1M: 25.5 GB in 3.3 ms).  FP64 is also close to the
+// FP64 pipe's rate (2 DFMA/clk/SM).  Every y_ij is accumulated in CSR order with FMA, so the
+// result is deterministic.
 //
 // Long rows (power-law degrees; CSR(A^T) of a matrix with popular columns holds
 // rows of up to ~10^6 entries) would leave one warp working long after the rest.
 // A plan built once per matrix cuts every row longer than kSpmmChunk entries into
-// chunks of kSpmmChunk: one warp per chunk writes a partial row, and a second
-// kernel adds each row's partials in chunk order (still deterministic).
+// chunks of kSpmmChunk: one sub-warp per chunk, in the first blocks of the rows' launch, writes a
+// partial row, and a second kernel adds each row's partials in chunk order (still deterministic).
 #include <climits>
 
 #include "tsvd_internal.cuh"
