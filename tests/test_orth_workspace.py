@@ -98,3 +98,18 @@ def test_blocks_sized_for_the_last_one_hold_the_earlier_ones(tsvd):
     for r, b in ((64, 64), (160, 32), (512, 64)):
         row = [least(q, r, b) for q in range(1_000, 400_000, 7_001)]
         assert row == sorted(row), (r, b)
+
+
+def test_python_call_takes_the_least_size_where_the_full_one_does_not_fit(monkeypatch):
+    import torch
+
+    from paper_2403_06218_gb300 import api
+
+    def ws(nbytes, dev):
+        if nbytes > 1_000:
+            raise torch.cuda.OutOfMemoryError("no room")
+        return nbytes
+    monkeypatch.setattr(api, "_ws", ws)
+    assert api._ws_or(5_000, 900, None) == 900 and api._ws_or(800, 700, None) == 800
+    with pytest.raises(torch.cuda.OutOfMemoryError):
+        api._ws_or(5_000, 2_000, None)
